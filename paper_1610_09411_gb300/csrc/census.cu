@@ -17,6 +17,7 @@
 //   Thm 13 5-cycles ............................ k_cycles5
 //   Thm 3 + App. B assembly .................... k_assemble
 #include "common.cuh"
+#include "core.cuh"
 #include "internal.h"
 
 #include <algorithm>
@@ -960,17 +961,23 @@ static constexpr int64_t PH_LARGE_W = PH_LARGE_SLOTS / 2;
 
 // w_i of every vertex with degree >= 2, appended to the list of its class
 // (roughly by decreasing rank, so the heaviest items come first)
-// Also the largest common-neighbour list (triangles on one edge) into cnts[7].
+// Also the largest common-neighbour list (triangles on one edge) into cnts[7]
+// and twice the number of diamonds, sum over slots of C(T, 2), into cnts[8].
 __global__ void k_pair_classify(DevGraph g, const uint32_t* T, int32_t* lists, unsigned long long* cnts,
                                 long long w_small, long long w_large, Owner own) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  unsigned long long dia = 0;
   for (int64_t k = warp; k < g.n; k += nwarps) {
     int64_t i = g.n - 1 - k;
     int64_t b0 = g.R[i], e0 = g.R[i + 1];
     unsigned tmax = 0;
-    for (int64_t p = b0 + lane; p < e0; p += 32) tmax = max(tmax, T[p]);
+    for (int64_t p = b0 + lane; p < e0; p += 32) {
+      const uint32_t t = T[p];
+      tmax = max(tmax, t);
+      dia += t < 2 ? 0 : (unsigned long long)t * (t - 1) / 2;
+    }
     tmax = __reduce_max_sync(0xffffffffu, tmax);
     if (lane == 0 && tmax) atomicMax(&cnts[7], (unsigned long long)tmax);
     if (e0 - b0 < 2 || !own.owns(i)) continue;
@@ -985,6 +992,8 @@ __global__ void k_pair_classify(DevGraph g, const uint32_t* T, int32_t* lists, u
       if (cls == 2) atomicMax(&cnts[6], w);    // the largest item, for the task buffers
     }
   }
+  dia = warp_sum_u64(dia);
+  if (lane == 0 && dia) atomicAdd(&cnts[8], dia);
 }
 
 // Open addressing in shared memory (keys -1 = empty), linear probing.  At most
@@ -1163,17 +1172,20 @@ __device__ __forceinline__ u128 pair_run_tasks(const DevGraph& g, const PairTask
 // k-th y; the whole warp then walks each y's common-neighbour list).
 template <class Get>
 __device__ __forceinline__ u128 pair_diamond_chunk(const DevGraph& g, const TriLists& tl3, const uint32_t* T,
-                                                   int64_t i, int64_t xb, int64_t r0, int64_t r1, Get&& get) {
+                                                   const CoreView& cv, int64_t i, int64_t xb, int64_t r0, int64_t r1,
+                                                   Get&& get) {
   const int lane = threadIdx.x & 31;
   const int32_t i32 = (int32_t)i;
   Sum128 n17;
   int64_t r = r0 + lane;
   int64_t vb_l = 0;
   uint32_t len_l = 0;
+  bool cut = false;                             // only the tips below the core: core.cu counts the others
   if (r < r1) {
     int64_t sxy = xb + tl3.P[r];                // slot (x -> y)
+    cut = i >= cv.h0 && g.C[sxy] >= cv.h0;
+    len_l = cut ? cv.low[sxy] : T[sxy];
     vb_l = tl3.off[sxy];
-    len_l = T[sxy];
   }
   // short lists: each lane walks its own, a few entries in flight, until it
   // passes i (no entry loaded beyond the next few); long ones: the whole warp
@@ -1202,8 +1214,8 @@ __device__ __forceinline__ u128 pair_diamond_chunk(const DevGraph& g, const TriL
   // one list at a time, in blocks of 32 x PAIR_ILP entries and then 4, 2, 1
   // and a last partial group of 32, so that no slot past the prefix is issued.
   const bool lng = r < r1 && len_l > PAIR_SHORT;
-  int pre_l = 0;
-  if (lng) {
+  int pre_l = lng && cut ? (int)len_l : 0;
+  if (lng && !cut) {
     const int32_t* L = tl3.U + vb_l;
     int lo = 0, hi = (int)len_l;
     while (lo < hi) {
@@ -1259,23 +1271,37 @@ __device__ __forceinline__ void pair_tri_range(const DevGraph& g, const TriLists
 }
 
 template <class Get>
-__device__ __forceinline__ u128 pair_diamonds(const DevGraph& g, const TriLists& tl3, const uint32_t* T, int64_t i,
-                                              int64_t b0, int64_t e0, int64_t gw, int64_t gnw, Get&& get) {
+__device__ __forceinline__ u128 pair_diamonds(const DevGraph& g, const TriLists& tl3, const uint32_t* T,
+                                              const CoreView& cv, int64_t i, int64_t b0, int64_t e0, int64_t gw,
+                                              int64_t gnw, Get&& get) {
   u128 n17 = 0;
+  if (cv.h0 <= 0) return n17;                   // every vertex is in the core
   for (int64_t p = b0 + gw; p < e0; p += gnw) {
     if (T[p] == 0) continue;
     int64_t xb, r0, r1;
     pair_tri_range(g, tl3, T, p, xb, r0, r1);
-    for (int64_t rb = r0; rb < r1; rb += 32) n17 += pair_diamond_chunk(g, tl3, T, i, xb, rb, min(rb + 32, r1), get);
+    for (int64_t rb = r0; rb < r1; rb += 32) n17 += pair_diamond_chunk(g, tl3, T, cv, i, xb, rb, min(rb + 32, r1), get);
   }
   return n17;
+}
+
+// W(i, j) of a core item for the core vertices j below it in the same graph
+// (thread tid of nthreads).  Entries whose W is zero may hold anything: no
+// diamond reads them.
+template <class Get>
+__device__ __forceinline__ void core_store_row(const CoreView& cv, int64_t i, int64_t tid, int64_t nthreads, Get&& get) {
+  if (i < cv.h0) return;
+  const int64_t t = i - cv.h0, row = cv.rowb[t];
+  const int32_t cnt = cv.li[t];
+  const int32_t* hl = cv.hl ? cv.hl + cv.hb[t] : nullptr;
+  for (int64_t k = tid; k < cnt; k += nthreads) cv.put(row + k, get(hl ? hl[k] : (int32_t)(cv.h0 + k)));
 }
 
 // Light and medium items: one CTA per item, W(i, .) in a shared-memory hash
 // table (SLOTS keys and counts) that is cleared after every item.
 template <int SLOTS>
 __global__ void k_pairs_hash(DevGraph g, const int32_t* items, int64_t nitems, unsigned long long* qctr,
-                             TriLists tl3, const uint32_t* T, AccSet acc, unsigned* status) {
+                             TriLists tl3, const uint32_t* T, CoreView cv, AccSet acc, unsigned* status) {
   extern __shared__ int32_t ph_smem[];
   int32_t* hk = ph_smem;
   uint32_t* hv = (uint32_t*)(ph_smem + SLOTS);
@@ -1297,13 +1323,17 @@ __global__ void k_pairs_hash(DevGraph g, const int32_t* items, int64_t nitems, u
       return atomicAdd(&hv[sl], 1u);
     }, [](int64_t, int64_t) { return false; });
     __syncthreads();
-    u128 n17 = pair_diamonds(g, tl3, T, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t {
+    u128 n17 = pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t {
       int sl = ph_find<SLOTS>(hk, j);
       if (sl < 0) { set_err(status, DEVERR_SCRATCH); return 2u; }
       return hv[sl];
     });
     __syncthreads();
-    for (int t = threadIdx.x; t < SLOTS; t += blockDim.x) { hk[t] = -1; hv[t] = 0u; }
+    for (int t = threadIdx.x; t < SLOTS; t += blockDim.x) {
+      if (i >= cv.h0 && hk[t] >= cv.h0) cv.put(cv.rowb[i - cv.h0] + cv.li[hk[t] - cv.h0], hv[t]);
+      hk[t] = -1;
+      hv[t] = 0u;
+    }
     la.v[0] += n13;
     la.v[1] += n17;
     block_item_flush(la, ids, acc, i, sh);
@@ -1330,7 +1360,7 @@ template <bool BIG, int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB) k_pairs_grp(DevGraph g, const int32_t* items,
                                                                          int64_t nitems, unsigned long long* qctr,
                                                                          TagScratch ts, TriLists tl3,
-                                                                         const uint32_t* T, AccSet acc,
+                                                                         const uint32_t* T, CoreView cv, AccSet acc,
                                                                          PairTasks pt, int64_t wlo, int win_words) {
   extern __shared__ uint32_t win[];
   __shared__ u128 sh[32];
@@ -1375,13 +1405,15 @@ __global__ void __launch_bounds__(THREADS, MINB) k_pairs_grp(DevGraph g, const i
     const unsigned long long nt1 = __ldcg(&pt.n[grp]);
     n13 += pair_run_tasks(g, pt, grp, nt1, gw, gnw, inc);
     cluster_barrier();
-    u128 n17 = pair_diamonds(g, tl3, T, i, b0, e0, gw, gnw, [&](int32_t j) -> uint32_t {
+    auto get = [&](int32_t j) -> uint32_t {
       if (j >= wlo && j < whi) {
         const int64_t k = j - wlo;
         return (win[k >> 1] >> (16u * (unsigned)(k & 1))) & 0xffffu;
       }
       return w.get_l2(j);
-    });
+    };
+    u128 n17 = pair_diamonds(g, tl3, T, cv, i, b0, e0, gw, gnw, get);
+    core_store_row(cv, i, (int64_t)crank * blockDim.x + threadIdx.x, (int64_t)csize * blockDim.x, get);
     la.v[0] += n13;
     la.v[1] += n17;
     block_item_flush(la, ids, acc, i, sh);
@@ -1510,7 +1542,7 @@ __device__ __forceinline__ u128 pair_wedges_win(const DevGraph& g, longlong2* cu
 template <bool BIG>
 __global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t* items, int64_t nitems,
                                                         unsigned long long* qctr, PairWin pw, TriLists tl3,
-                                                        const uint32_t* T, AccSet acc, PairTasks pt,
+                                                        const uint32_t* T, CoreView cv, AccSet acc, PairTasks pt,
                                                         unsigned* status) {
   extern __shared__ uint32_t win[];
   __shared__ u128 sh[32];
@@ -1595,7 +1627,7 @@ __global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t
       }
     }
     const uint32_t lo_top32 = (uint32_t)(pw.jbig - (ktop + 1) * S), S32 = (uint32_t)S;
-    u128 n17 = pair_diamonds(g, tl3, T, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t {
+    auto get = [&](int32_t j) -> uint32_t {
       // j < min(i, jbig) lies in the top window exactly when j - lo_top (mod 2^32) is below S
       const uint32_t q = (uint32_t)j - lo_top32;
       if (q < S32) return (win[q >> 1] >> ((q & 1u) << 4)) & 0xffffu;
@@ -1605,7 +1637,9 @@ __global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t
       }
       const uint32_t t = (uint32_t)j + (uint32_t)par;
       return (__ldcg(&g16[t >> 1]) >> ((t & 1u) << 4)) & 0xffffu;
-    });
+    };
+    u128 n17 = pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, get);
+    core_store_row(cv, i, threadIdx.x, blockDim.x, get);
     la.v[0] += n13;
     la.v[1] += n17;
     __syncthreads();                            // the diamond reads of the window are done
@@ -1628,50 +1662,72 @@ __global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t
 // ============================================================================
 static constexpr int WHEEL_WARP_MAX = 1024;     // centres up to this degree: warp items
 
-// Walks, for one centre c and one position pu, every k in N(c) cap N(u) below
-// u (a prefix of the list of slot c -> u) and every v in N(c) cap N(k) below u
-// (a prefix of the list of slot c -> k), calling visit(pv) once per pair with
-// pv the position of v in row c.  A warp takes the k's a0, a0 + astep, ...:
-// it fetches 32 of them at a time (lane l the l-th) and scans each v list with
-// WHEEL_ILP independent loads in flight per lane.
+// Core centres (core.cu) leave the 4-cycles whose low vertices (below h0; the
+// positions below pc) are none, one, or two opposite ones to the contraction.
+// What is left has two adjacent low vertices.  For u low, everything below u is
+// low and the rule above applies unchanged.  For u in the core, v is low and
+// with wL (wH) the number of k that are low (in the core and below u),
+// wL wH + C(wL, 2): the low k are counted first, then the core k read the counts.
+//
+// One of these walks for one u: for the k at entries [a0, a1) of the list Lu of
+// slot c -> u that are below kmax (the warp takes a0 + w, a0 + w + step, ...,
+// 32 at a time, lane l the l-th), every v below vmax in the list of slot
+// c -> k: visit(pv).  LEN gives the entries of that list that can lie below
+// vmax.  Lists of up to WHEEL_SHORT entries are walked by one lane each, longer
+// ones by the warp, with WHEEL_ILP independent loads in flight per lane.
 #ifndef ESC_WHEEL_ILP
 #define ESC_WHEEL_ILP 8
 #endif
 static constexpr int WHEEL_ILP = ESC_WHEEL_ILP;
+static constexpr uint32_t WHEEL_SHORT = 32;
 
 template <class Visit>
-__device__ __forceinline__ void wheel_links(const TriLists& tl3, const uint32_t* T, int64_t base, const int32_t* Lu,
-                                            uint32_t lenu, int pu, uint32_t a0, uint32_t astep, Visit&& visit) {
+__device__ __forceinline__ void wheel_walk(const TriLists& tl3, const uint32_t* LEN, int64_t base, const int32_t* Lu,
+                                           uint32_t a0, uint32_t a1, int kmax, int vmax, uint32_t w, uint32_t step,
+                                           Visit&& visit) {
   const int lane = threadIdx.x & 31;
-  for (uint32_t ab = a0; ab < lenu; ab += 32 * astep) {
-    uint32_t a = ab + lane * astep;
+  for (uint32_t ab = a0 + w; ab < a1; ab += 32 * step) {
+    const uint32_t a = ab + lane * step;
     const int32_t* Lk_l = tl3.P;
     uint32_t lk_l = 0;
-    bool live = a < lenu, in = false;
+    const bool live = a < a1;
+    bool in = false;
     if (live) {
-      int32_t pk = Lu[a];
-      if (pk < pu) {
+      const int32_t pk = Lu[a];
+      if (pk < kmax) {
         in = true;
         Lk_l = tl3.P + tl3.offp[base + pk];
-        lk_l = T[base + pk];
+        lk_l = LEN[base + pk];
       }
     }
-    unsigned m = __ballot_sync(0xffffffffu, in);
-    bool done = __any_sync(0xffffffffu, live && !in);   // the k list is sorted: later rounds are above u
+    const bool done = __any_sync(0xffffffffu, live && !in);   // the k list is sorted: later rounds are above kmax
+    if (lk_l <= WHEEL_SHORT) {
+      for (uint32_t t = 0; t < lk_l; t += 4) {
+        int32_t pv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) pv[u] = t + u < lk_l ? Lk_l[t + u] : 0x7fffffff;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (pv[u] < vmax) visit(pv[u]);
+        if (pv[3] >= vmax) break;
+      }
+      lk_l = 0;
+    }
+    unsigned m = __ballot_sync(0xffffffffu, lk_l > 0);
     while (m) {
-      int k = __ffs(m) - 1;
+      const int k = __ffs(m) - 1;
       m &= m - 1;
       const int32_t* Lk = reinterpret_cast<const int32_t*>(
           __shfl_sync(0xffffffffu, reinterpret_cast<uintptr_t>(Lk_l), k));
-      uint32_t lk = __shfl_sync(0xffffffffu, lk_l, k);
+      const uint32_t lk = __shfl_sync(0xffffffffu, lk_l, k);
       for (uint32_t tb = 0; tb < lk; tb += 32 * WHEEL_ILP) {
         int32_t pv[WHEEL_ILP];
         bool past = false;
 #pragma unroll
         for (int u = 0; u < WHEEL_ILP; ++u) {
-          uint32_t t = tb + lane + 32 * u;
+          const uint32_t t = tb + lane + 32 * u;
           pv[u] = t < lk ? Lk[t] : 0x7fffffff;
-          if (pv[u] >= pu) { pv[u] = -1; past = true; }
+          if (pv[u] >= vmax) { pv[u] = -1; past = true; }
         }
 #pragma unroll
         for (int u = 0; u < WHEEL_ILP; ++u)
@@ -1702,7 +1758,7 @@ __global__ void k_wheel_warp_counts(DevGraph g, int64_t c0, int64_t* item_cnt, O
 
 __global__ void __launch_bounds__(256, 6) k_wheels_warp(DevGraph g, int64_t c0, const int64_t* item_off,
                                                         unsigned long long* qctr, TriLists tl3, const uint32_t* T,
-                                                        AccSet acc) {
+                                                        CoreView cv, AccSet acc) {
   __shared__ u128 sh[32];
   __shared__ uint32_t scr_all[8][WHEEL_WARP_MAX];
   int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
@@ -1730,10 +1786,14 @@ __global__ void __launch_bounds__(256, 6) k_wheels_warp(DevGraph g, int64_t c0, 
     int d = (int)(g.R[c + 1] - base);
     int u0 = (int)(it - item_off[lo]) * WHEEL_WBLK;
     int u1 = min(d, u0 + WHEEL_WBLK);
+    const int pc = c >= cv.h0 ? d - cv.dh[c - cv.h0] : d;   // positions from pc on are in the core
     u128 n18 = 0;
     for (int pu = u0; pu < u1; ++pu) {
       uint32_t lenu = T[base + pu];
       if (lenu < 2) continue;
+      const bool top = pu >= pc;
+      const uint32_t lowu = top ? cv.low[base + pu] : lenu;
+      if (lowu == 0) continue;
       if (++tag == 0x10000u) {                           // tags exhausted: start over from zeroed counters
         __syncwarp();
         for (int i = lane; i < WHEEL_WARP_MAX; i += 32) scr[i] = 0;
@@ -1743,11 +1803,18 @@ __global__ void __launch_bounds__(256, 6) k_wheels_warp(DevGraph g, int64_t c0, 
       const int32_t* Lu = tl3.P + tl3.offp[base + pu];
       unsigned long long part = 0;
       const uint32_t t16 = tag << 16;
-      wheel_links(tl3, T, base, Lu, lenu, pu, 0u, 1u, [&](int32_t pv) {
+      wheel_walk(tl3, T, base, Lu, 0u, lowu, pu, min(pu, pc), 0u, 1u, [&](int32_t pv) {
         atomicMax(&scr[pv], t16);               // an older u's entry becomes a zero count of this one
         part += atomicAdd(&scr[pv], 1u) & 0xffffu;
       });
       __syncwarp();                             // this u's increments before the next u's tag
+      if (top && lowu < lenu) {
+        wheel_walk(tl3, cv.low, base, Lu, lowu, lenu, pu, pc, 0u, 1u, [&](int32_t pv) {
+          const uint32_t v = scr[pv];
+          if ((v & 0xffff0000u) == t16) part += v & 0xffffu;
+        });
+        __syncwarp();
+      }
       n18 += part;
     }
     la.v[0] += n18;
@@ -1757,82 +1824,111 @@ __global__ void __launch_bounds__(256, 6) k_wheels_warp(DevGraph g, int64_t c0, 
 }
 
 // Centres above WHEEL_WARP_MAX: work items (centre, block of WHEEL_CHUNK
-// positions u); counters in shared memory when the degree fits, otherwise in a
-// per-CTA global region.
-static constexpr int WHEEL_CHUNK = 64;
+// positions u) taken by a CTA of WHEEL_THREADS threads (one per SM: its shared
+// memory holds the counters).  The CTA's warps form groups that take different
+// u's, as many groups as counter arrays of pc positions fit: a core centre
+// leaves little work per u, so one warp per u (pc up to about 1,700) or four
+// keep more u's in flight than the whole CTA on one.
+static constexpr int WHEEL_CHUNK = 128;
+static constexpr int WHEEL_THREADS = 1024;
 
 // Counters are tagged with the u they count for, (tag << 16) | count in the
 // 32-bit shared-memory words and (tag << 32) | count in the 64-bit global ones
 // (counts there can pass 2^16); before each increment an atomicMax with the
 // current tag turns an older entry into a zero count, so no clearing pass
-// walks the lists a second time.  A CTA's tags grow with the u's it takes.
+// walks the lists a second time.  The tags of a CTA grow with its items and
+// within an item with u, whatever array an item's groups use.
 // win16: every count of the sweep stays below 2^16 (the largest common-
-// neighbour list is shorter), so large centres keep a shared-memory window.
-__global__ void k_wheels_cta(DevGraph g, int64_t c0, const int64_t* item_off, int64_t nitems,
-                             unsigned long long* qctr, TriLists tl3, const uint32_t* T, unsigned long long* gscr,
-                             int64_t gscr_stride, int smem_cap, AccSet acc, bool win16) {
+// neighbour list is shorter), so centres with more positions than the shared
+// memory holds keep a shared-memory window over the last smem_cap of them (the
+// highest ranks, where the common neighbours concentrate) and count the others
+// in global memory.
+__device__ __forceinline__ void wheel_group_sync(int gs, int grp) {
+  if (gs == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gs * 32) : "memory");
+}
+
+__global__ void __launch_bounds__(WHEEL_THREADS, 1) k_wheels_cta(DevGraph g, int64_t c0, const int64_t* item_off,
+                                                                int64_t nitems, unsigned long long* qctr, TriLists tl3,
+                                                                const uint32_t* T, CoreView cv,
+                                                                unsigned long long* gscr, int64_t gscr_stride,
+                                                                int smem_cap, AccSet acc, bool win16) {
   extern __shared__ uint32_t sscr[];
   __shared__ u128 sh[32];
   __shared__ int64_t sh_item;
-  int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int wid = threadIdx.x >> 5;
   const int ids[1] = {ACC_N18};
   LocalAcc<1> la;
   la.zero();
   unsigned long long* g64 = gscr + (int64_t)blockIdx.x * gscr_stride;
   for (int i = threadIdx.x; i < smem_cap; i += blockDim.x) sscr[i] = 0;
   __syncthreads();
-  uint32_t tag = 0;                             // the same in every thread of the CTA
+  uint32_t tag0 = 0;                            // tags used so far, the same in every thread of the CTA
   while (true) {
-    int64_t it = next_item(qctr, nitems, &sh_item);
+    int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers also end the last item's reads
     if (it < 0) break;
     it = nitems - 1 - it;                     // heaviest centres first
     // centre of item `it`: the last k with item_off[k] <= it (item_off over centres c0..n-1)
     int64_t lo = 0, hi = g.n - c0;
     while (hi - lo > 1) { int64_t mid = (lo + hi) >> 1; if (item_off[mid] <= it) lo = mid; else hi = mid; }
-    int64_t c = c0 + lo;
-    int64_t base = g.R[c];
-    int d = (int)(g.R[c + 1] - base);
-    int u0 = (int)(it - item_off[lo]) * WHEEL_CHUNK;
-    int u1 = min(d, u0 + WHEEL_CHUNK);
-    const bool in_smem = d <= smem_cap;
-    for (int pu = u0; pu < u1; ++pu) {
-      uint32_t lenu = T[base + pu];
+    const int64_t c = c0 + lo;
+    const int64_t base = g.R[c];
+    const int d = (int)(g.R[c + 1] - base);
+    const int u0 = (int)(it - item_off[lo]) * WHEEL_CHUNK;
+    const int u1 = min(d, u0 + WHEEL_CHUNK);
+    const int pc = c >= cv.h0 ? d - cv.dh[c - cv.h0] : d;   // positions from pc on are in the core
+    if (tag0 + WHEEL_CHUNK > 0xffffu) {         // tags used up: zero both counter sets, start over
+      for (int i = threadIdx.x; i < smem_cap; i += blockDim.x) sscr[i] = 0;
+      for (int64_t i = threadIdx.x; i < gscr_stride; i += blockDim.x) g64[i] = 0;
+      __syncthreads();
+      tag0 = 0;
+    }
+    const bool in_smem = pc <= smem_cap;
+    // warps per group: 1, 4, 8, 16 or 32 (groups of two would need more than the 15 named barriers)
+    int gs = WHEEL_THREADS / 32;
+    if ((int64_t)pc * 32 <= smem_cap) gs = 1;
+    else if ((int64_t)pc * 8 <= smem_cap) gs = 4;
+    else if ((int64_t)pc * 4 <= smem_cap) gs = 8;
+    else if ((int64_t)pc * 2 <= smem_cap) gs = 16;
+    const int grp = wid / gs, ngrp = WHEEL_THREADS / 32 / gs, gw = wid % gs;
+    uint32_t* scr = sscr + (in_smem ? (int64_t)grp * pc : 0);
+    for (int pu = u0 + grp; pu < u1; pu += ngrp) {
+      const uint32_t lenu = T[base + pu];
       if (lenu < 2) continue;
-      if (++tag > 0xffffu) {                    // tags used up: zero both counter sets, start over
-        for (int i = threadIdx.x; i < smem_cap; i += blockDim.x) sscr[i] = 0;
-        for (int64_t i = threadIdx.x; i < gscr_stride; i += blockDim.x) g64[i] = 0;
-        __syncthreads();
-        tag = 1;
-      }
+      const bool top = pu >= pc;
+      const uint32_t lowu = top ? cv.low[base + pu] : lenu;
+      if (lowu == 0) continue;
       const int32_t* Lu = tl3.P + tl3.offp[base + pu];
+      const uint32_t tag = tag0 + 1 + (uint32_t)(pu - u0), t16 = tag << 16;
+      const unsigned long long t32 = (unsigned long long)tag << 32;
+      const int wstart = in_smem ? 0 : (win16 ? pc - smem_cap : pc);
       unsigned long long part = 0;
-      if (in_smem) {
-        const uint32_t t16 = tag << 16;
-        wheel_links(tl3, T, base, Lu, lenu, pu, (uint32_t)wid, (uint32_t)nw, [&](int32_t pv) {
-          atomicMax(&sscr[pv], t16);
-          part += atomicAdd(&sscr[pv], 1u) & 0xffffu;
-        });
-      } else {
-        // a centre too large for shared memory: its last smem_cap positions
-        // (the highest ranks, where the common neighbours concentrate) stay
-        // there when every count fits 16 bits (win16), the rest in global memory
-        const unsigned long long t32 = (unsigned long long)tag << 32;
-        const uint32_t t16 = tag << 16;
-        const int wstart = win16 ? d - smem_cap : d;
-        wheel_links(tl3, T, base, Lu, lenu, pu, (uint32_t)wid, (uint32_t)nw, [&](int32_t pv) {
+      wheel_walk(tl3, T, base, Lu, 0u, lowu, pu, min(pu, pc), (uint32_t)gw, (uint32_t)gs, [&](int32_t pv) {
+        if (pv >= wstart) {
+          uint32_t* q = &scr[pv - wstart];
+          atomicMax(q, t16);
+          part += atomicAdd(q, 1u) & 0xffffu;
+        } else {
+          atomicMax(&g64[pv], t32);
+          part += (uint32_t)atomicAdd(&g64[pv], 1ull);
+        }
+      });
+      if (top && lowu < lenu) {
+        wheel_group_sync(gs, grp);              // every low k is counted
+        wheel_walk(tl3, cv.low, base, Lu, lowu, lenu, pu, pc, (uint32_t)gw, (uint32_t)gs, [&](int32_t pv) {
           if (pv >= wstart) {
-            uint32_t* c = &sscr[pv - wstart];
-            atomicMax(c, t16);
-            part += atomicAdd(c, 1u) & 0xffffu;
+            const uint32_t v = scr[pv - wstart];
+            if ((v & 0xffff0000u) == t16) part += v & 0xffffu;
           } else {
-            atomicMax(&g64[pv], t32);
-            part += (uint32_t)atomicAdd(&g64[pv], 1ull);
+            const unsigned long long v = __ldcg(&g64[pv]);
+            if ((v >> 32) == tag) part += (uint32_t)v;
           }
         });
       }
       la.v[0] += part;
-      __syncthreads();                          // the next u's tag must not meet this u's increments
+      wheel_group_sync(gs, grp);                // the next u's tag must not meet this u's counts
     }
+    tag0 += WHEEL_CHUNK;
     block_item_flush(la, ids, acc, c, sh);
   }
   final_flush(la, ids, acc, sh);
@@ -2148,8 +2244,8 @@ __global__ void k_assemble(const Acc128* acc_all, const unsigned long long* n_ar
   N[14] = A[ACC_N14];
   N[15] = A[ACC_N15];
   N[16] = A[ACC_N16A] - 12 * K4;
-  N[17] = A[ACC_N17];
-  N[18] = A[ACC_N18];
+  N[17] = A[ACC_N17] + A[ACC_N17H] / 2;
+  N[18] = A[ACC_N18] + A[ACC_N18H] / 4;
   N[19] = A[ACC_N19];
   N[20] = A[ACC_N20];
   N[21] = A[ACC_N21];
@@ -2564,7 +2660,7 @@ static cudaError_t plan_pair_clusters(bool big, int sms, size_t arr_bytes, int64
 
 static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGraph& g, const int32_t* items,
                                     int64_t nitems, unsigned long long* qctr, const TagScratch& ts,
-                                    const TriLists& tl3, const uint32_t* T, const AccSet& accs,
+                                    const TriLists& tl3, const uint32_t* T, const CoreView& cv, const AccSet& accs,
                                     const PairTasks& pt, cudaStream_t s) {
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[1];
@@ -2581,15 +2677,30 @@ static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGra
   cudaError_t e = cudaErrorInvalidValue;
 #define ESC_PG(k, t, b)                                                                                   \
   if (plan.shape == k)                                                                                    \
-    e = big ? cudaLaunchKernelEx(&lc, k_pairs_grp<true, t, b>, g, items, nitems, qctr, ts, tl3, T, accs, pt,     \
+    e = big ? cudaLaunchKernelEx(&lc, k_pairs_grp<true, t, b>, g, items, nitems, qctr, ts, tl3, T, cv, accs, pt, \
                                  plan.wlo, plan.win_words)                                                      \
-            : cudaLaunchKernelEx(&lc, k_pairs_grp<false, t, b>, g, items, nitems, qctr, ts, tl3, T, accs, pt,    \
+            : cudaLaunchKernelEx(&lc, k_pairs_grp<false, t, b>, g, items, nitems, qctr, ts, tl3, T, cv, accs, pt, \
                                  plan.wlo, plan.win_words);
   ESC_PAIR_SHAPES(ESC_PG)
 #undef ESC_PG
   note_launch();
   return e;
 }
+
+// The dense core: vertices of degree CORE_MIN_DEG or more, at most CORE_CAP of
+// a single graph, in graphs (or unions) of at least CORE_MIN_D diamonds and
+// CORE_D_PER_ENTRY per adjacency entry.  Below that the sweeps' diamonds cost
+// less than the core's launches and passes over the graph (census, ms, without
+// and with a core): ER(800, 0.15), 8e6 diamonds, 1.69 / 1.73; ER(500, 0.3),
+// 4e7 (503 per entry), 2.22 / 1.83; R-MAT 11, 2e7 (387), 3.62 / 2.07;
+// Chung-Lu n = 120,000, 5e8 (401), 18.2 / 16.4; Chung-Lu 2.3 n = 250,000, 5e8
+// (134), 52.5 / 52.7; Chung-Lu 2.5 n = 500,000, 9e7 (11), 97.5 / 100.1.
+// The degree limit hardly matters between 16 and 64 (R-MAT 16: 38.5 to 39.0 ms,
+// 96: 45.2), nor the cap from 16,384 up (R-MAT 19: 8,192 760 ms, 16,384 661 ms,
+// 32,768 656 ms); W takes 2 bytes x cap^2.
+static constexpr int CORE_MIN_DEG = 48, CORE_CAP = 16384, CORE_CHUNK_MB = 2048;
+static constexpr unsigned long long CORE_MIN_D = 1ull << 24, CORE_D_PER_ENTRY = 160;
+static constexpr size_t CORE_W_BYTES = (size_t)24 << 30;
 
 cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t nnz, const CensusConfig& cfg,
                        unsigned long long* d_out, unsigned* d_status, PerElement* pe_out, Oriented* or_out,
@@ -2821,9 +2932,9 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // pair-sweep items by wedge count (light / medium / heavy lists)
   DevBuf b_plist, b_pctr;
   ESC_TRY(b_plist.alloc(five ? sizeof(int32_t) * 3 * (size_t)(n + 1) : 16));
-  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 8));
-  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 8, s);
-  unsigned long long pcnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 9));
+  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 9, s);
+  unsigned long long pcnt[9] = {0};
   if (five && n > 0) {
     // item classes: hash capacities bound the light and medium classes
     // (ESC_PAIR_SMALL_W / ESC_PAIR_LARGE_W lower them for tuning)
@@ -2848,6 +2959,74 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     int64_t lo = 0, hi = n;
     while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= 65536) hi = mid; else lo = mid + 1; }
     jbig = lo;
+  }
+  // core vertices: their core neighbours, places in W and the prefix sums of the work
+  DevBuf b_cdh, b_cli, b_crow, b_coff, b_chl, b_chb, b_cwb, b_low, b_W, b_cblk, b_ctile, b_cb;
+  CoreView cv{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
+  std::vector<int64_t> coff;
+  int64_t wlen = 0;
+  int64_t ch = 0;
+  const int core_min_d = env_int("ESC_CORE_MIN_D", 0);
+  if (five && own.parts <= 1 && env_int("ESC_CORE", 2) != 1 &&
+      pcnt[8] / 2 >= (core_min_d ? (unsigned long long)core_min_d
+                                 : std::max(CORE_MIN_D, CORE_D_PER_ENTRY * (unsigned long long)nnz))) {
+    const int64_t min_deg = env_int("ESC_CORE_MIN_DEG", CORE_MIN_DEG);
+    int64_t lo = 0, hi = n;                     // first rank of degree >= min_deg
+    while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= min_deg) hi = mid; else lo = mid + 1; }
+    ch = n - lo;
+    if (G == 1) ch = std::min<int64_t>(ch, env_int("ESC_CORE_CAP", CORE_CAP));
+  }
+  if (ch > 0) {
+    ESC_TRY(b_cdh.alloc(sizeof(int32_t) * ch));
+    ESC_TRY(b_cli.alloc(sizeof(int32_t) * ch));
+    ESC_TRY(b_crow.alloc(sizeof(int64_t) * ch));
+    ESC_TRY(b_coff.alloc(sizeof(int64_t) * 4 * (ch + 1)));
+    cv.h0 = n - ch;
+    ESC_TRY(core_layout(g, cv.h0, G == 1, b_cdh.as<int32_t>(), b_cli.as<int32_t>(), b_crow.as<int64_t>(),
+                        b_coff.as<int64_t>(), sms, s));
+    if (G > 1) {
+      ESC_TRY(b_chl.alloc(sizeof(int32_t) * ch));
+      ESC_TRY(b_chb.alloc(sizeof(int64_t) * ch));
+      ESC_TRY(b_cwb.alloc(sizeof(int64_t) * (G + 1)));
+      ESC_TRY(core_union(accs.vg, G, cv.h0, ch, b_chl.as<int32_t>(), b_chb.as<int64_t>(), b_cli.as<int32_t>(),
+                         b_crow.as<int64_t>(), b_cwb.as<int64_t>(), arena, sms, s));
+      cudaMemcpyAsync(&wlen, b_cwb.as<int64_t>() + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    } else {
+      wlen = ch * ch;
+    }
+    coff.resize(4 * (size_t)(ch + 1));
+    cudaMemcpyAsync(coff.data(), b_coff.p, sizeof(int64_t) * 4 * (ch + 1), cudaMemcpyDeviceToHost, s);
+    ESC_TRY(cudaStreamSynchronize(s));
+  }
+  // the core's buffers; a core whose W would pass CORE_W_BYTES is left out
+  CoreChunks cchunks;
+  CoreBuffers cbuf;
+  if (ch > 0) {
+    cv.wide = jbig < n ? 1 : 0;
+    const size_t wb = (cv.wide ? sizeof(uint32_t) : sizeof(uint16_t)) * (size_t)(wlen + 1);
+    core_chunks(coff.data(), ch, (int64_t)env_int("ESC_CORE_CHUNK_MB", CORE_CHUNK_MB) << 20, &cchunks);
+    if (wb > CORE_W_BYTES || cchunks.max_tiles == 0) {
+      ch = 0;
+      cv.h0 = n;
+    } else {
+      ESC_TRY(b_low.alloc(sizeof(uint32_t) * (size_t)(nnz + 1)));
+      ESC_TRY(b_W.alloc(wb));
+      ESC_TRY(b_cblk.alloc(core_block_bytes(cchunks)));
+      ESC_TRY(b_ctile.alloc(sizeof(int4) * (size_t)cchunks.max_tiles));
+      cbuf.blocks = b_cblk.p;
+      cbuf.tiles = b_ctile.p;
+      if (cv.h0 > 0) {
+        ESC_TRY(b_cb.alloc((cv.wide ? sizeof(uint32_t) : sizeof(uint16_t)) * (size_t)(cchunks.max_tri + 2)));
+        cbuf.b = b_cb.p;
+      }
+      cv.low = b_low.as<uint32_t>();
+      cv.dh = b_cdh.as<int32_t>();
+      cv.li = b_cli.as<int32_t>();
+      cv.rowb = b_crow.as<int64_t>();
+      cv.hl = G > 1 ? b_chl.as<int32_t>() : nullptr;
+      cv.hb = G > 1 ? b_chb.as<int64_t>() : nullptr;
+      cv.W = b_W.p;
+    }
   }
   // the heavy pair items: clusters sharing one counter array each
   PairPlan pplan;
@@ -2930,9 +3109,9 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   }
   DevBuf b_io, b_gs;
   int64_t nitems_w = 0;
-  // counters in shared memory up to half the opt-in size: two CTAs per SM
-  int smem_cap = std::max(0, (smem_optin / 2 - 4096) / 4);
-  smem_cap = (int)std::min<int64_t>(smem_cap, maxdeg);
+  // counters in shared memory: one CTA per SM, and no more than eight arrays of
+  // the largest degree (small graphs leave room for the other sweeps' CTAs)
+  int smem_cap = (int)std::min<int64_t>(std::max(0, (smem_optin - 4096) / 4), 8 * maxdeg);
   int64_t gstride = maxdeg > smem_cap ? maxdeg : 1;
   size_t smem_w = sizeof(uint32_t) * (size_t)std::max(smem_cap, 1);
   std::vector<int64_t> item_off(n - c0 + 1, 0);
@@ -2942,8 +3121,8 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     nitems_w = item_off[n - c0];
     ESC_TRY(b_io.alloc(sizeof(int64_t) * (n - c0 + 1)));
     cudaMemcpyAsync(b_io.p, item_off.data(), sizeof(int64_t) * (n - c0 + 1), cudaMemcpyHostToDevice, s);
-    ESC_TRY(b_gs.alloc(sizeof(unsigned long long) * (size_t)gstride * 2 * sms + 16));
-    cudaMemsetAsync(b_gs.p, 0, sizeof(unsigned long long) * (size_t)gstride * 2 * sms + 16, s);
+    ESC_TRY(b_gs.alloc(sizeof(unsigned long long) * (size_t)gstride * sms + 16));
+    cudaMemsetAsync(b_gs.p, 0, sizeof(unsigned long long) * (size_t)gstride * sms + 16, s);
     ESC_TRY(allow_max_smem((const void*)k_wheels_cta, smem_optin));
   }
   DevBuf b_wo;                                 // warp wheel items: offsets over centres c0-1 .. 0
@@ -2961,6 +3140,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   if (five && n > 0)
     (k_tri_lists<<<grid_sweep, 512, smem_l, s>>>(g, ctr + 3, off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(),
                                                  b_gh.as<int32_t>(), ghash_cap, hcap_l, d_status), note_launch());
+  if (ch > 0) ESC_TRY(core_low(g, T, off, b_U.as<int32_t>(), cv.h0, b_low.as<uint32_t>(), sms, s));
   mark(4, 1, s);
   StreamSet ss_all;
   cudaStream_t s1 = s, s2 = s, s3 = s, s4 = s;
@@ -2974,14 +3154,15 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // wheels (Thm 11): the longest phase, started first
   mark(6, 0, s3);
   if (five && c0 < n)
-    (k_wheels_cta<<<2 * sms, 512, smem_w, s3>>>(g, c0, b_io.as<int64_t>(), nitems_w, ctr + 5, tl3, T,
+    (k_wheels_cta<<<(unsigned)std::min<int64_t>(sms, std::max<int64_t>(nitems_w, 1)), WHEEL_THREADS, smem_w, s3>>>(
+                                            g, c0, b_io.as<int64_t>(), nitems_w, ctr + 5, tl3, T, cv,
                                             b_gs.as<unsigned long long>(), gstride, smem_cap, accs,
                                             pcnt[7] < 65536 && env_int("ESC_WHEEL_WINDOW", 2) != 1), note_launch());
   if (five && c0 > 0) {
     int per_sm = 1;
     ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wheels_warp, 256, 0));
     (k_wheels_warp<<<(unsigned)std::max(1, per_sm) * sms, 256, 0, s3>>>(g, c0, b_wo.as<int64_t>(), ctr + 7, tl3, T,
-                                                                          accs), note_launch());
+                                                                          cv, accs), note_launch());
   }
   mark(6, 1, s3);
   // pairs (Thms 11, 12); 16-bit counters when no degree reaches 2^16 (then no W(i,j) can)
@@ -2995,7 +3176,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_hash<PH_SMALL_SLOTS>, PH_SMALL_THREADS,
                                                             sm0));
       unsigned grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, (int64_t)pcnt[0]);
-      (k_pairs_hash<PH_SMALL_SLOTS><<<grid, PH_SMALL_THREADS, sm0, s>>>(g, pl, (int64_t)pcnt[0], pq + 0, tl3, T, accs,
+      (k_pairs_hash<PH_SMALL_SLOTS><<<grid, PH_SMALL_THREADS, sm0, s>>>(g, pl, (int64_t)pcnt[0], pq + 0, tl3, T, cv, accs,
                                                                        d_status), note_launch());
     }
     if (pcnt[1] > 0) {
@@ -3006,20 +3187,23 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
                                                             sm1));
       unsigned grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, (int64_t)pcnt[1]);
       (k_pairs_hash<PH_LARGE_SLOTS><<<grid, PH_LARGE_THREADS, sm1, s>>>(g, pl + n, (int64_t)pcnt[1], pq + 1, tl3, T,
-                                                                       accs, d_status), note_launch());
+                                                                       cv, accs, d_status), note_launch());
     }
     if (pcnt[2] > 0 && pplan.windowed) {
       const size_t smw = sizeof(uint32_t) * (size_t)pplan.win_words;
       if (jbig < n)
         (k_pairs_win<true><<<pplan.nclusters, pplan.threads, smw, s>>>(g, pl + 2 * n, (int64_t)pcnt[2], pq + 2, pwin,
-                                                                      tl3, T, accs, ptasks, d_status), note_launch());
+                                                                      tl3, T, cv, accs, ptasks, d_status), note_launch());
       else
         (k_pairs_win<false><<<pplan.nclusters, pplan.threads, smw, s>>>(g, pl + 2 * n, (int64_t)pcnt[2], pq + 2, pwin,
-                                                                       tl3, T, accs, ptasks, d_status), note_launch());
+                                                                       tl3, T, cv, accs, ptasks, d_status), note_launch());
     } else if (pcnt[2] > 0) {
-      ESC_TRY(launch_pairs_grp(jbig < n, pplan, g, pl + 2 * n, (int64_t)pcnt[2], pq + 2, tsB, tl3, T, accs, ptasks,
+      ESC_TRY(launch_pairs_grp(jbig < n, pplan, g, pl + 2 * n, (int64_t)pcnt[2], pq + 2, tsB, tl3, T, cv, accs, ptasks,
                                s));
     }
+    if (ch > 0)
+      ESC_TRY(core_run(g, cv, T, offp, b_P.as<int32_t>(), b_coff.as<int64_t>(), coff.data(), cchunks, cbuf, accs,
+                       d_status, sms, smem_optin, s));
   }
   mark(5, 1, s);
   // cliques and per-triangle sums (Thms 6, 7, 10, 14)

@@ -34,6 +34,8 @@ enum AccId {
   ACC_TD,         // sum_i t_i d_i
   ACC_DP,         // sum over out-edges a -> b of (d+(a) - 1) d+(b)   directed 3-paths i <- a -> b -> j
   ACC_DBP,        // sum over directed triangles of C(apexes above, 2)  directed bipyramids
+  ACC_N17H,       // 2 x the core's share of N17 (core.cu)
+  ACC_N18H,       // 4 x the core's share of N18
   ACC_COUNT
 };
 
@@ -177,6 +179,23 @@ struct DevGraph {
 __device__ __forceinline__ int64_t dg_deg(const DevGraph& g, int64_t v) { return g.R[v + 1] - g.R[v]; }
 __device__ __forceinline__ int64_t dg_outdeg(const DevGraph& g, int64_t v) { return g.R[v + 1] - g.op[v]; }
 
+// The dense core (core.cu): the ranks from h0 on, n when a graph has none.
+struct CoreView {
+  int64_t h0;
+  const uint32_t* low;    // per slot whose entry is in the core: common neighbours of the edge below h0
+  const int32_t* dh;      // per core vertex (rank - h0): core neighbours
+  const int32_t* li;      // core vertices of the same graph below it
+  const int64_t* rowb;    // start of its row in W
+  const int32_t* hl;      // union of graphs: the core ranks by graph (null for a single graph: rank h0 + k)
+  const int64_t* hb;      // union: start of its graph's ranks in hl
+  void* W;                // wedge counts W(i, j) of the core pairs j < i of one graph
+  int wide;               // 32-bit entries instead of 16-bit ones
+  __device__ __forceinline__ void put(int64_t e, uint32_t v) const {
+    if (wide) ((uint32_t*)W)[e] = v;
+    else ((uint16_t*)W)[e] = (uint16_t)v;
+  }
+};
+
 // lower_bound of key in sorted C[lo, hi)
 __device__ __forceinline__ int64_t lower_bound_i32(const int32_t* a, int64_t lo, int64_t hi, int32_t key) {
   while (lo < hi) {
@@ -211,6 +230,7 @@ enum DevErr : unsigned {
   DEVERR_SCRATCH = 1u << 0,   // a scratch capacity was exceeded
   DEVERR_BOUNDS = 1u << 1,    // an index fell outside its array
   DEVERR_OVERFLOW = 1u << 2,  // a per-element counter overflowed
+  DEVERR_TIMEOUT = 1u << 3,   // a bounded wait ran out
 };
 
 __device__ __forceinline__ void set_err(unsigned* st, unsigned bit) { atomicOr(st, bit); }

@@ -45,6 +45,12 @@ escape_status from_cuda(cudaError_t e) {
   return ESCAPE_ECUDA;
 }
 
+// the device status word of a census
+escape_status from_status(unsigned h) {
+  if (h == 0) return ESCAPE_OK;
+  return h == DEVERR_TIMEOUT ? ESCAPE_ETIMEOUT : ESCAPE_EINTERNAL;
+}
+
 void free_pe(escape_graph* g) {
   cudaFree(g->pe.Te); cudaFree(g->pe.C4e); cudaFree(g->pe.K4e);
   cudaFree(g->pe.tv); cudaFree(g->pe.C4v); cudaFree(g->pe.K4v);
@@ -299,7 +305,7 @@ escape_status census_one(escape_graph* g, const int64_t* d_rp, const int32_t* d_
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstat, d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     st = from_cuda(e);
-    if (st == ESCAPE_OK && hstat != 0) st = ESCAPE_EINTERNAL;
+    if (st == ESCAPE_OK) st = from_status(hstat);
     if (st == ESCAPE_OK) {
       *out = tmp;
       for (int i = 0; i < 4; ++i) g->basis[i] = basis[i];
@@ -540,7 +546,7 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
       if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       st = from_cuda(e);
-      if (st == ESCAPE_OK && h) st = ESCAPE_EINTERNAL;
+      if (st == ESCAPE_OK) st = from_status(h);
     }
   }
   cudaFree(d_voff); cudaFree(d_rp); cudaFree(d_col); cudaFree(d_status); cudaFree(d_out);
@@ -698,7 +704,7 @@ escape_status escape_census5_part(escape_graph* g, int32_t part, int32_t parts, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     st = from_cuda(e);
-    if (st == ESCAPE_OK && h) st = ESCAPE_EINTERNAL;
+    if (st == ESCAPE_OK) st = from_status(h);
     if (st == ESCAPE_OK) *out = tmp;
   }
   cudaFree(d_acc);
