@@ -812,9 +812,12 @@ __device__ __forceinline__ long long ld_cluster_s64(const void* p, unsigned rank
 // ============================================================================
 // Thm 5: 4-cycles.  For the highest vertex i and each j < i,
 // w(i,j) = |{k in N(i) cap N(j) : k < i}| (out-wedges and in-out wedges);
-// C4 = sum C(w,2).  Per element: every wedge i - k - j adds w-1 to edges
-// (i,k), (k,j) and vertex k; every j adds C(w,2) to vertices i and j.
-// CTA per i, dense per-CTA counters over j with a touched list.
+// C4 = sum C(w,2), the sum of the values the increments return.  Per edge: every
+// wedge i - k - j adds w-1 to edges (i,k) and (k,j); C4(v) is half the sum over
+// the edges of v (a 4-cycle has two edges at each of its vertices), so no
+// counter per vertex is touched.  Light and medium items count in a hash table
+// (k_cycles4_hash), heavy ones in windows (k_cycles4_win) or, in a union of
+// graphs, in tagged counters (k_cycles4_tag).
 // ============================================================================
 #ifndef ESC_SWEEP_ILP
 #define ESC_SWEEP_ILP 8
@@ -828,104 +831,10 @@ static constexpr int PAIR_ILP = ESC_PAIR_ILP;
 static_assert(PAIR_ILP >= 1 && PAIR_ILP <= 8, "pair_range sums at most 8 values of C(old, 2) in 64 bits");
 
 struct SweepScratch {
-  uint32_t* cnt;       // per CTA: n counters (kept zero between items)
-  int32_t* touched;    // per CTA: n entries
-  uint32_t* cnt2;      // second counter array (5-cycles)
-  int32_t* touched2;
-  unsigned* ntouched;  // per CTA: 2 counters
+  uint32_t* cnt2;      // per CTA: n counters of P2 (kept zero between items)
+  int32_t* touched2;   // per CTA: n entries
   int64_t n;
 };
-
-template <bool BIG>
-__global__ void k_cycles4(DevGraph g, unsigned long long* qctr, TagScratch ts, unsigned long long* C4raw,
-                          unsigned long long* C4v, AccSet acc, Owner own) {
-  __shared__ u128 sh[32];
-  __shared__ int64_t sh_item;
-  TaggedCounters<BIG> w(ts);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  u128 c4sum = 0;
-  while (true) {
-    int64_t it = next_item(qctr, own.count(g.n), &sh_item);
-    if (it < 0) break;
-    int64_t i = own.item(g.n, it);
-    int64_t b0 = g.R[i], e0 = g.op[i];
-    if (e0 == b0) continue;           // no lower neighbours
-    if (w.next(g.n)) __syncthreads();
-    // pass 1: wedge counts w(i, j).  C(w, 2) at j is the sum of the values the
-    // increments of j return, so each increment adds its old value to C4(j)
-    // at once and no second pass over the touched j's is needed.  The lists
-    // N(k) below i are fetched 32 per warp (lane l the l-th), SWEEP_ILP
-    // entries in flight per lane.
-    u128 mine = 0;
-    for (int64_t pbase = b0 + wid; pbase < e0; pbase += (int64_t)nw * 32) {
-      int64_t p = pbase + (int64_t)lane * nw;
-      int64_t kb_l = 0, ke_l = 0;
-      if (p < e0) {
-        kb_l = g.R[g.C[p]];
-        ke_l = g.rev[p];                        // N(k) below i ends at the slot of i
-      }
-      int kmax = (int)min((int64_t)32, (e0 - pbase + nw - 1) / nw);
-      for (int kk = 0; kk < kmax; ++kk) {
-        int64_t kb = __shfl_sync(0xffffffffu, kb_l, kk), ke = __shfl_sync(0xffffffffu, ke_l, kk);
-        for (int64_t q = kb + lane; q < ke; q += 32 * SWEEP_ILP) {
-          int32_t jj[SWEEP_ILP];
-          uint32_t oo[SWEEP_ILP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < ke ? g.C[q + 32 * u] : -1;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) oo[u] = jj[u] >= 0 ? w.inc(jj[u]) : 0u;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u)
-            if (oo[u]) {
-              atomicAdd(&C4v[jj[u]], (unsigned long long)oo[u]);
-              mine += oo[u];
-            }
-        }
-      }
-    }
-    u128 tot = block_sum_u128(mine, sh);        // its barriers also end pass 1
-    if (threadIdx.x == 0) {
-      if (tot) atomicAdd(&C4v[i], (unsigned long long)tot);
-      if (acc.vg) acc_add(acc_of(acc, i), ACC_C4, tot);
-      else c4sum += tot;
-    }
-    // pass 3: per-edge counts, the lists fetched as in pass 1
-    for (int64_t pbase = b0 + wid; pbase < e0; pbase += (int64_t)nw * 32) {
-      int64_t p_l = pbase + (int64_t)lane * nw;
-      int64_t kb_l = 0, ke_l = 0;
-      int32_t k_l = 0;
-      if (p_l < e0) {
-        k_l = g.C[p_l];
-        kb_l = g.R[k_l];
-        ke_l = g.rev[p_l];
-      }
-      int kmax = (int)min((int64_t)32, (e0 - pbase + nw - 1) / nw);
-      for (int kk = 0; kk < kmax; ++kk) {
-        int64_t kb = __shfl_sync(0xffffffffu, kb_l, kk), ke = __shfl_sync(0xffffffffu, ke_l, kk);
-        unsigned long long sk = 0;
-        for (int64_t q = kb + lane; q < ke; q += 32 * SWEEP_ILP) {
-          int32_t jj[SWEEP_ILP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < ke ? g.C[q + 32 * u] : -1;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) {
-            if (jj[u] < 0) continue;
-            unsigned long long c = w.get(jj[u]) - 1;
-            if (c) { atomicAdd(&C4raw[q + 32 * u], c); sk += c; }
-          }
-        }
-        sk = warp_sum_u64(sk);
-        int32_t k = __shfl_sync(0xffffffffu, k_l, kk);
-        if (lane == 0 && sk) {
-          atomicAdd(&C4raw[pbase + (int64_t)kk * nw], sk);
-          atomicAdd(&C4v[k], sk);
-        }
-      }
-    }
-    __syncthreads();                            // the next item's counts must not meet these reads
-  }
-  if (threadIdx.x == 0 && !acc.vg) acc_add(acc.base, ACC_C4, c4sum);
-}
 
 // Per-edge common-neighbour lists (built by the triangle-list pass).
 struct TriLists {
@@ -947,89 +856,183 @@ struct TriLists {
 // ============================================================================
 
 
-// Items are split by their wedge count w_i = sum_{c in N(i)} |N(c) below i|
-// (the number of W(i, .) increments, so also a bound on the distinct j):
-//   light  (w_i <= PH_SMALL_W): one CTA, W(i, .) in a shared-memory hash table
-//   medium (w_i <= PH_LARGE_W): one CTA, a larger shared-memory hash table
-//   heavy:                      a cluster of CTAs shares one tagged counter
-//                               array in global memory, and only as many
-//                               clusters run as keep their arrays within L2
-static constexpr int PH_SMALL_SLOTS = 4096, PH_SMALL_THREADS = 256;
-static constexpr int PH_LARGE_SLOTS = 16384, PH_LARGE_THREADS = 512;
-static constexpr int64_t PH_SMALL_W = PH_SMALL_SLOTS / 2;     // load factor <= 1/2
-static constexpr int64_t PH_LARGE_W = PH_LARGE_SLOTS / 2;
+// Items of the pair, 4-cycle and 5-cycle sweeps are split by the number w_i of
+// their counter increments, which with the size of the graph also bounds the
+// distinct counters m_i = min(w_i, n):
+//   light:   m_i <= IT_LIGHT_M and w_i <= 4 IT_LIGHT_M: one CTA of 64 threads
+//   medium:  m_i <= IT_MEDIUM_M: one CTA of 512 threads
+//   heavy:   the rest
+// Light and medium items count in a packed shared-memory hash table of 2 m_i
+// words or more (a power of two), cleared for the item: small items clear
+// little and keep many CTAs on an SM.  An item whose degree does not fit the
+// count bits of a packed word is heavy.  What bounded the sweeps before: one
+// 512-thread CTA per vertex with counters in global memory, most of whose time
+// went to barriers and latency on vertices of a few dozen edges (alone, ms,
+// before and after): Chung-Lu 2.3 n = 625,000 5-cycles 34.7 / 17.6, 4-cycles
+// 16.7 / 6.2; Chung-Lu 2.1 n = 262,144 9.6 / 6.6 and 6.5 / 2.0; R-MAT 19 70 / 58
+// and 56 / 20; 256 graphs of 20 to 200 vertices 1.03 / 0.36 and 0.40 / 0.14.
+static constexpr int IT_LIGHT_LOG = 11, IT_MEDIUM_LOG = 14, IT_MIN_LOG = 7;
+static constexpr int IT_LIGHT_THREADS = 64, IT_MEDIUM_THREADS = 512;
+static constexpr long long IT_LIGHT_M = 1ll << (IT_LIGHT_LOG - 1);
+static constexpr long long IT_MEDIUM_M = 1ll << (IT_MEDIUM_LOG - 1);
+static constexpr long long IT5_MEDIUM_M = IT_MEDIUM_M / 2;   // the 5-cycle sweep has two tables
 
-// w_i of every vertex with degree >= 2, appended to the list of its class
-// (roughly by decreasing rank, so the heaviest items come first)
-// Also the largest common-neighbour list (triangles on one edge) into cnts[7]
-// and twice the number of diamonds, sum over slots of C(T, 2), into cnts[8].
-__global__ void k_pair_classify(DevGraph g, const uint32_t* T, int32_t* lists, unsigned long long* cnts,
-                                long long w_small, long long w_large, Owner own) {
+// A packed item: rank in the low 32 bits, log2 of the table size(s) above.
+__host__ __device__ __forceinline__ int64_t item_rank(unsigned long long it) { return (int64_t)(it & 0xffffffffull); }
+__host__ __device__ __forceinline__ int item_log(unsigned long long it) { return (int)((it >> 32) & 0xff); }
+__host__ __device__ __forceinline__ int item_log2(unsigned long long it) { return (int)((it >> 40) & 0xff); }
+
+// Open addressing in shared memory, key and count in one 32-bit word: key << cb
+// | count, all ones = empty.  Half the space and half the accesses of separate
+// key and count words.  Every key is below 2^(32 - cb) - 1 and every count
+// below 2^cb - 1 (ranks below n, counts at most the item's degree: the host
+// and the classification see to it), so no used word is all ones.
+struct PackedHash {
+  uint32_t* tab;
+  int cb, log;
+  static constexpr uint32_t EMPTY = 0xffffffffu;
+  __device__ __forceinline__ uint32_t slot(int32_t j) const { return ((uint32_t)j * 0x9E3779B1u) >> (32 - log); }
+  __device__ __forceinline__ void clear(int tid, int nthreads) const {
+    uint4* t4 = reinterpret_cast<uint4*>(tab);
+    for (int t = tid; t < (1 << log) / 4; t += nthreads) t4[t] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+  }
+  // the count before; full: the table has no room (never: sized by m_i)
+  __device__ __forceinline__ uint32_t inc(int32_t j, bool& full) const {
+    const uint32_t m = (1u << log) - 1u, cm = (1u << cb) - 1u;
+    uint32_t sl = slot(j);
+    for (uint32_t probe = 0; probe <= m; ++probe) {
+      uint32_t w = *(volatile uint32_t*)&tab[sl];
+      if (w == EMPTY) {
+        w = atomicCAS(&tab[sl], EMPTY, ((uint32_t)j << cb) | 1u);
+        if (w == EMPTY) return 0u;
+      }
+      if ((w >> cb) == (uint32_t)j) return atomicAdd(&tab[sl], 1u) & cm;
+      sl = (sl + 1u) & m;
+    }
+    full = true;
+    return 0u;
+  }
+  // the count (0 when j was never counted)
+  __device__ __forceinline__ uint32_t get(int32_t j) const {
+    const uint32_t m = (1u << log) - 1u;
+    uint32_t sl = slot(j);
+    for (uint32_t probe = 0; probe <= m; ++probe) {
+      const uint32_t w = tab[sl];
+      if (w == EMPTY) return 0u;
+      if ((w >> cb) == (uint32_t)j) return w & ((1u << cb) - 1u);
+      sl = (sl + 1u) & m;
+    }
+    return 0u;
+  }
+};
+
+// log2 of a table for m counters (load factor at most 1/2)
+__device__ __forceinline__ int table_log(unsigned long long m) {
+  const int l = m <= 1 ? 1 : 65 - __clzll((long long)(m - 1));   // ceil(log2(2 m))
+  return max(l, IT_MIN_LOG);
+}
+
+// One sweep's item lists (light, medium, heavy; n entries each) and counters:
+// cnt[0..2] list lengths, cnt[3..5] the queues, cnt[6] the largest heavy item.
+struct ItemLists {
+  unsigned long long* list;
+  unsigned long long* cnt;
+};
+__device__ __forceinline__ void item_append(const ItemLists& il, int64_t n, int64_t i, unsigned long long w,
+                                            unsigned long long m1, unsigned long long m2, long long light_m,
+                                            long long medium_m, bool fits) {
+  const unsigned long long m = max(m1, m2);
+  const int cls = !fits ? 2
+                        : ((long long)m <= light_m && (long long)w <= 4 * light_m
+                               ? 0
+                               : ((long long)m <= medium_m ? 1 : 2));
+  unsigned long long v = (unsigned long long)i;
+  if (cls < 2) v |= ((unsigned long long)table_log(m1) << 32) | ((unsigned long long)table_log(m2) << 40);
+  il.list[(int64_t)cls * n + (int64_t)atomicAdd(&il.cnt[cls], 1ull)] = v;
+  if (cls == 2) atomicMax(&il.cnt[6], w);        // for the task buffers
+}
+
+// Pair items: w_i = sum_{c in N(i)} |N(c) below i| of every vertex with degree
+// >= 2 (roughly by decreasing rank, so the heaviest items come first).
+// Also the largest common-neighbour list (triangles on one edge) into cnt[7]
+// and twice the number of diamonds, sum over slots of C(T, 2), into cnt[8].
+__global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, long long light_m, long long medium_m,
+                                int cb, const int32_t* vg, const unsigned long long* n_arr, Owner own) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long dia = 0;
+  unsigned tmax = 0;
   for (int64_t k = warp; k < g.n; k += nwarps) {
     int64_t i = g.n - 1 - k;
     int64_t b0 = g.R[i], e0 = g.R[i + 1];
-    unsigned tmax = 0;
+    unsigned long long w = 0;
+    const bool mine = e0 - b0 >= 2 && own.owns(i);
     for (int64_t p = b0 + lane; p < e0; p += 32) {
       const uint32_t t = T[p];
       tmax = max(tmax, t);
       dia += t < 2 ? 0 : (unsigned long long)t * (t - 1) / 2;
+      if (mine) w += (unsigned long long)(g.rev[p] - g.R[g.C[p]]);
     }
-    tmax = __reduce_max_sync(0xffffffffu, tmax);
-    if (lane == 0 && tmax) atomicMax(&cnts[7], (unsigned long long)tmax);
-    if (e0 - b0 < 2 || !own.owns(i)) continue;
-    unsigned long long w = 0;
-    for (int64_t p = b0 + lane; p < e0; p += 32) w += (unsigned long long)(g.rev[p] - g.R[g.C[p]]);
     w = warp_sum_u64(w);
-    w = __shfl_sync(0xffffffffu, w, 0);
-    if (w == 0) continue;
-    int cls = (long long)w <= w_small ? 0 : ((long long)w <= w_large ? 1 : 2);
-    if (lane == 0) {
-      lists[(int64_t)cls * g.n + (int64_t)atomicAdd(&cnts[cls], 1ull)] = (int32_t)i;
-      if (cls == 2) atomicMax(&cnts[6], w);    // the largest item, for the task buffers
+    if (lane == 0 && w) {
+      const unsigned long long m = min(w, min((unsigned long long)i, vg ? n_arr[vg[i]] : ~0ull));
+      item_append(il, g.n, i, w, m, m, light_m, medium_m, (unsigned long long)(e0 - b0) < (1u << cb) - 1u);
     }
   }
   dia = warp_sum_u64(dia);
-  if (lane == 0 && dia) atomicAdd(&cnts[8], dia);
+  if (lane == 0 && dia) atomicAdd(&il.cnt[8], dia);
+  tmax = __reduce_max_sync(0xffffffffu, tmax);
+  if (lane == 0 && tmax) atomicMax(&il.cnt[7], (unsigned long long)tmax);
 }
 
-// Open addressing in shared memory (keys -1 = empty), linear probing.  At most
-// half the slots are ever used, so a probe sequence ends within the table.
-template <int SLOTS>
-__device__ __forceinline__ int ph_insert(int32_t* hk, int32_t j) {
-  constexpr int LOG = __builtin_ctz(SLOTS);
-  uint32_t sl = ((uint32_t)j * 0x9E3779B1u) >> (32 - LOG);
-  volatile int32_t* vk = hk;
-  for (int probe = 0; probe < SLOTS; ++probe) {
-    int32_t k = vk[sl];
-    if (k == j) return (int)sl;
-    if (k == -1) {
-      int32_t old = atomicCAS(&hk[sl], -1, j);
-      if (old == -1 || old == j) return (int)sl;
+// 4-cycle items (w4_i = sum over k in N-(i) of |N(k) below i|) and, unless
+// only4, 5-cycle items (the increments of w'(i, .) and of P2(i, .), see
+// k_cycles5).
+__global__ void k_cycle_classify(DevGraph g, ItemLists i4, ItemLists i5, bool only4, long long light_m,
+                                 long long medium_m4, long long medium_m5, int cb, const int32_t* vg,
+                                 const unsigned long long* n_arr, Owner own) {
+  int lane = threadIdx.x & 31;
+  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t k = warp; k < g.n; k += nwarps) {
+    const int64_t i = g.n - 1 - k;
+    if (!own.owns(i)) continue;
+    const int64_t b0 = g.R[i], o = g.op[i], e0 = g.R[i + 1];
+    if (o == b0) continue;                      // no lower neighbour
+    unsigned long long w4 = 0, w5 = 0, p2 = 0;
+    for (int64_t p = b0 + lane; p < e0; p += 32) {
+      const int32_t c = g.C[p];
+      const int64_t cr = g.R[c], ce = g.R[c + 1];
+      if (p < o) {
+        w4 += (unsigned long long)(g.rev[p] - cr);
+        w5 += (unsigned long long)(ce - cr);
+        p2 += (unsigned long long)(ce - g.op[c]);
+      } else {
+        if (only4) break;
+        w5 += (unsigned long long)(ce - g.op[c]);
+      }
     }
-    sl = (sl + 1) & (SLOTS - 1);
+    w4 = warp_sum_u64(w4);
+    w5 = warp_sum_u64(w5);
+    p2 = warp_sum_u64(p2);
+    if (lane) continue;
+    const unsigned long long ng = vg ? n_arr[vg[i]] : (unsigned long long)g.n;
+    const bool fits = (unsigned long long)(e0 - b0) < (1u << cb) - 1u;
+    if (w4) {
+      const unsigned long long m = min(w4, min((unsigned long long)i, ng));
+      item_append(i4, g.n, i, w4, m, m, light_m, medium_m4, fits);
+    }
+    // P2 counts the slot of i itself once per a: with nothing else, no path leaves it
+    if (!only4 && p2 > (unsigned long long)(o - b0))
+      item_append(i5, g.n, i, w5 + p2, min(w5, ng), min(p2, ng), light_m, medium_m5, fits);
   }
-  return -1;
-}
-template <int SLOTS>
-__device__ __forceinline__ int ph_find(const int32_t* hk, int32_t j) {
-  constexpr int LOG = __builtin_ctz(SLOTS);
-  uint32_t sl = ((uint32_t)j * 0x9E3779B1u) >> (32 - LOG);
-  for (int probe = 0; probe < SLOTS; ++probe) {
-    int32_t k = hk[sl];
-    if (k == j) return (int)sl;
-    if (k == -1) return -1;
-    sl = (sl + 1) & (SLOTS - 1);
-  }
-  return -1;
 }
 
 // The two passes of one item i, shared by both forms of the sweep.  Warp
 // `gw` of `gnw` (the warps of a CTA, or of a whole cluster) takes its share:
-//   inc(j) counts the wedge i - c - j and returns W(i,j) before it;
+//   inc(j) counts the wedge i - c - j and returns its term of the sum, a
+//   function of the count before it (pair_c2 for N13, the count itself for C4);
 //   get(j) returns W(i,j) after every increment.
 // Pass 1: W(i,.) from every wedge i - c - j (c in N(i), j in N(c), j < i);
 // C(W,3) is accumulated on the fly as the sum of C(old, 2).  The lists N(c) are
@@ -1073,7 +1076,7 @@ __device__ __forceinline__ u128 pair_range(const DevGraph& g, int64_t cb, int64_
     unsigned long long blk = 0;                 // at most 8 terms below 2^61 (a count is below 2^31)
 #pragma unroll
     for (int u = 0; u < PAIR_ILP; ++u)
-      if (jj[u] >= 0) blk += pair_c2(inc(jj[u]));
+      if (jj[u] >= 0) blk += inc(jj[u]);
     n13.add(blk);
   }
   return n13.get();
@@ -1106,7 +1109,7 @@ __device__ __forceinline__ u128 pair_wedges(const DevGraph& g, int64_t b0, int64
         unsigned long long blk = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (jj[u] >= 0) blk += pair_c2(inc(jj[u]));
+          if (jj[u] >= 0) blk += inc(jj[u]);
         sh13.add(blk);
       }
       n13 += sh13.get();
@@ -1297,45 +1300,42 @@ __device__ __forceinline__ void core_store_row(const CoreView& cv, int64_t i, in
   for (int64_t k = tid; k < cnt; k += nthreads) cv.put(row + k, get(hl ? hl[k] : (int32_t)(cv.h0 + k)));
 }
 
-// Light and medium items: one CTA per item, W(i, .) in a shared-memory hash
-// table (SLOTS keys and counts) that is cleared after every item.
-template <int SLOTS>
-__global__ void k_pairs_hash(DevGraph g, const int32_t* items, int64_t nitems, unsigned long long* qctr,
-                             TriLists tl3, const uint32_t* T, CoreView cv, AccSet acc, unsigned* status) {
-  extern __shared__ int32_t ph_smem[];
-  int32_t* hk = ph_smem;
-  uint32_t* hv = (uint32_t*)(ph_smem + SLOTS);
+// Light and medium items: one CTA of THREADS threads per item, W(i, .) in a
+// packed hash table.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_pairs_hash(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                       unsigned long long* qctr, int cb, int max_log, TriLists tl3,
+                                                       const uint32_t* T, CoreView cv, AccSet acc, unsigned* status) {
+  extern __shared__ uint4 hash_smem[];
   __shared__ u128 sh[32];
   __shared__ int64_t sh_item;
-  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int wid = threadIdx.x >> 5, nw = THREADS / 32;
+  PackedHash H{reinterpret_cast<uint32_t*>(hash_smem), cb, 0};
   const int ids[2] = {ACC_N13, ACC_N17};
   LocalAcc<2> la;
   la.zero();
-  for (int t = threadIdx.x; t < SLOTS; t += blockDim.x) { hk[t] = -1; hv[t] = 0u; }
   while (true) {
-    int64_t it = next_item(qctr, nitems, &sh_item);     // its barriers publish the cleared table
+    int64_t it = next_item(qctr, nitems, &sh_item);     // its barriers end the last item's reads
     if (it < 0) break;
-    const int64_t i = items[it];
+    const int64_t i = item_rank(items[it]);
     const int64_t b0 = g.R[i], e0 = g.R[i + 1];
-    u128 n13 = pair_wedges(g, b0, e0, wid, nw, [&](int32_t j) -> uint32_t {
-      int sl = ph_insert<SLOTS>(hk, j);
-      if (sl < 0) { set_err(status, DEVERR_SCRATCH); return 0u; }
-      return atomicAdd(&hv[sl], 1u);
+    H.log = min(max_log, item_log(items[it]));
+    H.clear(threadIdx.x, THREADS);
+    __syncthreads();
+    bool full = false;
+    la.v[0] += pair_wedges(g, b0, e0, wid, nw, [&](int32_t j) -> unsigned long long {
+      return pair_c2(H.inc(j, full));
     }, [](int64_t, int64_t) { return false; });
+    if (full) set_err(status, DEVERR_SCRATCH);
     __syncthreads();
-    u128 n17 = pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t {
-      int sl = ph_find<SLOTS>(hk, j);
-      if (sl < 0) { set_err(status, DEVERR_SCRATCH); return 2u; }
-      return hv[sl];
-    });
-    __syncthreads();
-    for (int t = threadIdx.x; t < SLOTS; t += blockDim.x) {
-      if (i >= cv.h0 && hk[t] >= cv.h0) cv.put(cv.rowb[i - cv.h0] + cv.li[hk[t] - cv.h0], hv[t]);
-      hk[t] = -1;
-      hv[t] = 0u;
-    }
-    la.v[0] += n13;
-    la.v[1] += n17;
+    la.v[1] += pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t { return H.get(j); });
+    if (i >= cv.h0)
+      for (int t = threadIdx.x; t < (1 << H.log); t += THREADS) {
+        const uint32_t w = H.tab[t];
+        const int64_t j = (int64_t)(w >> cb);
+        if (w != PackedHash::EMPTY && j >= cv.h0)
+          cv.put(cv.rowb[i - cv.h0] + cv.li[j - cv.h0], w & ((1u << cb) - 1u));
+      }
     block_item_flush(la, ids, acc, i, sh);
   }
   final_flush(la, ids, acc, sh);
@@ -1357,7 +1357,7 @@ __global__ void k_pairs_hash(DevGraph g, const int32_t* items, int64_t nitems, u
 // 20) -- live in shared memory as 16-bit counts, two to a word, cleared for
 // every item (a count there is at most the rank's degree, below 2^16).
 template <bool BIG, int THREADS, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) k_pairs_grp(DevGraph g, const int32_t* items,
+__global__ void __launch_bounds__(THREADS, MINB) k_pairs_grp(DevGraph g, const unsigned long long* items,
                                                                          int64_t nitems, unsigned long long* qctr,
                                                                          TagScratch ts, TriLists tl3,
                                                                          const uint32_t* T, CoreView cv, AccSet acc,
@@ -1382,20 +1382,20 @@ __global__ void __launch_bounds__(THREADS, MINB) k_pairs_grp(DevGraph g, const i
     cluster_barrier();                         // also: the last item's reads are done
     const long long it = ld_cluster_s64(&sh_item, 0);
     if (it >= nitems) break;
-    const int64_t i = items[it];
+    const int64_t i = item_rank(items[it]);
     const int64_t b0 = g.R[i], e0 = g.R[i + 1];
     if (w.next_shared(ts.n, crank, csize)) cluster_barrier();
     if (win_words > 0) {
       for (int t = threadIdx.x; t < win_words; t += blockDim.x) win[t] = 0u;
       cluster_barrier();
     }
-    auto inc = [&](int32_t j) -> uint32_t {
+    auto inc = [&](int32_t j) -> unsigned long long {
       if (j >= wlo && j < whi) {
         const int64_t k = j - wlo;
         const unsigned sh16 = 16u * (unsigned)(k & 1);
-        return (atomicAdd(&win[k >> 1], 1u << sh16) >> sh16) & 0xffffu;
+        return pair_c2((atomicAdd(&win[k >> 1], 1u << sh16) >> sh16) & 0xffffu);
       }
-      return w.inc(j);
+      return pair_c2(w.inc(j));
     };
     u128 n13 = pair_wedges(g, b0, e0, gw, gnw, inc,
                            [&](int64_t cb, int64_t ce) { return pair_defer(pt, grp, cb, ce); });
@@ -1513,7 +1513,7 @@ __device__ __forceinline__ u128 pair_wedges_win(const DevGraph& g, longlong2* cu
         unsigned long long blk = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (u < stop) blk += pair_c2(inc(jj[u]));
+          if (u < stop) blk += inc(jj[u]);
         sh13.add(blk);
         if (stop < 4) {
           q += stop;
@@ -1539,71 +1539,69 @@ __device__ __forceinline__ u128 pair_wedges_win(const DevGraph& g, longlong2* cu
   return n13;
 }
 
+// The windows of one item: every wedge i - c - j with c in C[b0 .. e0) is
+// counted; term(old) is summed.  get(j) of the result reads the counts.
 template <bool BIG>
-__global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t* items, int64_t nitems,
-                                                        unsigned long long* qctr, PairWin pw, TriLists tl3,
-                                                        const uint32_t* T, CoreView cv, AccSet acc, PairTasks pt,
-                                                        unsigned* status) {
-  extern __shared__ uint32_t win[];
-  __shared__ u128 sh[32];
-  __shared__ int64_t sh_item;
-  __shared__ int sh_flag[2];                   // a window took increments (windows alternate)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int64_t grp = blockIdx.x;
-  const int64_t S = 2 * (int64_t)pw.win_words;
-  const int64_t par = pw.jbig & 1;
-  uint32_t* g16 = pw.g16 + grp * pw.g16_words + pw.woff;
-  uint4* const win4 = reinterpret_cast<uint4*>(win);
-  const int nv = pw.win_words >> 2;
-  longlong2* curs = pw.curs + grp * pw.curs_cap;
-  unsigned long long* side = pw.side + grp * (pw.n - pw.jbig);
+struct WinItem {
+  const PairWin& pw;
+  uint32_t* win;
+  uint32_t* g16;
+  longlong2* curs;
+  unsigned long long* side;
   uint32_t tag = 0;
-  const int ids[2] = {ACC_N13, ACC_N17};
-  LocalAcc<2> la;
-  la.zero();
-  for (int t = threadIdx.x; t < nv; t += blockDim.x) win4[t] = make_uint4(0u, 0u, 0u, 0u);
-  if (threadIdx.x == 0) sh_flag[0] = sh_flag[1] = 0;
-  while (true) {
-    const int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers publish the cleared window
-    if (it < 0) break;
-    const int64_t i = items[it];
-    const int64_t b0 = g.R[i], e0 = g.R[i + 1];
-    if (e0 - b0 > pw.curs_cap) {                // never: sized by the largest degree
-      if (threadIdx.x == 0) set_err(status, DEVERR_SCRATCH);
-      continue;
-    }
+  int64_t S, par, ktop = 0;
+  bool top_touched = false;
+  __device__ WinItem(const PairWin& p, uint32_t* w) : pw(p), win(w) {
+    const int64_t grp = blockIdx.x;
+    S = 2 * (int64_t)pw.win_words;
+    par = pw.jbig & 1;
+    g16 = pw.g16 + grp * pw.g16_words + pw.woff;
+    curs = pw.curs + grp * pw.curs_cap;
+    side = pw.side + grp * (pw.n - pw.jbig);
+  }
+  __device__ __forceinline__ void clear_window() {
+    uint4* const win4 = reinterpret_cast<uint4*>(win);
+    for (int t = threadIdx.x; t < (pw.win_words >> 2); t += blockDim.x) win4[t] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  template <class Term>
+  __device__ __forceinline__ u128 count(const DevGraph& g, const PairTasks& pt, int64_t i, int64_t b0, int64_t e0,
+                                        int* sh_flag, Term&& term) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int64_t grp = blockIdx.x;
+    uint4* const win4 = reinterpret_cast<uint4*>(win);
+    const int nv = pw.win_words >> 2;
     if (BIG && ++tag == 0xffffffffu) {          // tags used up: zero the 64-bit counters
       for (int64_t t = threadIdx.x; t < pw.n - pw.jbig; t += blockDim.x) side[t] = 0ull;
       tag = 1;
       __syncthreads();
     }
     const int64_t top = min(i, pw.jbig);        // ranks [0, top) are counted in windows
-    const int64_t ktop = (pw.jbig - top) / S;   // the window of rank top - 1
+    ktop = (pw.jbig - top) / S;                 // the window of rank top - 1
     const int64_t kbot = max(ktop, (pw.jbig - 1 - pw.n0) / S);   // the window of rank n0
-    u128 n13 = 0;
-    bool top_touched = false;
+    u128 sum = 0;
+    top_touched = false;
     for (int64_t k = kbot; k >= ktop; --k) {
       const int64_t lo = pw.jbig - (k + 1) * S;
       const uint32_t lo32 = (uint32_t)lo;       // -S <= lo < 2^31: 32-bit differences below
       const bool last = k == ktop;
       const int32_t hi = last ? 0x7fffffff : (int32_t)(pw.jbig - k * S);
       bool tch = false;
-      auto inc = [&](int32_t j) -> uint32_t {
+      auto inc = [&](int32_t j) -> unsigned long long {
         tch = true;
         if (BIG && j >= pw.jbig) {
           unsigned long long* q = &side[j - pw.jbig];
           atomicMax(q, (unsigned long long)tag << 32);
-          return (uint32_t)atomicAdd(q, 1ull);
+          return term((uint32_t)atomicAdd(q, 1ull));
         }
         const uint32_t q = (uint32_t)j - lo32;  // in [0, S)
         const unsigned s16 = (q & 1u) << 4;
-        return (atomicAdd(&win[q >> 1], 1u << s16) >> s16) & 0xffffu;
+        return term((atomicAdd(&win[q >> 1], 1u << s16) >> s16) & 0xffffu);
       };
-      n13 += pair_wedges_win(g, curs, b0, e0, wid, nw, k == kbot, last, hi, inc,
+      sum += pair_wedges_win(g, curs, b0, e0, wid, nw, k == kbot, last, hi, inc,
                              [&](int64_t cb, int64_t ce) { return pair_defer(pt, grp, cb, ce); });
       __syncthreads();                          // the window's long lists are appended as tasks
       const unsigned long long nt = __ldcg(&pt.n[grp]);
-      n13 += pair_run_tasks(g, pt, grp, nt, wid, nw, inc);
+      sum += pair_run_tasks(g, pt, grp, nt, wid, nw, inc);
       if (__any_sync(0xffffffffu, tch) && lane == 0) sh_flag[k & 1] = 1;
       __syncthreads();                          // the window's counts are complete; every thread has read nt
       const bool touched = sh_flag[k & 1] != 0;
@@ -1626,26 +1624,217 @@ __global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const int32_t
         __syncthreads();
       }
     }
-    const uint32_t lo_top32 = (uint32_t)(pw.jbig - (ktop + 1) * S), S32 = (uint32_t)S;
-    auto get = [&](int32_t j) -> uint32_t {
-      // j < min(i, jbig) lies in the top window exactly when j - lo_top (mod 2^32) is below S
-      const uint32_t q = (uint32_t)j - lo_top32;
-      if (q < S32) return (win[q >> 1] >> ((q & 1u) << 4)) & 0xffffu;
-      if (BIG && j >= pw.jbig) {
-        const unsigned long long v = __ldcg(&side[j - pw.jbig]);
-        return (uint32_t)(v >> 32) == tag ? (uint32_t)v : 0u;
-      }
-      const uint32_t t = (uint32_t)j + (uint32_t)par;
-      return (__ldcg(&g16[t >> 1]) >> ((t & 1u) << 4)) & 0xffffu;
-    };
-    u128 n17 = pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, get);
-    core_store_row(cv, i, threadIdx.x, blockDim.x, get);
-    la.v[0] += n13;
-    la.v[1] += n17;
-    __syncthreads();                            // the diamond reads of the window are done
-    if (top_touched)
-      for (int t = threadIdx.x; t < nv; t += blockDim.x) win4[t] = make_uint4(0u, 0u, 0u, 0u);
+    return sum;
+  }
+  __device__ __forceinline__ uint32_t get(int32_t j) const {
+    // j < min(i, jbig) lies in the top window exactly when j - lo_top (mod 2^32) is below S
+    const uint32_t q = (uint32_t)j - (uint32_t)(pw.jbig - (ktop + 1) * S);
+    if (q < (uint32_t)S) return (win[q >> 1] >> ((q & 1u) << 4)) & 0xffffu;
+    if (BIG && j >= pw.jbig) {
+      const unsigned long long v = __ldcg(&side[j - pw.jbig]);
+      return (uint32_t)(v >> 32) == tag ? (uint32_t)v : 0u;
+    }
+    const uint32_t t = (uint32_t)j + (uint32_t)par;
+    return (__ldcg(&g16[t >> 1]) >> ((t & 1u) << 4)) & 0xffffu;
+  }
+  // after the last get (a barrier between)
+  __device__ __forceinline__ void done(int* sh_flag) {
+    if (top_touched) clear_window();
     if (threadIdx.x == 0) sh_flag[0] = sh_flag[1] = 0;
+  }
+};
+
+template <bool BIG>
+__global__ void __launch_bounds__(1024, 1) k_pairs_win(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                        unsigned long long* qctr, PairWin pw, TriLists tl3,
+                                                        const uint32_t* T, CoreView cv, AccSet acc, PairTasks pt,
+                                                        unsigned* status) {
+  extern __shared__ uint32_t win[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  __shared__ int sh_flag[2];                   // a window took increments (windows alternate)
+  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  WinItem<BIG> wi(pw, win);
+  const int ids[2] = {ACC_N13, ACC_N17};
+  LocalAcc<2> la;
+  la.zero();
+  wi.clear_window();
+  if (threadIdx.x == 0) sh_flag[0] = sh_flag[1] = 0;
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers publish the cleared window
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.R[i + 1];
+    if (e0 - b0 > pw.curs_cap) {                // never: sized by the largest degree
+      if (threadIdx.x == 0) set_err(status, DEVERR_SCRATCH);
+      continue;
+    }
+    la.v[0] += wi.count(g, pt, i, b0, e0, sh_flag, [](uint32_t old) { return pair_c2(old); });
+    auto get = [&](int32_t j) -> uint32_t { return wi.get(j); };
+    la.v[1] += pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, get);
+    core_store_row(cv, i, threadIdx.x, blockDim.x, get);
+    __syncthreads();                            // the diamond reads of the window are done
+    wi.done(sh_flag);
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// ---------------------------------------------------------------- 4-cycles
+// Second pass of one item (Thm 5's rule): every wedge i - k - j adds
+// w(i,j) - 1 to the edges (i,k) and (k,j).  Lists of up to PAIR_SHORT entries
+// are walked by one lane each, longer ones by the warp.
+template <class Get>
+__device__ __forceinline__ void cycle4_edges(const DevGraph& g, int64_t b0, int64_t e0, int64_t gw, int64_t gnw,
+                                             unsigned long long* C4raw, Get&& get) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t pbase = b0 + gw; pbase < e0; pbase += gnw * 32) {
+    const int64_t p = pbase + (int64_t)lane * gnw;
+    int64_t kb_l = 0;
+    int len_l = 0;
+    if (p < e0) {
+      kb_l = g.R[g.C[p]];
+      len_l = (int)(g.rev[p] - kb_l);           // N(k) below i ends at the slot of i
+    }
+    if (len_l <= PAIR_SHORT) {
+      unsigned long long sk = 0;
+      for (int q = 0; q < len_l; q += 4) {
+        int32_t jj[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) jj[u] = q + u < len_l ? g.C[kb_l + q + u] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (jj[u] >= 0) {
+            const unsigned long long c = get(jj[u]) - 1u;
+            if (c) {
+              atomicAdd(&C4raw[kb_l + q + u], c);
+              sk += c;
+            }
+          }
+      }
+      if (sk) atomicAdd(&C4raw[p], sk);
+    }
+    unsigned longm = __ballot_sync(0xffffffffu, len_l > PAIR_SHORT);
+    while (longm) {
+      const int k = __ffs(longm) - 1;
+      longm &= longm - 1;
+      const int64_t kb = __shfl_sync(0xffffffffu, kb_l, k);
+      const int len = __shfl_sync(0xffffffffu, len_l, k);
+      const int32_t* L = g.C + kb;
+      unsigned long long sk = 0;
+      for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
+        int32_t jj[SWEEP_ILP];
+#pragma unroll
+        for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < SWEEP_ILP; ++u)
+          if (jj[u] >= 0) {
+            const unsigned long long c = get(jj[u]) - 1u;
+            if (c) {
+              atomicAdd(&C4raw[kb + q + 32 * u], c);
+              sk += c;
+            }
+          }
+      }
+      sk = warp_sum_u64(sk);
+      if (lane == 0 && sk) atomicAdd(&C4raw[pbase + (int64_t)k * gnw], sk);
+    }
+  }
+}
+
+// Heavy items of a single graph: the wedges to lower neighbours counted in the
+// same windows as the pair sweep's.
+template <bool BIG>
+__global__ void __launch_bounds__(1024, 1) k_cycles4_win(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                          unsigned long long* qctr, PairWin pw, PairTasks pt,
+                                                          unsigned long long* C4raw, AccSet acc, unsigned* status) {
+  extern __shared__ uint32_t win[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  __shared__ int sh_flag[2];
+  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  WinItem<BIG> wi(pw, win);
+  const int ids[1] = {ACC_C4};
+  LocalAcc<1> la;
+  la.zero();
+  wi.clear_window();
+  if (threadIdx.x == 0) sh_flag[0] = sh_flag[1] = 0;
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.op[i];
+    if (e0 - b0 > pw.curs_cap) {
+      if (threadIdx.x == 0) set_err(status, DEVERR_SCRATCH);
+      continue;
+    }
+    const u128 c4 = wi.count(g, pt, i, b0, e0, sh_flag, [](uint32_t old) { return (unsigned long long)old; });
+    la.v[0] += c4;
+    if (__syncthreads_or(c4 != 0)) cycle4_edges(g, b0, e0, wid, nw, C4raw, [&](int32_t j) { return wi.get(j); });
+    __syncthreads();
+    wi.done(sh_flag);
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Heavy items of a union: dense tagged counters per CTA.
+template <bool BIG>
+__global__ void __launch_bounds__(512, 2) k_cycles4_tag(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                        unsigned long long* qctr, TagScratch ts,
+                                                        unsigned long long* C4raw, AccSet acc) {
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  TaggedCounters<BIG> w(ts);
+  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int ids[1] = {ACC_C4};
+  LocalAcc<1> la;
+  la.zero();
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.op[i];
+    if (w.next(g.n)) __syncthreads();
+    const u128 c4 = pair_wedges(g, b0, e0, wid, nw, [&](int32_t j) -> unsigned long long { return w.inc(j); },
+                                [](int64_t, int64_t) { return false; });
+    la.v[0] += c4;
+    if (__syncthreads_or(c4 != 0)) cycle4_edges(g, b0, e0, wid, nw, C4raw, [&](int32_t j) { return w.get(j); });
+    block_item_flush(la, ids, acc, i, sh);
+    __syncthreads();                            // the next item's counts must not meet these reads
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Light and medium items: one CTA of THREADS threads per item, w(i, .) in a
+// packed hash table.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_cycles4_hash(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                         unsigned long long* qctr, int cb, int max_log,
+                                                         unsigned long long* C4raw, AccSet acc, unsigned* status) {
+  extern __shared__ uint4 hash_smem[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  const int wid = threadIdx.x >> 5, nw = THREADS / 32;
+  PackedHash H{reinterpret_cast<uint32_t*>(hash_smem), cb, 0};
+  const int ids[1] = {ACC_C4};
+  LocalAcc<1> la;
+  la.zero();
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.op[i];
+    H.log = min(max_log, item_log(items[it]));
+    H.clear(threadIdx.x, THREADS);
+    __syncthreads();
+    bool full = false;
+    const u128 c4 = pair_wedges(g, b0, e0, wid, nw, [&](int32_t j) -> unsigned long long {
+      return H.inc(j, full);
+    }, [](int64_t, int64_t) { return false; });
+    if (full) set_err(status, DEVERR_SCRATCH);
+    la.v[0] += c4;
+    if (__syncthreads_or(c4 != 0)) cycle4_edges(g, b0, e0, wid, nw, C4raw, [&](int32_t j) { return H.get(j); });
     block_item_flush(la, ids, acc, i, sh);
   }
   final_flush(la, ids, acc, sh);
@@ -1942,113 +2131,229 @@ __global__ void __launch_bounds__(WHEEL_THREADS, 1) k_wheels_cta(DevGraph g, int
 // The paths whose own a or b is counted by w' are the directed tailed
 // triangles, subtracted through ACC_N8Z (pass A).
 // ============================================================================
-template <bool BIG>
-__global__ void __launch_bounds__(512, 2) k_cycles5(DevGraph g, unsigned long long* qctr, TagScratch ts,
-                                                   SweepScratch ss, AccSet acc, Owner own) {
+// The lists N+(b) of up to 32 vertices b (lane l holds the l-th list [cb_l, ce_l)
+// and its factor f_l; empty lists have cb_l = ce_l): sum of f * get(j) over
+// their entries.  Lists of up to PAIR_SHORT entries are walked by one lane each.
+template <class Get>
+__device__ __forceinline__ u128 cycle5_lists(const DevGraph& g, int64_t cb_l, int64_t ce_l, uint32_t f_l, Get&& get) {
+  const int lane = threadIdx.x & 31;
+  const int len_l = (int)(ce_l - cb_l);
+  u128 sum = 0;
+  if (len_l <= PAIR_SHORT) {
+    const int32_t* L = g.C + cb_l;
+    unsigned long long s_ = 0;
+    for (int q = 0; q < len_l; q += 4) {
+      int32_t jj[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) jj[u] = q + u < len_l ? L[q + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (jj[u] >= 0) s_ += get(jj[u]);
+    }
+    sum += (u128)s_ * f_l;
+  }
+  unsigned longm = __ballot_sync(0xffffffffu, len_l > PAIR_SHORT);
+  while (longm) {
+    const int k = __ffs(longm) - 1;
+    longm &= longm - 1;
+    const int32_t* L = g.C + __shfl_sync(0xffffffffu, cb_l, k);
+    const int len = __shfl_sync(0xffffffffu, len_l, k);
+    const uint32_t f = __shfl_sync(0xffffffffu, f_l, k);
+    unsigned long long s_ = 0;
+    for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
+      int32_t jj[SWEEP_ILP];
+#pragma unroll
+      for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
+#pragma unroll
+      for (int u = 0; u < SWEEP_ILP; ++u)
+        if (jj[u] >= 0) s_ += get(jj[u]);
+    }
+    sum += (u128)s_ * f;
+  }
+  return sum;
+}
+
+// visit(j) for every entry of up to 32 lists (lane l holds the l-th), short
+// ones by one lane each.
+template <class Visit>
+__device__ __forceinline__ void lists_each(const DevGraph& g, int64_t cb_l, int64_t ce_l, Visit&& visit) {
+  const int lane = threadIdx.x & 31;
+  const int len_l = (int)(ce_l - cb_l);
+  if (len_l <= PAIR_SHORT) {
+    const int32_t* L = g.C + cb_l;
+    for (int q = 0; q < len_l; q += 4) {
+      int32_t jj[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) jj[u] = q + u < len_l ? L[q + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (jj[u] >= 0) visit(jj[u]);
+    }
+  }
+  unsigned longm = __ballot_sync(0xffffffffu, len_l > PAIR_SHORT);
+  while (longm) {
+    const int k = __ffs(longm) - 1;
+    longm &= longm - 1;
+    const int32_t* L = g.C + __shfl_sync(0xffffffffu, cb_l, k);
+    const int len = __shfl_sync(0xffffffffu, len_l, k);
+    for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
+      int32_t jj[SWEEP_ILP];
+#pragma unroll
+      for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
+#pragma unroll
+      for (int u = 0; u < SWEEP_ILP; ++u)
+        if (jj[u] >= 0) visit(jj[u]);
+    }
+  }
+}
+
+// The increments of one item: w'(i, .) from c < i (every j in N(c)) and c > i
+// (j in N+(c)); P2(i, .) from a in N-(i) (b in N+(a)).  j = b = i is left out.
+template <class IncW, class IncP>
+__device__ __forceinline__ void cycle5_counts(const DevGraph& g, int64_t i, int64_t b0, int64_t o, int64_t e0,
+                                              int64_t gw, int64_t gnw, IncW&& incw, IncP&& incp) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t pbase = b0 + gw; pbase < e0; pbase += gnw * 32) {
+    const int64_t p = pbase + (int64_t)lane * gnw;
+    int64_t cb_l = 0, ce_l = 0, cm_l = 0;       // the list; from cm_l on also P2
+    if (p < e0) {
+      const int32_t c = g.C[p];
+      const int64_t co = g.op[c];
+      ce_l = g.R[c + 1];
+      cb_l = p < o ? g.R[c] : co;
+      cm_l = p < o ? co : ce_l;
+    }
+    lists_each(g, cb_l, ce_l, [&](int32_t j) { if (j != i) incw(j); });
+    lists_each(g, cm_l, ce_l, [&](int32_t j) { if (j != i) incp(j); });
+  }
+}
+
+// Light and medium items: one CTA of THREADS threads per item, w'(i, .) and
+// P2(i, .) in two packed hash tables; the distinct b are the used words of the
+// second.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_cycles5_hash(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                         unsigned long long* qctr, int cb, int max_log, AccSet acc,
+                                                         unsigned* status) {
+  extern __shared__ uint4 hash_smem[];
   __shared__ u128 sh[32];
   __shared__ int64_t sh_item;
-  TaggedCounters<BIG> wp(ts);                                                         // w'(i, .)
-  uint32_t* p2 = ss.cnt2 + (int64_t)blockIdx.x * ss.n;                            // P2(i, .), with a list
-  int32_t* tl2 = ss.touched2 + (int64_t)blockIdx.x * ss.n;
-  unsigned* nt = ss.ntouched + 2 * blockIdx.x;
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = THREADS / 32;
+  PackedHash Hw{reinterpret_cast<uint32_t*>(hash_smem), cb, 0}, Hp = Hw;
   const int ids[1] = {ACC_N8M};
   LocalAcc<1> la;
   la.zero();
   while (true) {
-    int64_t it = next_item(qctr, own.count(g.n), &sh_item);
+    const int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers end the last item's reads
     if (it < 0) break;
-    int64_t i = own.item(g.n, it);
-    int64_t b0 = g.R[i], o = g.op[i], e0 = g.R[i + 1];
-    if (o == b0) continue;                      // needs an in-neighbour a
-    wp.next(ts.n);
-    if (threadIdx.x == 0) nt[1] = 0;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], o = g.op[i], e0 = g.R[i + 1];
+    Hw.log = min(max_log, item_log(items[it]));
+    Hp.log = min(max_log, item_log2(items[it]));
+    Hp.tab = Hw.tab + (1 << Hw.log);
+    Hw.clear(threadIdx.x, THREADS);
+    Hp.clear(threadIdx.x, THREADS);
     __syncthreads();
-    // w'(i, .): c < i -> every j in N(c); c > i -> j in N+(c).  Lists are
-    // fetched 32 per warp (lane k the k-th), SWEEP_ILP entries in flight per lane.
-    for (int64_t pbase = b0 + wid; pbase < e0; pbase += (int64_t)nw * 32) {
-      int64_t p = pbase + (int64_t)lane * nw;
-      int64_t cb_l = 0, ce_l = 0;
-      if (p < e0) {
-        int32_t c = g.C[p];
-        cb_l = (p < o) ? g.R[c] : g.op[c];
-        ce_l = g.R[c + 1];
-      }
-      int kmax = (int)min((int64_t)32, (e0 - pbase + nw - 1) / nw);
-      for (int k = 0; k < kmax; ++k) {
-        int64_t cb = __shfl_sync(0xffffffffu, cb_l, k), ce = __shfl_sync(0xffffffffu, ce_l, k);
-        const int32_t* L = g.C + cb;            // 32-bit offsets: a row has fewer than 2^31 entries
-        const int len = (int)(ce - cb);
-        for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
-          int32_t jj[SWEEP_ILP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : (int32_t)i;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u)
-            if (jj[u] != i) wp.add(jj[u]);
-        }
-      }
-    }
-    // P2(i, .): a in N-(i), b in N+(a)
-    for (int64_t pbase = b0 + wid; pbase < o; pbase += (int64_t)nw * 32) {
-      int64_t p = pbase + (int64_t)lane * nw;
-      int64_t cb_l = 0, ce_l = 0;
-      if (p < o) {
-        int32_t a = g.C[p];
-        cb_l = g.op[a];
-        ce_l = g.R[a + 1];
-      }
-      int kmax = (int)min((int64_t)32, (o - pbase + nw - 1) / nw);
-      for (int k = 0; k < kmax; ++k) {
-        int64_t cb = __shfl_sync(0xffffffffu, cb_l, k), ce = __shfl_sync(0xffffffffu, ce_l, k);
-        const int32_t* L = g.C + cb;
-        const int len = (int)(ce - cb);
-        for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
-          int32_t bb[SWEEP_ILP];
-          uint32_t oo[SWEEP_ILP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) bb[u] = q + 32 * u < len ? L[q + 32 * u] : (int32_t)i;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) oo[u] = bb[u] != i ? atomicAdd(&p2[bb[u]], 1u) : 1u;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) warp_append(tl2, &nt[1], oo[u] == 0, bb[u]);
-        }
-      }
-    }
+    bool full = false;
+    cycle5_counts(g, i, b0, o, e0, wid, nw, [&](int32_t j) { Hw.inc(j, full); }, [&](int32_t j) { Hp.inc(j, full); });
+    if (full) set_err(status, DEVERR_SCRATCH);
     __syncthreads();
-    unsigned n2 = nt[1];
-    // sum over the distinct b of P2(i, b) * sum_{j in N+(b)} w'(i, j); the
-    // b's are fetched 32 per warp
-    for (unsigned tb = (unsigned)wid * 32; tb < n2; tb += (unsigned)nw * 32) {
-      unsigned t = tb + lane;
+    for (int tb = wid * 32; tb < (1 << Hp.log); tb += THREADS) {
+      const uint32_t w = Hp.tab[tb + lane];
+      const bool used = w != PackedHash::EMPTY;
+      if (!__any_sync(0xffffffffu, used)) continue;
       int64_t cb_l = 0, ce_l = 0;
-      uint32_t pk_l = 0;
-      if (t < n2) {
-        int32_t b = tl2[t];
+      if (used) {
+        const int32_t b = (int32_t)(w >> cb);
         cb_l = g.op[b];
         ce_l = g.R[b + 1];
-        pk_l = p2[b];
       }
-      int kmax = (int)min(32u, n2 - tb);
-      for (int k = 0; k < kmax; ++k) {
-        int64_t cb = __shfl_sync(0xffffffffu, cb_l, k), ce = __shfl_sync(0xffffffffu, ce_l, k);
-        uint32_t pk = __shfl_sync(0xffffffffu, pk_l, k);
-        unsigned long long s_ = 0;
-        const int32_t* L = g.C + cb;
-        const int len = (int)(ce - cb);
-        for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
-          int32_t jj[SWEEP_ILP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
-#pragma unroll
-          for (int u = 0; u < SWEEP_ILP; ++u)
-            if (jj[u] >= 0) s_ += wp.get(jj[u]);
-        }
-        la.v[0] += (u128)s_ * pk;
+      la.v[0] += cycle5_lists(g, cb_l, ce_l, w & ((1u << cb) - 1u), [&](int32_t j) -> uint32_t { return Hw.get(j); });
+    }
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Heavy items: one 1024-thread CTA per SM.  The counts of the ranks
+// [wlo, jbig) -- the top ones below the 64-bit side array, where the j, two
+// steps up the order from a, concentrate -- live in shared memory, w'(i, r) in
+// the low and P2(i, r) in the high 16 bits of a word (both at most the rank's
+// degree, below 2^16); lower ranks use tagged counters and a touched list in
+// global memory.
+template <bool BIG>
+__global__ void __launch_bounds__(1024, 1) k_cycles5(DevGraph g, const unsigned long long* items, int64_t nitems,
+                                                     unsigned long long* qctr, TagScratch ts, SweepScratch ss,
+                                                     AccSet acc, int64_t wlo, int win_words) {
+  extern __shared__ uint32_t win[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  __shared__ unsigned nt;
+  TaggedCounters<BIG> wp(ts);                                                         // w'(i, .) outside the window
+  uint32_t* p2 = ss.cnt2 + (int64_t)blockIdx.x * ss.n;                            // P2(i, .) there, with a list
+  int32_t* tl2 = ss.touched2 + (int64_t)blockIdx.x * ss.n;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t wlo32 = (uint32_t)wlo, nwin = (uint32_t)win_words;
+  const int ids[1] = {ACC_N8M};
+  LocalAcc<1> la;
+  la.zero();
+  for (int t = threadIdx.x; t < win_words; t += blockDim.x) win[t] = 0u;
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], o = g.op[i], e0 = g.R[i + 1];
+    wp.next(ts.n);
+    if (threadIdx.x == 0) nt = 0;
+    __syncthreads();
+    cycle5_counts(g, i, b0, o, e0, wid, nw,
+                  [&](int32_t j) {
+                    const uint32_t q = (uint32_t)j - wlo32;
+                    if (q < nwin) atomicAdd(&win[q], 1u);
+                    else wp.add(j);
+                  },
+                  [&](int32_t b) {
+                    const uint32_t q = (uint32_t)b - wlo32;
+                    if (q < nwin) {
+                      atomicAdd(&win[q], 1u << 16);
+                    } else {
+                      const bool first = atomicAdd(&p2[b], 1u) == 0;
+                      if (first) tl2[atomicAdd(&nt, 1u)] = b;
+                    }
+                  });
+    __syncthreads();
+    auto get = [&](int32_t j) -> uint32_t {
+      const uint32_t q = (uint32_t)j - wlo32;
+      return q < nwin ? win[q] & 0xffffu : wp.get(j);
+    };
+    // sum over the distinct b of P2(i, b) * sum_{j in N+(b)} w'(i, j)
+    const unsigned n2 = nt;
+    for (uint32_t tb = (uint32_t)wid * 32; tb < nwin; tb += (uint32_t)nw * 32) {
+      const uint32_t f = tb + lane < nwin ? win[tb + lane] >> 16 : 0u;
+      if (!__any_sync(0xffffffffu, f != 0)) continue;
+      int64_t cb_l = 0, ce_l = 0;
+      if (f) {
+        const int64_t b = wlo + tb + lane;
+        cb_l = g.op[b];
+        ce_l = g.R[b + 1];
       }
+      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, get);
+    }
+    for (unsigned tb = (unsigned)wid * 32; tb < n2; tb += (unsigned)nw * 32) {
+      const unsigned t = tb + lane;
+      int64_t cb_l = 0, ce_l = 0;
+      uint32_t f = 0;
+      if (t < n2) {
+        const int32_t b = tl2[t];
+        cb_l = g.op[b];
+        ce_l = g.R[b + 1];
+        f = p2[b];
+      }
+      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, get);
     }
     __syncthreads();
     for (unsigned t = threadIdx.x; t < n2; t += blockDim.x) p2[tl2[t]] = 0;
+    for (int t = threadIdx.x; t < win_words; t += blockDim.x) win[t] = 0u;
     block_item_flush(la, ids, acc, i, sh);
     __syncthreads();
   }
@@ -2560,8 +2865,7 @@ static const void* pairs_grp_fn(bool big, int shape) {
 // The windowed form (k_pairs_win, the default): one 1024-thread CTA per SM,
 // the window as wide as shared memory allows, but no wider than the ranks
 // [n0, jbig) need.
-static cudaError_t plan_pair_windows(bool big, int sms, int64_t n0, int64_t jbig, int smem_optin, PairPlan* plan) {
-  const void* k = big ? (const void*)k_pairs_win<true> : (const void*)k_pairs_win<false>;
+static cudaError_t plan_pair_windows(const void* k, int sms, int64_t n0, int64_t jbig, int smem_optin, PairPlan* plan) {
   cudaFuncAttributes fa;
   ESC_TRY(cudaFuncGetAttributes(&fa, k));
   ESC_TRY(allow_max_smem(k, smem_optin));     // the limit is the same for every graph
@@ -2594,7 +2898,10 @@ static cudaError_t plan_pair_clusters(bool big, int sms, size_t arr_bytes, int64
   // is twice as wide as two 512-thread CTAs' each); without the window,
   // (512, 2).
   const int wmode = env_int("ESC_PAIR_WINDOW", union_of_graphs ? 2 : 3);
-  if (wmode >= 3 && env_int("ESC_PAIR_CLUSTER", 1) == 1) return plan_pair_windows(big, sms, n0, jbig, smem_optin, plan);
+  if (wmode >= 3 && env_int("ESC_PAIR_CLUSTER", 1) == 1) {
+    const void* kw = big ? (const void*)k_pairs_win<true> : (const void*)k_pairs_win<false>;
+    return plan_pair_windows(kw, sms, n0, jbig, smem_optin, plan);
+  }
   const bool window = env_int("ESC_PAIR_CLUSTER", 1) == 1 && wmode != 1;
   plan->shape = std::min(2, env_int("ESC_PAIR_SHAPE", window ? 3 : 2) - 1);
   plan->threads = plan->shape == 2 ? 1024 : 512;
@@ -2658,7 +2965,7 @@ static cudaError_t plan_pair_clusters(bool big, int sms, size_t arr_bytes, int64
   return cudaSuccess;
 }
 
-static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGraph& g, const int32_t* items,
+static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGraph& g, const unsigned long long* items,
                                     int64_t nitems, unsigned long long* qctr, const TagScratch& ts,
                                     const TriLists& tl3, const uint32_t* T, const CoreView& cv, const AccSet& accs,
                                     const PairTasks& pt, cudaStream_t s) {
@@ -2777,7 +3084,6 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   cudaMemsetAsync(T, 0, sizeof(uint32_t) * (nnz + 1), s);
   cudaMemsetAsync(K4e, 0, sizeof(unsigned long long) * (nnz + 1), s);
   cudaMemsetAsync(C4e, 0, sizeof(unsigned long long) * (nnz + 1), s);
-  cudaMemsetAsync(C4v, 0, sizeof(unsigned long long) * (n + 1), s);
   cudaMemsetAsync(acc, 0, sizeof(Acc128) * ACC_COUNT * G, s);
   DevBuf b_vg, b_narr, b_marr;
   ESC_TRY(b_narr.alloc(sizeof(unsigned long long) * G));
@@ -2908,11 +3214,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // With four_only, only the 4-cycle sweep runs; the lists, pairs, wheels and
   // 5-cycles (and their work space) are skipped.
   const bool five = !cfg.four_only;
-  DevBuf b_cntA, b_cntB, b_cntC, b_cntD, b_tlD, b_ntC;
-  size_t sw = five ? sizeof(uint32_t) * (size_t)n * grid_sweep + 16 : 16;
-  ESC_TRY(b_cntD.alloc(sw)); ESC_TRY(b_tlD.alloc(sw));
-  ESC_TRY(b_ntC.alloc(sizeof(unsigned) * 2 * grid_sweep));
-  cudaMemsetAsync(b_cntD.p, 0, sw, s);
+  DevBuf b_cntA, b_cntB, b_cntC, b_cntD, b_tlD;
 
   // common-neighbour list offsets and sizes
   DevBuf b_off, b_offp, b_U, b_P, b_gh;
@@ -2929,21 +3231,33 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     cudaMemcpyAsync(&ulen, off + nnz, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(&plen, offp + nnz, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   }
-  // pair-sweep items by wedge count (light / medium / heavy lists)
-  DevBuf b_plist, b_pctr;
-  ESC_TRY(b_plist.alloc(five ? sizeof(int32_t) * 3 * (size_t)(n + 1) : 16));
-  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 9));
-  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 9, s);
-  unsigned long long pcnt[9] = {0};
-  if (five && n > 0) {
-    // item classes: hash capacities bound the light and medium classes
-    // (ESC_PAIR_SMALL_W / ESC_PAIR_LARGE_W lower them for tuning)
-    const long long w_small = std::min<long long>(PH_SMALL_W, env_int("ESC_PAIR_SMALL_W", PH_SMALL_W + 1) - 1);
-    const long long w_large = std::min<long long>(PH_LARGE_W, env_int("ESC_PAIR_LARGE_W", PH_LARGE_W + 1) - 1);
-    (k_pair_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T, b_plist.as<int32_t>(),
-                                                                b_pctr.as<unsigned long long>(), w_small,
-                                                                std::max(w_small, w_large), own), note_launch());
-    cudaMemcpyAsync(pcnt, b_pctr.p, sizeof(pcnt), cudaMemcpyDeviceToHost, s);
+  // items of the pair, 4-cycle and 5-cycle sweeps (light / medium / heavy lists)
+  DevBuf b_plist, b_list4, b_list5, b_pctr;
+  const size_t list_b = sizeof(unsigned long long) * 3 * (size_t)(n + 1);
+  ESC_TRY(b_plist.alloc(five ? list_b : 16));
+  ESC_TRY(b_list4.alloc(list_b));
+  ESC_TRY(b_list5.alloc(five ? list_b : 16));
+  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 27));
+  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 27, s);
+  ItemLists ilp{b_plist.as<unsigned long long>(), b_pctr.as<unsigned long long>()};
+  ItemLists il4{b_list4.as<unsigned long long>(), ilp.cnt + 9}, il5{b_list5.as<unsigned long long>(), ilp.cnt + 18};
+  unsigned long long cnts[27] = {0};
+  const unsigned long long *pcnt = cnts, *cnt4 = cnts + 9, *cnt5 = cnts + 18;
+  // count bits of a packed word: every rank is below 2^(32 - cb) - 1
+  int cb = 31;
+  while (cb > 1 && n >= ((int64_t)1 << (32 - cb)) - 1) --cb;
+  if (n > 0) {
+    // ESC_PAIR_SMALL_W / ESC_PAIR_LARGE_W and ESC_CYCLE_SMALL_W / ESC_CYCLE_LARGE_W lower the classes' limits (tests)
+    const unsigned long long* n_arr = b_narr.as<unsigned long long>();
+    auto limit = [](const char* name, long long m) { return std::min<long long>(m, env_int(name, (int)m + 1) - 1); };
+    if (five)
+      (k_pair_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
+           g, T, ilp, limit("ESC_PAIR_SMALL_W", IT_LIGHT_M), limit("ESC_PAIR_LARGE_W", IT_MEDIUM_M), cb, accs.vg, n_arr,
+           own), note_launch());
+    (k_cycle_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
+         g, il4, il5, !five, limit("ESC_CYCLE_SMALL_W", IT_LIGHT_M), limit("ESC_CYCLE_LARGE_W", IT_MEDIUM_M),
+         limit("ESC_CYCLE_LARGE_W", IT5_MEDIUM_M), cb, accs.vg, n_arr, own), note_launch());
+    cudaMemcpyAsync(cnts, b_pctr.p, sizeof(cnts), cudaMemcpyDeviceToHost, s);
   }
   std::vector<int64_t> hR(n + 1, 0);
   if (n > 0) cudaMemcpyAsync(hR.data(), o.R, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s);
@@ -3031,12 +3345,14 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // the heavy pair items: clusters sharing one counter array each
   PairPlan pplan;
   int64_t n0 = 0;                               // first rank of degree >= 1 (lower ranks are never counted)
-  if (five && pcnt[2] > 0) {
+  if (n > 0) {
     {
       int64_t lo = 0, hi = n;
       while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= 1) hi = mid; else lo = mid + 1; }
       n0 = lo;
     }
+  }
+  if (five && pcnt[2] > 0) {
     size_t arr_bytes = sizeof(uint32_t) * (size_t)std::max<int64_t>(jbig - n0, 0) +
                        sizeof(unsigned long long) * (size_t)(n - jbig);
     ESC_TRY(plan_pair_clusters(jbig < n, sms, arr_bytes, n0, jbig, smem_optin, cfg.num_graphs > 1, &pplan));
@@ -3053,42 +3369,73 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     ptasks.q = b_ptq.as<long long>();
     ptasks.n = b_ptn.as<unsigned long long>();
   }
-  size_t sw32 = sizeof(uint32_t) * (size_t)jbig * grid_sweep + 16;
-  size_t sw64 = sizeof(unsigned long long) * (size_t)(n - jbig) * grid_sweep + 16;
+  // heavy 4-cycle items: windows for a single graph, tagged counters for a union
+  const bool win4 = cnt4[2] > 0 && G == 1, tag4 = cnt4[2] > 0 && G > 1;
+  PairPlan plan4;
+  DevBuf b_ptq4, b_ptn4;
+  PairTasks ptasks4{nullptr, nullptr, 0};
+  if (win4) {
+    ESC_TRY(plan_pair_windows(jbig < n ? (const void*)k_cycles4_win<true> : (const void*)k_cycles4_win<false>, sms, n0,
+                              jbig, smem_optin, &plan4));
+    ptasks4.cap = (int64_t)(cnt4[6] / PAIR_TASK) + maxdeg + 1;
+    ESC_TRY(b_ptq4.alloc(sizeof(long long) * 2 * (size_t)ptasks4.cap * plan4.nclusters));
+    ESC_TRY(b_ptn4.alloc(sizeof(unsigned long long) * (size_t)plan4.nclusters));
+    cudaMemsetAsync(b_ptn4.p, 0, sizeof(unsigned long long) * (size_t)plan4.nclusters, s);
+    ptasks4.q = b_ptq4.as<long long>();
+    ptasks4.n = b_ptn4.as<unsigned long long>();
+  }
+  // heavy 5-cycle items: a shared-memory window over the top ranks, one CTA per SM
+  // (ESC_CYCLE_WIN_WORDS: a narrower one, so that small graphs count outside it too; tests)
+  const int win5_words = (int)std::min<int64_t>(
+      std::min((smem_optin - 4096) / 4, env_int("ESC_CYCLE_WIN_WORDS", 1 << 30)), std::max<int64_t>(jbig - n0, 1));
+  const int64_t wlo5 = jbig - win5_words;
+  const bool heavy5 = five && cnt5[2] > 0, below5 = heavy5 && (wlo5 > n0 || jbig < n);   // some counters outside it
+  size_t sw32 = tag4 ? sizeof(uint32_t) * (size_t)jbig * grid_sweep + 16 : 16;
+  size_t sw64 = tag4   ? sizeof(unsigned long long) * (size_t)(n - jbig) * grid_sweep + 16
+                : win4 ? sizeof(unsigned long long) * (size_t)(n - jbig) * plan4.nclusters + 16
+                       : 16;
   size_t sw32p = five && !pplan.windowed ? sizeof(uint32_t) * (size_t)jbig * pplan.nclusters + 16 : 16;
   size_t sw64p = five ? sizeof(unsigned long long) * (size_t)(n - jbig) * pplan.nclusters + 16 : 16;
-  size_t sw32c = five ? sw32 : 16, sw64c = five ? sw64 : 16;
+  size_t sw32c = below5 ? sizeof(uint32_t) * (size_t)jbig * sms + 16 : 16;
+  size_t sw64c = below5 ? sizeof(unsigned long long) * (size_t)(n - jbig) * sms + 16 : 16;
+  size_t swp2 = below5 ? sizeof(uint32_t) * (size_t)n * sms + 16 : 16;
   DevBuf b_bigA, b_bigB, b_bigC;
   ESC_TRY(b_cntA.alloc(sw32)); ESC_TRY(b_bigA.alloc(sw64));
   ESC_TRY(b_cntB.alloc(sw32p)); ESC_TRY(b_bigB.alloc(sw64p));
   ESC_TRY(b_cntC.alloc(sw32c)); ESC_TRY(b_bigC.alloc(sw64c));
-  cudaMemsetAsync(b_cntA.p, 0, sw32, s);
-  cudaMemsetAsync(b_cntB.p, 0, sw32p, s);
-  cudaMemsetAsync(b_cntC.p, 0, sw32c, s);
-  cudaMemsetAsync(b_bigA.p, 0, sw64, s);
-  cudaMemsetAsync(b_bigB.p, 0, sw64p, s);
-  cudaMemsetAsync(b_bigC.p, 0, sw64c, s);
+  ESC_TRY(b_cntD.alloc(swp2)); ESC_TRY(b_tlD.alloc(swp2));
+  auto zero = [&](const DevBuf& b, size_t bytes) {
+    if (bytes > 16) cudaMemsetAsync(b.p, 0, bytes, s);
+  };
+  zero(b_cntA, sw32); zero(b_bigA, sw64);
+  zero(b_cntB, sw32p); zero(b_bigB, sw64p);
+  zero(b_cntC, sw32c); zero(b_bigC, sw64c);
+  zero(b_cntD, swp2);
   TagScratch tsA{b_cntA.as<uint32_t>(), b_bigA.as<unsigned long long>(), jbig, n};
   TagScratch tsB{b_cntB.as<uint32_t>(), b_bigB.as<unsigned long long>(), jbig, n};
   // the windowed heavy items: per CTA the dense 16-bit counts and the list cursors
-  DevBuf b_g16, b_curs;
-  PairWin pwin{};
-  if (five && pplan.windowed) {
-    pwin.g16_words = ((n + 2) / 2 + 4 + 3) & ~(int64_t)3;
-    pwin.curs_cap = std::max<int64_t>(maxdeg, 1);
-    ESC_TRY(b_g16.alloc(sizeof(uint32_t) * (size_t)pwin.g16_words * pplan.nclusters));
-    ESC_TRY(b_curs.alloc(sizeof(longlong2) * (size_t)pwin.curs_cap * pplan.nclusters));
-    pwin.g16 = b_g16.as<uint32_t>();
-    pwin.curs = b_curs.as<longlong2>();
-    pwin.side = b_bigB.as<unsigned long long>();      // zeroed above
-    pwin.jbig = jbig;
-    pwin.n = n;
-    pwin.n0 = n0;
-    pwin.win_words = pplan.win_words;
-    pwin.woff = (int)((4 - (((jbig + (jbig & 1)) >> 1) & 3)) & 3);
-  }
-  TagScratch tsC{b_cntC.as<uint32_t>(), b_bigC.as<unsigned long long>(), jbig, n};
-  SweepScratch ssC{nullptr, nullptr, b_cntD.as<uint32_t>(), b_tlD.as<int32_t>(), b_ntC.as<unsigned>(), n};
+  DevBuf b_g16, b_curs, b_g16_4, b_curs4;
+  PairWin pwin{}, pwin4{};
+  auto windows = [&](const PairPlan& pl, DevBuf& bg, DevBuf& bc, unsigned long long* side, PairWin* pw) -> cudaError_t {
+    pw->g16_words = ((n + 2) / 2 + 4 + 3) & ~(int64_t)3;
+    pw->curs_cap = std::max<int64_t>(maxdeg, 1);
+    ESC_TRY(bg.alloc(sizeof(uint32_t) * (size_t)pw->g16_words * pl.nclusters));
+    ESC_TRY(bc.alloc(sizeof(longlong2) * (size_t)pw->curs_cap * pl.nclusters));
+    pw->g16 = bg.as<uint32_t>();
+    pw->curs = bc.as<longlong2>();
+    pw->side = side;                            // zeroed above
+    pw->jbig = jbig;
+    pw->n = n;
+    pw->n0 = n0;
+    pw->win_words = pl.win_words;
+    pw->woff = (int)((4 - (((jbig + (jbig & 1)) >> 1) & 3)) & 3);
+    return cudaSuccess;
+  };
+  if (five && pplan.windowed) ESC_TRY(windows(pplan, b_g16, b_curs, b_bigB.as<unsigned long long>(), &pwin));
+  if (win4) ESC_TRY(windows(plan4, b_g16_4, b_curs4, b_bigA.as<unsigned long long>(), &pwin4));
+  // with every counted rank in the window nothing is kept outside it (no array, so none to zero)
+  TagScratch tsC{b_cntC.as<uint32_t>(), b_bigC.as<unsigned long long>(), below5 ? jbig : 0, below5 ? n : 0};
+  SweepScratch ssC{b_cntD.as<uint32_t>(), b_tlD.as<int32_t>(), below5 ? n : 0};
   const int hcap_l = 8192;
   int64_t ghash_cap = pow2_at_least((int)std::max<int64_t>(2 * maxdeg, 2));
   if (2 * maxdeg <= hcap_l) ghash_cap = 2;
@@ -3167,27 +3514,28 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   mark(6, 1, s3);
   // pairs (Thms 11, 12); 16-bit counters when no degree reaches 2^16 (then no W(i,j) can)
   mark(5, 0, s);
+  // CTAs that fit the device at once, at most one per item
+  auto fill = [&](const void* k, int threads, size_t smem, int64_t items, unsigned* grid) -> cudaError_t {
+    ESC_TRY(allow_max_smem(k, smem_optin));
+    int per_sm = 1;
+    ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem));
+    *grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, items);
+    return cudaSuccess;
+  };
+  const size_t sm_light = sizeof(uint32_t) << IT_LIGHT_LOG, sm_medium = sizeof(uint32_t) << IT_MEDIUM_LOG;
+  unsigned grid_i = 1;
   if (five && n > 0) {
-    unsigned long long* pq = b_pctr.as<unsigned long long>() + 3;     // queue counters of the three lists
-    const int32_t* pl = b_plist.as<int32_t>();
+    unsigned long long* pq = ilp.cnt + 3;       // queue counters of the three lists
+    const unsigned long long* pl = ilp.list;
     if (pcnt[0] > 0) {
-      const size_t sm0 = (sizeof(int32_t) + sizeof(uint32_t)) * PH_SMALL_SLOTS;
-      int per_sm = 1;
-      ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_hash<PH_SMALL_SLOTS>, PH_SMALL_THREADS,
-                                                            sm0));
-      unsigned grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, (int64_t)pcnt[0]);
-      (k_pairs_hash<PH_SMALL_SLOTS><<<grid, PH_SMALL_THREADS, sm0, s>>>(g, pl, (int64_t)pcnt[0], pq + 0, tl3, T, cv, accs,
-                                                                       d_status), note_launch());
+      ESC_TRY(fill((const void*)k_pairs_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)pcnt[0], &grid_i));
+      (k_pairs_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s>>>(
+           g, pl, (int64_t)pcnt[0], pq + 0, cb, IT_LIGHT_LOG, tl3, T, cv, accs, d_status), note_launch());
     }
     if (pcnt[1] > 0) {
-      const size_t sm1 = (sizeof(int32_t) + sizeof(uint32_t)) * PH_LARGE_SLOTS;
-      ESC_TRY(allow_max_smem((const void*)k_pairs_hash<PH_LARGE_SLOTS>, smem_optin));
-      int per_sm = 1;
-      ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_hash<PH_LARGE_SLOTS>, PH_LARGE_THREADS,
-                                                            sm1));
-      unsigned grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, (int64_t)pcnt[1]);
-      (k_pairs_hash<PH_LARGE_SLOTS><<<grid, PH_LARGE_THREADS, sm1, s>>>(g, pl + n, (int64_t)pcnt[1], pq + 1, tl3, T,
-                                                                       cv, accs, d_status), note_launch());
+      ESC_TRY(fill((const void*)k_pairs_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)pcnt[1], &grid_i));
+      (k_pairs_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s>>>(
+           g, pl + n, (int64_t)pcnt[1], pq + 1, cb, IT_MEDIUM_LOG, tl3, T, cv, accs, d_status), note_launch());
     }
     if (pcnt[2] > 0 && pplan.windowed) {
       const size_t smw = sizeof(uint32_t) * (size_t)pplan.win_words;
@@ -3232,20 +3580,65 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // 4-cycles (Thm 5)
   mark(3, 0, s2);
   if (n > 0) {
-    if (jbig < n)
-      (k_cycles4<true><<<grid_sweep, 512, 0, s2>>>(g, ctr + 2, tsA, C4e, C4v, accs, own), note_launch());
-    else
-      (k_cycles4<false><<<grid_sweep, 512, 0, s2>>>(g, ctr + 2, tsA, C4e, C4v, accs, own), note_launch());
+    unsigned long long* q4 = il4.cnt + 3;
+    const unsigned long long* l4 = il4.list;
+    if (win4) {
+      const size_t smw = sizeof(uint32_t) * (size_t)plan4.win_words;
+      if (jbig < n)
+        (k_cycles4_win<true><<<plan4.nclusters, plan4.threads, smw, s2>>>(
+             g, l4 + 2 * n, (int64_t)cnt4[2], q4 + 2, pwin4, ptasks4, C4e, accs, d_status), note_launch());
+      else
+        (k_cycles4_win<false><<<plan4.nclusters, plan4.threads, smw, s2>>>(
+             g, l4 + 2 * n, (int64_t)cnt4[2], q4 + 2, pwin4, ptasks4, C4e, accs, d_status), note_launch());
+    } else if (tag4) {
+      if (jbig < n)
+        (k_cycles4_tag<true><<<grid_sweep, 512, 0, s2>>>(g, l4 + 2 * n, (int64_t)cnt4[2], q4 + 2, tsA, C4e, accs),
+         note_launch());
+      else
+        (k_cycles4_tag<false><<<grid_sweep, 512, 0, s2>>>(g, l4 + 2 * n, (int64_t)cnt4[2], q4 + 2, tsA, C4e, accs),
+         note_launch());
+    }
+    if (cnt4[1] > 0) {
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt4[1], &grid_i));
+      (k_cycles4_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s2>>>(
+           g, l4 + n, (int64_t)cnt4[1], q4 + 1, cb, IT_MEDIUM_LOG, C4e, accs, d_status), note_launch());
+    }
+    if (cnt4[0] > 0) {
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)cnt4[0], &grid_i));
+      (k_cycles4_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s2>>>(
+           g, l4, (int64_t)cnt4[0], q4 + 0, cb, IT_LIGHT_LOG, C4e, accs, d_status), note_launch());
+    }
     (k_fold_u64<<<grid_for(n * 32, TPB, sms), TPB, 0, s2>>>(g, C4e), note_launch());
+    (k_vertex_sum_div<<<grid_for(n * 32, TPB, sms), TPB, 0, s2>>>(g, C4e, C4v, 2), note_launch());
   }
   mark(3, 1, s2);
   // 5-cycles (Thm 13)
   mark(7, 0, s4);
   if (five && n > 0) {
-    if (jbig < n)
-      (k_cycles5<true><<<grid_sweep, 512, 0, s4>>>(g, ctr + 6, tsC, ssC, accs, own), note_launch());
-    else
-      (k_cycles5<false><<<grid_sweep, 512, 0, s4>>>(g, ctr + 6, tsC, ssC, accs, own), note_launch());
+    unsigned long long* q5 = il5.cnt + 3;
+    const unsigned long long* l5 = il5.list;
+    if (heavy5) {
+      const size_t smw = sizeof(uint32_t) * (size_t)win5_words;
+      const void* k5 = jbig < n ? (const void*)k_cycles5<true> : (const void*)k_cycles5<false>;
+      ESC_TRY(allow_max_smem(k5, smem_optin));
+      const unsigned grid5 = (unsigned)std::min<int64_t>(sms, (int64_t)cnt5[2]);
+      if (jbig < n)
+        (k_cycles5<true><<<grid5, 1024, smw, s4>>>(g, l5 + 2 * n, (int64_t)cnt5[2], q5 + 2, tsC, ssC, accs, wlo5,
+                                                   win5_words), note_launch());
+      else
+        (k_cycles5<false><<<grid5, 1024, smw, s4>>>(g, l5 + 2 * n, (int64_t)cnt5[2], q5 + 2, tsC, ssC, accs, wlo5,
+                                                    win5_words), note_launch());
+    }
+    if (cnt5[1] > 0) {                          // two tables of half the size
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt5[1], &grid_i));
+      (k_cycles5_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s4>>>(
+           g, l5 + n, (int64_t)cnt5[1], q5 + 1, cb, IT_MEDIUM_LOG - 1, accs, d_status), note_launch());
+    }
+    if (cnt5[0] > 0) {
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, 2 * sm_light, (int64_t)cnt5[0], &grid_i));
+      (k_cycles5_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, 2 * sm_light, s4>>>(
+           g, l5, (int64_t)cnt5[0], q5 + 0, cb, IT_LIGHT_LOG, accs, d_status), note_launch());
+    }
   }
   mark(7, 1, s4);
   ESC_TRY(ss_all.join_into(s));
