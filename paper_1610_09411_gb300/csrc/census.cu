@@ -2648,6 +2648,12 @@ __global__ void k_graph_sizes(const int64_t* voff, const int64_t* rp, int num_gr
   m_arr[k] = (unsigned long long)((rp[voff[k + 1]] - rp[voff[k]]) / 2);
 }
 
+__global__ void k_set_sizes(unsigned long long n, unsigned long long m, unsigned long long* n_arr,
+                            unsigned long long* m_arr) {
+  *n_arr = n;
+  *m_arr = m;
+}
+
 // item lists of pass A/B: vertices by out-degree class
 // small / large: d+ up to small_max or above (vertices with d+ >= 2); the
 // small ones are also split by d- for the clique pass: up to warp_din in wsmall
@@ -2693,14 +2699,7 @@ __global__ void k_clique_dims(DevGraph g, unsigned long long* out) {
 
 
 // ---------------------------------------------------------------- buffers
-// Device buffers of one census.  Repeated censuses would otherwise pay dozens
-// of cudaMalloc / cudaFree calls each (cudaFree synchronises the device), so
-// buffers released by a census are kept in a per-device cache, up to
-// kCacheCap bytes, and handed to later ones: a request takes the smallest
-// cached buffer that is large enough and at most twice the size.  Release
-// happens only after the census's stream has drained (CacheScope), so a
-// buffer never changes hands while kernels may still use it.  If cudaMalloc
-// fails, the cache is emptied and the allocation tried once more.
+// The device-buffer cache declared in internal.h.
 static constexpr size_t kCacheCap = (size_t)8 << 30;
 
 class BufCache {
@@ -2742,111 +2741,130 @@ class BufCache {
   std::multimap<size_t, void*> free_[64];
   size_t bytes_[64] = {};
 };
-static BufCache g_cache;
+// never destroyed: a handle freed during process exit may still come here
+static BufCache& buf_cache() {
+  static BufCache* c = new BufCache;
+  return *c;
+}
 
-// Buffers released inside a scope wait until the scope ends, and the scope
-// ends by draining its stream.
-struct CacheScope;
 static thread_local CacheScope* t_scope = nullptr;
-struct CacheScope {
-  cudaStream_t s;
-  int dev = 0;
-  CacheScope* prev;
-  std::vector<std::pair<void*, size_t>> pending;
-  explicit CacheScope(cudaStream_t st) : s(st), prev(t_scope) {
-    cudaGetDevice(&dev);
-    t_scope = this;
-  }
-  ~CacheScope() {
-    cudaStreamSynchronize(s);
-    for (auto& pb : pending) g_cache.put(dev, pb.first, pb.second);
-    t_scope = prev;
-  }
-};
+CacheScope::CacheScope(cudaStream_t st) : s(st), prev(t_scope) { t_scope = this; }
+CacheScope::~CacheScope() {
+  cudaStreamSynchronize(s);
+  for (auto& b : pending) buf_cache().put(b.dev, b.p, b.bytes);
+  t_scope = prev;
+}
 
-struct DevBuf {
-  void* p = nullptr;
-  size_t bytes = 0;
-  ~DevBuf() {
-    if (!p) return;
-    if (t_scope) t_scope->pending.emplace_back(p, bytes);
-    else cudaFree(p);
-  }
-  cudaError_t alloc(size_t b) {
-    b = ((b > 0 ? b : 16) + 255) & ~(size_t)255;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    size_t got = 0;
-    if ((p = g_cache.get(dev, b, &got)) != nullptr) {
-      bytes = got;
-      return cudaSuccess;
-    }
-    cudaError_t e = cudaMalloc(&p, b);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      g_cache.clear(dev);
-      e = cudaMalloc(&p, b);
-    }
-    if (e != cudaSuccess) {
-      p = nullptr;
-      return e;
-    }
-    bytes = b;
+void DevBuf::release() {
+  if (!p) return;
+  if (t_scope) t_scope->pending.push_back({p, bytes, dev});
+  else buf_cache().put(dev, p, bytes);
+  p = nullptr;
+  bytes = 0;
+}
+cudaError_t DevBuf::alloc(size_t b) {
+  release();
+  b = ((b > 0 ? b : 16) + 255) & ~(size_t)255;
+  cudaGetDevice(&dev);
+  size_t got = 0;
+  if ((p = buf_cache().get(dev, b, &got)) != nullptr) {
+    bytes = got;
     return cudaSuccess;
   }
-  template <class T> T* as() { return (T*)p; }
-};
+  cudaError_t e = cudaMalloc(&p, b);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    buf_cache().clear(dev);
+    e = cudaMalloc(&p, b);
+  }
+  if (e != cudaSuccess) {
+    p = nullptr;
+    return e;
+  }
+  bytes = b;
+  return cudaSuccess;
+}
 
 #define ESC_TRY(x) do { cudaError_t _e = (x); if (_e != cudaSuccess) return _e; } while (0)
 
-// Side streams for the concurrent phases; events order them after / before
-// the caller's stream.  Destroyed when the census returns, after each has
-// drained: on an early error return the caller's stream may not have joined
-// them, and the buffers their kernels use go back to the cache only after
-// this destructor (they are declared before the StreamSet).
-struct StreamSet {
+// Side streams and events for the concurrent phases; events order them after /
+// before the caller's stream.  Creating them costs more than a small census
+// computes (four streams, 0.1 ms), so sets are kept for later censuses, at most
+// kStreamSets per device; a census holds one to itself.  A set goes back after
+// its streams have drained: on an early error return the caller's stream may
+// not have joined them, and the buffers their kernels use go back to the cache
+// only after this destructor (they are declared before the StreamSet).
+struct SideStreams {
   cudaStream_t st[4] = {nullptr, nullptr, nullptr, nullptr};
-  int count = 0;
+  cudaEvent_t fork = nullptr, join[4] = {nullptr, nullptr, nullptr, nullptr};
+};
+static constexpr size_t kStreamSets = 8;
+static std::mutex g_sides_mu;
+static std::vector<SideStreams>& side_pool(int dev) {
+  static auto* pools = new std::vector<SideStreams>[64];
+  return pools[dev & 63];
+}
+struct StreamSet {
+  SideStreams ss;
+  int count = 0, dev = 0;
   ~StreamSet() {
-    for (int i = 0; i < count; ++i) {
-      cudaStreamSynchronize(st[i]);
-      cudaStreamDestroy(st[i]);
+    if (!count) return;
+    bool ok = count == 4;
+    for (int i = 0; i < count; ++i) ok = cudaStreamSynchronize(ss.st[i]) == cudaSuccess && ok;
+    if (ok) {
+      std::lock_guard<std::mutex> lk(g_sides_mu);
+      auto& pool = side_pool(dev);
+      if (pool.size() < kStreamSets) {
+        pool.push_back(ss);
+        return;
+      }
     }
+    for (int i = 0; i < 4; ++i) {
+      if (ss.st[i]) cudaStreamDestroy(ss.st[i]);
+      if (ss.join[i]) cudaEventDestroy(ss.join[i]);
+    }
+    if (ss.fork) cudaEventDestroy(ss.fork);
   }
-  // prio[i] != 0: the device's greatest (most urgent) priority, else its least
-  cudaError_t create(int k, const int* urgent) {
+  // urgent[i] != 0: the device's greatest (most urgent) priority, else its least
+  // (the same flags at every call)
+  cudaError_t create(const int (&urgent)[4]) {
+    cudaGetDevice(&dev);
+    {
+      std::lock_guard<std::mutex> lk(g_sides_mu);
+      auto& pool = side_pool(dev);
+      if (!pool.empty()) {
+        ss = pool.back();
+        pool.pop_back();
+        count = 4;
+        return cudaSuccess;
+      }
+    }
     int least = 0, greatest = 0;
     cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    for (int i = 0; i < k; ++i) {
-      cudaError_t e = cudaStreamCreateWithPriority(&st[i], cudaStreamNonBlocking, urgent[i] ? greatest : least);
-      if (e != cudaSuccess) return e;
-      count = i + 1;
+    cudaError_t e = cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming);
+    count = 0;
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+      e = cudaEventCreateWithFlags(&ss.join[i], cudaEventDisableTiming);
+      if (e == cudaSuccess)
+        e = cudaStreamCreateWithPriority(&ss.st[i], cudaStreamNonBlocking, urgent[i] ? greatest : least);
+      if (e == cudaSuccess) count = i + 1;
     }
-    return cudaSuccess;
+    return e;
   }
-  // every stream in `to` waits for the work enqueued on `from` so far
-  cudaError_t fork_from(cudaStream_t from, std::initializer_list<cudaStream_t> to) {
-    cudaEvent_t e;
-    cudaError_t r = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-    if (r != cudaSuccess) return r;
-    r = cudaEventRecord(e, from);
-    for (cudaStream_t t : to)
-      if (r == cudaSuccess) r = cudaStreamWaitEvent(t, e, 0);
-    cudaEventDestroy(e);
+  // the side streams wait for the work enqueued on `from` so far
+  cudaError_t fork_from(cudaStream_t from) {
+    cudaError_t r = cudaEventRecord(ss.fork, from);
+    for (int i = 0; i < count && r == cudaSuccess; ++i) r = cudaStreamWaitEvent(ss.st[i], ss.fork, 0);
     return r;
   }
   // `into` waits for everything enqueued on the side streams
   cudaError_t join_into(cudaStream_t into) {
-    for (int i = 0; i < count; ++i) {
-      cudaEvent_t e;
-      cudaError_t r = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-      if (r != cudaSuccess) return r;
-      r = cudaEventRecord(e, st[i]);
-      if (r == cudaSuccess) r = cudaStreamWaitEvent(into, e, 0);
-      cudaEventDestroy(e);
-      if (r != cudaSuccess) return r;
+    cudaError_t r = cudaSuccess;
+    for (int i = 0; i < count && r == cudaSuccess; ++i) {
+      r = cudaEventRecord(ss.join[i], ss.st[i]);
+      if (r == cudaSuccess) r = cudaStreamWaitEvent(into, ss.join[i], 0);
     }
-    return cudaSuccess;
+    return r;
   }
 };
 
@@ -3037,6 +3055,19 @@ static constexpr int CORE_MIN_DEG = 48, CORE_CAP = 16384, CORE_CHUNK_MB = 2048;
 static constexpr unsigned long long CORE_MIN_D = 1ull << 24, CORE_D_PER_ENTRY = 160;
 static constexpr size_t CORE_W_BYTES = (size_t)24 << 30;
 
+// App. B's matrices are constants of the pattern catalogue (the embedding
+// counts take the host 0.85 ms): built once per process.
+static const ConvTables& conversion_tables() {
+  static const ConvTables tabs = [] {
+    ConvTables t;
+    conversion_inverse(3, t.a3);
+    conversion_inverse(4, t.a4);
+    conversion_inverse(5, t.a5);
+    return t;
+  }();
+  return tabs;
+}
+
 cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t nnz, const CensusConfig& cfg,
                        unsigned long long* d_out, unsigned* d_status, PerElement* pe_out, Oriented* or_out,
                        cudaStream_t s) {
@@ -3126,10 +3157,8 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
                                                    b_marr.as<unsigned long long>()), note_launch());
     accs.vg = b_vg.as<int32_t>();
   } else {
-    unsigned long long nm[2] = {(unsigned long long)n, (unsigned long long)(nnz / 2)};
-    cudaMemcpyAsync(b_narr.p, &nm[0], sizeof(unsigned long long), cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(b_marr.p, &nm[1], sizeof(unsigned long long), cudaMemcpyHostToDevice, s);
-    ESC_TRY(cudaStreamSynchronize(s));   // nm lives on this stack frame
+    (k_set_sizes<<<1, 1, 0, s>>>((unsigned long long)n, (unsigned long long)(nnz / 2), b_narr.as<unsigned long long>(),
+                                 b_marr.as<unsigned long long>()), note_launch());
   }
   cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * 16, s);
   // a census split over parts: the sweeps take the owned items only, and the
@@ -3521,9 +3550,9 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   cudaStream_t s1 = s, s2 = s, s3 = s, s4 = s;
   if (!cfg.serial_phases) {
     const int urgent[4] = {0, 0, 1, 0};
-    ESC_TRY(ss_all.create(4, urgent));
-    s1 = ss_all.st[0]; s2 = ss_all.st[1]; s3 = ss_all.st[2]; s4 = ss_all.st[3];
-    ESC_TRY(ss_all.fork_from(s, {s1, s2, s3, s4}));
+    ESC_TRY(ss_all.create(urgent));
+    s1 = ss_all.ss.st[0]; s2 = ss_all.ss.st[1]; s3 = ss_all.ss.st[2]; s4 = ss_all.ss.st[3];
+    ESC_TRY(ss_all.fork_from(s));
   }
 
   // wheels (Thm 11): the longest phase, started first
@@ -3680,10 +3709,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   } else {
     if (n > 0)
       (k_edge_sums<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T, C4e, K4e, tv, C4v, K4v, accs), note_launch());
-    ConvTables tabs;
-    conversion_inverse(3, tabs.a3);
-    conversion_inverse(4, tabs.a4);
-    conversion_inverse(5, tabs.a5);
+    const ConvTables& tabs = conversion_tables();
     (k_assemble<<<(G + 63) / 64, 64, 0, s>>>(acc, b_narr.as<unsigned long long>(), b_marr.as<unsigned long long>(),
                                             G, tabs, d_out, (u128*)cfg.d_basis), note_launch());
   }
@@ -3691,16 +3717,22 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
 
   if (pe_out) {
     // hand the per-element arrays over to the caller (ownership moves)
-    pe_out->Te = T; b_T.p = nullptr;
-    pe_out->C4e = C4e; b_C4e.p = nullptr;
-    pe_out->K4e = K4e; b_K4e.p = nullptr;
-    pe_out->tv = tv; b_tv.p = nullptr;
-    pe_out->C4v = C4v; b_C4v.p = nullptr;
-    pe_out->K4v = K4v; b_K4v.p = nullptr;
+    pe_out->Te = T;
+    pe_out->C4e = C4e;
+    pe_out->K4e = K4e;
+    pe_out->tv = tv;
+    pe_out->C4v = C4v;
+    pe_out->K4v = K4v;
+    for (DevBuf* b : {&b_T, &b_C4e, &b_K4e, &b_tv, &b_C4v, &b_K4v}) pe_out->own.push_back(std::move(*b));
   }
   if (or_out) {
-    *or_out = o;
-    b_perm.p = b_rank.p = b_R.p = b_C.p = b_op.p = b_rev.p = nullptr;
+    or_out->perm = o.perm;
+    or_out->rank = o.rank;
+    or_out->R = o.R;
+    or_out->C = o.C;
+    or_out->op = o.op;
+    or_out->rev = o.rev;
+    for (DevBuf* b : {&b_perm, &b_rank, &b_R, &b_C, &b_op, &b_rev}) or_out->own.push_back(std::move(*b));
   }
   ESC_TRY(cudaStreamSynchronize(s));   // scratch buffers are freed on return
   return cudaGetLastError();
@@ -3727,10 +3759,7 @@ cudaError_t run_census_finish(const Oriented& o, int64_t n, int64_t nnz, const P
     (k_edge_sums<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, pe.Te, pe.C4e, pe.K4e, pe.tv, pe.C4v, pe.K4v, accs),
      note_launch());
   }
-  ConvTables tabs;
-  conversion_inverse(3, tabs.a3);
-  conversion_inverse(4, tabs.a4);
-  conversion_inverse(5, tabs.a5);
+  const ConvTables& tabs = conversion_tables();
   (k_assemble<<<1, 64, 0, s>>>(b_acc.as<Acc128>(), b_nm.as<unsigned long long>(), b_nm.as<unsigned long long>() + 1,
                                1, tabs, d_out, nullptr), note_launch());
   ESC_TRY(cudaStreamSynchronize(s));   // nm lives on this stack frame

@@ -12,8 +12,9 @@
 
 struct escape_graph {
   int64_t n = 0, nnz = 0;
-  int64_t* d_rp = nullptr;     // input CSR, original ids
-  int32_t* d_col = nullptr;
+  esc::DevBuf b_rp, b_col;     // input CSR, original ids
+  const int64_t* d_rp = nullptr;
+  const int32_t* d_col = nullptr;
   int device = 0, sms = 1;
   int keep_pe = 0, cta_per_sm = 2, serial = -1;   // serial: 1 on, 0 off, -1 by graph size
   bool has_pe = false;
@@ -52,11 +53,7 @@ escape_status from_status(unsigned h) {
 }
 
 void free_pe(escape_graph* g) {
-  cudaFree(g->pe.Te); cudaFree(g->pe.C4e); cudaFree(g->pe.K4e);
-  cudaFree(g->pe.tv); cudaFree(g->pe.C4v); cudaFree(g->pe.K4v);
   g->pe = esc::PerElement{};
-  cudaFree(g->ori.perm); cudaFree(g->ori.rank); cudaFree(g->ori.R); cudaFree(g->ori.C);
-  cudaFree(g->ori.op); cudaFree(g->ori.rev);
   g->ori = esc::Oriented{};
   g->has_pe = false;
 }
@@ -273,11 +270,13 @@ cudaError_t fetch_row_ptr(const int64_t* d_rp, int64_t rows, std::vector<int64_t
 escape_status census_one(escape_graph* g, const int64_t* d_rp, const int32_t* d_col, int64_t n, int64_t nnz,
                          escape_census* out, cudaStream_t s, bool keep, esc::PerElement* pe, esc::Oriented* ori,
                          float* phase_ms, int* nphase, bool four_only = false) {
-  unsigned long long* d_out = nullptr;
-  unsigned* d_status = nullptr;
-  cudaError_t e = cudaMalloc(&d_out, sizeof(escape_census) + sizeof(escape_u128) * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&d_status, sizeof(unsigned));
-  if (e != cudaSuccess) { cudaFree(d_out); return from_cuda(e); }
+  esc::CacheScope scope(s);
+  esc::DevBuf b_out, b_status;
+  cudaError_t e = b_out.alloc(sizeof(escape_census) + sizeof(escape_u128) * 4);
+  if (e == cudaSuccess) e = b_status.alloc(sizeof(unsigned));
+  if (e != cudaSuccess) return from_cuda(e);
+  unsigned long long* d_out = b_out.as<unsigned long long>();
+  unsigned* d_status = b_status.as<unsigned>();
   cudaMemsetAsync(d_status, 0, sizeof(unsigned), s);
   cudaEvent_t evs[18];
   int nev = phase_ms ? 18 : 0;
@@ -322,8 +321,6 @@ escape_status census_one(escape_graph* g, const int64_t* d_rp, const int32_t* d_
     *nphase = phases;
     for (int i = 0; i < nev; ++i) cudaEventDestroy(evs[i]);
   }
-  cudaFree(d_out);
-  cudaFree(d_status);
   return st;
 }
 
@@ -373,13 +370,15 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
     }
     if (!row_ptr_ok(h, n, nnz)) { delete g; return ESCAPE_EINVAL; }
   }
-  int64_t* d_rp = nullptr;
-  int32_t* d_col = nullptr;
-  unsigned* d_status = nullptr;
-  cudaError_t e = cudaMalloc(&d_rp, sizeof(int64_t) * (n + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&d_col, sizeof(int32_t) * (nnz > 0 ? nnz : 1));
-  if (e == cudaSuccess) e = cudaMalloc(&d_status, sizeof(unsigned));
-  if (e != cudaSuccess) { cudaFree(d_rp); cudaFree(d_col); delete g; return from_cuda(e); }
+  esc::CacheScope scope(s);                     // ends after the handle's buffers below have been moved or released
+  esc::DevBuf b_rp, b_col, b_status;
+  cudaError_t e = b_rp.alloc(sizeof(int64_t) * (n + 1));
+  if (e == cudaSuccess) e = b_col.alloc(sizeof(int32_t) * (nnz > 0 ? nnz : 1));
+  if (e == cudaSuccess) e = b_status.alloc(sizeof(unsigned));
+  if (e != cudaSuccess) { delete g; return from_cuda(e); }
+  int64_t* d_rp = b_rp.as<int64_t>();
+  int32_t* d_col = b_col.as<int32_t>();
+  unsigned* d_status = b_status.as<unsigned>();
   cudaMemcpyKind kind = dev_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (n > 0) e = cudaMemcpyAsync(d_rp, row_ptr, sizeof(int64_t) * (n + 1), kind, s);
   else e = cudaMemsetAsync(d_rp, 0, sizeof(int64_t), s);
@@ -389,20 +388,17 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
   if (st == ESCAPE_OK && (flags & ESCAPE_NORMALIZE)) {
     esc::DeviceArena arena;
     size_t ab = (size_t)(2 * nnz + 16) * 8 * 3 + (size_t)((2 * nnz) / 4096 + 2) * 256 * 8 * 2 + (1 << 22);
-    e = cudaMalloc(&arena.base, ab);
+    esc::DevBuf b_arena, nrp, ncol;
+    e = b_arena.alloc(ab);
     if (e == cudaSuccess) {
+      arena.base = b_arena.as<char>();
       arena.cap = ab;
-      int64_t *nrp = nullptr;
-      int32_t* ncol = nullptr;
       int64_t nnz2 = 0;
       e = esc::normalize_csr(n, nnz, d_rp, d_col, &nrp, &ncol, &nnz2, d_status, arena, s, g->sms);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-      cudaFree(arena.base);
       if (e == cudaSuccess) {
-        cudaFree(d_rp);
-        cudaFree(d_col);
-        d_rp = nrp;
-        d_col = ncol;
+        std::swap(b_rp, nrp);
+        std::swap(b_col, ncol);
         nnz = nnz2;
       }
     }
@@ -418,12 +414,13 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
     st = from_cuda(e);
     if (st == ESCAPE_OK && h) st = ESCAPE_EINVAL;
   }
-  cudaFree(d_status);
-  if (st != ESCAPE_OK) { cudaFree(d_rp); cudaFree(d_col); delete g; return st; }
+  if (st != ESCAPE_OK) { delete g; return st; }
   g->n = n;
   g->nnz = nnz;
-  g->d_rp = d_rp;
-  g->d_col = d_col;
+  g->b_rp = std::move(b_rp);
+  g->b_col = std::move(b_col);
+  g->d_rp = g->b_rp.as<int64_t>();
+  g->d_col = g->b_col.as<int32_t>();
   *out = g;
   return ESCAPE_OK;
 }
@@ -488,15 +485,17 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
   cudaMemcpyKind kind = dev_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   cudaError_t e = cudaSuccess;
   // device copies: offsets, rows, entries turned into union ids
-  int64_t *d_voff = nullptr, *d_rp = nullptr;
-  int32_t* d_col = nullptr;
-  unsigned* d_status = nullptr;
-  unsigned long long* d_out = nullptr;
-  e = cudaMalloc(&d_voff, sizeof(int64_t) * (num_graphs + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&d_rp, sizeof(int64_t) * (rows + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&d_col, sizeof(int32_t) * (nnz > 0 ? nnz : 1));
-  if (e == cudaSuccess) e = cudaMalloc(&d_status, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMalloc(&d_out, sizeof(escape_census) * num_graphs);
+  esc::CacheScope scope(s);
+  esc::DevBuf b_voff, b_rp, b_col, b_status, b_out;
+  e = b_voff.alloc(sizeof(int64_t) * (num_graphs + 1));
+  if (e == cudaSuccess) e = b_rp.alloc(sizeof(int64_t) * (rows + 1));
+  if (e == cudaSuccess) e = b_col.alloc(sizeof(int32_t) * (nnz > 0 ? nnz : 1));
+  if (e == cudaSuccess) e = b_status.alloc(sizeof(unsigned));
+  if (e == cudaSuccess) e = b_out.alloc(sizeof(escape_census) * num_graphs);
+  int64_t *d_voff = b_voff.as<int64_t>(), *d_rp = b_rp.as<int64_t>();
+  int32_t* d_col = b_col.as<int32_t>();
+  unsigned* d_status = b_status.as<unsigned>();
+  unsigned long long* d_out = b_out.as<unsigned long long>();
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_voff, voff_h, sizeof(int64_t) * (num_graphs + 1), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_rp, rp_h, sizeof(int64_t) * (rows + 1), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && nnz > 0) e = cudaMemcpyAsync(d_col, col, sizeof(int32_t) * nnz, kind, s);
@@ -510,16 +509,21 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
   if (st == ESCAPE_OK && (flags & ESCAPE_NORMALIZE)) {
     esc::DeviceArena arena;
     size_t ab = (size_t)(2 * nnz + 16) * 8 * 3 + (size_t)((2 * nnz) / 4096 + 2) * 256 * 8 * 2 + (1 << 22);
-    e = cudaMalloc(&arena.base, ab);
+    esc::DevBuf b_arena, nrp, ncol;
+    e = b_arena.alloc(ab);
     if (e == cudaSuccess) {
+      arena.base = b_arena.as<char>();
       arena.cap = ab;
-      int64_t* nrp = nullptr;
-      int32_t* ncol = nullptr;
       int64_t nnz2 = 0;
       e = esc::normalize_csr(rows, nnz, d_rp, d_col, &nrp, &ncol, &nnz2, d_status, arena, s, sms);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-      cudaFree(arena.base);
-      if (e == cudaSuccess) { cudaFree(d_rp); cudaFree(d_col); d_rp = nrp; d_col = ncol; nnz = nnz2; }
+      if (e == cudaSuccess) {
+        std::swap(b_rp, nrp);
+        std::swap(b_col, ncol);
+        d_rp = b_rp.as<int64_t>();
+        d_col = b_col.as<int32_t>();
+        nnz = nnz2;
+      }
     }
     st = from_cuda(e);
   } else if (st == ESCAPE_OK) {
@@ -549,7 +553,6 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
       if (st == ESCAPE_OK) st = from_status(h);
     }
   }
-  cudaFree(d_voff); cudaFree(d_rp); cudaFree(d_col); cudaFree(d_status); cudaFree(d_out);
   return st;
 }
 
@@ -631,14 +634,14 @@ escape_status escape_per_element(escape_graph* g, uint64_t* tri_e, uint64_t* c4_
                                  uint64_t* c4_v, uint64_t* k4_v, void* stream) {
   if (!g || !g->has_pe) return ESCAPE_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  unsigned long long *dT = nullptr, *dC = nullptr, *dK = nullptr, *vt = nullptr, *vc = nullptr, *vk = nullptr;
+  esc::CacheScope scope(s);
+  esc::DevBuf bufs[6];
   size_t eb = sizeof(unsigned long long) * (g->nnz + 1), vb = sizeof(unsigned long long) * (g->n + 1);
-  cudaError_t e = cudaMalloc(&dT, eb);
-  if (e == cudaSuccess) e = cudaMalloc(&dC, eb);
-  if (e == cudaSuccess) e = cudaMalloc(&dK, eb);
-  if (e == cudaSuccess) e = cudaMalloc(&vt, vb);
-  if (e == cudaSuccess) e = cudaMalloc(&vc, vb);
-  if (e == cudaSuccess) e = cudaMalloc(&vk, vb);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 6 && e == cudaSuccess; ++k) e = bufs[k].alloc(k < 3 ? eb : vb);
+  unsigned long long *dT = bufs[0].as<unsigned long long>(), *dC = bufs[1].as<unsigned long long>(),
+                     *dK = bufs[2].as<unsigned long long>(), *vt = bufs[3].as<unsigned long long>(),
+                     *vc = bufs[4].as<unsigned long long>(), *vk = bufs[5].as<unsigned long long>();
   if (e == cudaSuccess && g->n > 0) {
     (k_map_edges<<<(unsigned)std::min<int64_t>((g->n * 32 + 255) / 256, 65535), 256, 0, s>>>(
         g->d_rp, g->d_col, g->n, g->ori.rank, g->ori.R, g->ori.C, g->pe.Te, g->pe.C4e, g->pe.K4e, dT, dC, dK), esc::note_launch());
@@ -653,7 +656,6 @@ escape_status escape_per_element(escape_graph* g, uint64_t* tri_e, uint64_t* c4_
   if (e == cudaSuccess && c4_v && g->n) e = cudaMemcpyAsync(c4_v, vc, sizeof(uint64_t) * g->n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && k4_v && g->n) e = cudaMemcpyAsync(k4_v, vk, sizeof(uint64_t) * g->n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(dT); cudaFree(dC); cudaFree(dK); cudaFree(vt); cudaFree(vc); cudaFree(vk);
   return from_cuda(e);
 }
 
@@ -676,12 +678,14 @@ escape_status escape_census5_part(escape_graph* g, int32_t part, int32_t parts, 
   g->has_basis = false;
   g->has_part = false;
   long long l0 = esc::launches_so_far();
-  unsigned long long *d_acc = nullptr, *d_out = nullptr;
-  unsigned* d_status = nullptr;
   const int nsum = esc::census_sum_count();
-  cudaError_t e = cudaMalloc(&d_acc, sizeof(escape_u128) * nsum);
-  if (e == cudaSuccess) e = cudaMalloc(&d_out, sizeof(escape_census));
-  if (e == cudaSuccess) e = cudaMalloc(&d_status, sizeof(unsigned));
+  esc::CacheScope scope(s);
+  esc::DevBuf b_acc, b_out, b_status;
+  cudaError_t e = b_acc.alloc(sizeof(escape_u128) * nsum);
+  if (e == cudaSuccess) e = b_out.alloc(sizeof(escape_census));
+  if (e == cudaSuccess) e = b_status.alloc(sizeof(unsigned));
+  unsigned long long *d_acc = b_acc.as<unsigned long long>(), *d_out = b_out.as<unsigned long long>();
+  unsigned* d_status = b_status.as<unsigned>();
   if (e == cudaSuccess) e = cudaMemsetAsync(d_status, 0, sizeof(unsigned), s);
   escape_status st = from_cuda(e);
   if (st == ESCAPE_OK) {
@@ -707,9 +711,6 @@ escape_status escape_census5_part(escape_graph* g, int32_t part, int32_t parts, 
     if (st == ESCAPE_OK) st = from_status(h);
     if (st == ESCAPE_OK) *out = tmp;
   }
-  cudaFree(d_acc);
-  cudaFree(d_out);
-  cudaFree(d_status);
   g->launches = esc::launches_so_far() - l0;
   if (st == ESCAPE_OK) g->has_part = true;
   else free_pe(g);
@@ -740,10 +741,12 @@ escape_status escape_census5_finish(escape_graph* g, const escape_part* total, e
   if (!g || !total || !out || !g->has_part) return ESCAPE_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   long long l0 = esc::launches_so_far();
-  unsigned long long *d_acc = nullptr, *d_out = nullptr;
   const int nsum = esc::census_sum_count();
-  cudaError_t e = cudaMalloc(&d_acc, sizeof(escape_u128) * nsum);
-  if (e == cudaSuccess) e = cudaMalloc(&d_out, sizeof(escape_census));
+  esc::CacheScope scope(s);
+  esc::DevBuf b_acc, b_out;
+  cudaError_t e = b_acc.alloc(sizeof(escape_u128) * nsum);
+  if (e == cudaSuccess) e = b_out.alloc(sizeof(escape_census));
+  unsigned long long *d_acc = b_acc.as<unsigned long long>(), *d_out = b_out.as<unsigned long long>();
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_acc, total->sums, sizeof(escape_u128) * nsum, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = esc::run_census_finish(g->ori, g->n, g->nnz, g->pe, d_acc, d_out, g->sms, s);
   escape_census tmp;
@@ -751,8 +754,6 @@ escape_status escape_census5_finish(escape_graph* g, const escape_part* total, e
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   escape_status st = from_cuda(e);
   if (st == ESCAPE_OK) *out = tmp;
-  cudaFree(d_acc);
-  cudaFree(d_out);
   g->launches = esc::launches_so_far() - l0;
   free_pe(g);
   g->has_part = false;
@@ -766,11 +767,7 @@ escape_status escape_last_basis_counts(const escape_graph* g, escape_u128* out) 
 }
 
 void escape_free(escape_graph* g) {
-  if (!g) return;
-  free_pe(g);
-  cudaFree(g->d_rp);
-  cudaFree(g->d_col);
-  delete g;
+  delete g;                                     // its buffers go to the cache: every call on it has waited for its work
 }
 
 }  // extern "C"

@@ -4,6 +4,8 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <utility>
+#include <vector>
 
 namespace esc {
 
@@ -25,6 +27,45 @@ struct DeviceArena {
   void release(size_t m) { top = m; }
 };
 
+// Device buffers.  Repeated calls would otherwise pay dozens of cudaMalloc /
+// cudaFree calls each (cudaFree synchronises the device), so released buffers
+// are kept in a per-device cache, up to 8 GiB, and handed to later ones: a
+// request takes the smallest cached buffer that is large enough and at most
+// twice the size.  If cudaMalloc fails, the cache is emptied and the allocation
+// tried once more.  A buffer released inside a CacheScope goes back when the
+// scope ends, after the scope's stream has drained, so it never changes hands
+// while kernels may still use it; one released outside any scope goes back at
+// once (nothing may be in flight on it: every entry point waits for its work).
+struct DevBuf {
+  void* p = nullptr;
+  size_t bytes = 0;
+  int dev = 0;
+  DevBuf() = default;
+  DevBuf(const DevBuf&) = delete;
+  DevBuf& operator=(const DevBuf&) = delete;
+  DevBuf(DevBuf&& o) noexcept : p(o.p), bytes(o.bytes), dev(o.dev) { o.p = nullptr; o.bytes = 0; }
+  DevBuf& operator=(DevBuf&& o) noexcept {
+    std::swap(p, o.p);
+    std::swap(bytes, o.bytes);
+    std::swap(dev, o.dev);
+    return *this;
+  }
+  ~DevBuf() { release(); }
+  cudaError_t alloc(size_t b);
+  void release();
+  template <class T> T* as() const { return (T*)p; }
+};
+struct CacheScope {
+  struct Held { void* p; size_t bytes; int dev; };
+  cudaStream_t s;
+  CacheScope* prev;
+  std::vector<Held> pending;
+  explicit CacheScope(cudaStream_t st);
+  ~CacheScope();
+  CacheScope(const CacheScope&) = delete;
+  CacheScope& operator=(const CacheScope&) = delete;
+};
+
 // The degree-ordered graph in rank space (Sec. 3.2).
 struct Oriented {
   int32_t* perm = nullptr;   // n: original id of each rank
@@ -33,6 +74,7 @@ struct Oriented {
   int32_t* C = nullptr;      // nnz
   int64_t* op = nullptr;     // n
   int64_t* rev = nullptr;    // nnz
+  std::vector<DevBuf> own;   // the buffers behind them, when a handle keeps them
 };
 
 // Counts kernel launches made by this thread (reported per census call).
@@ -46,8 +88,8 @@ cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, bool 
                                cudaStream_t s);
 cudaError_t radix_sort(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* tv, int64_t n, int bits,
                        DeviceArena& arena, cudaStream_t s);
-cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const int32_t* col_in, int64_t** rp_out,
-                          int32_t** col_out, int64_t* nnz_out, unsigned* d_status, DeviceArena& arena,
+cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const int32_t* col_in, DevBuf* rp_out,
+                          DevBuf* col_out, int64_t* nnz_out, unsigned* d_status, DeviceArena& arena,
                           cudaStream_t s, int sms);
 cudaError_t validate_csr(int64_t n, const int64_t* rp, const int32_t* col, unsigned* d_status, cudaStream_t s,
                          int sms);
@@ -63,6 +105,7 @@ struct PerElement {
   unsigned long long* tv = nullptr;   // n: triangles at each vertex
   unsigned long long* C4v = nullptr;  // n
   unsigned long long* K4v = nullptr;  // n
+  std::vector<DevBuf> own;            // the buffers behind them
 };
 
 struct CensusTimings {

@@ -328,7 +328,7 @@ static unsigned grid_for(int64_t n, int threads, int sms) {
 
 // ---------------------------------------------------------------- public (internal) entry points
 cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const int32_t* col_in,
-                          int64_t** rp_out, int32_t** col_out, int64_t* nnz_out, unsigned* d_status,
+                          DevBuf* rp_out, DevBuf* col_out, int64_t* nnz_out, unsigned* d_status,
                           DeviceArena& arena, cudaStream_t s, int sms) {
   int vb = bits_for(n > 1 ? n : 2);
   int64_t cnt = 2 * nnz_in;
@@ -348,18 +348,16 @@ cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const
   cudaMemcpyAsync(&nnz, flag + cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
-  int64_t* rp = nullptr;
-  int32_t* col = nullptr;
-  e = cudaMalloc(&rp, sizeof(int64_t) * (n + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&col, sizeof(int32_t) * (nnz > 0 ? nnz : 1));
-  if (e != cudaSuccess) { cudaFree(rp); return e; }
+  e = rp_out->alloc(sizeof(int64_t) * (n + 1));
+  if (e == cudaSuccess) e = col_out->alloc(sizeof(int32_t) * (nnz > 0 ? nnz : 1));
+  if (e != cudaSuccess) return e;
+  int64_t* rp = rp_out->as<int64_t>();
+  int32_t* col = col_out->as<int32_t>();
   cudaMemsetAsync(rp, 0, sizeof(int64_t) * (n + 1), s);
   if (cnt > 0) (k_compact_csr<<<grid_for(cnt, 256, sms), 256, 0, s>>>(keys, flag, cnt, vb, col, rp), note_launch());
   e = exclusive_scan_i64(rp, rp, n, true, arena, s);
-  if (e != cudaSuccess) { cudaFree(rp); cudaFree(col); return e; }
+  if (e != cudaSuccess) return e;
   arena.release(mark);
-  *rp_out = rp;
-  *col_out = col;
   *nnz_out = nnz;
   return cudaGetLastError();
 }
