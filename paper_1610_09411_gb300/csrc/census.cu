@@ -252,12 +252,22 @@ __global__ void k_vertex_from_edges_T(DevGraph g, const uint32_t* T, unsigned lo
   }
 }
 
-__global__ void k_sym_u64(DevGraph g, unsigned long long* E) {
+// 4-cliques per edge: the canonical slot holds those whose lowest vertex lies
+// below the core (all of them without one), H2 (slots from r0 on, or null) twice
+// those inside the core; their sum goes to both slots.
+__global__ void k_sym_K4(DevGraph g, unsigned long long* E, const unsigned long long* H2, int64_t r0) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = warp; v < g.n; v += nwarps)
-    for (int64_t p = g.op[v] + lane; p < g.R[v + 1]; p += 32) E[g.rev[p]] = E[p];
+    for (int64_t p = g.op[v] + lane; p < g.R[v + 1]; p += 32) {
+      unsigned long long e = E[p];
+      if (H2 && p >= r0) {
+        e += H2[p - r0] / 2;
+        E[p] = e;
+      }
+      E[g.rev[p]] = e;
+    }
 }
 
 // 4-cycle per-edge counts arrive in either slot of an edge: fold them.
@@ -313,62 +323,25 @@ struct CliqueScratch {
 };
 
 // Bytes of the clique pass's work space for out-degree d (B, K4 accumulators,
-// hash of 2 x pow2(2d) ints, T values).  B rows are clique_stride(d) words
-// apart: an odd stride, so the lanes of a warp reading word w of 32 different
-// rows hit different shared-memory banks (an even stride of 2^k words puts them
-// on 32 / 2^k banks).
+// hash of 2 x pow2(2d) ints, T and degree of x's out-neighbours).  B rows are
+// clique_stride(d) words apart: an odd stride, so the lanes of a warp reading
+// word w of 32 different rows hit different shared-memory banks (an even stride
+// of 2^k words puts them on 32 / 2^k banks).
 static inline __host__ __device__ int clique_stride(int d) { return ((d + 63) >> 6) | 1; }
 static constexpr int CLQ_MAX_WARPS = 16;         // warps of a CTA of the clique pass (512 threads)
 static inline size_t clique_space(int d) {
   int h = 1;
   while (h < 2 * d) h <<= 1;
   return sizeof(uint64_t) * ((size_t)d * clique_stride(d) + d) + sizeof(int32_t) * (2 * (size_t)h) +
-         sizeof(uint32_t) * d;
+         sizeof(uint32_t) * 2 * (size_t)((d + 1) & ~1);
 }
-
-// B rows are symmetric (row a = every neighbour of v_a inside N+(x)); W words
-// per row, RS words apart.
-// with_k5: count the candidates c above b (for DBP); lane_k5: also count the
-// 5-cliques here, one lane per edge (else k5_warp does it for the warp).
-__device__ __forceinline__ void clique_edge(const uint64_t* B, int W, int RS, int a, int b, const uint64_t* Da,
-                                            const uint64_t* Db, int DW, bool with_k5, bool lane_k5,
-                                            unsigned long long& alpha_out, unsigned long long& beta_out,
-                                            unsigned long long& k5_out, unsigned long long& above_out) {
-  const uint64_t* ra = B + (int64_t)a * RS;
-  const uint64_t* rb = B + (int64_t)b * RS;
-  unsigned long long alpha = 0, k5 = 0, above = 0;
-#pragma unroll 4
-  for (int w = 0; w < W; ++w) alpha += __popcll(ra[w] & rb[w]);
-  // 5-cliques with lowest vertex x and next two v_a < v_b: every c in the
-  // common neighbourhood above b, then every l adjacent to a, b, c above c
-  int w0 = with_k5 ? (b + 1) >> 6 : W;
-  for (int w = w0; w < W; ++w) {
-    uint64_t cm = ra[w] & rb[w];
-    if (w == w0) cm &= ~0ull << ((b + 1) & 63);
-    above += __popcll(cm);
-    while (lane_k5 && cm) {
-      int c = w * 64 + __ffsll((long long)cm) - 1;
-      cm &= cm - 1;
-      const uint64_t* rc = B + (int64_t)c * RS;
-      int u = (c + 1) >> 6;
-      if (u < W) k5 += __popcll(ra[u] & rb[u] & rc[u] & (~0ull << ((c + 1) & 63)));
-      // the remaining words four at a time (independent loads in flight)
-      for (++u; u + 4 <= W; u += 4)
-        k5 += __popcll(ra[u] & rb[u] & rc[u]) + __popcll(ra[u + 1] & rb[u + 1] & rc[u + 1]) +
-              __popcll(ra[u + 2] & rb[u + 2] & rc[u + 2]) + __popcll(ra[u + 3] & rb[u + 3] & rc[u + 3]);
-      for (; u < W; ++u) k5 += __popcll(ra[u] & rb[u] & rc[u]);
-    }
-  }
-  unsigned long long beta = 0;
-  if (Da) {
-#pragma unroll 8
-    for (int w = 0; w < DW; ++w) beta += __popcll(Da[w] & Db[w]);
-  }
-  alpha_out = alpha;
-  beta_out = beta;
-  k5_out = k5;
-  above_out = above;
-}
+// per warp: a batch of CLQ_BATCH vertices b and their prefix sums (5-cliques);
+// also the queue of edges waiting for a full warp (32 + 31 entries of two ints)
+static constexpr int CLQ_BATCH_WORDS = 4, CLQ_BATCH = 64 * CLQ_BATCH_WORDS;
+struct CliqueWarp {
+  uint32_t pre[CLQ_BATCH];
+  uint8_t b[CLQ_BATCH];            // from the first vertex of the batch
+};
 
 // Position of the k-th (0-based) set bit of m (k < popc(m)).
 __device__ __forceinline__ int select32(unsigned m, int k) {
@@ -387,85 +360,137 @@ __device__ __forceinline__ int select64(uint64_t x, int k) {
   const int c = __popc((unsigned)x);
   return k < c ? select32((unsigned)x, k) : 32 + select32((unsigned)(x >> 32), k - c);
 }
+// bits above position b (of the word that holds position b + 1)
+__device__ __forceinline__ uint64_t above_mask(int b) { return ~0ull << ((b + 1) & 63); }
 
-// 5-cliques (Thm 14) of the edges (a, b) of G[N+(x)] that the lanes hold
-// (want: an edge with at least two candidates), one edge at a time for the
-// whole warp: the candidates c (common neighbours of v_a and v_b above b) are
-// taken 32 at a time, lane k the k-th, and each lane counts the common
-// neighbours of v_a, v_b and v_c above c.  Consecutive candidates lie in the
-// same or neighbouring words, so the lanes' word loops nearly coincide.  The
-// common neighbourhood of a and b goes to the warp's buffer mb (W <= 32 words).
-__device__ __forceinline__ unsigned long long k5_warp(const uint64_t* B, int W, int RS, int a, int b_l, bool want_l,
-                                                      uint64_t* mb) {
+// 5-cliques (Thm 14) whose two lowest vertices are x and v_a, by one warp: for
+// every b above a in row a, the candidates c are the common neighbours of v_a
+// and v_b above b, and each pair (b, c) adds the common neighbours of the three
+// above c.  The b come in batches of CLQ_BATCH_WORDS words of row a; the pairs
+// of a batch, numbered through by the prefix sums of |candidates|, are split
+// evenly over the lanes, so every lane walks about the same number of pairs and
+// nothing is shared per edge (one edge at a time for the whole warp cost some
+// 150 warp instructions per edge before its first candidate: k_clique_large on
+// R-MAT 19 149 -> 116 ms, on 96 graphs of up to 2,000 vertices 70 -> 41 ms; with
+// the 4-cliques and N20 of the core taken from its contraction 94 and 28.5 ms).
+// dbp += C(candidates, 2) per edge (directed bipyramids).
+__device__ __forceinline__ void k5_row(const uint64_t* B, int W, int RS, int a, CliqueWarp* cw, unsigned long long& k5,
+                                       u128& dbp) {
   const int lane = threadIdx.x & 31;
   const uint64_t* ra = B + (int64_t)a * RS;
-  unsigned long long k5 = 0;
-  unsigned todo = __ballot_sync(0xffffffffu, want_l);
-  while (todo) {
-    const int k = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const int b = __shfl_sync(0xffffffffu, b_l, k);
-    const uint64_t* rb = B + (int64_t)b * RS;
-    const int w0 = (b + 1) >> 6;
+  for (int wb = (a + 1) >> 6; wb < W; wb += CLQ_BATCH_WORDS) {
     uint64_t m = 0;
-    if (lane >= w0 && lane < W) {
-      m = ra[lane] & rb[lane];
-      if (lane == w0) m &= ~0ull << ((b + 1) & 63);
+    if (lane < CLQ_BATCH_WORDS && wb + lane < W) {
+      m = ra[wb + lane];
+      if (wb + lane == (a + 1) >> 6) m &= above_mask(a);
     }
-    if (lane < W) mb[lane] = m;
-    __syncwarp();
     const int cnt = __popcll(m);
-    int incl = cnt;
+    const int c0 = __shfl_sync(0xffffffffu, cnt, 0), c1 = c0 + __shfl_sync(0xffffffffu, cnt, 1),
+              c2 = c1 + __shfl_sync(0xffffffffu, cnt, 2), s = c2 + __shfl_sync(0xffffffffu, cnt, 3);
+    unsigned total = 0;
+    for (int t0 = 0; t0 < s; t0 += 32) {
+      const int t = t0 + lane;
+      const int wq = t < c0 ? 0 : (t < c1 ? 1 : (t < c2 ? 2 : 3));
+      const uint64_t mw = __shfl_sync(0xffffffffu, m, wq);
+      unsigned n = 0;
+      int b = 0;
+      if (t < s) {
+        b = (wb + wq) * 64 + select64(mw, t - (wq == 0 ? 0 : (wq == 1 ? c0 : (wq == 2 ? c1 : c2))));
+        const uint64_t* rb = B + (int64_t)b * RS;
+        int u = (b + 1) >> 6;
+        if (u < W) n = __popcll(ra[u] & rb[u] & above_mask(b));
+        for (++u; u < W; ++u) n += __popcll(ra[u] & rb[u]);
+        if (n >= 2) dbp += (unsigned long long)n * (n - 1) / 2;
+        else n = 0;                             // a lone candidate closes no 5-clique
+      }
+      unsigned incl = n;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (t < s) {
+        cw->b[t] = (uint8_t)(b - wb * 64);
+        cw->pre[t] = total + incl - n;
+      }
+      total += __shfl_sync(0xffffffffu, incl, 31);
     }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const int kth = t0 + lane;
-      int wq = w0;                              // the word of candidate kth: words whose candidates all precede it
-      for (int u = w0; u < W; ++u) wq += __shfl_sync(0xffffffffu, incl, u) <= kth ? 1 : 0;
-      wq = min(wq, W - 1);
-      const int before = __shfl_sync(0xffffffffu, incl, wq) - __shfl_sync(0xffffffffu, cnt, wq);
-      if (kth < total) {
-        const int c = wq * 64 + select64(mb[wq], kth - before);
-        const uint64_t* rc = B + (int64_t)c * RS;
-        int u = (c + 1) >> 6;
-        unsigned long long part = 0;
-        if (u < W) part = __popcll(mb[u] & rc[u] & (~0ull << ((c + 1) & 63)));
-        for (++u; u + 4 <= W; u += 4)
-          part += __popcll(mb[u] & rc[u]) + __popcll(mb[u + 1] & rc[u + 1]) + __popcll(mb[u + 2] & rc[u + 2]) +
-                  __popcll(mb[u + 3] & rc[u + 3]);
-        for (; u < W; ++u) part += __popcll(mb[u] & rc[u]);
-        k5 += part;
+    __syncwarp();
+    const unsigned share = (total + 31) / 32, p0 = min(total, lane * share), p1 = min(total, p0 + share);
+    if (p0 < p1) {
+      int lo = 0, hi = s;                       // the b of pair p0: the last t with pre[t] <= p0
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (cw->pre[mid] <= p0) lo = mid; else hi = mid;
+      }
+      int t = lo, skip = (int)(p0 - cw->pre[t]);
+      unsigned left = p1 - p0;
+      while (true) {
+        const int b = wb * 64 + cw->b[t];
+        const uint64_t* rb = B + (int64_t)b * RS;
+        unsigned here = min(left, (t + 1 < s ? cw->pre[t + 1] : total) - cw->pre[t] - (unsigned)skip);
+        left -= here;
+        int w = (b + 1) >> 6;
+        uint64_t cm = here ? ra[w] & rb[w] & above_mask(b) : 0;
+        while (here) {
+          const int c_w = __popcll(cm);
+          if (skip >= c_w) {                    // also: the word is used up
+            skip -= c_w;
+            ++w;
+            cm = ra[w] & rb[w];
+            continue;
+          }
+          if (skip) {
+            cm &= ~0ull << select64(cm, skip);
+            skip = 0;
+          }
+          const int c = w * 64 + __ffsll((long long)cm) - 1;
+          cm &= cm - 1;
+          --here;
+          const uint64_t* rc = B + (int64_t)c * RS;
+          int u = (c + 1) >> 6;
+          unsigned part = u < W ? __popcll(ra[u] & rb[u] & rc[u] & above_mask(c)) : 0u;
+          for (++u; u < W; ++u) part += __popcll(ra[u] & rb[u] & rc[u]);
+          k5 += part;
+        }
+        if (!left) break;
+        skip = 0;
+        ++t;
       }
     }
-    __syncwarp();                               // the buffer is read before the next edge writes it
+    __syncwarp();                               // the batch is read before the next one is written
   }
-  return k5;
 }
 
-// Work-space layout of the CTA path: B (d x W u64), K4 accumulators (d u64),
-// hash (2 x hcap ints), T of x's out-edges (d u32), in shared memory; for
-// out-degrees whose bit matrix does not fit there (GLOBAL_B), the same layout
-// in a per-CTA region of global memory (cs.G, cs.g_words words per CTA).
+// Work-space layout of the CTA path: B (d x RS u64, rows symmetric: row a = every
+// neighbour of v_a inside N+(x)), K4 accumulators (d u64), hash (2 x hcap
+// ints), T of x's out-edges and degree of its out-neighbours (d u32 each), in
+// shared memory; for out-degrees whose bit matrix does not fit there (GLOBAL_B),
+// the same layout in a per-CTA region of global memory (cs.G, cs.g_words words
+// per CTA).  The per-warp batches follow in shared memory.
 // A launch takes the items with dlo < d+ <= dmax and skips the others.
+// five: also what only the 5-vertex counts need (beta, the triangle sums, the
+// 5-cliques).  From rank core0 on, the 4-cliques and N20 come from the dense
+// core (core.cu): no alpha, beta or D.
 template <bool GLOBAL_B>
-__global__ void k_clique_large(DevGraph g, const int32_t* items, int64_t nitems, unsigned long long* qctr,
-                               const uint32_t* T, unsigned long long* K4e, AccSet acc, CliqueScratch cs,
-                               int hash_cap, int dlo, int dmax, unsigned* status, bool with_k5) {
+__global__ void __launch_bounds__(512, 1) k_clique_large(DevGraph g, const int32_t* items, int64_t nitems,
+                                                         unsigned long long* qctr, const uint32_t* T,
+                                                         unsigned long long* K4e, AccSet acc, CliqueScratch cs,
+                                                         int hash_cap, int dlo, int dmax, unsigned* status, bool five,
+                                                         int64_t core0) {
   extern __shared__ uint64_t smem64[];
   __shared__ u128 sh[32];
   __shared__ int64_t sh_item;
-  __shared__ uint64_t s_mb[CLQ_MAX_WARPS][32];   // k5_warp's buffers
+  __shared__ int sh_row;
   const int RS_cap = clique_stride(dmax);
   uint64_t* B = GLOBAL_B ? cs.G + (int64_t)blockIdx.x * cs.g_words : smem64;   // dmax * RS_cap
   unsigned long long* k4x = (unsigned long long*)(B + (int64_t)dmax * RS_cap);  // dmax
   int32_t* hk = (int32_t*)(k4x + dmax);                        // hash_cap
   int32_t* hv = hk + hash_cap;                                 // hash_cap
-  uint32_t* Tx = (uint32_t*)(hv + hash_cap);                   // dmax
+  uint32_t* Tx = (uint32_t*)(hv + hash_cap);                   // dmax, even
+  uint32_t* dv = Tx + ((dmax + 1) & ~1);                       // dmax, even
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  CliqueWarp* cw = reinterpret_cast<CliqueWarp*>(GLOBAL_B ? (void*)smem64 : (void*)(dv + ((dmax + 1) & ~1))) + wid;
   uint64_t* D = cs.D + (int64_t)blockIdx.x * cs.d_words;
   const int ids[6] = {ACC_K4, ACC_N20, ACC_N10A, ACC_N16A, ACC_N21, ACC_DBP};
   LocalAcc<6> la;
@@ -481,8 +506,9 @@ __global__ void k_clique_large(DevGraph g, const int32_t* items, int64_t nitems,
     int W = (d + 63) >> 6;
     const int RS = clique_stride(d);
     int DW = (din + 63) >> 6;
-    bool use_beta = din > 0 && (int64_t)d * DW <= cs.d_words;
-    if (din > 0 && !use_beta && threadIdx.x == 0) set_err(status, DEVERR_SCRATCH);
+    const bool k4_here = x < core0;
+    bool use_beta = five && k4_here && din > 0 && (int64_t)d * DW <= cs.d_words;
+    if (five && k4_here && din > 0 && !use_beta && threadIdx.x == 0) set_err(status, DEVERR_SCRATCH);
     int hsz = pow2_at_least(2 * d);
     PosHash H{hk, hv, hsz - 1};
     for (int i = threadIdx.x; i < hsz; i += blockDim.x) hk[i] = -1;
@@ -490,17 +516,29 @@ __global__ void k_clique_large(DevGraph g, const int32_t* items, int64_t nitems,
     for (int i = threadIdx.x; i < d; i += blockDim.x) { k4x[i] = 0; Tx[i] = T[o + i]; }
     if (use_beta)
       for (int64_t i = threadIdx.x; i < (int64_t)d * DW; i += blockDim.x) D[i] = 0;
+    if (threadIdx.x == 0) sh_row = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < d; i += blockDim.x) H.insert(g.C[o + i], i);
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+      const int32_t v = g.C[o + i];
+      H.insert(v, i);
+      dv[i] = (uint32_t)(g.R[v + 1] - g.R[v]);
+    }
     __syncthreads();
-    // build B
+    unsigned long long dx = (unsigned long long)(g.R[x + 1] - g.R[x]);
+    // build B; every hit (a, b) is the triangle {x, v_a, v_b}: its N10 and N16 terms
     for (int a = wid; a < d; a += nw) {
       int32_t v = g.C[o + a];
+      const unsigned long long dva = dv[a], txa = Tx[a];
       for (int64_t q = g.op[v] + lane; q < g.R[v + 1]; q += 32) {
         int b = H.find(g.C[q]);
         if (b >= 0) {
           atomicOr((unsigned long long*)&B[(int64_t)a * RS + (b >> 6)], 1ull << (b & 63));
           atomicOr((unsigned long long*)&B[(int64_t)b * RS + (a >> 6)], 1ull << (a & 63));
+          if (five) {
+            const unsigned long long tab = T[q], txb = Tx[b], dvb = dv[b];
+            la.v[2] += (u128)(tab - 1) * (dx - 2) + (u128)(txb - 1) * (dva - 2) + (u128)(txa - 1) * (dvb - 2);   // N10
+            la.v[3] += (u128)(txa - 1) * (txb - 1) + (u128)(txa - 1) * (tab - 1) + (u128)(txb - 1) * (tab - 1);  // N16
+          }
         }
       }
     }
@@ -515,47 +553,79 @@ __global__ void k_clique_large(DevGraph g, const int32_t* items, int64_t nitems,
       }
     }
     __syncthreads();
-    unsigned long long dx = (unsigned long long)(g.R[x + 1] - g.R[x]);
-    // edges (a, b) of G[N+(x)]: scan N+(v_a) again to get the slot of (v_a, v_b);
-    // the lanes step together so that k5_warp can take the 5-cliques
-    const bool warp_k5 = with_k5 && !GLOBAL_B && W <= 32 && nw <= CLQ_MAX_WARPS;
-    for (int a = wid; a < d; a += nw) {
+    // alpha and beta of the edges (a, b) of G[N+(x)]: N+(v_a) is scanned again
+    // for the slot of (v_a, v_b); hits wait in the warp's queue until 32 of them
+    // fill a warp (about a third of the entries are hits)
+    int32_t* qb = reinterpret_cast<int32_t*>(cw);            // b of the waiting edges
+    int32_t* qo = qb + 64;                                   // and their offsets in N+(v_a)
+    for (int a = wid; a < (k4_here ? d : 0); a += nw) {
       int32_t v = g.C[o + a];
-      unsigned long long dva = (unsigned long long)(g.R[v + 1] - g.R[v]);
+      const int64_t q0 = g.op[v];
+      const int len = (int)(g.R[v + 1] - q0);
+      const uint64_t* ra = B + (int64_t)a * RS;
+      const uint64_t* Da = use_beta ? D + (int64_t)a * DW : nullptr;
       unsigned long long k4a = 0;
-      const int64_t qe = g.R[v + 1];
-      for (int64_t qb = g.op[v]; qb < qe; qb += 32) {
-        const int64_t q = qb + lane;
+      int fill = 0;                                          // the same on every lane
+      for (int e = 0; e < len || fill > 0; e += 32) {
         int b = -1;
-        int32_t w = 0;
-        if (q < qe) {
-          w = g.C[q];
-          b = H.find(w);
-        }
-        unsigned long long above = 0;
+        if (e + lane < len) b = H.find(g.C[q0 + e + lane]);
+        const unsigned hm = __ballot_sync(0xffffffffu, b >= 0);
         if (b >= 0) {
-          unsigned long long alpha, beta, k5;
-          clique_edge(B, W, RS, a, b, use_beta ? D + (int64_t)a * DW : nullptr,
-                      use_beta ? D + (int64_t)b * DW : nullptr, DW, with_k5, with_k5 && !warp_k5, alpha, beta, k5,
-                      above);
-          la.v[5] += ch2(above);                                  // directed bipyramids on this triangle
-          unsigned long long dvb = (unsigned long long)(g.R[w + 1] - g.R[w]);
-          unsigned long long tab = T[q], txa = Tx[a], txb = Tx[b];
-          la.v[0] += alpha;                                       // 3 x K4
-          la.v[1] += ch2(alpha + beta);                           // N20
-          la.v[2] += (u128)(tab - 1) * (dx - 2) + (u128)(txb - 1) * (dva - 2) + (u128)(txa - 1) * (dvb - 2);   // N10
-          la.v[3] += (u128)(txa - 1) * (txb - 1) + (u128)(txa - 1) * (tab - 1) + (u128)(txb - 1) * (tab - 1);  // N16
-          la.v[4] += k5;                                          // N21 (zero when k5_warp counts them)
+          const int at = fill + __popc(hm & ((1u << lane) - 1u));
+          qb[at] = b;
+          qo[at] = e + lane;
+        }
+        fill += __popc(hm);
+        if (fill < 32 && e + 32 < len) continue;
+        __syncwarp();
+        if (lane < fill) {
+          const int bb = qb[lane];
+          const int64_t q = q0 + qo[lane];
+          const uint64_t* rb = B + (int64_t)bb * RS;
+          unsigned long long alpha = 0, beta = 0;
+#pragma unroll 4
+          for (int w = 0; w < W; ++w) alpha += __popcll(ra[w] & rb[w]);
+          if (use_beta) {
+            const uint64_t* Db = D + (int64_t)bb * DW;
+#pragma unroll 8
+            for (int w = 0; w < DW; ++w) beta += __popcll(Da[w] & Db[w]);
+          }
+          la.v[0] += alpha;                                  // 3 x K4
+          if (five) la.v[1] += ch2(alpha + beta);            // N20
           if (alpha) {
             atomicAdd(&K4e[q], alpha);
-            atomicAdd(&k4x[b], alpha);
+            atomicAdd(&k4x[bb], alpha);
             k4a += alpha;
           }
         }
-        if (warp_k5) la.v[4] += k5_warp(B, W, RS, a, b, b >= 0 && above >= 2, s_mb[wid]);
+        // the rest moves to the front
+        const int rest = max(fill - 32, 0);
+        int32_t mb = 0, mo = 0;
+        if (lane < rest) {
+          mb = qb[32 + lane];
+          mo = qo[32 + lane];
+        }
+        __syncwarp();
+        if (lane < rest) {
+          qb[lane] = mb;
+          qo[lane] = mo;
+        }
+        fill = rest;
       }
       k4a = warp_sum_u64(k4a);
       if (lane == 0 && k4a) atomicAdd(&k4x[a], k4a);
+      __syncwarp();
+    }
+    if (five) {                                 // rows handed out one by one: low rows hold most of the work
+      unsigned long long k5 = 0;
+      while (true) {
+        int a = 0;
+        if (lane == 0) a = atomicAdd(&sh_row, 1);
+        a = __shfl_sync(0xffffffffu, a, 0);
+        if (a >= d) break;
+        k5_row(B, W, RS, a, cw, k5, la.v[5]);
+      }
+      la.v[4] += k5;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < d; i += blockDim.x)
@@ -577,7 +647,8 @@ static constexpr int CLQ_ILP = 4;
 
 __global__ void __launch_bounds__(CLQ_WARPS * 32, 4) k_clique_warp(DevGraph g, const int32_t* items, int64_t nitems,
                                                                 unsigned long long* qctr, const uint32_t* T,
-                                                                unsigned long long* K4e, AccSet acc, bool with_k5) {
+                                                                unsigned long long* K4e, AccSet acc, bool with_k5,
+                                                                int64_t core0) {
   __shared__ u128 sh[32];
   __shared__ int32_t sL[CLQ_WARPS][32];
   __shared__ uint32_t sT[CLQ_WARPS][32];
@@ -607,7 +678,8 @@ __global__ void __launch_bounds__(CLQ_WARPS * 32, 4) k_clique_warp(DevGraph g, c
     int64_t o = g.op[x], ib = g.R[x];
     int d = (int)(g.R[x + 1] - o);
     int din = (int)(o - ib);
-    int DW = (din + 63) >> 6;
+    const bool k4_here = x < core0;                   // else 4-cliques and N20 come from the core
+    const int DW = with_k5 && k4_here ? (din + 63) >> 6 : 0;   // beta only feeds N20
     int32_t va = lane < d ? g.C[o + lane] : 0x7fffffff;
     L[lane] = va;
     sT[wl][lane] = lane < d ? T[o + lane] : 0u;
@@ -635,7 +707,7 @@ __global__ void __launch_bounds__(CLQ_WARPS * 32, 4) k_clique_warp(DevGraph g, c
       }
     }
     // D: in-neighbour y (index k) marks bit k of D_a for every v_a in N+(y)
-    for (int k = lane; k < din; k += 32) {
+    for (int k = lane; k < (DW ? din : 0); k += 32) {
       int32_t y = g.C[ib + k];
       int64_t q1 = g.R[y + 1];
       for (int64_t q = g.op[y]; q < q1; q += CLQ_ILP) {
@@ -673,12 +745,14 @@ __global__ void __launch_bounds__(CLQ_WARPS * 32, 4) k_clique_warp(DevGraph g, c
         }
         unsigned long long dvb = (unsigned long long)(g.R[w + 1] - g.R[w]);
         unsigned long long tab = T[q], txb = sT[wl][b];
-        la.v[0] += alpha;                                         // 3 x K4
-        la.v[1] += ch2(alpha + beta);                             // N20
+        if (k4_here) {
+          la.v[0] += alpha;                                       // 3 x K4
+          la.v[1] += ch2(alpha + beta);                           // N20
+        }
         la.v[2] += (u128)(tab - 1) * (dx - 2) + (u128)(txb - 1) * (dva - 2) + (u128)(txa - 1) * (dvb - 2);   // N10
         la.v[3] += (u128)(txa - 1) * (txb - 1) + (u128)(txa - 1) * (tab - 1) + (u128)(txb - 1) * (tab - 1);  // N16
         la.v[4] += k5;                                            // N21
-        if (alpha) {
+        if (alpha && k4_here) {
           atomicAdd(&K4e[q], alpha);
           atomicAdd(&K[b], alpha);
           k4a += alpha;
@@ -2558,7 +2632,7 @@ __global__ void k_assemble(const Acc128* acc_all, const unsigned long long* n_ar
   }
   u128 n = n_arr[k], m = m_arr[k];
   u128 W = A[ACC_W], T = A[ACC_T], TT = A[ACC_TT], C4 = A[ACC_C4], D = A[ACC_D];
-  u128 K4 = A[ACC_K4] / 3, S3 = A[ACC_S3];
+  u128 K4 = (A[ACC_K4] + A[ACC_K4H] / 4) / 3, S3 = A[ACC_S3];
   u128 P4 = A[ACC_P4A] - 3 * T;
   u128 N[35];
   N[1] = A[ACC_S4];
@@ -2580,7 +2654,7 @@ __global__ void k_assemble(const Acc128* acc_all, const unsigned long long* n_ar
   N[17] = A[ACC_N17] + A[ACC_N17H] / 2;
   N[18] = A[ACC_N18] + A[ACC_N18H] / 4;
   N[19] = A[ACC_N19];
-  N[20] = A[ACC_N20];
+  N[20] = A[ACC_N20] + A[ACC_N20H] / 3;
   N[21] = A[ACC_N21];
   N[22] = cnk(n, 5);
   N[23] = n >= 2 ? m * cnk(n - 2, 3) : 0;
@@ -3238,17 +3312,18 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   // larger ones (dense graphs) use a per-CTA region of global memory
   int dsplit = dmax;
   while (dsplit > SMALL_DPLUS + 1 &&
-         clique_space(dsplit) + 1024 + sizeof(uint64_t) * 32 * CLQ_MAX_WARPS > (size_t)smem_optin)
+         clique_space(dsplit) + 1024 + sizeof(CliqueWarp) * CLQ_MAX_WARPS > (size_t)smem_optin)
     --dsplit;
   const int dmax_s = std::min(dmax, dsplit);
   int hcap_b = pow2_at_least(2 * dmax_s);
-  size_t smem_b = clique_space(dmax_s);
+  size_t smem_b = clique_space(dmax_s) + sizeof(CliqueWarp) * 8;
   ESC_TRY(allow_max_smem((const void*)k_clique_large<false>, smem_optin));
   // as many 256-thread CTAs per SM as registers and the bit matrix allow;
   // one 512-thread CTA per SM when fewer than two fit (large bit matrices)
   int clq_threads = 256, clq_per_sm = 1;
   ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clq_per_sm, k_clique_large<false>, clq_threads, smem_b));
   if (clq_per_sm < 2) {
+    smem_b = clique_space(dmax_s) + sizeof(CliqueWarp) * CLQ_MAX_WARPS;
     clq_threads = 512;
     clq_per_sm = 1;
   }
@@ -3332,7 +3407,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     jbig = lo;
   }
   // core vertices: their core neighbours, places in W and the prefix sums of the work
-  DevBuf b_cdh, b_cli, b_crow, b_coff, b_chl, b_chb, b_cwb, b_low, b_W, b_cblk, b_ctile, b_cb;
+  DevBuf b_cdh, b_cli, b_crow, b_coff, b_chl, b_chb, b_cwb, b_low, b_W, b_cblk, b_ctile, b_cb, b_cbits, b_ck4;
   CoreView cv{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
   std::vector<int64_t> coff;
   int64_t wlen = 0;
@@ -3384,6 +3459,12 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       ESC_TRY(b_W.alloc(wb));
       ESC_TRY(b_cblk.alloc(core_block_bytes(cchunks)));
       ESC_TRY(b_ctile.alloc(sizeof(int4) * (size_t)cchunks.max_tiles));
+      ESC_TRY(b_cbits.alloc(core_bit_bytes(cchunks)));
+      cbuf.k4_0 = hR[cv.h0];
+      ESC_TRY(b_ck4.alloc(sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1)));
+      cudaMemsetAsync(b_ck4.p, 0, sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1), s);
+      cbuf.k4 = b_ck4.p;
+      cbuf.bits = b_cbits.p;
       cbuf.blocks = b_cblk.p;
       cbuf.tiles = b_ctile.p;
       if (cv.h0 > 0) {
@@ -3615,23 +3696,19 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   mark(2, 0, s1);
   if (nitems_b > 0)
     (k_clique_large<false><<<(unsigned)std::min<int64_t>(blocks_b, nitems_b), clq_threads, smem_b, s1>>>(
-        g, b_items.as<int32_t>(), nitems_b, ctr + 1, T, K4e, accs, cs, hcap_b, -1, dmax_s, d_status, five),
+        g, b_items.as<int32_t>(), nitems_b, ctr + 1, T, K4e, accs, cs, hcap_b, -1, dmax_s, d_status, five, cv.h0),
      note_launch());
   if (nitems_b > 0 && blocks_g > 0)
-    (k_clique_large<true><<<(unsigned)std::min<int64_t>(blocks_g, nitems_b), 512, 0, s1>>>(
+    (k_clique_large<true><<<(unsigned)std::min<int64_t>(blocks_g, nitems_b), 512, sizeof(CliqueWarp) * CLQ_MAX_WARPS,
+                            s1>>>(
         g, b_items.as<int32_t>(), nitems_b, ctr + 9, T, K4e, accs, cs, pow2_at_least(2 * dmax), dsplit, dmax,
-        d_status, five), note_launch());
+        d_status, five, cv.h0), note_launch());
   if (nwsmall > 0) {
     int per_sm = 1;
     ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_clique_warp, CLQ_WARPS * 32, 0));
     unsigned grid_w = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, (nwsmall + CLQ_WARPS - 1) / CLQ_WARPS);
     (k_clique_warp<<<grid_w, CLQ_WARPS * 32, 0, s1>>>(g, b_wsmall.as<int32_t>(), nwsmall, ctr + 8, T, K4e, accs,
-                                                      five), note_launch());
-  }
-  if (n > 0) {
-    (k_sym_u64<<<grid_for(n * 32, TPB, sms), TPB, 0, s1>>>(g, K4e), note_launch());
-    if (!cfg.partial)                          // a part's K4 sums are divided once every part's are in
-      (k_vertex_sum_div<<<grid_for(n * 32, TPB, sms), TPB, 0, s1>>>(g, K4e, K4v, 3), note_launch());
+                                                      five, cv.h0), note_launch());
   }
   mark(2, 1, s1);
   // 4-cycles (Thm 5)
@@ -3702,6 +3779,12 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
 
   // ---------------- closed forms over vertices and edges, then assembly
   mark(8, 0, s);
+  if (n > 0) {
+    (k_sym_K4<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, K4e, (const unsigned long long*)cbuf.k4, cbuf.k4_0),
+     note_launch());
+    if (!cfg.partial)                          // a part's K4 sums are divided once every part's are in
+      (k_vertex_sum_div<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, K4e, K4v, 3), note_launch());
+  }
   if (cfg.partial) {
     // one part of a split census: its raw sums; the closed forms need every
     // part's per-element counts and run in run_census_finish

@@ -36,6 +36,8 @@ enum AccId {
   ACC_DBP,        // sum over directed triangles of C(apexes above, 2)  directed bipyramids
   ACC_N17H,       // 2 x the core's share of N17 (core.cu)
   ACC_N18H,       // 4 x the core's share of N18
+  ACC_N20H,       // 3 x the core's share of N20
+  ACC_K4H,        // 12 x the 4-cliques inside the core
   ACC_COUNT
 };
 

@@ -14,6 +14,12 @@
 //       edge inside H (seen from both ends) .... 1/2 sum_{u>v} (W(u,v) - 2) M
 //       edge from c to below h0 ................ sum_{u>v} (W(u,v) - 2) b
 // With Y = M + 2b that is 1/2 sum (W - 2) Y and 1/4 sum (Y^2 - Y - 2 b^2).
+// For adjacent u and v, M + b is K4(t) of the triangle t = {c, u, v} (Thm 7), and
+// M counts the 4-cliques of t inside H, so over the adjacent pairs
+//   N20, triangles inside H ........ 1/3 sum C(M + b, 2)     (t is seen from three centres)
+//   K4 inside H .................... 1/12 sum M
+//   K4(c, u) inside H .............. 1/2 sum_v M
+// and the clique pass leaves these to the core for lowest vertices in H.
 // Every diamond and cycle not named here (a tip below h0; both ends of the edge
 // below h0; two adjacent cycle vertices below h0; a centre below h0) is counted
 // by the sweeps in census.cu, which skip the ones named here.
@@ -41,6 +47,7 @@ namespace esc {
 
 static constexpr int CORE_BLK = 128;                       // rows and columns of an operand block
 static constexpr int CORE_BLK_BYTES = CORE_BLK * CORE_BLK;
+static constexpr int CORE_BIT_WORDS = CORE_BLK * 4;        // words of bits per operand block
 static constexpr int CORE_TN = 256;                        // columns of an output tile (two blocks)
 static constexpr int CORE_STAGES = 4;
 static constexpr int CORE_STAGE_BYTES = 3 * CORE_BLK_BYTES;   // one block of rows, two of columns
@@ -226,7 +233,7 @@ __global__ void __launch_bounds__(256) k_core_mixed(DevGraph g, const uint32_t* 
 __global__ void __launch_bounds__(256) k_core_build(DevGraph g, const uint32_t* T, const int64_t* offp,
                                                     const int32_t* P, int64_t h0, int64_t h, const int32_t* dh,
                                                     const int64_t* off, int64_t s0, int64_t s1, int bit_words,
-                                                    uint8_t* blocks, int4* tiles) {
+                                                    uint8_t* blocks, uint32_t* bitm, int4* tiles) {
   extern __shared__ uint32_t core_bits[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t *rb_off = off, *blk_off = off + (h + 1), *tile_off = off + 2 * (h + 1);
@@ -240,6 +247,7 @@ __global__ void __launch_bounds__(256) k_core_build(DevGraph g, const uint32_t* 
   const int64_t blk0 = blk_off[s] - blk_off[s0];
   uint8_t* out = blocks + (blk0 + (int64_t)rb * nb) * CORE_BLK_BYTES;
   uint32_t* bits = core_bits + wid * bit_words;
+  uint32_t* bout = bitm + (blk0 + (int64_t)rb * nb) * CORE_BIT_WORDS;   // rows of 4 nb words
   for (int r = wid; r < CORE_BLK; r += 8) {
     const int a = rb * CORE_BLK + r;
     for (int i = lane; i < nb * 4; i += 32) bits[i] = 0u;
@@ -253,6 +261,7 @@ __global__ void __launch_bounds__(256) k_core_build(DevGraph g, const uint32_t* 
       }
     }
     __syncwarp();
+    for (int j = lane; j < nb * 4; j += 32) bout[r * (nb * 4) + j] = bits[j];
     for (int j = lane; j < nb * 8; j += 32) {
       const uint32_t x = bits[j >> 1] >> ((j & 1) * 16);
       uint4 o;                                  // bit -> byte 0x38 (1.0 in e4m3)
@@ -353,8 +362,10 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // so that the lanes of a warp read W(v, .) and b(v, .) along their rows.
 // Every wait is bounded: a wait that runs out sets the status word and ends the
 // CTA's work.  One centre with d = 16,000 runs at 3.4 PFLOP/s; the many smaller
-// centres of R-MAT 19 (3.3e13 multiply-adds in its triangle's tiles) take 38 ms
-// and are bound by the reads of W and b per entry, not by the MMAs.
+// centres of R-MAT 19 (3.3e13 multiply-adds in its triangle's tiles) take 42 ms
+// and are bound by the scattered sectors of W (512 MB, beyond L2) that the
+// entries read, not by the MMAs; the adjacency bits, N20 and the 4-clique sums
+// cost 4 ms of it and save the clique pass 22 ms.
 template <typename WT> struct CoreSum { typedef uint32_t type; };   // 32 terms below 2^18
 template <> struct CoreSum<uint32_t> { typedef unsigned long long type; };
 // barrier of the eight reading warps; true when ok holds on every thread
@@ -372,7 +383,8 @@ static constexpr size_t CORE_SMEM = 1024 + (size_t)CORE_STAGES * CORE_STAGE_BYTE
 template <typename WT, bool HASB>
 __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreView cv, const int4* tiles,
                                                               int64_t ntiles, const uint8_t* blocks,
-                                                              const WT* b_all, const int64_t* tri_off, int64_t s0,
+                                                              const uint32_t* bitm, unsigned long long* k4,
+                                                              int64_t k4_0, const WT* b_all, const int64_t* tri_off, int64_t s0,
                                                               AccSet acc, unsigned* status) {
   extern __shared__ uint8_t core_smem_raw[];
   __shared__ CoreBars bars;
@@ -401,8 +413,8 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  const int ids[2] = {ACC_N17H, ACC_N18H};
-  LocalAcc<2> la;
+  const int ids[4] = {ACC_N17H, ACC_N18H, ACC_N20H, ACC_K4H};
+  LocalAcc<4> la;
   la.zero();
   const int64_t step = gridDim.x;
   if (wid == CORE_EPI_WARPS) {                  // ------------ operand copies
@@ -502,7 +514,13 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
       }
       const int d = td.z, u = (td.w & 0xffff) * CORE_BLK + quad * 32 + lane, v0 = (td.w >> 16) * CORE_TN;
       const WT* bc = HASB ? b_all + (tri_off[td.y] - tri_off[s0]) : nullptr;
-      unsigned long long swy = 0, syy = 0, sy = 0, sbb = 0;
+      // adjacency bits of the warp's 32 rows, one word per column; the slots from
+      // pos on lead to vertices above c
+      const int64_t c = g.n - 1 - td.y;
+      const int nb = (d + CORE_BLK - 1) / CORE_BLK, pos = d - (int)(g.R[c + 1] - g.op[c]);
+      const uint32_t* bw = bitm + (int64_t)td.x * CORE_BIT_WORDS + (td.w & 0xffff) * 4 + quad;
+      unsigned long long* k4c = k4 + (g.R[c + 1] - d - k4_0);
+      unsigned long long swy = 0, syy = 0, sy = 0, sbb = 0, s20 = 0, sk = 0;
       const bool ok = mb_wait(smem_u32(&bars.accf[buf]), (it >> 1) & 1);
       tc_fence_after();
       const WT* const* wr = wrow + buf * CORE_TN;
@@ -515,6 +533,11 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
         uint32_t m[QC];
         tmem_ld(m, tmem + buf * CORE_TN + q0 + ((uint32_t)(quad * 32) << 16));
         uint32_t w[QC], bb[HASB ? QC : 1];
+        uint32_t adj = 0, col = 0;              // lane l: the bits and the M sum of column vb + l
+        if (lane < QC) {
+          const int v = vb + lane;              // padded rows are zero
+          adj = __ldg(bw + (int64_t)(v / CORE_BLK) * nb * CORE_BIT_WORDS + (v % CORE_BLK) * (nb * 4));
+        }
         const bool full = vb > u && vb + QC - 1 < d;
 #pragma unroll
         for (int q = 0; q < QC; ++q) {
@@ -532,22 +555,34 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
           const bool on = full || (vb + q > u && vb + q < d);
           // an integer below 2^23 in fp32: its low mantissa bits after adding 2^23
           uint32_t y = on ? __float_as_uint(__uint_as_float(m[q]) + 8388608.0f) & 0x7fffffu : 0u;
+          const bool ad = ((__shfl_sync(0xffffffffu, adj, q) >> lane) & 1u) != 0;
+          const uint32_t mk = ad ? y : 0u;
+          const uint32_t cs = __reduce_add_sync(0xffffffffu, mk);
+          if (lane == q) col = cs;
+          sk += mk;
+          uint32_t k = mk;
           if (HASB) {
             const uint32_t b = bb[HASB ? q : 0];
             y += 2 * b;
             sbb += (unsigned long long)b * b;
+            if (ad) k += b;
           }
+          s20 += (unsigned long long)k * (k - 1u);   // k = 0: 0 x (2^32 - 1)
           swy += (unsigned long long)w[q] * y;
           syy += (unsigned long long)y * y;
           sy32 += y;
         }
         sy += sy32;
+        if (col && vb + lane >= pos) atomicAdd(&k4c[vb + lane], (unsigned long long)col);
       }
+      if (sk && u >= pos) atomicAdd(&k4c[u], sk);
       tc_fence_before();
       __syncwarp();
       if (lane == 0 && ok) mb_arrive(smem_u32(&bars.acce[buf]));
       la.v[0] += swy - 2 * sy;                  // 2 x N17: W >= 2 wherever Y > 0
       la.v[1] += syy - sy - 2 * sbb;            // 4 x N18
+      la.v[2] += s20 / 2;                       // 3 x N20
+      la.v[3] += sk;                            // 12 x K4
       warp_item_flush(la, ids, acc, g.n - 1 - td.y);
       if (more) {
         wrow[(buf ^ 1) * CORE_TN + tid] = Wm + (lv1 >= 0 ? cv.rowb[lv1] : 0);
@@ -630,6 +665,7 @@ void core_chunks(const int64_t* off, int64_t h, int64_t cap_bytes, CoreChunks* c
   }
 }
 size_t core_block_bytes(const CoreChunks& ck) { return (size_t)ck.max_blocks * CORE_BLK_BYTES; }
+size_t core_bit_bytes(const CoreChunks& ck) { return (size_t)ck.max_blocks * CORE_BIT_WORDS * sizeof(uint32_t); }
 
 template <typename WT>
 static cudaError_t core_run_as(const DevGraph& g, const CoreView& cv, const uint32_t* T, const int64_t* offp,
@@ -656,17 +692,21 @@ static cudaError_t core_run_as(const DevGraph& g, const CoreView& cv, const uint
       (k_core_mixed<WT><<<(unsigned)(s1 - s0), 256, 0, s>>>(g, T, offp, P, cv.h0, cv.dh, d_tri, s0, b), note_launch());
     }
     (k_core_build<<<(unsigned)(rb[s1] - rb[s0]), 256, smem_b, s>>>(g, T, offp, P, cv.h0, h, cv.dh, d_off, s0, s1,
-                                                                   bit_words, (uint8_t*)cb.blocks, (int4*)cb.tiles),
+                                                                   bit_words, (uint8_t*)cb.blocks, (uint32_t*)cb.bits,
+                                                                   (int4*)cb.tiles),
      note_launch());
     const unsigned grid = (unsigned)std::min<int64_t>(sms, nt);
     if (b)
       (k_core_mma<WT, true><<<grid, CORE_THREADS, CORE_SMEM, s>>>(g, cv, (const int4*)cb.tiles, nt,
-                                                                  (const uint8_t*)cb.blocks, b, d_tri, s0, acc, status),
+                                                                  (const uint8_t*)cb.blocks, (const uint32_t*)cb.bits,
+                                                                  (unsigned long long*)cb.k4, cb.k4_0, b, d_tri, s0, acc,
+                                                                  status),
        note_launch());
     else
       (k_core_mma<WT, false><<<grid, CORE_THREADS, CORE_SMEM, s>>>(g, cv, (const int4*)cb.tiles, nt,
-                                                                   (const uint8_t*)cb.blocks, nullptr, d_tri, s0, acc,
-                                                                   status),
+                                                                   (const uint8_t*)cb.blocks, (const uint32_t*)cb.bits,
+                                                                   (unsigned long long*)cb.k4, cb.k4_0, nullptr, d_tri,
+                                                                   s0, acc, status),
        note_launch());
     e = cudaGetLastError();
   }

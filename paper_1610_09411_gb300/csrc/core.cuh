@@ -16,7 +16,10 @@ struct CoreChunks {
 };
 struct CoreBuffers {
   void* blocks = nullptr;          // core_block_bytes(chunks)
+  void* bits = nullptr;            // core_bit_bytes(chunks): the same matrices as bits
   void* tiles = nullptr;           // 16 bytes x max_tiles
+  void* k4 = nullptr;              // zeroed u64 per slot from k4_0, the first one of rank h0
+  int64_t k4_0 = 0;
   void* b = nullptr;               // max_tri counts as wide as W's; null when no vertex lies below the core
 };
 
@@ -30,7 +33,8 @@ cudaError_t core_low(const DevGraph& g, const uint32_t* T, const int64_t* off, c
                      uint32_t* low, int sms, cudaStream_t s);
 void core_chunks(const int64_t* off, int64_t h, int64_t cap_bytes, CoreChunks* ck);
 size_t core_block_bytes(const CoreChunks& ck);
-// every chunk's contraction; adds to ACC_N17H and ACC_N18H
+size_t core_bit_bytes(const CoreChunks& ck);
+// every chunk's contraction; adds to ACC_N17H, ACC_N18H, ACC_N20H, ACC_K4H and k4
 cudaError_t core_run(const DevGraph& g, const CoreView& cv, const uint32_t* T, const int64_t* offp, const int32_t* P,
                      const int64_t* d_off, const int64_t* off, const CoreChunks& ck, const CoreBuffers& cb,
                      const AccSet& acc, unsigned* status, int sms, int smem_optin, cudaStream_t s);
