@@ -201,7 +201,7 @@ escape_status escape_last_basis_counts(const escape_graph* g, escape_u128* out);
  * Work space is one fixed device array of ESCAPE_NOALLOC_MAX_N x 64 words
  * (8 MiB) inside the library, shared by every call: calls whose GPU work
  * overlaps (on different streams or threads) race and must be serialised by
- * the caller.  Each call clears the work space and the outputs before
+ * the caller.  Each call sets up the work space and clears the outputs before
  * counting.  The array takes its device memory when the library's device
  * code is loaded on a device -- with CUDA's lazy module loading, during the
  * first call on that device -- and keeps it until the process exits; so make

@@ -9,32 +9,43 @@
 //
 // The counting is the 4-cycle rule of the main library (for the highest
 // vertex i of a 4-cycle and the opposite vertex j, the number of middles
-// below i), run here directly on the caller's CSR with the degree order
-// computed on the fly instead of renaming vertices.
+// below i), run here directly on the caller's CSR: the degree order is a key per
+// vertex, (row length, id) in one 32-bit word.
+//
+// All counters are in shared memory: a vertex of at most 32 neighbours has at
+// most 32 x 32 wedges to lower vertices (a middle has no more neighbours than
+// it), counted by one warp in a packed hash table; the others take one CTA with
+// a counter and a place in the touched list for every vertex (6 bytes x 32,768).
+// Chung-Lu n = 30,011 (232,000 edges): 0.59 ms, against 4.85 ms with 32 CTAs
+// counting in global memory and two row lengths read per comparison; the heavy
+// vertices take 0.42 ms of it, bound by the latency of their list walks.
 #include "../../include/escape.h"
 #include "common.cuh"
 #include "internal.h"
 
+#include <algorithm>
 #include <mutex>
 
 namespace {
 
-constexpr int NA_CTAS = 32;                         // persistent CTAs
-constexpr int NA_THREADS = 512;
 constexpr int64_t NA_MAX_N = ESCAPE_NOALLOC_MAX_N;  // vertices
-// Work space shared by every call on this device: per CTA a counter array and
-// a touched list of NA_MAX_N entries each (8 MiB in total), then a header of
-// 64 words (work counter, status).
-constexpr int64_t NA_WORDS = (int64_t)NA_CTAS * NA_MAX_N * 2 + 64;
+constexpr int NA_LIGHT_DEG = 32, NA_LIGHT_WARPS = 8, NA_LIGHT_LOG = 11, NA_HEAVY_THREADS = 1024;
+constexpr int NA_ILP = 4;
+// Work space shared by every call on this device (8 MiB reserved): a header of
+// 64 words (heavy items, queue, status), the order keys and the list of heavy
+// vertices.
+constexpr int64_t NA_WORDS = (int64_t)64 * NA_MAX_N + 64;
 static __device__ __align__(256) unsigned int g_noalloc_scratch[NA_WORDS];
+struct NaSpace {
+  unsigned int *heavy_n, *queue, *status, *key;
+  int32_t* heavy;
+};
+NaSpace na_space(unsigned int* base) {
+  return NaSpace{base, base + 1, base + 2, base + 64, (int32_t*)(base + 64 + NA_MAX_N)};
+}
 
 std::mutex g_mu;
 void* g_addr[64] = {nullptr};     // device address of g_noalloc_scratch, per device
-
-__device__ __forceinline__ bool na_prec(const int64_t* rp, int64_t a, int64_t b) {
-  int64_t da = rp[a + 1] - rp[a], db = rp[b + 1] - rp[b];
-  return da < db || (da == db && a < b);
-}
 
 // Row v's entry range, clamped: an offset outside [0, rp[n]] or a row that
 // ends before it starts sets the status word and reads as an empty row, so no
@@ -50,73 +61,197 @@ __device__ __forceinline__ void na_row(const int64_t* rp, int64_t n, int64_t v, 
   }
 }
 
-__global__ void k_cycles4_noalloc(const int64_t* rp, const int32_t* col, int64_t n, unsigned int* scratch,
-                                  unsigned long long* c4v, unsigned long long* c4_total) {
-  __shared__ u128 sh[32];
-  __shared__ int64_t sh_item;
-  unsigned int* w = scratch + (int64_t)blockIdx.x * NA_MAX_N;
-  int32_t* tl = (int32_t*)(scratch + (int64_t)NA_CTAS * NA_MAX_N + (int64_t)blockIdx.x * NA_MAX_N);
-  unsigned int* hdr = scratch + (int64_t)NA_CTAS * NA_MAX_N * 2;
-  unsigned long long* ctr = (unsigned long long*)hdr;          // hdr[0..1]
-  unsigned int* status = hdr + 2;
-  __shared__ unsigned int nt;
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  u128 total = 0;
-  while (true) {
-    if (threadIdx.x == 0) sh_item = (int64_t)atomicAdd(ctr, 1ull);
-    __syncthreads();
-    int64_t i = sh_item;
-    __syncthreads();
-    if (i >= n) break;
-    if (threadIdx.x == 0) nt = 0;
-    __syncthreads();
-    int64_t ib, ie;
-    na_row(rp, n, i, ib, ie, status);
-    // pass 1: wedges i - k - j with k, j below i in the degree order
-    for (int64_t p = ib + wid; p < ie; p += nw) {
-      int32_t k = col[p];
-      if (k < 0 || k >= n) { if (lane == 0) atomicOr(status, 1u); continue; }
-      if (!na_prec(rp, k, i)) continue;
-      int64_t kb, ke;
-      na_row(rp, n, k, kb, ke, status);
-      for (int64_t q = kb + lane; q < ke; q += 32) {
-        int32_t j = col[q];
-        if (j < 0 || j >= n) { atomicOr(status, 1u); continue; }
-        if (j == i || !na_prec(rp, j, i)) continue;
-        if (atomicAdd(&w[j], 1u) == 0) tl[atomicAdd(&nt, 1u)] = j;
+// Order keys and zeroed outputs.  A row is at most n - 1 < 2^15 entries long in a
+// simple graph; longer ones (malformed) share the largest length.
+__global__ void k_na_prep(const int64_t* rp, int64_t n, NaSpace ns, unsigned long long* c4v,
+                          unsigned long long* c4_total) {
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v == 0) *c4_total = 0;
+  if (v >= n) return;
+  int64_t b, e;
+  na_row(rp, n, v, b, e, ns.status);
+  ns.key[v] = ((unsigned int)min(e - b, (int64_t)0x1ffff) << 15) | (unsigned int)v;
+  c4v[v] = 0;
+}
+
+__device__ __forceinline__ int na_len(unsigned int key) { return (int)(key >> 15); }
+
+// One warp per vertex of at most NA_LIGHT_DEG neighbours (lane l takes the l-th
+// one's row); the other vertices go to the heavy list.
+__global__ void __launch_bounds__(NA_LIGHT_WARPS * 32) k_na_light(const int64_t* rp, const int32_t* col, int64_t n,
+                                                                 NaSpace ns, unsigned long long* c4v,
+                                                                 unsigned long long* c4_total) {
+  extern __shared__ uint4 na_smem[];
+  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+  uint32_t* tab = reinterpret_cast<uint32_t*>(na_smem) + (wl << NA_LIGHT_LOG);
+  const int64_t nwarps = (int64_t)gridDim.x * NA_LIGHT_WARPS;
+  unsigned long long total = 0;
+  for (int64_t i = (int64_t)blockIdx.x * NA_LIGHT_WARPS + wl; i < n; i += nwarps) {
+    const unsigned int ki = ns.key[i];
+    const int d = na_len(ki);
+    if (d > NA_LIGHT_DEG) {
+      if (lane == 0) ns.heavy[atomicAdd(ns.heavy_n, 1u)] = (int32_t)i;
+      continue;
+    }
+    int64_t b, e, kb = 0, ke = 0;
+    na_row(rp, n, i, b, e, ns.status);
+    int32_t k = -1;
+    if (lane < d && b + lane < e) {
+      k = col[b + lane];
+      if (k < 0 || k >= n) {
+        atomicOr(ns.status, 1u);
+        k = -1;
+      } else if (ns.key[k] < ki) {
+        na_row(rp, n, k, kb, ke, ns.status);
       }
     }
-    __syncthreads();
-    unsigned int ntc = nt;
-    // pass 2: C(w, 2) to i and j
-    u128 mine = 0;
-    for (unsigned int t = threadIdx.x; t < ntc; t += blockDim.x) {
-      int32_t j = tl[t];
-      unsigned long long c = (unsigned long long)w[j] * (w[j] - 1) / 2;
-      if (c) { atomicAdd(&c4v[j], c); mine += c; }
-    }
-    u128 s = block_sum_u128(mine, sh);
-    if (threadIdx.x == 0) { if (s) atomicAdd(&c4v[i], (unsigned long long)s); total += s; }
-    // pass 3: w - 1 to every middle k
-    for (int64_t p = ib + wid; p < ie; p += nw) {
-      int32_t k = col[p];
-      if (k < 0 || k >= n || !na_prec(rp, k, i)) continue;
-      unsigned long long sk = 0;
-      int64_t kb, ke;
-      na_row(rp, n, k, kb, ke, status);
-      for (int64_t q = kb + lane; q < ke; q += 32) {
-        int32_t j = col[q];
-        if (j < 0 || j >= n || j == i || !na_prec(rp, j, i)) continue;
-        sk += w[j] - 1;
+    if (d < 2) continue;
+    // key << 16 | count: ids below 2^15 and counts of at most 2^10, so no used word is all ones
+    const int log = max(7, 32 - __clz(2 * d * d - 1));
+    const uint32_t mask = (1u << log) - 1u;
+    for (int t = lane; t < (1 << log) / 4; t += 32)
+      reinterpret_cast<uint4*>(tab)[t] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncwarp();
+    auto slot_of = [&](int32_t j, bool insert) -> int {
+      uint32_t sl = ((uint32_t)j * 0x9E3779B1u) >> (32 - log);
+      for (uint32_t probe = 0; probe <= mask; ++probe) {
+        uint32_t w = *(volatile uint32_t*)&tab[sl];
+        if (w == ~0u) {
+          if (!insert) return -1;
+          w = atomicCAS(&tab[sl], ~0u, (uint32_t)j << 16);
+          if (w == ~0u) return (int)sl;
+        }
+        if ((w >> 16) == (uint32_t)j) return (int)sl;
+        sl = (sl + 1u) & mask;
       }
-      sk = warp_sum_u64(sk);
-      if (lane == 0 && sk) atomicAdd(&c4v[k], sk);
+      return -1;
+    };
+    for (int64_t q = kb; q < ke; ++q) {
+      const int32_t j = col[q];
+      if (j < 0 || j >= n) {
+        atomicOr(ns.status, 1u);
+        continue;
+      }
+      if (j == i || ns.key[j] >= ki) continue;
+      const int sl = slot_of(j, true);
+      if (sl >= 0) atomicAdd(&tab[sl], 1u);
     }
-    __syncthreads();
-    for (unsigned int t = threadIdx.x; t < ntc; t += blockDim.x) w[tl[t]] = 0;
-    __syncthreads();
+    __syncwarp();
+    unsigned long long sk = 0;
+    for (int64_t q = kb; q < ke; ++q) {
+      const int32_t j = col[q];
+      if (j < 0 || j >= n || j == i || ns.key[j] >= ki) continue;
+      const int sl = slot_of(j, false);
+      if (sl >= 0) sk += (tab[sl] & 0xffffu) - 1u;
+    }
+    if (sk) atomicAdd(&c4v[k], sk);
+    unsigned long long mine = 0;
+    for (int t = lane; t <= (int)mask; t += 32) {
+      const uint32_t w = tab[t];
+      if (w == ~0u) continue;
+      const unsigned long long c = (unsigned long long)(w & 0xffffu) * ((w & 0xffffu) - 1u) / 2;
+      if (c) {
+        atomicAdd(&c4v[w >> 16], c);
+        mine += c;
+      }
+    }
+    mine = warp_sum_u64(mine);
+    if (lane == 0 && mine) atomicAdd(&c4v[i], mine);
+    total += mine;                              // valid on lane 0
+    __syncwarp();                               // the table is read before the next item clears it
   }
   // each 4-cycle is counted once, at its highest vertex
+  if (lane == 0 && total) atomicAdd(c4_total, total);
+}
+
+// One CTA per heavy vertex: counters of every vertex and the touched list in
+// shared memory.
+__global__ void __launch_bounds__(NA_HEAVY_THREADS, 1) k_na_heavy(const int64_t* rp, const int32_t* col, int64_t n,
+                                                                 NaSpace ns, unsigned long long* c4v,
+                                                                 unsigned long long* c4_total) {
+  extern __shared__ uint4 na_smem[];
+  __shared__ u128 sh[32];
+  __shared__ unsigned int sh_item, nt;
+  uint32_t* w = reinterpret_cast<uint32_t*>(na_smem);
+  uint16_t* tl = reinterpret_cast<uint16_t*>(w + n);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned int items = *ns.heavy_n;
+  u128 total = 0;
+  for (int64_t t = threadIdx.x; t < n; t += blockDim.x) w[t] = 0;
+  while (true) {
+    if (threadIdx.x == 0) {
+      sh_item = atomicAdd(ns.queue, 1u);
+      nt = 0;
+    }
+    __syncthreads();
+    const unsigned int it = sh_item;
+    if (it >= items) break;
+    const int64_t i = ns.heavy[it];
+    const unsigned int ki = ns.key[i];
+    int64_t ib, ie;
+    na_row(rp, n, i, ib, ie, ns.status);
+    // one pass over the wedges i - k - j with k, j below i; `first` counts them
+    auto wedges = [&](bool first) {
+      for (int64_t p = ib + wid; p < ie; p += nw) {
+        const int32_t k = col[p];
+        if (k < 0 || k >= n) {
+          if (lane == 0) atomicOr(ns.status, 1u);
+          continue;
+        }
+        if (ns.key[k] >= ki) continue;
+        int64_t kb, ke;
+        na_row(rp, n, k, kb, ke, ns.status);
+        unsigned long long sk = 0;
+        for (int64_t q = kb + lane; q < ke; q += 32 * NA_ILP) {
+          int32_t j[NA_ILP];
+          unsigned int kj[NA_ILP];
+#pragma unroll
+          for (int u = 0; u < NA_ILP; ++u) j[u] = q + 32 * u < ke ? col[q + 32 * u] : (int32_t)i;
+#pragma unroll
+          for (int u = 0; u < NA_ILP; ++u) {
+            if (j[u] < 0 || j[u] >= n) {
+              atomicOr(ns.status, 1u);
+              j[u] = (int32_t)i;
+            }
+            kj[u] = ns.key[j[u]];               // i itself is not below i
+          }
+#pragma unroll
+          for (int u = 0; u < NA_ILP; ++u) {
+            if (kj[u] >= ki) continue;
+            if (first) {
+              if (atomicAdd(&w[j[u]], 1u) == 0) tl[atomicAdd(&nt, 1u)] = (uint16_t)j[u];
+            } else {
+              sk += w[j[u]] - 1u;
+            }
+          }
+        }
+        if (!first) {
+          sk = warp_sum_u64(sk);
+          if (lane == 0 && sk) atomicAdd(&c4v[k], sk);
+        }
+      }
+    };
+    wedges(true);
+    __syncthreads();
+    const unsigned int ntc = nt;
+    wedges(false);                              // w - 1 to every middle k
+    __syncthreads();
+    u128 mine = 0;                              // C(w, 2) to i and j
+    for (unsigned int t = threadIdx.x; t < ntc; t += blockDim.x) {
+      const int32_t j = tl[t];
+      const unsigned long long c = (unsigned long long)w[j] * (w[j] - 1) / 2;
+      w[j] = 0;
+      if (c) {
+        atomicAdd(&c4v[j], c);
+        mine += c;
+      }
+    }
+    const u128 s = block_sum_u128(mine, sh);    // its barriers also end the reads of nt and sh_item
+    if (threadIdx.x == 0) {
+      if (s) atomicAdd(&c4v[i], (unsigned long long)s);
+      total += s;
+    }
+  }
   if (threadIdx.x == 0 && total) atomicAdd(c4_total, (unsigned long long)total);
 }
 
@@ -142,21 +277,32 @@ extern "C" escape_status escape_cycles4_noalloc(int64_t n, const int64_t* row_pt
     }
     base = g_addr[dev];
   }
-  unsigned int* scratch = (unsigned int*)base;
-  // everything the kernel expects to start at zero: counters, header, outputs
-  e = cudaMemsetAsync(scratch, 0, sizeof(unsigned int) * (size_t)NA_WORDS, s);
-  if (e == cudaSuccess && n > 0) e = cudaMemsetAsync(c4_v, 0, sizeof(uint64_t) * (size_t)n, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c4_total, 0, sizeof(uint64_t), s);
+  const NaSpace ns = na_space((unsigned int*)base);
+  int sms = 1;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // the header starts at zero; keys, lists and outputs are written by the kernels
+  e = cudaMemsetAsync(base, 0, sizeof(unsigned int) * 64, s);
+  if (n == 0 && e == cudaSuccess) e = cudaMemsetAsync(c4_total, 0, sizeof(uint64_t), s);
+  const size_t sm_light = (sizeof(uint32_t) << NA_LIGHT_LOG) * NA_LIGHT_WARPS;
+  const size_t sm_heavy = (sizeof(uint32_t) + sizeof(uint16_t)) * (size_t)NA_MAX_N;
+  if (n > 0) {                                  // the same limits at every call
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_na_light, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_light);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_na_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_heavy);
+  }
   if (e != cudaSuccess) { cudaGetLastError(); esc::note_cuda_error(e); return ESCAPE_ECUDA; }
   if (n > 0) {
-    k_cycles4_noalloc<<<NA_CTAS, NA_THREADS, 0, s>>>(row_ptr, col, n, scratch, (unsigned long long*)c4_v,
-                                                     (unsigned long long*)c4_total);
+    unsigned long long *v = (unsigned long long*)c4_v, *tot = (unsigned long long*)c4_total;
+    const unsigned warps_grid = (unsigned)std::min<int64_t>((n + NA_LIGHT_WARPS - 1) / NA_LIGHT_WARPS, (int64_t)sms * 3);
+    k_na_prep<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(row_ptr, n, ns, v, tot);
+    k_na_light<<<warps_grid, NA_LIGHT_WARPS * 32, sm_light, s>>>(row_ptr, col, n, ns, v, tot);
+    k_na_heavy<<<(unsigned)sms, NA_HEAVY_THREADS, (sizeof(uint32_t) + sizeof(uint16_t)) * (size_t)((n + 1) & ~1ll), s>>>(
+        row_ptr, col, n, ns, v, tot);
   }
   unsigned int status = 0;
   e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&status, scratch + (int64_t)NA_CTAS * NA_MAX_N * 2 + 2, sizeof(unsigned int),
-                        cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, ns.status, sizeof(unsigned int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) { cudaGetLastError(); esc::note_cuda_error(e); return ESCAPE_ECUDA; }
   return status ? ESCAPE_EINVAL : ESCAPE_OK;
