@@ -2594,7 +2594,7 @@ __global__ void k_edge_sums(DevGraph g, const uint32_t* T, const unsigned long l
 }
 
 // ============================================================================
-// Assembly (Thm 3, App. A; Thms 4, 8-14; App. B).  One thread; all arithmetic
+// Assembly (Thm 3, App. A; Thms 4, 8-14; App. B).  All arithmetic
 // modulo 2^128, which is exact because every final count is below 2^127.
 // out: induced c3[4], c4[11], c5[34], then non-induced n3, n4, n5 (u128 each).
 // ============================================================================
@@ -2612,85 +2612,93 @@ __device__ __forceinline__ u128 cnk(u128 n, int k) {
   return r;
 }
 
-// One thread per graph: graph k reads accumulator row k and writes result k.
+// One CTA of ASM_THREADS threads per graph: graph k reads accumulator row k and
+// writes result k.  Every non-induced count and every row of the conversion is
+// one thread's (128-bit products and divisions by one thread took 54 us).
 // basis_all (optional): per graph the four counts the runtime is linear in
 // (Sec. 8's runtime fit): W, D, directed 3-paths, directed bipyramids.
-__global__ void k_assemble(const Acc128* acc_all, const unsigned long long* n_arr, const unsigned long long* m_arr,
-                           int num_graphs, ConvTables tabs, unsigned long long* out_all, u128* basis_all) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= num_graphs) return;
-  const Acc128* acc = acc_all + (int64_t)k * ACC_COUNT;
-  unsigned long long* out = out_all + (int64_t)k * 2 * 98;
-  u128 A[ACC_COUNT];
-  for (int i = 0; i < ACC_COUNT; ++i) A[i] = ((u128)acc[i].hi << 64) | acc[i].lo;
-  if (basis_all) {
-    u128* bo = basis_all + (int64_t)k * 4;
-    bo[0] = A[ACC_W];
-    bo[1] = A[ACC_D];
-    bo[2] = A[ACC_DP];
-    bo[3] = A[ACC_DBP];
-  }
-  u128 n = n_arr[k], m = m_arr[k];
-  u128 W = A[ACC_W], T = A[ACC_T], TT = A[ACC_TT], C4 = A[ACC_C4], D = A[ACC_D];
-  u128 K4 = (A[ACC_K4] + A[ACC_K4H] / 4) / 3, S3 = A[ACC_S3];
-  u128 P4 = A[ACC_P4A] - 3 * T;
-  u128 N[35];
-  N[1] = A[ACC_S4];
-  N[2] = A[ACC_N2A] - 2 * TT;
-  N[3] = A[ACC_N3A] - 4 * C4 - 2 * TT - 3 * T;
-  N[4] = A[ACC_N4];
-  N[5] = A[ACC_N5A] - 4 * D;
-  N[6] = A[ACC_N6A] - 2 * D;
-  N[7] = A[ACC_N7A] - 2 * D;
-  N[8] = A[ACC_N8M] - A[ACC_N8Z];
-  N[9] = A[ACC_N9A] - 2 * D;
-  N[10] = A[ACC_N10A] - 12 * K4;
-  N[11] = A[ACC_N11];
-  N[12] = A[ACC_N12A] - 4 * D;
-  N[13] = A[ACC_N13];
-  N[14] = A[ACC_N14];
-  N[15] = A[ACC_N15];
-  N[16] = A[ACC_N16A] - 12 * K4;
-  N[17] = A[ACC_N17] + A[ACC_N17H] / 2;
-  N[18] = A[ACC_N18] + A[ACC_N18H] / 4;
-  N[19] = A[ACC_N19];
-  N[20] = A[ACC_N20] + A[ACC_N20H] / 3;
-  N[21] = A[ACC_N21];
-  N[22] = cnk(n, 5);
-  N[23] = n >= 2 ? m * cnk(n - 2, 3) : 0;
-  N[24] = n >= 4 ? (cnk(m, 2) - W) * (n - 4) : 0;
-  N[25] = n >= 3 ? W * cnk(n - 3, 2) : 0;
-  N[26] = n >= 3 ? T * cnk(n - 3, 2) : 0;
-  N[27] = n >= 4 ? S3 * (n - 4) : 0;
-  N[28] = n >= 4 ? P4 * (n - 4) : 0;
-  N[29] = n >= 4 ? TT * (n - 4) : 0;
-  N[30] = n >= 4 ? C4 * (n - 4) : 0;
-  N[31] = n >= 4 ? D * (n - 4) : 0;
-  N[32] = n >= 4 ? K4 * (n - 4) : 0;
-  N[33] = W * m - A[ACC_D2D] - A[ACC_DNBR] + 2 * W + 3 * T;
-  N[34] = T * m - A[ACC_TD] + 3 * T;
-  u128 n4[11] = {S3, P4, TT, C4, D, K4, cnk(n, 4), n >= 2 ? m * cnk(n - 2, 2) : 0, cnk(m, 2) - W,
-                 n >= 3 ? W * (n - 3) : 0, n >= 3 ? T * (n - 3) : 0};
-  u128 n3[4] = {cnk(n, 3), n >= 2 ? m * (n - 2) : 0, W, T};
-  // induced = A^-1 * non-induced (signed integer matrix, arithmetic mod 2^128)
-  u128* o = (u128*)out;
-  for (int i = 0; i < 4; ++i) {
-    u128 s = 0;
-    for (int j = 0; j < 4; ++j) s += (u128)(__int128)tabs.a3[i * 4 + j] * n3[j];
-    o[i] = s;
-    o[49 + i] = n3[i];
-  }
-  for (int i = 0; i < 11; ++i) {
-    u128 s = 0;
-    for (int j = 0; j < 11; ++j) s += (u128)(__int128)tabs.a4[i * 11 + j] * n4[j];
-    o[4 + i] = s;
-    o[49 + 4 + i] = n4[i];
-  }
-  for (int i = 0; i < 34; ++i) {
-    u128 s = 0;
-    for (int j = 0; j < 34; ++j) s += (u128)(__int128)tabs.a5[i * 34 + j] * N[j + 1];
-    o[15 + i] = s;
-    o[49 + 15 + i] = N[i + 1];
+static constexpr int ASM_THREADS = 64;
+__global__ void __launch_bounds__(ASM_THREADS) k_assemble(const Acc128* acc_all, const unsigned long long* n_arr,
+                                                         const unsigned long long* m_arr, int num_graphs,
+                                                         ConvTables tabs, unsigned long long* out_all,
+                                                         u128* basis_all) {
+  __shared__ u128 A[ACC_COUNT], cnt[49];        // cnt: n3[4], n4[11], n5[34]
+  const int t = threadIdx.x;
+  for (int k = blockIdx.x; k < num_graphs; k += gridDim.x) {
+    const Acc128* acc = acc_all + (int64_t)k * ACC_COUNT;
+    __syncthreads();                            // the last graph's counts are read
+    if (t < ACC_COUNT) A[t] = ((u128)acc[t].hi << 64) | acc[t].lo;
+    __syncthreads();
+    if (basis_all && t < 4)
+      basis_all[(int64_t)k * 4 + t] = t == 0 ? A[ACC_W] : (t == 1 ? A[ACC_D] : (t == 2 ? A[ACC_DP] : A[ACC_DBP]));
+    const u128 n = n_arr[k], m = m_arr[k];
+    const u128 W = A[ACC_W], T = A[ACC_T], TT = A[ACC_TT], C4 = A[ACC_C4], D = A[ACC_D], S3 = A[ACC_S3];
+    const u128 K4 = (A[ACC_K4] + A[ACC_K4H] / 4) / 3, P4 = A[ACC_P4A] - 3 * T;
+    u128 v = 0;
+    switch (t) {
+      case 0: v = cnk(n, 3); break;
+      case 1: v = n >= 2 ? m * (n - 2) : 0; break;
+      case 2: v = W; break;
+      case 3: v = T; break;
+      case 4: v = S3; break;
+      case 5: v = P4; break;
+      case 6: v = TT; break;
+      case 7: v = C4; break;
+      case 8: v = D; break;
+      case 9: v = K4; break;
+      case 10: v = cnk(n, 4); break;
+      case 11: v = n >= 2 ? m * cnk(n - 2, 2) : 0; break;
+      case 12: v = cnk(m, 2) - W; break;
+      case 13: v = n >= 3 ? W * (n - 3) : 0; break;
+      case 14: v = n >= 3 ? T * (n - 3) : 0; break;
+      // 5-vertex patterns 1 .. 34
+      case 15: v = A[ACC_S4]; break;
+      case 16: v = A[ACC_N2A] - 2 * TT; break;
+      case 17: v = A[ACC_N3A] - 4 * C4 - 2 * TT - 3 * T; break;
+      case 18: v = A[ACC_N4]; break;
+      case 19: v = A[ACC_N5A] - 4 * D; break;
+      case 20: v = A[ACC_N6A] - 2 * D; break;
+      case 21: v = A[ACC_N7A] - 2 * D; break;
+      case 22: v = A[ACC_N8M] - A[ACC_N8Z]; break;
+      case 23: v = A[ACC_N9A] - 2 * D; break;
+      case 24: v = A[ACC_N10A] - 12 * K4; break;
+      case 25: v = A[ACC_N11]; break;
+      case 26: v = A[ACC_N12A] - 4 * D; break;
+      case 27: v = A[ACC_N13]; break;
+      case 28: v = A[ACC_N14]; break;
+      case 29: v = A[ACC_N15]; break;
+      case 30: v = A[ACC_N16A] - 12 * K4; break;
+      case 31: v = A[ACC_N17] + A[ACC_N17H] / 2; break;
+      case 32: v = A[ACC_N18] + A[ACC_N18H] / 4; break;
+      case 33: v = A[ACC_N19]; break;
+      case 34: v = A[ACC_N20] + A[ACC_N20H] / 3; break;
+      case 35: v = A[ACC_N21]; break;
+      case 36: v = cnk(n, 5); break;
+      case 37: v = n >= 2 ? m * cnk(n - 2, 3) : 0; break;
+      case 38: v = n >= 4 ? (cnk(m, 2) - W) * (n - 4) : 0; break;
+      case 39: v = n >= 3 ? W * cnk(n - 3, 2) : 0; break;
+      case 40: v = n >= 3 ? T * cnk(n - 3, 2) : 0; break;
+      case 41: v = n >= 4 ? S3 * (n - 4) : 0; break;
+      case 42: v = n >= 4 ? P4 * (n - 4) : 0; break;
+      case 43: v = n >= 4 ? TT * (n - 4) : 0; break;
+      case 44: v = n >= 4 ? C4 * (n - 4) : 0; break;
+      case 45: v = n >= 4 ? D * (n - 4) : 0; break;
+      case 46: v = n >= 4 ? K4 * (n - 4) : 0; break;
+      case 47: v = W * m - A[ACC_D2D] - A[ACC_DNBR] + 2 * W + 3 * T; break;
+      case 48: v = T * m - A[ACC_TD] + 3 * T; break;
+    }
+    if (t < 49) cnt[t] = v;
+    __syncthreads();
+    // induced = A^-1 * non-induced (signed integer matrix, arithmetic mod 2^128)
+    if (t < 49) {
+      const int first = t < 4 ? 0 : (t < 15 ? 4 : 15), len = t < 4 ? 4 : (t < 15 ? 11 : 34);
+      const long long* row = (t < 4 ? tabs.a3 : (t < 15 ? tabs.a4 : tabs.a5)) + (t - first) * len;
+      u128 s = 0;
+      for (int j = 0; j < len; ++j) s += (u128)(__int128)row[j] * cnt[first + j];
+      u128* o = (u128*)(out_all + (int64_t)k * 2 * 98);
+      o[t] = s;
+      o[49 + t] = cnt[t];
+    }
   }
 }
 
@@ -3793,7 +3801,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     if (n > 0)
       (k_edge_sums<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T, C4e, K4e, tv, C4v, K4v, accs), note_launch());
     const ConvTables& tabs = conversion_tables();
-    (k_assemble<<<(G + 63) / 64, 64, 0, s>>>(acc, b_narr.as<unsigned long long>(), b_marr.as<unsigned long long>(),
+    (k_assemble<<<(unsigned)std::min(G, 65535), ASM_THREADS, 0, s>>>(acc, b_narr.as<unsigned long long>(), b_marr.as<unsigned long long>(),
                                             G, tabs, d_out, (u128*)cfg.d_basis), note_launch());
   }
   mark(8, 1, s);
@@ -3843,7 +3851,7 @@ cudaError_t run_census_finish(const Oriented& o, int64_t n, int64_t nnz, const P
      note_launch());
   }
   const ConvTables& tabs = conversion_tables();
-  (k_assemble<<<1, 64, 0, s>>>(b_acc.as<Acc128>(), b_nm.as<unsigned long long>(), b_nm.as<unsigned long long>() + 1,
+  (k_assemble<<<1, ASM_THREADS, 0, s>>>(b_acc.as<Acc128>(), b_nm.as<unsigned long long>(), b_nm.as<unsigned long long>() + 1,
                                1, tabs, d_out, nullptr), note_launch());
   ESC_TRY(cudaStreamSynchronize(s));   // nm lives on this stack frame
   return cudaGetLastError();

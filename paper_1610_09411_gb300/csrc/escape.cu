@@ -404,7 +404,7 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
     }
     st = from_cuda(e);
   } else if (st == ESCAPE_OK) {
-    e = esc::validate_csr(n, d_rp, d_col, d_status, s, g->sms);
+    e = esc::validate_csr(n, nnz, d_rp, d_col, d_status, s, g->sms);
     st = from_cuda(e);
   }
   if (st == ESCAPE_OK) {
@@ -527,7 +527,7 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
     }
     st = from_cuda(e);
   } else if (st == ESCAPE_OK) {
-    st = from_cuda(esc::validate_csr(rows, d_rp, d_col, d_status, s, sms));
+    st = from_cuda(esc::validate_csr(rows, nnz, d_rp, d_col, d_status, s, sms));
   }
   if (st == ESCAPE_OK) {
     unsigned h = 0;

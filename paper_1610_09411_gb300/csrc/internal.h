@@ -87,12 +87,12 @@ int bits_for(int64_t n);
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, bool with_total, DeviceArena& arena,
                                cudaStream_t s);
 cudaError_t radix_sort(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* tv, int64_t n, int bits,
-                       DeviceArena& arena, cudaStream_t s);
+                       DeviceArena& arena, cudaStream_t s, int low = 0);
 cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const int32_t* col_in, DevBuf* rp_out,
                           DevBuf* col_out, int64_t* nnz_out, unsigned* d_status, DeviceArena& arena,
                           cudaStream_t s, int sms);
-cudaError_t validate_csr(int64_t n, const int64_t* rp, const int32_t* col, unsigned* d_status, cudaStream_t s,
-                         int sms);
+cudaError_t validate_csr(int64_t n, int64_t nnz, const int64_t* rp, const int32_t* col, unsigned* d_status,
+                         cudaStream_t s, int sms);
 cudaError_t orient(const int64_t* rp, const int32_t* col, int64_t n, int64_t nnz, Oriented& o, DeviceArena& arena,
                    cudaStream_t s, int sms);
 

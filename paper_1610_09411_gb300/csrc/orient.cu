@@ -131,18 +131,35 @@ __global__ void k_rs_hist(const uint64_t* keys, int64_t n, int shift, int64_t nt
   for (int d = threadIdx.x; d < RS_BINS; d += blockDim.x) counts[(int64_t)d * ntiles + blockIdx.x] = h[d];
 }
 
-__global__ void k_rs_scatter(const uint64_t* keys, const uint32_t* vals, uint64_t* okeys, uint32_t* ovals,
-                             int64_t n, int shift, int64_t ntiles, const int64_t* offs) {
+// The tile's keys are read once, RS_ROUNDS loads in flight per lane, and kept in
+// registers for the counting and the scattering pass (with a load per key and
+// pass in the two serial loops, one tile took 20 us).
+__global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t* keys, const uint32_t* vals, uint64_t* okeys,
+                                                          uint32_t* ovals, int64_t n, int shift, int64_t ntiles,
+                                                          const int64_t* offs) {
   __shared__ unsigned wh[RS_WARPS][RS_BINS];
   __shared__ int64_t wbase[RS_WARPS][RS_BINS];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < RS_WARPS * RS_BINS; i += blockDim.x) (&wh[0][0])[i] = 0;
-  __syncthreads();
   int64_t wstart = (int64_t)blockIdx.x * RS_TILE + (int64_t)w * (RS_ROUNDS * 32);
+  uint64_t key[RS_ROUNDS];
+  uint32_t val[RS_ROUNDS];
+#pragma unroll
   for (int r = 0; r < RS_ROUNDS; ++r) {
-    int64_t i = wstart + r * 32 + lane;
-    if (i < n) atomicAdd(&wh[w][(keys[i] >> shift) & 0xff], 1u);
+    const int64_t i = wstart + r * 32 + lane;
+    key[r] = i < n ? keys[i] : 0;
   }
+  if (vals) {
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+      const int64_t i = wstart + r * 32 + lane;
+      val[r] = i < n ? vals[i] : 0;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < RS_ROUNDS; ++r)
+    if (wstart + r * 32 + lane < n) atomicAdd(&wh[w][(key[r] >> shift) & 0xff], 1u);
   __syncthreads();
   for (int d = threadIdx.x; d < RS_BINS; d += blockDim.x) {
     int64_t run = offs[(int64_t)d * ntiles + blockIdx.x];
@@ -150,11 +167,10 @@ __global__ void k_rs_scatter(const uint64_t* keys, const uint32_t* vals, uint64_
   }
   __syncthreads();
   unsigned lt = (1u << lane) - 1u;
+#pragma unroll
   for (int r = 0; r < RS_ROUNDS; ++r) {
-    int64_t i = wstart + r * 32 + lane;
-    bool valid = i < n;
-    uint64_t key = valid ? keys[i] : 0;
-    unsigned dig = valid ? (unsigned)((key >> shift) & 0xff) : 0x100u + lane;   // invalid lanes match nobody
+    const bool valid = wstart + r * 32 + lane < n;
+    unsigned dig = valid ? (unsigned)((key[r] >> shift) & 0xff) : 0x100u + lane;   // invalid lanes match nobody
     unsigned peers = __match_any_sync(0xffffffffu, dig);
     int rank = __popc(peers & lt);
     int64_t dst = 0;
@@ -163,26 +179,26 @@ __global__ void k_rs_scatter(const uint64_t* keys, const uint32_t* vals, uint64_
     if (valid && rank == 0) wbase[w][dig] += __popc(peers);
     __syncwarp();
     if (valid) {
-      okeys[dst] = key;
-      if (vals) ovals[dst] = vals[i];
+      okeys[dst] = key[r];
+      if (vals) ovals[dst] = val[r];
     }
   }
 }
 
-// Stable sort of (keys, vals) by the low `bits` bits of the key.  The result
+// Stable sort of (keys, vals) by the bits [low, bits) of the key.  The result
 // ends in `keys`/`vals`; `tk`/`tv` are scratch of the same size.
 cudaError_t radix_sort(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* tv, int64_t n, int bits,
-                       DeviceArena& arena, cudaStream_t s) {
-  if (n <= 1 || bits <= 0) return cudaSuccess;
+                       DeviceArena& arena, cudaStream_t s, int low) {
+  if (n <= 1 || bits <= low) return cudaSuccess;
   int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
   size_t mark = arena.mark();
   int64_t* counts = (int64_t*)arena.alloc(sizeof(int64_t) * (RS_BINS * ntiles + 1));
   if (!counts) return cudaErrorMemoryAllocation;
   uint64_t *ka = keys, *kb = tk;
   uint32_t *va = vals, *vb = tv;
-  int passes = (bits + 7) / 8;
+  int passes = (bits - low + 7) / 8;
   for (int p = 0; p < passes; ++p) {
-    int shift = p * 8;
+    int shift = low + p * 8;
     (k_rs_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, n, shift, ntiles, counts), note_launch());
     cudaError_t e = exclusive_scan_i64(counts, counts, RS_BINS * ntiles, false, arena, s);
     if (e != cudaSuccess) return e;
@@ -244,19 +260,36 @@ __global__ void k_compact_csr(const uint64_t* keys, const int64_t* pos, int64_t 
   }
 }
 
-// Input already simple?  Rows non-decreasing, ids in range, sorted strictly,
-// no loops, symmetric.
-__global__ void k_validate(const int64_t* rp, const int32_t* col, int64_t n, unsigned* st) {
-  int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += stride) {
-    int64_t b = rp[u], e = rp[u + 1];
-    if (e < b) { set_err(st, DEVERR_BOUNDS); continue; }
-    for (int64_t p = b; p < e; ++p) {
-      int32_t v = col[p];
-      if (v < 0 || v >= n || v == u || (p > b && v <= col[p - 1])) { set_err(st, DEVERR_BOUNDS); break; }
-      int64_t q = lower_bound_i32(col, rp[v], rp[v + 1], (int32_t)u);
-      if (q >= rp[v + 1] || col[q] != (int32_t)u) { set_err(st, DEVERR_BOUNDS); break; }
+// Input already simple?  Ids in range, rows sorted strictly, no loops,
+// symmetric (the row offsets themselves are checked on the host).  One thread per
+// entry: a CTA takes VAL_TILE consecutive entries, finds the rows they span, and
+// each thread its row between them (one thread per row left the rest waiting for
+// the hub's: a serving step of 8 requests 2.1 ms).
+static constexpr int VAL_THREADS = 256, VAL_TILE = 2048;
+__global__ void __launch_bounds__(VAL_THREADS) k_validate(const int64_t* rp, const int32_t* col, int64_t n,
+                                                         unsigned* st) {
+  __shared__ int64_t sh_row[2];
+  const int64_t nnz = rp[n];
+  for (int64_t t0 = (int64_t)blockIdx.x * VAL_TILE; t0 < nnz; t0 += (int64_t)gridDim.x * VAL_TILE) {
+    const int64_t t1 = min(nnz, t0 + VAL_TILE);
+    if (threadIdx.x < 2) {                      // the row of the first and of the last entry: the last u with rp[u] <= p
+      const int64_t p = threadIdx.x ? t1 - 1 : t0;
+      int64_t lo = 0, hi = n;
+      while (hi - lo > 1) { const int64_t mid = (lo + hi) >> 1; if (rp[mid] <= p) lo = mid; else hi = mid; }
+      sh_row[threadIdx.x] = lo;
     }
+    __syncthreads();
+    const int64_t r0 = sh_row[0], r1 = sh_row[1];
+    for (int64_t p = t0 + threadIdx.x; p < t1; p += VAL_THREADS) {
+      int64_t lo = r0, hi = r1 + 1;
+      while (hi - lo > 1) { const int64_t mid = (lo + hi) >> 1; if (rp[mid] <= p) lo = mid; else hi = mid; }
+      const int64_t u = lo;
+      const int32_t v = col[p];
+      if (v < 0 || v >= n || v == u || (p > rp[u] && v <= col[p - 1])) { set_err(st, DEVERR_BOUNDS); continue; }
+      const int64_t e = rp[v + 1], q = lower_bound_i32(col, rp[v], e, (int32_t)u);
+      if (q >= e || col[q] != (int32_t)u) set_err(st, DEVERR_BOUNDS);
+    }
+    __syncthreads();                            // the rows are read before the next tile's are written
   }
 }
 
@@ -282,15 +315,21 @@ __global__ void k_ranks(const uint32_t* sorted_ids, const uint64_t* sorted_deg, 
   }
 }
 
+// Entry u -> v becomes the key (rank of v, rank of u), written at the place of
+// row rank(u): the array is sorted by its low part, so a stable sort by the high
+// part alone (half the radix passes) leaves every row of the rank-space graph
+// together and sorted (the graph is symmetric: row v's sources are its
+// neighbours).
 __global__ void k_rank_edge_keys(const int64_t* rp, const int32_t* col, int64_t n, const int32_t* rank,
-                                 int vb, uint64_t* keys) {
+                                 const int64_t* R, int vb, uint64_t* keys) {
   // one warp per original row
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int lane = threadIdx.x & 31;
   for (int64_t u = warp; u < n; u += nwarps) {
-    uint64_t ru = (uint64_t)rank[u];
-    for (int64_t p = rp[u] + lane; p < rp[u + 1]; p += 32) keys[p] = (ru << vb) | (uint64_t)rank[col[p]];
+    const uint64_t ru = (uint64_t)rank[u];
+    const int64_t to = R[ru] - rp[u];
+    for (int64_t p = rp[u] + lane; p < rp[u + 1]; p += 32) keys[to + p] = ((uint64_t)rank[col[p]] << vb) | ru;
   }
 }
 
@@ -362,9 +401,10 @@ cudaError_t normalize_csr(int64_t n, int64_t nnz_in, const int64_t* rp_in, const
   return cudaGetLastError();
 }
 
-cudaError_t validate_csr(int64_t n, const int64_t* rp, const int32_t* col, unsigned* d_status, cudaStream_t s,
-                         int sms) {
-  if (n > 0) (k_validate<<<grid_for(n, 128, sms), 128, 0, s>>>(rp, col, n, d_status), note_launch());
+cudaError_t validate_csr(int64_t n, int64_t nnz, const int64_t* rp, const int32_t* col, unsigned* d_status,
+                         cudaStream_t s, int sms) {
+  if (n > 0 && nnz > 0)
+    (k_validate<<<grid_for(nnz, VAL_TILE, sms), VAL_THREADS, 0, s>>>(rp, col, n, d_status), note_launch());
   return cudaGetLastError();
 }
 
@@ -381,7 +421,7 @@ cudaError_t orient(const int64_t* rp, const int32_t* col, int64_t n, int64_t nnz
   cudaError_t e;
   // 1. rank vertices by (degree, id): stable sort of degrees with ids as values
   if (n > 0) (k_degree_keys<<<grid_for(n, 256, sms), 256, 0, s>>>(rp, n, keys, vals), note_launch());
-  int dbits = bits_for(nnz + 2);
+  const int dbits = bits_for((nnz < n ? nnz : n) + 2);   // a degree is below n
   e = radix_sort(keys, vals, tk, tv, n, dbits, arena, s);
   if (e != cudaSuccess) return e;
   if (n > 0) (k_ranks<<<grid_for(n, 256, sms), 256, 0, s>>>(vals, keys, n, o.perm, o.rank, o.R), note_launch());
@@ -391,8 +431,8 @@ cudaError_t orient(const int64_t* rp, const int32_t* col, int64_t n, int64_t nnz
   // 3. renamed entries sorted by (row rank, neighbour rank)
   int vb = bits_for(n > 1 ? n : 2);
   if (nnz > 0) {
-    (k_rank_edge_keys<<<grid_for(n * 32, 256, sms), 256, 0, s>>>(rp, col, n, o.rank, vb, keys), note_launch());
-    e = radix_sort(keys, nullptr, tk, nullptr, nnz, 2 * vb, arena, s);
+    (k_rank_edge_keys<<<grid_for(n * 32, 256, sms), 256, 0, s>>>(rp, col, n, o.rank, o.R, vb, keys), note_launch());
+    e = radix_sort(keys, nullptr, tk, nullptr, nnz, 2 * vb, arena, s, vb);
     if (e != cudaSuccess) return e;
     (k_keys_to_col<<<grid_for(nnz, 256, sms), 256, 0, s>>>(keys, nnz, vb, o.C), note_launch());
   }
