@@ -462,6 +462,76 @@ __device__ __forceinline__ void k5_row(const uint64_t* B, int W, int RS, int a, 
   }
 }
 
+// The same for rows of at most WW words: lane t of a warp takes the t-th of 32
+// consecutive b and all its candidates, with the candidate set in registers, and
+// every candidate adds the whole of its intersection with it, above and below
+// (each pair of adjacent candidates twice): no masks and the same word loop in
+// every lane, at six instructions a word instead of twelve.  k5x2 += 2 x the
+// 5-cliques.
+template <int WW>
+__device__ __forceinline__ void k5_row_reg(const uint64_t* B, int W, int RS, int a, unsigned long long& k5x2, u128& dbp) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t* ra = B + (int64_t)a * RS;
+  uint64_t m = 0;                               // lane l: word l of row a above a
+  if (lane < W) {
+    m = ra[lane];
+    const int w0 = (a + 1) >> 6;
+    if (lane < w0) m = 0;
+    else if (lane == w0) m &= above_mask(a);
+  }
+  const int cnt = __popcll(m);
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < WW; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const int s = __shfl_sync(0xffffffffu, incl, WW - 1);
+  for (int t0 = 0; t0 < s; t0 += 32) {
+    const int t = t0 + lane;
+    int wq = 0;
+#pragma unroll
+    for (int u = 0; u < WW - 1; ++u) wq += __shfl_sync(0xffffffffu, incl, u) <= t ? 1 : 0;
+    const uint64_t mw = __shfl_sync(0xffffffffu, m, wq);
+    const int before = __shfl_sync(0xffffffffu, incl - cnt, wq);
+    const int b = t < s ? wq * 64 + select64(mw, t - before) : a;
+    const int u0 = __shfl_sync(0xffffffffu, (b + 1) >> 6, 0);   // lane 0 holds the lowest b
+    const uint64_t* rb = B + (int64_t)b * RS;
+    uint64_t S[WW];
+    int n = 0;
+#pragma unroll
+    for (int u = 0; u < WW; ++u) {
+      S[u] = 0;
+      if (u >= u0 && u < W) {
+        const int wb = (b + 1) >> 6;
+        uint64_t x = ra[u] & rb[u];
+        if (u < wb || t >= s) x = 0;
+        else if (u == wb) x &= above_mask(b);
+        S[u] = x;
+        n += __popcll(x);
+      }
+    }
+    if (n >= 2) dbp += (unsigned long long)n * (n - 1) / 2;
+    else n = 0;                                 // a lone candidate closes no 5-clique
+    int w = (b + 1) >> 6;
+    uint64_t cm = n ? ra[w] & rb[w] & above_mask(b) : 0;
+    unsigned part = 0;                          // below 2^32: n <= 64 WW candidates of as many neighbours
+    while (n > 0) {
+      while (!cm) {
+        ++w;
+        cm = ra[w] & rb[w];
+      }
+      const uint64_t* rc = B + (int64_t)(w * 64 + __ffsll((long long)cm) - 1) * RS;
+      cm &= cm - 1;
+      --n;
+#pragma unroll
+      for (int u = 0; u < WW; ++u)
+        if (u >= u0 && u < W) part += __popcll(S[u] & rc[u]);
+    }
+    k5x2 += part;
+  }
+}
+
 // Work-space layout of the CTA path: B (d x RS u64, rows symmetric: row a = every
 // neighbour of v_a inside N+(x)), K4 accumulators (d u64), hash (2 x hcap
 // ints), T of x's out-edges and degree of its out-neighbours (d u32 each), in
@@ -617,15 +687,18 @@ __global__ void __launch_bounds__(512, 1) k_clique_large(DevGraph g, const int32
       __syncwarp();
     }
     if (five) {                                 // rows handed out one by one: low rows hold most of the work
-      unsigned long long k5 = 0;
+      unsigned long long k5 = 0, k5x2 = 0;
       while (true) {
         int a = 0;
         if (lane == 0) a = atomicAdd(&sh_row, 1);
         a = __shfl_sync(0xffffffffu, a, 0);
         if (a >= d) break;
-        k5_row(B, W, RS, a, cw, k5, la.v[5]);
+        if (!GLOBAL_B && W <= 4) k5_row_reg<4>(B, W, RS, a, k5x2, la.v[5]);
+        else if (!GLOBAL_B && W <= 8) k5_row_reg<8>(B, W, RS, a, k5x2, la.v[5]);
+        else if (!GLOBAL_B && W <= 12) k5_row_reg<12>(B, W, RS, a, k5x2, la.v[5]);
+        else k5_row(B, W, RS, a, cw, k5, la.v[5]);
       }
-      la.v[4] += k5;
+      la.v[4] += k5 + k5x2 / 2;                 // a lane's sum of two-fold counts is even
     }
     __syncthreads();
     for (int i = threadIdx.x; i < d; i += blockDim.x)
@@ -2466,19 +2539,74 @@ __global__ void __launch_bounds__(1024, 1) k_cycles5(DevGraph g, const unsigned 
 // Per-edge common-neighbour lists (the per-edge triangle lists of Thm 7),
 // stored sorted: the id list once per undirected edge (addressed from both
 // slots), and for each slot (u -> v) the positions in row u of the same
-// vertices.  Built per higher endpoint y: N(y) goes into a hash table (vertex
-// -> position in row y), and for every lower neighbour x the row N(x) is
-// filtered through it; a hit at index q of row x has position q - R[x] there.
+// vertices.  Edges without a triangle are skipped.  By the higher endpoint y:
+//   degree <= TL_LIGHT: one thread per edge merges the two short rows;
+//   above: one CTA per y, N(y) in a hash table (vertex -> position in row y); for
+//     every lower neighbour x the row N(x) is filtered through it; a hit at
+//     index q of row x has position q - R[x] there.
+// One CTA for every y, with the offsets of each x fetched before its row, was
+// bound by latency: R-MAT 19 41 ms, Chung-Lu 2.3 n = 625,000 6.4 ms.
 // ============================================================================
-__global__ void k_tri_lists(DevGraph g, unsigned long long* qctr, const int64_t* off, const int64_t* offp,
-                            const uint32_t* T, int32_t* U, int32_t* P, int32_t* ghash, int64_t ghash_cap,
-                            int hash_cap, unsigned* status) {
+static constexpr int TL_LIGHT = 64, TL_TILE = 2048, TL_ILP = 4;
+
+// Slots [0, slots) are the rows of the vertices of degree <= TL_LIGHT.
+__global__ void __launch_bounds__(256) k_tri_lists_light(DevGraph g, int64_t rows, int64_t slots, const int64_t* off,
+                                                        const int64_t* offp, const uint32_t* T, int32_t* U, int32_t* P,
+                                                        unsigned* status) {
+  __shared__ int64_t sh_row[2];
+  for (int64_t t0 = (int64_t)blockIdx.x * TL_TILE; t0 < slots; t0 += (int64_t)gridDim.x * TL_TILE) {
+    const int64_t t1 = min(slots, t0 + TL_TILE);
+    if (threadIdx.x < 2) {                      // rows of the first and last slot: the last y with R[y] <= p
+      const int64_t p = threadIdx.x ? t1 - 1 : t0;
+      int64_t lo = 0, hi = rows;
+      while (hi - lo > 1) { const int64_t mid = (lo + hi) >> 1; if (g.R[mid] <= p) lo = mid; else hi = mid; }
+      sh_row[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    const int64_t r0 = sh_row[0], r1 = sh_row[1];
+    for (int64_t p = t0 + threadIdx.x; p < t1; p += blockDim.x) {
+      const uint32_t expect = T[p];
+      if (expect == 0) continue;
+      int64_t lo = r0, hi = r1 + 1;
+      while (hi - lo > 1) { const int64_t mid = (lo + hi) >> 1; if (g.R[mid] <= p) lo = mid; else hi = mid; }
+      const int64_t y = lo;
+      const int32_t x = g.C[p];
+      if (x > y) continue;                      // once per edge, at its higher endpoint
+      const int64_t yb = g.R[y], xb = g.R[x], cs = g.rev[p];
+      const int dy = (int)(g.R[y + 1] - yb), dx = (int)(g.R[x + 1] - xb);
+      const int64_t out = off[cs], outx = offp[cs], outy = offp[p];
+      uint32_t k = 0;
+      int i = 0, j = 0;
+      while (i < dx && j < dy) {
+        const int32_t a = g.C[xb + i], c = g.C[yb + j];
+        if (a == c) {
+          if (k < expect) {
+            U[out + k] = a;
+            P[outx + k] = i;
+            P[outy + k] = j;
+          }
+          ++k;
+        }
+        i += a <= c ? 1 : 0;
+        j += c <= a ? 1 : 0;
+      }
+      if (k != expect) set_err(status, DEVERR_BOUNDS);
+    }
+    __syncthreads();                            // the rows are read before the next tile's are written
+  }
+}
+
+// Vertices n - 1 down to r0.
+__global__ void __launch_bounds__(512) k_tri_lists(DevGraph g, int64_t r0, unsigned long long* qctr, const int64_t* off,
+                                                  const int64_t* offp, const uint32_t* T, int32_t* U, int32_t* P,
+                                                  int32_t* ghash, int64_t ghash_cap, int hash_cap, unsigned* status) {
   extern __shared__ int32_t smem[];
   __shared__ int64_t sh_item;
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
   int32_t* gk = ghash + (int64_t)blockIdx.x * 2 * ghash_cap;
   while (true) {
-    int64_t it = next_item(qctr, g.n, &sh_item);
+    int64_t it = next_item(qctr, g.n - r0, &sh_item);
     if (it < 0) break;
     int64_t y = g.n - 1 - it;
     int64_t yb = g.R[y], yo = g.op[y], ye = g.R[y + 1];
@@ -2495,33 +2623,52 @@ __global__ void k_tri_lists(DevGraph g, unsigned long long* qctr, const int64_t*
     __syncthreads();
     for (int i = threadIdx.x; i < dy; i += blockDim.x) H.insert(g.C[yb + i], i);
     __syncthreads();
-    for (int64_t p = yb + wid; p < yo; p += nw) {   // x in N-(y); p = slot (y -> x)
-      int32_t x = g.C[p];
-      int64_t cs = g.rev[p];                        // canonical slot (x -> y)
-      int64_t out = off[cs], outx = offp[cs], outy = offp[p];
-      uint32_t expect = T[cs];
-      uint32_t written = 0;
-      int64_t xb = g.R[x];
-      for (int64_t base = xb; base < g.R[x + 1]; base += 32) {
-        int64_t q = base + lane;
-        int32_t py = -1, z = -1;
-        if (q < g.R[x + 1]) {
-          z = g.C[q];
-          py = H.find(z);
-        }
-        bool hit = py >= 0;
-        unsigned hm = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-          unsigned k = written + __popc(hm & ((1u << lane) - 1u));
-          if (k < expect) {
-            U[out + k] = z;
-            P[outx + k] = (int32_t)(q - xb);
-            P[outy + k] = py;
+    // x in N-(y), p = slot (y -> x): a warp fetches what it needs of 32 of them at
+    // once (lane l the l-th), then filters their rows one by one
+    for (int64_t pbase = yb + wid; pbase < yo; pbase += (int64_t)nw * 32) {
+      const int64_t p = pbase + (int64_t)lane * nw;
+      uint32_t expect_l = p < yo ? T[p] : 0u;
+      int64_t xb_l = 0, out_l = 0, outx_l = 0, outy_l = 0;
+      int len_l = 0;
+      if (expect_l) {
+        const int32_t x = g.C[p];
+        const int64_t cs = g.rev[p];            // canonical slot (x -> y)
+        xb_l = g.R[x];
+        len_l = (int)(g.R[x + 1] - xb_l);
+        out_l = off[cs];
+        outx_l = offp[cs];
+        outy_l = offp[p];
+      }
+      unsigned m = __ballot_sync(0xffffffffu, expect_l != 0);
+      while (m) {
+        const int k = __ffs(m) - 1;
+        m &= m - 1;
+        const uint32_t expect = __shfl_sync(0xffffffffu, expect_l, k);
+        const int len = __shfl_sync(0xffffffffu, len_l, k);
+        const int32_t* L = g.C + __shfl_sync(0xffffffffu, xb_l, k);
+        const int64_t out = __shfl_sync(0xffffffffu, out_l, k), outx = __shfl_sync(0xffffffffu, outx_l, k),
+                      outy = __shfl_sync(0xffffffffu, outy_l, k);
+        uint32_t written = 0;
+        for (int q = lane; q - lane < len && written < expect; q += 32 * TL_ILP) {
+          int32_t z[TL_ILP], py[TL_ILP];
+#pragma unroll
+          for (int u = 0; u < TL_ILP; ++u) z[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
+#pragma unroll
+          for (int u = 0; u < TL_ILP; ++u) py[u] = z[u] >= 0 ? H.find(z[u]) : -1;
+#pragma unroll
+          for (int u = 0; u < TL_ILP; ++u) {
+            const unsigned hm = __ballot_sync(0xffffffffu, py[u] >= 0);
+            const uint32_t at = written + __popc(hm & lt);
+            if (py[u] >= 0 && at < expect) {
+              U[out + at] = z[u];
+              P[outx + at] = q + 32 * u;
+              P[outy + at] = py[u];
+            }
+            written += __popc(hm);
           }
         }
-        written += __popc(hm);
+        if (lane == 0 && written != expect) set_err(status, DEVERR_BOUNDS);
       }
-      if (lane == 0 && written != expect) set_err(status, DEVERR_BOUNDS);
     }
     __syncthreads();
   }
@@ -3631,8 +3778,17 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   //   s1, s2, s4 (least urgent): cliques, 4-cycles, 5-cycles; s joins all.
   mark(4, 0, s);
   if (five && n > 0)
-    (k_tri_lists<<<grid_sweep, 512, smem_l, s>>>(g, ctr + 3, off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(),
-                                                 b_gh.as<int32_t>(), ghash_cap, hcap_l, d_status), note_launch());
+  {
+    int64_t lo = 0, hi = n;                     // first rank of degree > TL_LIGHT
+    while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] > TL_LIGHT) hi = mid; else lo = mid + 1; }
+    if (lo < n)
+      (k_tri_lists<<<(unsigned)std::min<int64_t>(grid_sweep, n - lo), 512, smem_l, s>>>(
+           g, lo, ctr + 3, off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(), b_gh.as<int32_t>(), ghash_cap, hcap_l,
+           d_status), note_launch());
+    if (hR[lo] > 0)
+      (k_tri_lists_light<<<(unsigned)std::min<int64_t>((hR[lo] + TL_TILE - 1) / TL_TILE, (int64_t)sms * 8), 256, 0, s>>>(
+           g, lo, hR[lo], off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(), d_status), note_launch());
+  }
   if (ch > 0) ESC_TRY(core_low(g, T, off, b_U.as<int32_t>(), cv.h0, b_low.as<uint32_t>(), sms, s));
   mark(4, 1, s);
   StreamSet ss_all;

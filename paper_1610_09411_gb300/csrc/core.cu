@@ -180,7 +180,8 @@ __global__ void k_core_low(DevGraph g, const uint32_t* T, const int64_t* off, co
 // vertices adjacent to both (a suffix of the position list of slot c -> k) add
 // one to b at each of their pairs.  b is a triangle of counts as wide as W's
 // (16 bits, two to a word, when no degree reaches 2^16: b(u, v) < d_c).  One
-// CTA per centre, one warp per k.
+// CTA per centre, one warp for 32 k's.
+static constexpr int CORE_SHORT = 8;
 template <typename WT>
 __global__ void __launch_bounds__(256) k_core_mixed(DevGraph g, const uint32_t* T, const int64_t* offp,
                                                     const int32_t* P, int64_t h0, const int32_t* dh,
@@ -207,18 +208,39 @@ __global__ void __launch_bounds__(256) k_core_mixed(DevGraph g, const uint32_t* 
       st_l = o + lo;
       cnt_l = len - lo;
     }
-    unsigned m = __ballot_sync(0xffffffffu, cnt_l >= 2);
+    // short suffixes: each lane its own pairs; long ones: the warp, one at a time
+    auto add = [&](int64_t v, int64_t u) {
+      const int64_t e = v * (v - 1) / 2 + u;
+      if (sizeof(WT) == 2) atomicAdd(&b[e >> 1], 1u << (16 * (int)(e & 1)));
+      else atomicAdd(&b[e], 1u);
+    };
+    if (cnt_l >= 2 && cnt_l <= CORE_SHORT) {
+      const int32_t* L = P + st_l;
+      int32_t e[CORE_SHORT];
+#pragma unroll
+      for (int y = 0; y < CORE_SHORT; ++y) e[y] = y < cnt_l ? L[y] - (int32_t)pc : 0;
+#pragma unroll
+      for (int y = 1; y < CORE_SHORT; ++y)
+#pragma unroll
+        for (int x = 0; x < y; ++x)
+          if (y < cnt_l) add(e[y], e[x]);
+    }
+    unsigned m = __ballot_sync(0xffffffffu, cnt_l > CORE_SHORT);
     while (m) {
       const int q = __ffs(m) - 1;
       m &= m - 1;
       const int32_t* L = P + __shfl_sync(0xffffffffu, st_l, q);
       const int cnt = __shfl_sync(0xffffffffu, cnt_l, q);
-      for (int y = 1; y < cnt; ++y) {
-        const int64_t v = L[y] - pc, row = v * (v - 1) / 2;
-        for (int x = lane; x < y; x += 32) {
-          const int64_t e = row + (L[x] - pc);
-          if (sizeof(WT) == 2) atomicAdd(&b[e >> 1], 1u << (16 * (int)(e & 1)));
-          else atomicAdd(&b[e], 1u);
+      for (int x0 = 0; x0 < cnt; x0 += 32) {    // 32 entries x against every later y
+        const int64_t u = x0 + lane < cnt ? L[x0 + lane] - pc : 0;
+        for (int yb = x0; yb < cnt; yb += 32) {
+          const int32_t v_l = yb + lane < cnt ? L[yb + lane] - (int32_t)pc : 0;
+          const int ye = min(32, cnt - yb);
+#pragma unroll 4
+          for (int y = 0; y < ye; ++y) {
+            const int64_t v = __shfl_sync(0xffffffffu, v_l, y);
+            if (x0 + lane < yb + y) add(v, u);
+          }
         }
       }
     }
