@@ -1073,6 +1073,35 @@ struct PackedHash {
   }
 };
 
+// Places within the own graph.  A graph of up to DIRECT_N vertices has a counter
+// for each of them in shared memory, and its medium items count without hashing
+// (k_*_direct): of a single graph the place is the rank; of a union li gives
+// it, and g.J holds the entries' places.
+// A probe loop ends with the slowest of 32 lanes, and the 64 KB table left three
+// CTAs on an SM.  Census of 96 graphs of 20 to 2,000 vertices 145 -> 107 ms (its
+// 5-cycle items took 43 ms), of ER(800, 0.15) 1.39 -> 1.27 ms (5-cycles 0.21 ->
+// 0.10).
+struct LocalIds {
+  const int32_t *li, *hl;                       // place of a rank; ranks by graph (null: one graph)
+  const int64_t* hb;                            // first entry in hl of the graph of a rank
+  const int32_t* vg;
+  const unsigned long long* n_arr;
+  int n;
+  __device__ __forceinline__ int size(int64_t i) const { return li ? (int)n_arr[vg[i]] : n; }
+  __device__ __forceinline__ int32_t place(int64_t j) const { return li ? li[j] : (int32_t)j; }
+  __device__ __forceinline__ int64_t start(int64_t i) const { return li ? hb[i] : 0; }
+  __device__ __forceinline__ int64_t rank(int64_t start, int32_t t) const { return li ? hl[start + t] : t; }
+};
+static constexpr int DIRECT_N = 8192;
+__global__ void k_local_entries(const int32_t* C, int64_t nnz, const int32_t* li, int32_t* J) {
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
+    J[p] = li[C[p]];
+}
+__device__ __forceinline__ void direct_clear(uint32_t* tab, int ng) {   // the table's size is a multiple of 4 words
+  for (int t = threadIdx.x; t < (ng + 3) / 4; t += blockDim.x)
+    reinterpret_cast<uint4*>(tab)[t] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // log2 of a table for m counters (load factor at most 1/2)
 __device__ __forceinline__ int table_log(unsigned long long m) {
   const int l = m <= 1 ? 1 : 65 - __clzll((long long)(m - 1));   // ceil(log2(2 m))
@@ -1087,9 +1116,9 @@ struct ItemLists {
 };
 __device__ __forceinline__ void item_append(const ItemLists& il, int64_t n, int64_t i, unsigned long long w,
                                             unsigned long long m1, unsigned long long m2, long long light_m,
-                                            long long medium_m, bool fits) {
+                                            long long medium_m, bool fits, bool direct) {
   const unsigned long long m = max(m1, m2);
-  const int cls = !fits ? 2
+  const int cls = !fits ? (direct && (long long)m <= medium_m ? 1 : 2)   // no count bits in a direct counter
                         : ((long long)m <= light_m && (long long)w <= 4 * light_m
                                ? 0
                                : ((long long)m <= medium_m ? 1 : 2));
@@ -1104,7 +1133,7 @@ __device__ __forceinline__ void item_append(const ItemLists& il, int64_t n, int6
 // Also the largest common-neighbour list (triangles on one edge) into cnt[7]
 // and twice the number of diamonds, sum over slots of C(T, 2), into cnt[8].
 __global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, long long light_m, long long medium_m,
-                                int cb, const int32_t* vg, const unsigned long long* n_arr, Owner own) {
+                                int cb, const int32_t* vg, const unsigned long long* n_arr, bool direct, Owner own) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1124,7 +1153,7 @@ __global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, lon
     w = warp_sum_u64(w);
     if (lane == 0 && w) {
       const unsigned long long m = min(w, min((unsigned long long)i, vg ? n_arr[vg[i]] : ~0ull));
-      item_append(il, g.n, i, w, m, m, light_m, medium_m, (unsigned long long)(e0 - b0) < (1u << cb) - 1u);
+      item_append(il, g.n, i, w, m, m, light_m, medium_m, (unsigned long long)(e0 - b0) < (1u << cb) - 1u, direct);
     }
   }
   dia = warp_sum_u64(dia);
@@ -1138,7 +1167,7 @@ __global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, lon
 // k_cycles5).
 __global__ void k_cycle_classify(DevGraph g, ItemLists i4, ItemLists i5, bool only4, long long light_m,
                                  long long medium_m4, long long medium_m5, int cb, const int32_t* vg,
-                                 const unsigned long long* n_arr, Owner own) {
+                                 const unsigned long long* n_arr, bool direct, Owner own) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1168,11 +1197,11 @@ __global__ void k_cycle_classify(DevGraph g, ItemLists i4, ItemLists i5, bool on
     const bool fits = (unsigned long long)(e0 - b0) < (1u << cb) - 1u;
     if (w4) {
       const unsigned long long m = min(w4, min((unsigned long long)i, ng));
-      item_append(i4, g.n, i, w4, m, m, light_m, medium_m4, fits);
+      item_append(i4, g.n, i, w4, m, m, light_m, medium_m4, fits, direct);
     }
     // P2 counts the slot of i itself once per a: with nothing else, no path leaves it
     if (!only4 && p2 > (unsigned long long)(o - b0))
-      item_append(i5, g.n, i, w5 + p2, min(w5, ng), min(p2, ng), light_m, medium_m5, fits);
+      item_append(i5, g.n, i, w5 + p2, min(w5, ng), min(p2, ng), light_m, medium_m5, fits, direct);
   }
 }
 
@@ -1213,7 +1242,7 @@ __device__ __forceinline__ unsigned long long pair_c2(uint32_t old) {
 template <class Inc>
 __device__ __forceinline__ u128 pair_range(const DevGraph& g, int64_t cb, int64_t ce, Inc&& inc) {
   const int lane = threadIdx.x & 31;
-  const int32_t* L = g.C + cb;
+  const int32_t* L = g.J + cb;
   const int len = (int)(ce - cb);
   Sum128 n13;
   for (int q = lane; q < len; q += 32 * PAIR_ILP) {
@@ -1246,7 +1275,7 @@ __device__ __forceinline__ u128 pair_wedges(const DevGraph& g, int64_t b0, int64
     }
     // short lists: each lane its own; the others one at a time by the warp
     if (ce_l - cb_l <= PAIR_SHORT) {
-      const int32_t* L = g.C + cb_l;
+      const int32_t* L = g.J + cb_l;
       const int len = (int)(ce_l - cb_l);
       Sum128 sh13;
       for (int q = 0; q < len; q += 4) {
@@ -1454,6 +1483,37 @@ __device__ __forceinline__ void core_store_row(const CoreView& cv, int64_t i, in
 // list, 87% of the warps' time went to waiting for it: Chung-Lu 2.3
 // n = 625,000, medium items 31.4 -> 8.9 ms; the census 117 -> 95.5 ms).
 static constexpr int PH_PIECE = 128, PH_LONG = 64;
+struct LongLists {
+  longlong2 list[PH_LONG];
+  unsigned n;                                   // zero before the barrier that precedes the item's wedges
+};
+template <class Inc>
+__device__ __forceinline__ u128 pair_wedges_shared(const DevGraph& g, int64_t b0, int64_t e0, int wid, int nw,
+                                                   LongLists& ll, Inc&& inc) {
+  const int lane = threadIdx.x & 31;
+  u128 sum = pair_wedges(g, b0, e0, wid, nw, inc, [&](int64_t cb, int64_t ce) {
+    if (ce - cb <= PH_PIECE) return false;
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(&ll.n, 1u);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at >= PH_LONG) return false;            // no room: the warp walks the list itself
+    if (lane == 0) ll.list[at] = make_longlong2(cb, ce);
+    return true;
+  });
+  __syncthreads();
+  // the long lists in pieces of PH_PIECE entries, piece by piece over the warps
+  const int nl = (int)min(ll.n, (unsigned)PH_LONG);
+  for (int l = 0, w = wid; l < nl; ++l) {
+    const longlong2 r = ll.list[l];
+    const int np = (int)((r.y - r.x + PH_PIECE - 1) / PH_PIECE);
+    for (; w < np; w += nw) {
+      const int64_t a = r.x + (int64_t)w * PH_PIECE;
+      sum += pair_range(g, a, min((int64_t)r.y, a + PH_PIECE), inc);
+    }
+    w -= np;
+  }
+  return sum;
+}
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) k_pairs_hash(DevGraph g, const unsigned long long* items, int64_t nitems,
                                                        unsigned long long* qctr, int cb, int max_log, TriLists tl3,
@@ -1461,9 +1521,8 @@ __global__ void __launch_bounds__(THREADS) k_pairs_hash(DevGraph g, const unsign
   extern __shared__ uint4 hash_smem[];
   __shared__ u128 sh[32];
   __shared__ int64_t sh_item;
-  __shared__ longlong2 s_long[PH_LONG];
-  __shared__ unsigned n_long;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = THREADS / 32;
+  __shared__ LongLists ll;
+  const int wid = threadIdx.x >> 5, nw = THREADS / 32;
   PackedHash H{reinterpret_cast<uint32_t*>(hash_smem), cb, 0};
   const int ids[2] = {ACC_N13, ACC_N17};
   LocalAcc<2> la;
@@ -1475,31 +1534,11 @@ __global__ void __launch_bounds__(THREADS) k_pairs_hash(DevGraph g, const unsign
     const int64_t b0 = g.R[i], e0 = g.R[i + 1];
     H.log = min(max_log, item_log(items[it]));
     H.clear(threadIdx.x, THREADS);
-    if (threadIdx.x == 0) n_long = 0;
+    if (threadIdx.x == 0) ll.n = 0;
     __syncthreads();
     bool full = false;
     auto inc = [&](int32_t j) -> unsigned long long { return pair_c2(H.inc(j, full)); };
-    la.v[0] += pair_wedges(g, b0, e0, wid, nw, inc, [&](int64_t cb_, int64_t ce) {
-      if (ce - cb_ <= PH_PIECE) return false;
-      unsigned at = 0;
-      if (lane == 0) at = atomicAdd(&n_long, 1u);
-      at = __shfl_sync(0xffffffffu, at, 0);
-      if (at >= PH_LONG) return false;          // no room: the warp walks the list itself
-      if (lane == 0) s_long[at] = make_longlong2(cb_, ce);
-      return true;
-    });
-    __syncthreads();
-    // the long lists in pieces of PH_PIECE entries, piece by piece over the warps
-    const int nl = (int)min(n_long, (unsigned)PH_LONG);
-    for (int l = 0, w = wid; l < nl; ++l) {
-      const longlong2 r = s_long[l];
-      const int np = (int)((r.y - r.x + PH_PIECE - 1) / PH_PIECE);
-      for (; w < np; w += nw) {
-        const int64_t a = r.x + (int64_t)w * PH_PIECE;
-        la.v[0] += pair_range(g, a, min((int64_t)r.y, a + PH_PIECE), inc);
-      }
-      w -= np;
-    }
+    la.v[0] += pair_wedges_shared(g, b0, e0, wid, nw, ll, inc);
     if (full) set_err(status, DEVERR_SCRATCH);
     __syncthreads();
     la.v[1] += pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t { return H.get(j); });
@@ -1510,6 +1549,46 @@ __global__ void __launch_bounds__(THREADS) k_pairs_hash(DevGraph g, const unsign
         if (w != PackedHash::EMPTY && j >= cv.h0)
           cv.put(cv.rowb[i - cv.h0] + cv.li[j - cv.h0], w & ((1u << cb) - 1u));
       }
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Medium items of small graphs: a counter per vertex of the graph.
+__global__ void __launch_bounds__(IT_MEDIUM_THREADS) k_pairs_direct(DevGraph g, const unsigned long long* items,
+                                                                   int64_t nitems, unsigned long long* qctr,
+                                                                   LocalIds lc, TriLists tl3, const uint32_t* T,
+                                                                   CoreView cv, AccSet acc) {
+  extern __shared__ uint4 hash_smem[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  __shared__ LongLists ll;
+  uint32_t* tab = reinterpret_cast<uint32_t*>(hash_smem);
+  const int wid = threadIdx.x >> 5, nw = IT_MEDIUM_THREADS / 32;
+  const int ids[2] = {ACC_N13, ACC_N17};
+  LocalAcc<2> la;
+  la.zero();
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers end the last item's reads
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.R[i + 1];
+    const int ng = lc.size(i);
+    direct_clear(tab, ng);
+    if (threadIdx.x == 0) ll.n = 0;
+    __syncthreads();
+    la.v[0] += pair_wedges_shared(g, b0, e0, wid, nw, ll, [&](int32_t j) { return pair_c2(atomicAdd(&tab[j], 1u)); });
+    __syncthreads();
+    la.v[1] += pair_diamonds(g, tl3, T, cv, i, b0, e0, wid, nw, [&](int32_t j) -> uint32_t { return tab[lc.place(j)]; });
+    if (i >= cv.h0) {
+      const int64_t s0 = lc.start(i);
+      for (int t = threadIdx.x; t < ng; t += IT_MEDIUM_THREADS) {
+        const uint32_t w = tab[t];
+        if (!w) continue;
+        const int64_t j = lc.rank(s0, t);
+        if (j >= cv.h0) cv.put(cv.rowb[i - cv.h0] + cv.li[j - cv.h0], w);
+      }
+    }
     block_item_flush(la, ids, acc, i, sh);
   }
   final_flush(la, ids, acc, sh);
@@ -1673,7 +1752,7 @@ __device__ __forceinline__ u128 pair_wedges_win(const DevGraph& g, longlong2* cu
     }
     int64_t cn_l = ce_l;                        // the lane's new cursor
     if (ce_l - cb_l <= PAIR_SHORT) {            // short: each lane walks its own list up to hi
-      const int32_t* L = g.C + cb_l;
+      const int32_t* L = g.J + cb_l;
       const int len = (int)(ce_l - cb_l);
       Sum128 sh13;
       int q = 0;
@@ -1876,7 +1955,7 @@ __device__ __forceinline__ void cycle4_edges(const DevGraph& g, int64_t b0, int6
       for (int q = 0; q < len_l; q += 4) {
         int32_t jj[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) jj[u] = q + u < len_l ? g.C[kb_l + q + u] : -1;
+        for (int u = 0; u < 4; ++u) jj[u] = q + u < len_l ? g.J[kb_l + q + u] : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (jj[u] >= 0) {
@@ -1895,7 +1974,7 @@ __device__ __forceinline__ void cycle4_edges(const DevGraph& g, int64_t b0, int6
       longm &= longm - 1;
       const int64_t kb = __shfl_sync(0xffffffffu, kb_l, k);
       const int len = __shfl_sync(0xffffffffu, len_l, k);
-      const int32_t* L = g.C + kb;
+      const int32_t* L = g.J + kb;
       unsigned long long sk = 0;
       for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
         int32_t jj[SWEEP_ILP];
@@ -2010,6 +2089,36 @@ __global__ void __launch_bounds__(THREADS) k_cycles4_hash(DevGraph g, const unsi
     if (full) set_err(status, DEVERR_SCRATCH);
     la.v[0] += c4;
     if (__syncthreads_or(c4 != 0)) cycle4_edges(g, b0, e0, wid, nw, C4raw, [&](int32_t j) { return H.get(j); });
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Medium items of small graphs: a counter per vertex of the graph.
+__global__ void __launch_bounds__(IT_MEDIUM_THREADS) k_cycles4_direct(DevGraph g, const unsigned long long* items,
+                                                                     int64_t nitems, unsigned long long* qctr,
+                                                                     LocalIds lc, unsigned long long* C4raw,
+                                                                     AccSet acc) {
+  extern __shared__ uint4 hash_smem[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  uint32_t* tab = reinterpret_cast<uint32_t*>(hash_smem);
+  const int wid = threadIdx.x >> 5, nw = IT_MEDIUM_THREADS / 32;
+  const int ids[1] = {ACC_C4};
+  LocalAcc<1> la;
+  la.zero();
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]);
+    const int64_t b0 = g.R[i], e0 = g.op[i];
+    direct_clear(tab, lc.size(i));
+    __syncthreads();
+    const u128 c4 = pair_wedges(g, b0, e0, wid, nw,
+                                [&](int32_t j) -> unsigned long long { return atomicAdd(&tab[j], 1u); },
+                                [](int64_t, int64_t) { return false; });
+    la.v[0] += c4;
+    if (__syncthreads_or(c4 != 0)) cycle4_edges(g, b0, e0, wid, nw, C4raw, [&](int32_t j) { return tab[j]; });
     block_item_flush(la, ids, acc, i, sh);
   }
   final_flush(la, ids, acc, sh);
@@ -2315,7 +2424,7 @@ __device__ __forceinline__ u128 cycle5_lists(const DevGraph& g, int64_t cb_l, in
   const int len_l = (int)(ce_l - cb_l);
   u128 sum = 0;
   if (len_l <= PAIR_SHORT) {
-    const int32_t* L = g.C + cb_l;
+    const int32_t* L = g.J + cb_l;
     unsigned long long s_ = 0;
     for (int q = 0; q < len_l; q += 4) {
       int32_t jj[4];
@@ -2331,7 +2440,7 @@ __device__ __forceinline__ u128 cycle5_lists(const DevGraph& g, int64_t cb_l, in
   while (longm) {
     const int k = __ffs(longm) - 1;
     longm &= longm - 1;
-    const int32_t* L = g.C + __shfl_sync(0xffffffffu, cb_l, k);
+    const int32_t* L = g.J + __shfl_sync(0xffffffffu, cb_l, k);
     const int len = __shfl_sync(0xffffffffu, len_l, k);
     const uint32_t f = __shfl_sync(0xffffffffu, f_l, k);
     unsigned long long s_ = 0;
@@ -2355,7 +2464,7 @@ __device__ __forceinline__ void lists_each(const DevGraph& g, int64_t cb_l, int6
   const int lane = threadIdx.x & 31;
   const int len_l = (int)(ce_l - cb_l);
   if (len_l <= PAIR_SHORT) {
-    const int32_t* L = g.C + cb_l;
+    const int32_t* L = g.J + cb_l;
     for (int q = 0; q < len_l; q += 4) {
       int32_t jj[4];
 #pragma unroll
@@ -2369,7 +2478,7 @@ __device__ __forceinline__ void lists_each(const DevGraph& g, int64_t cb_l, int6
   while (longm) {
     const int k = __ffs(longm) - 1;
     longm &= longm - 1;
-    const int32_t* L = g.C + __shfl_sync(0xffffffffu, cb_l, k);
+    const int32_t* L = g.J + __shfl_sync(0xffffffffu, cb_l, k);
     const int len = __shfl_sync(0xffffffffu, len_l, k);
     for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
       int32_t jj[SWEEP_ILP];
@@ -2383,9 +2492,10 @@ __device__ __forceinline__ void lists_each(const DevGraph& g, int64_t cb_l, int6
 }
 
 // The increments of one item: w'(i, .) from c < i (every j in N(c)) and c > i
-// (j in N+(c)); P2(i, .) from a in N-(i) (b in N+(a)).  j = b = i is left out.
+// (j in N+(c)); P2(i, .) from a in N-(i) (b in N+(a)).  j = b = i (as g.J names
+// the item) is left out.
 template <class IncW, class IncP>
-__device__ __forceinline__ void cycle5_counts(const DevGraph& g, int64_t i, int64_t b0, int64_t o, int64_t e0,
+__device__ __forceinline__ void cycle5_counts(const DevGraph& g, int32_t i, int64_t b0, int64_t o, int64_t e0,
                                               int64_t gw, int64_t gnw, IncW&& incw, IncP&& incp) {
   const int lane = threadIdx.x & 31;
   for (int64_t pbase = b0 + gw; pbase < e0; pbase += gnw * 32) {
@@ -2430,7 +2540,7 @@ __global__ void __launch_bounds__(THREADS) k_cycles5_hash(DevGraph g, const unsi
     Hp.clear(threadIdx.x, THREADS);
     __syncthreads();
     bool full = false;
-    cycle5_counts(g, i, b0, o, e0, wid, nw, [&](int32_t j) { Hw.inc(j, full); }, [&](int32_t j) { Hp.inc(j, full); });
+    cycle5_counts(g, (int32_t)i, b0, o, e0, wid, nw, [&](int32_t j) { Hw.inc(j, full); }, [&](int32_t j) { Hp.inc(j, full); });
     if (full) set_err(status, DEVERR_SCRATCH);
     __syncthreads();
     for (int tb = wid * 32; tb < (1 << Hp.log); tb += THREADS) {
@@ -2444,6 +2554,49 @@ __global__ void __launch_bounds__(THREADS) k_cycles5_hash(DevGraph g, const unsi
         ce_l = g.R[b + 1];
       }
       la.v[0] += cycle5_lists(g, cb_l, ce_l, w & ((1u << cb) - 1u), [&](int32_t j) -> uint32_t { return Hw.get(j); });
+    }
+    block_item_flush(la, ids, acc, i, sh);
+  }
+  final_flush(la, ids, acc, sh);
+}
+
+// Medium items of small graphs: w'(i, .) in the low and P2(i, .) in the high 16
+// bits of a counter per vertex of the graph (both below its size, at most
+// DIRECT_N).  Each warp takes every 16th b, so that the long lists N+(b) of
+// neighbouring ranks go to different warps.
+__global__ void __launch_bounds__(IT_MEDIUM_THREADS) k_cycles5_direct(DevGraph g, const unsigned long long* items,
+                                                                     int64_t nitems, unsigned long long* qctr,
+                                                                     LocalIds lc, AccSet acc) {
+  extern __shared__ uint4 hash_smem[];
+  __shared__ u128 sh[32];
+  __shared__ int64_t sh_item;
+  uint32_t* tab = reinterpret_cast<uint32_t*>(hash_smem);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = IT_MEDIUM_THREADS / 32;
+  const int ids[1] = {ACC_N8M};
+  LocalAcc<1> la;
+  la.zero();
+  while (true) {
+    const int64_t it = next_item(qctr, nitems, &sh_item);   // its barriers end the last item's reads
+    if (it < 0) break;
+    const int64_t i = item_rank(items[it]), s0 = lc.start(i);
+    const int64_t b0 = g.R[i], o = g.op[i], e0 = g.R[i + 1];
+    const int ng = lc.size(i);
+    direct_clear(tab, ng);
+    __syncthreads();
+    cycle5_counts(g, lc.place(i), b0, o, e0, wid, nw, [&](int32_t j) { atomicAdd(&tab[j], 1u); },
+                  [&](int32_t b) { atomicAdd(&tab[b], 1u << 16); });
+    __syncthreads();
+    for (int tb = wid; tb < ng; tb += nw * 32) {
+      const int t = tb + lane * nw;
+      const uint32_t f = t < ng ? tab[t] >> 16 : 0u;
+      if (!__any_sync(0xffffffffu, f != 0)) continue;
+      int64_t cb_l = 0, ce_l = 0;
+      if (f) {
+        const int64_t b = lc.rank(s0, t);
+        cb_l = g.op[b];
+        ce_l = g.R[b + 1];
+      }
+      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, [&](int32_t j) -> uint32_t { return tab[j] & 0xffffu; });
     }
     block_item_flush(la, ids, acc, i, sh);
   }
@@ -2481,7 +2634,7 @@ __global__ void __launch_bounds__(1024, 1) k_cycles5(DevGraph g, const unsigned 
     wp.next(ts.n);
     if (threadIdx.x == 0) nt = 0;
     __syncthreads();
-    cycle5_counts(g, i, b0, o, e0, wid, nw,
+    cycle5_counts(g, (int32_t)i, b0, o, e0, wid, nw,
                   [&](int32_t j) {
                     const uint32_t q = (uint32_t)j - wlo32;
                     if (q < nwin) atomicAdd(&win[q], 1u);
@@ -2909,8 +3062,9 @@ __global__ void k_split_items(DevGraph g, int32_t* small, int32_t* large, int32_
   }
 }
 
-// max over vertices of d+ x ceil(d- / 64) (words of the D bit sets) and max d+
-__global__ void k_clique_dims(DevGraph g, unsigned long long* out) {
+// max over vertices of d+ x ceil(d- / 64) (words of the D bit sets) and of d+;
+// the largest graph's vertices
+__global__ void k_clique_dims(DevGraph g, const unsigned long long* n_arr, int num_graphs, unsigned long long* out) {
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned long long mw = 0, md = 0;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < g.n; x += stride) {
@@ -2922,8 +3076,12 @@ __global__ void k_clique_dims(DevGraph g, unsigned long long* out) {
     }
     if (dp > md) md = dp;
   }
-  atomicMax(&out[0], mw);
-  atomicMax(&out[1], md);
+  unsigned long long mg = 0;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < num_graphs; k += stride)
+    if (n_arr[k] > mg) mg = n_arr[k];
+  if (mw) atomicMax(&out[0], mw);
+  if (md) atomicMax(&out[1], md);
+  if (mg) atomicMax(&out[2], mg);
 }
 
 
@@ -3350,7 +3508,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   ESC_TRY(orient(rp, col, n, nnz, o, arena, s, sms));
   mark(0, 1, s);
 
-  DevGraph g{n, nnz, o.R, o.C, o.op, o.rev};
+  DevGraph g{n, nnz, o.R, o.C, o.op, o.rev, o.C};
   const int TPB = 256;
   // ---------------- per-element arrays and accumulators
   DevBuf b_T, b_K4e, b_C4e, b_tv, b_C4v, b_K4v, b_acc, b_ctr;
@@ -3410,17 +3568,18 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   ESC_TRY(b_wsmall.alloc(sizeof(int32_t) * (n + 1)));
   ESC_TRY(b_csmall.alloc(sizeof(int32_t) * (n + 1)));
   ESC_TRY(b_clarge.alloc(sizeof(int32_t) * (n + 1)));
-  ESC_TRY(b_dims.alloc(sizeof(unsigned long long) * 2));
-  cudaMemsetAsync(b_dims.p, 0, sizeof(unsigned long long) * 2, s);
+  ESC_TRY(b_dims.alloc(sizeof(unsigned long long) * 3));
+  cudaMemsetAsync(b_dims.p, 0, sizeof(unsigned long long) * 3, s);
   if (n > 0) {
     (k_split_items<<<grid_for(n, TPB, sms), TPB, 0, s>>>(g, b_small.as<int32_t>(), b_large.as<int32_t>(),
                                                           b_wsmall.as<int32_t>(), b_csmall.as<int32_t>(),
                                                           b_clarge.as<int32_t>(), ctr, SMALL_DPLUS,
                                                           std::min(CLQ_WARP_DIN, env_int("ESC_CLQ_WARP_DIN", CLQ_WARP_DIN)),
                                                           own), note_launch());
-    (k_clique_dims<<<grid_for(n, TPB, sms), TPB, 0, s>>>(g, b_dims.as<unsigned long long>()), note_launch());
+    (k_clique_dims<<<grid_for(n, TPB, sms), TPB, 0, s>>>(g, b_narr.as<unsigned long long>(), G,
+                                                         b_dims.as<unsigned long long>()), note_launch());
   }
-  unsigned long long hcnt[16] = {0}, dims[2] = {0, 0};
+  unsigned long long hcnt[16] = {0}, dims[3] = {0, 0, 0};
   cudaMemcpyAsync(hcnt, ctr, sizeof(hcnt), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(dims, b_dims.p, sizeof(dims), cudaMemcpyDeviceToHost, s);
   ESC_TRY(cudaStreamSynchronize(s));
@@ -3528,6 +3687,31 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 27, s);
   ItemLists ilp{b_plist.as<unsigned long long>(), b_pctr.as<unsigned long long>()};
   ItemLists il4{b_list4.as<unsigned long long>(), ilp.cnt + 9}, il5{b_list5.as<unsigned long long>(), ilp.cnt + 18};
+  // small graphs (a union's member for member): medium items count by place in
+  // the graph; the places of a union take a sort of its vertices by graph
+  // (ESC_DIRECT=1: never; tests)
+  const bool direct = dims[2] <= (unsigned long long)DIRECT_N && (G == 1 || (nnz >= 4 * n && G <= n)) &&
+                      env_int("ESC_DIRECT", 2) != 1;
+  const size_t sm_direct = sizeof(uint32_t) * (((size_t)dims[2] + 3) & ~(size_t)3);
+  DevBuf b_lli, b_lhl, b_lhb, b_lrow, b_lwb, b_lJ;
+  LocalIds lc{nullptr, nullptr, nullptr, accs.vg, b_narr.as<unsigned long long>(), (int)std::min<int64_t>(n, DIRECT_N)};
+  DevGraph gd = g;                              // entries by place
+  if (direct && G > 1 && n > 0) {
+    ESC_TRY(b_lli.alloc(sizeof(int32_t) * n));
+    ESC_TRY(b_lhl.alloc(sizeof(int32_t) * n));
+    ESC_TRY(b_lhb.alloc(sizeof(int64_t) * n));
+    ESC_TRY(b_lrow.alloc(sizeof(int64_t) * n));
+    ESC_TRY(b_lwb.alloc(sizeof(int64_t) * (G + 1)));
+    ESC_TRY(b_lJ.alloc(sizeof(int32_t) * (nnz + 1)));
+    ESC_TRY(core_union(accs.vg, G, 0, n, b_lhl.as<int32_t>(), b_lhb.as<int64_t>(), b_lli.as<int32_t>(),
+                       b_lrow.as<int64_t>(), b_lwb.as<int64_t>(), arena, sms, s));
+    (k_local_entries<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(o.C, nnz, b_lli.as<int32_t>(), b_lJ.as<int32_t>()),
+     note_launch());
+    lc.li = b_lli.as<int32_t>();
+    lc.hl = b_lhl.as<int32_t>();
+    lc.hb = b_lhb.as<int64_t>();
+    gd.J = b_lJ.as<int32_t>();
+  }
   unsigned long long cnts[27] = {0};
   const unsigned long long *pcnt = cnts, *cnt4 = cnts + 9, *cnt5 = cnts + 18;
   // count bits of a packed word: every rank is below 2^(32 - cb) - 1
@@ -3540,10 +3724,10 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     if (five)
       (k_pair_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
            g, T, ilp, limit("ESC_PAIR_SMALL_W", IT_LIGHT_M), limit("ESC_PAIR_LARGE_W", IT_MEDIUM_M), cb, accs.vg, n_arr,
-           own), note_launch());
+           direct, own), note_launch());
     (k_cycle_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
          g, il4, il5, !five, limit("ESC_CYCLE_SMALL_W", IT_LIGHT_M), limit("ESC_CYCLE_LARGE_W", IT_MEDIUM_M),
-         limit("ESC_CYCLE_LARGE_W", IT5_MEDIUM_M), cb, accs.vg, n_arr, own), note_launch());
+         limit("ESC_CYCLE_LARGE_W", direct ? IT_MEDIUM_M : IT5_MEDIUM_M), cb, accs.vg, n_arr, direct, own), note_launch());
     cudaMemcpyAsync(cnts, b_pctr.p, sizeof(cnts), cudaMemcpyDeviceToHost, s);
   }
   std::vector<int64_t> hR(n + 1, 0);
@@ -3834,7 +4018,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       (k_pairs_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s>>>(
            g, pl, (int64_t)pcnt[0], pq + 0, cb, IT_LIGHT_LOG, tl3, T, cv, accs, d_status), note_launch());
     }
-    if (pcnt[1] > 0) {
+    if (pcnt[1] > 0 && direct) {
+      ESC_TRY(fill((const void*)k_pairs_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)pcnt[1], &grid_i));
+      (k_pairs_direct<<<grid_i, IT_MEDIUM_THREADS, sm_direct, s>>>(gd, pl + n, (int64_t)pcnt[1], pq + 1, lc, tl3, T, cv,
+                                                                 accs), note_launch());
+    } else if (pcnt[1] > 0) {
       ESC_TRY(fill((const void*)k_pairs_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)pcnt[1], &grid_i));
       (k_pairs_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s>>>(
            g, pl + n, (int64_t)pcnt[1], pq + 1, cb, IT_MEDIUM_LOG, tl3, T, cv, accs, d_status), note_launch());
@@ -3896,7 +4084,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
         (k_cycles4_tag<false><<<grid_sweep, 512, 0, s2>>>(g, l4 + 2 * n, (int64_t)cnt4[2], q4 + 2, tsA, C4e, accs),
          note_launch());
     }
-    if (cnt4[1] > 0) {
+    if (cnt4[1] > 0 && direct) {
+      ESC_TRY(fill((const void*)k_cycles4_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt4[1], &grid_i));
+      (k_cycles4_direct<<<grid_i, IT_MEDIUM_THREADS, sm_direct, s2>>>(gd, l4 + n, (int64_t)cnt4[1], q4 + 1, lc, C4e,
+                                                                    accs), note_launch());
+    } else if (cnt4[1] > 0) {
       ESC_TRY(fill((const void*)k_cycles4_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt4[1], &grid_i));
       (k_cycles4_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s2>>>(
            g, l4 + n, (int64_t)cnt4[1], q4 + 1, cb, IT_MEDIUM_LOG, C4e, accs, d_status), note_launch());
@@ -3927,7 +4119,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
         (k_cycles5<false><<<grid5, 1024, smw, s4>>>(g, l5 + 2 * n, (int64_t)cnt5[2], q5 + 2, tsC, ssC, accs, wlo5,
                                                     win5_words), note_launch());
     }
-    if (cnt5[1] > 0) {                          // two tables of half the size
+    if (cnt5[1] > 0 && direct) {
+      ESC_TRY(fill((const void*)k_cycles5_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt5[1], &grid_i));
+      (k_cycles5_direct<<<grid_i, IT_MEDIUM_THREADS, sm_direct, s4>>>(gd, l5 + n, (int64_t)cnt5[1], q5 + 1, lc, accs),
+       note_launch());
+    } else if (cnt5[1] > 0) {                   // two tables of half the size
       ESC_TRY(fill((const void*)k_cycles5_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt5[1], &grid_i));
       (k_cycles5_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s4>>>(
            g, l5 + n, (int64_t)cnt5[1], q5 + 1, cb, IT_MEDIUM_LOG - 1, accs, d_status), note_launch());
@@ -3993,7 +4189,7 @@ cudaError_t run_census_finish(const Oriented& o, int64_t n, int64_t nnz, const P
                               const unsigned long long* d_acc, unsigned long long* d_out, int sms, cudaStream_t s) {
   CacheScope cache_scope(s);
   const int TPB = 256;
-  DevGraph g{n, nnz, o.R, o.C, o.op, o.rev};
+  DevGraph g{n, nnz, o.R, o.C, o.op, o.rev, o.C};
   DevBuf b_acc, b_nm;
   ESC_TRY(b_acc.alloc(sizeof(Acc128) * ACC_COUNT));
   ESC_TRY(b_nm.alloc(sizeof(unsigned long long) * 2));

@@ -176,6 +176,7 @@ struct DevGraph {
   const int32_t* C;     // nnz neighbours (ranks), sorted per row
   const int64_t* op;    // n: first out-neighbour position of each row
   const int64_t* rev;   // nnz: slot of the reverse entry
+  const int32_t* J;     // nnz neighbours as the sweeps' counters index them: C, or the places within the entry's own graph
 };
 
 __device__ __forceinline__ int64_t dg_deg(const DevGraph& g, int64_t v) { return g.R[v + 1] - g.R[v]; }
