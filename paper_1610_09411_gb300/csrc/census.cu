@@ -1021,8 +1021,14 @@ __global__ void k_list_records(DevGraph g, const uint32_t* T, const int64_t* off
 // their counter increments, which with the size of the graph also bounds the
 // distinct counters m_i = min(w_i, n):
 //   light:   m_i <= IT_LIGHT_M and w_i <= 4 IT_LIGHT_M: one CTA of 64 threads
+//   mid:     m_i <= half of medium's: one CTA of 256 threads
 //   medium:  m_i <= IT_MEDIUM_M: one CTA of 512 threads
+//   large:   m_i <= IT_LARGE_M, pair items of single graphs that take several
+//            windows: one CTA of 1024 threads
 //   heavy:   the rest
+// Chung-Lu 2.3 n = 625,000 census 90.2 -> 82.5 ms with mid and large beside the
+// others: an item waits for its chain of barriers and list reads, so what counts
+// is how many are in flight and that their lists are walked once.
 // Light and medium items count in a packed shared-memory hash table of 2 m_i
 // words or more (a power of two), cleared for the item: small items clear
 // little and keep many CTAs on an SM.  An item whose degree does not fit the
@@ -1032,8 +1038,9 @@ __global__ void k_list_records(DevGraph g, const uint32_t* T, const int64_t* off
 // before and after): Chung-Lu 2.3 n = 625,000 5-cycles 34.7 / 17.6, 4-cycles
 // 16.7 / 6.2; Chung-Lu 2.1 n = 262,144 9.6 / 6.6 and 6.5 / 2.0; R-MAT 19 70 / 58
 // and 56 / 20; 256 graphs of 20 to 200 vertices 1.03 / 0.36 and 0.40 / 0.14.
-static constexpr int IT_LIGHT_LOG = 11, IT_MEDIUM_LOG = 14, IT_MIN_LOG = 7;
-static constexpr int IT_LIGHT_THREADS = 64, IT_MEDIUM_THREADS = 512;
+static constexpr int IT_LIGHT_LOG = 11, IT_MID_LOG = 13, IT_MEDIUM_LOG = 14, IT_LARGE_LOG = 15, IT_MIN_LOG = 7;
+static constexpr int IT_LIGHT_THREADS = 64, IT_MID_THREADS = 256, IT_MEDIUM_THREADS = 512, IT_LARGE_THREADS = 1024;
+static constexpr long long IT_LARGE_M = 3ll << (IT_LARGE_LOG - 2);
 static constexpr long long IT_LIGHT_M = 1ll << (IT_LIGHT_LOG - 1);
 static constexpr long long IT_MEDIUM_M = 1ll << (IT_MEDIUM_LOG - 1);
 static constexpr long long IT5_MEDIUM_M = IT_MEDIUM_M / 2;   // the 5-cycle sweep has two tables
@@ -1122,23 +1129,28 @@ __device__ __forceinline__ int table_log(unsigned long long m) {
   return max(l, IT_MIN_LOG);
 }
 
-// One sweep's item lists (light, medium, heavy; n entries each) and counters:
-// cnt[0..2] list lengths, cnt[3..5] the queues, cnt[6] the largest heavy item.
+// One sweep's item lists (light, medium, heavy, mid, large; n entries each) and
+// counters: cnt[0..2] the first three lists' lengths, cnt[3..5] their queues,
+// cnt[6] the largest heavy item, cnt[9..10] the last two's lengths, cnt[11..12]
+// their queues.
+static constexpr int IT_LISTS = 5, IT_CNT = 13;
 struct ItemLists {
   unsigned long long* list;
   unsigned long long* cnt;
 };
 __device__ __forceinline__ void item_append(const ItemLists& il, int64_t n, int64_t i, unsigned long long w,
                                             unsigned long long m1, unsigned long long m2, long long light_m,
-                                            long long medium_m, bool fits, bool direct) {
+                                            long long medium_m, long long large_m, bool fits, bool direct) {
   const unsigned long long m = max(m1, m2);
-  const int cls = !fits ? (direct && (long long)m <= medium_m ? 1 : 2)   // no count bits in a direct counter
-                        : ((long long)m <= light_m && (long long)w <= 4 * light_m
-                               ? 0
-                               : ((long long)m <= medium_m ? 1 : 2));
+  int cls = 2;
+  if (!fits) cls = direct && (long long)m <= medium_m ? 1 : 2;   // no count bits in a direct counter
+  else if ((long long)m <= light_m && (long long)w <= 4 * light_m) cls = 0;
+  else if ((long long)m <= medium_m / 2 && !direct) cls = 3;
+  else if ((long long)m <= medium_m) cls = 1;
+  else if ((long long)m <= large_m) cls = 4;
   unsigned long long v = (unsigned long long)i;
-  if (cls < 2) v |= ((unsigned long long)table_log(m1) << 32) | ((unsigned long long)table_log(m2) << 40);
-  il.list[(int64_t)cls * n + (int64_t)atomicAdd(&il.cnt[cls], 1ull)] = v;
+  if (cls != 2) v |= ((unsigned long long)table_log(m1) << 32) | ((unsigned long long)table_log(m2) << 40);
+  il.list[(int64_t)cls * n + (int64_t)atomicAdd(&il.cnt[cls < 3 ? cls : cls + 6], 1ull)] = v;
   if (cls == 2) atomicMax(&il.cnt[6], w);        // for the task buffers
 }
 
@@ -1147,7 +1159,8 @@ __device__ __forceinline__ void item_append(const ItemLists& il, int64_t n, int6
 // Also the largest common-neighbour list (triangles on one edge) into cnt[7]
 // and twice the number of diamonds, sum over slots of C(T, 2), into cnt[8].
 __global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, long long light_m, long long medium_m,
-                                int cb, const int32_t* vg, const unsigned long long* n_arr, bool direct, Owner own) {
+                                long long large_m, int cb, const int32_t* vg, const unsigned long long* n_arr,
+                                bool direct, Owner own) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1167,7 +1180,7 @@ __global__ void k_pair_classify(DevGraph g, const uint32_t* T, ItemLists il, lon
     w = warp_sum_u64(w);
     if (lane == 0 && w) {
       const unsigned long long m = min(w, min((unsigned long long)i, vg ? n_arr[vg[i]] : ~0ull));
-      item_append(il, g.n, i, w, m, m, light_m, medium_m, (unsigned long long)(e0 - b0) < (1u << cb) - 1u, direct);
+      item_append(il, g.n, i, w, m, m, light_m, medium_m, large_m, (unsigned long long)(e0 - b0) < (1u << cb) - 1u, direct);
     }
   }
   dia = warp_sum_u64(dia);
@@ -1211,11 +1224,11 @@ __global__ void k_cycle_classify(DevGraph g, ItemLists i4, ItemLists i5, bool on
     const bool fits = (unsigned long long)(e0 - b0) < (1u << cb) - 1u;
     if (w4) {
       const unsigned long long m = min(w4, min((unsigned long long)i, ng));
-      item_append(i4, g.n, i, w4, m, m, light_m, medium_m4, fits, direct);
+      item_append(i4, g.n, i, w4, m, m, light_m, medium_m4, 0, fits, direct);
     }
     // P2 counts the slot of i itself once per a: with nothing else, no path leaves it
     if (!only4 && p2 > (unsigned long long)(o - b0))
-      item_append(i5, g.n, i, w5 + p2, min(w5, ng), min(p2, ng), light_m, medium_m5, fits, direct);
+      item_append(i5, g.n, i, w5 + p2, min(w5, ng), min(p2, ng), light_m, medium_m5, 0, fits, direct);
   }
 }
 
@@ -3713,14 +3726,14 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   }
   // items of the pair, 4-cycle and 5-cycle sweeps (light / medium / heavy lists)
   DevBuf b_plist, b_list4, b_list5, b_pctr;
-  const size_t list_b = sizeof(unsigned long long) * 3 * (size_t)(n + 1);
+  const size_t list_b = sizeof(unsigned long long) * IT_LISTS * (size_t)(n + 1);
   ESC_TRY(b_plist.alloc(five ? list_b : 16));
   ESC_TRY(b_list4.alloc(list_b));
   ESC_TRY(b_list5.alloc(five ? list_b : 16));
-  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 27));
-  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 27, s);
+  ESC_TRY(b_pctr.alloc(sizeof(unsigned long long) * 3 * IT_CNT));
+  cudaMemsetAsync(b_pctr.p, 0, sizeof(unsigned long long) * 3 * IT_CNT, s);
   ItemLists ilp{b_plist.as<unsigned long long>(), b_pctr.as<unsigned long long>()};
-  ItemLists il4{b_list4.as<unsigned long long>(), ilp.cnt + 9}, il5{b_list5.as<unsigned long long>(), ilp.cnt + 18};
+  ItemLists il4{b_list4.as<unsigned long long>(), ilp.cnt + IT_CNT}, il5{b_list5.as<unsigned long long>(), ilp.cnt + 2 * IT_CNT};
   // small graphs (a union's member for member): medium items count by place in
   // the graph; the places of a union take a sort of its vertices by graph
   // (ESC_DIRECT=1: never; tests)
@@ -3746,8 +3759,10 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     lc.hb = b_lhb.as<int64_t>();
     gd.J = b_lJ.as<int32_t>();
   }
-  unsigned long long cnts[27] = {0};
-  const unsigned long long *pcnt = cnts, *cnt4 = cnts + 9, *cnt5 = cnts + 18;
+  unsigned long long cnts[3 * IT_CNT] = {0};
+  const unsigned long long *pcnt = cnts, *cnt4 = cnts + IT_CNT, *cnt5 = cnts + 2 * IT_CNT;
+  // a single graph of more ranks than a window: heavy items walk their lists once per window
+  const bool large_pairs = G == 1 && n > 2 * (int64_t)std::min((smem_optin - 4096) / 4, env_int("ESC_PAIR_WIN_WORDS", 1 << 30));
   // count bits of a packed word: every rank is below 2^(32 - cb) - 1
   int cb = 31;
   while (cb > 1 && n >= ((int64_t)1 << (32 - cb)) - 1) --cb;
@@ -3757,8 +3772,8 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     auto limit = [](const char* name, long long m) { return std::min<long long>(m, env_int(name, (int)m + 1) - 1); };
     if (five)
       (k_pair_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
-           g, T, ilp, limit("ESC_PAIR_SMALL_W", IT_LIGHT_M), limit("ESC_PAIR_LARGE_W", IT_MEDIUM_M), cb, accs.vg, n_arr,
-           direct, own), note_launch());
+           g, T, ilp, limit("ESC_PAIR_SMALL_W", IT_LIGHT_M), limit("ESC_PAIR_LARGE_W", IT_MEDIUM_M),
+           large_pairs ? limit("ESC_PAIR_LARGE_W", IT_LARGE_M) : 0, cb, accs.vg, n_arr, direct, own), note_launch());
     (k_cycle_classify<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(
          g, il4, il5, !five, limit("ESC_CYCLE_SMALL_W", IT_LIGHT_M), limit("ESC_CYCLE_LARGE_W", IT_MEDIUM_M),
          limit("ESC_CYCLE_LARGE_W", direct ? IT_MEDIUM_M : IT5_MEDIUM_M), cb, accs.vg, n_arr, direct, own), note_launch());
@@ -4047,15 +4062,26 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     *grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, items);
     return cudaSuccess;
   };
-  const size_t sm_light = sizeof(uint32_t) << IT_LIGHT_LOG, sm_medium = sizeof(uint32_t) << IT_MEDIUM_LOG;
+  const size_t sm_light = sizeof(uint32_t) << IT_LIGHT_LOG, sm_mid = sizeof(uint32_t) << IT_MID_LOG,
+               sm_medium = sizeof(uint32_t) << IT_MEDIUM_LOG, sm_large = sizeof(uint32_t) << IT_LARGE_LOG;
   unsigned grid_i = 1;
   if (five && n > 0) {
-    unsigned long long* pq = ilp.cnt + 3;       // queue counters of the three lists
+    unsigned long long* pq = ilp.cnt + 3;       // queue counters of the first three lists
     const unsigned long long* pl = ilp.list;
     if (pcnt[0] > 0) {
       ESC_TRY(fill((const void*)k_pairs_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)pcnt[0], &grid_i));
       (k_pairs_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s>>>(
            g, pl, (int64_t)pcnt[0], pq + 0, cb, IT_LIGHT_LOG, tl3, T, cv, accs, d_status), note_launch());
+    }
+    if (pcnt[9] > 0) {
+      ESC_TRY(fill((const void*)k_pairs_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)pcnt[9], &grid_i));
+      (k_pairs_hash<IT_MID_THREADS><<<grid_i, IT_MID_THREADS, sm_mid, s>>>(
+           g, pl + 3 * n, (int64_t)pcnt[9], ilp.cnt + 11, cb, IT_MID_LOG, tl3, T, cv, accs, d_status), note_launch());
+    }
+    if (pcnt[10] > 0) {
+      ESC_TRY(fill((const void*)k_pairs_hash<IT_LARGE_THREADS>, IT_LARGE_THREADS, sm_large, (int64_t)pcnt[10], &grid_i));
+      (k_pairs_hash<IT_LARGE_THREADS><<<grid_i, IT_LARGE_THREADS, sm_large, s>>>(
+           g, pl + 4 * n, (int64_t)pcnt[10], ilp.cnt + 12, cb, IT_LARGE_LOG, tl3, T, cv, accs, d_status), note_launch());
     }
     if (pcnt[1] > 0 && direct) {
       ESC_TRY(fill((const void*)k_pairs_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)pcnt[1], &grid_i));
@@ -4132,6 +4158,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       (k_cycles4_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s2>>>(
            g, l4 + n, (int64_t)cnt4[1], q4 + 1, cb, IT_MEDIUM_LOG, C4e, accs, d_status), note_launch());
     }
+    if (cnt4[9] > 0) {
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt4[9], &grid_i));
+      (k_cycles4_hash<IT_MID_THREADS><<<grid_i, IT_MID_THREADS, sm_mid, s2>>>(
+           g, l4 + 3 * n, (int64_t)cnt4[9], il4.cnt + 11, cb, IT_MID_LOG, C4e, accs, d_status), note_launch());
+    }
     if (cnt4[0] > 0) {
       ESC_TRY(fill((const void*)k_cycles4_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)cnt4[0], &grid_i));
       (k_cycles4_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s2>>>(
@@ -4166,6 +4197,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       ESC_TRY(fill((const void*)k_cycles5_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt5[1], &grid_i));
       (k_cycles5_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s4>>>(
            g, l5 + n, (int64_t)cnt5[1], q5 + 1, cb, IT_MEDIUM_LOG - 1, accs, d_status), note_launch());
+    }
+    if (cnt5[9] > 0) {
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt5[9], &grid_i));
+      (k_cycles5_hash<IT_MID_THREADS><<<grid_i, IT_MID_THREADS, sm_mid, s4>>>(
+           g, l5 + 3 * n, (int64_t)cnt5[9], il5.cnt + 11, cb, IT_MID_LOG - 1, accs, d_status), note_launch());
     }
     if (cnt5[0] > 0) {
       ESC_TRY(fill((const void*)k_cycles5_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, 2 * sm_light, (int64_t)cnt5[0], &grid_i));

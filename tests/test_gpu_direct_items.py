@@ -72,3 +72,14 @@ def test_sparse_union_with_more_graphs_than_edges():
     graphs = [gg.empty(1)] * 40 + [gg.path(4), gg.cycle(5), gg.empty(0), gg.complete(4)]
     for g, r in zip(graphs, gpu_batch(graphs)):
         assert_same_census(r, oracle.census(g))
+
+
+@pytest.mark.parametrize("words", [4000, None], ids=["large_hash", "one_window"])
+def test_large_pair_items_match_the_oracle(words, monkeypatch):
+    """Pair items of 8,193 to 24,576 counters: hashed when a window does not
+    hold the graph's ranks."""
+    from paper_1610_09411_gb300 import escape as esc
+    if words:
+        monkeypatch.setenv("ESC_PAIR_WIN_WORDS", str(words))
+    g = gg.chung_lu(26001, 2.1, 12, 3000, 9)
+    assert_same_census(esc.census(g.row_ptr, g.col, n=g.n), oracle.census(g))
