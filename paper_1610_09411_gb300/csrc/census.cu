@@ -2462,10 +2462,14 @@ __global__ void __launch_bounds__(WHEEL_THREADS, 1) k_wheels_cta(DevGraph g, int
 // The paths whose own a or b is counted by w' are the directed tailed
 // triangles, subtracted through ACC_N8Z (pass A).
 // ============================================================================
+template <bool BIG> struct CountSum { typedef uint32_t type; };
+template <> struct CountSum<true> { typedef unsigned long long type; };
+
 // The lists N+(b) of up to 32 vertices b (lane l holds the l-th list [cb_l, ce_l)
 // and its factor f_l; empty lists have cb_l = ce_l): sum of f * get(j) over
 // their entries.  Lists of up to PAIR_SHORT entries are walked by one lane each.
-template <class Get>
+// Blk holds the sum of SWEEP_ILP counts: 32 bits where a count is below 2^16.
+template <typename Blk, class Get>
 __device__ __forceinline__ u128 cycle5_lists(const DevGraph& g, int64_t cb_l, int64_t ce_l, uint32_t f_l, Get&& get) {
   const int lane = threadIdx.x & 31;
   const int len_l = (int)(ce_l - cb_l);
@@ -2490,15 +2494,32 @@ __device__ __forceinline__ u128 cycle5_lists(const DevGraph& g, int64_t cb_l, in
     const int32_t* L = g.J + __shfl_sync(0xffffffffu, cb_l, k);
     const int len = __shfl_sync(0xffffffffu, len_l, k);
     const uint32_t f = __shfl_sync(0xffffffffu, f_l, k);
+    // whole groups without a test per entry (R-MAT 19 5-cycles 57.3 -> 53.0 ms)
     unsigned long long s_ = 0;
-    for (int q = lane; q < len; q += 32 * SWEEP_ILP) {
+    int q = 0;
+    for (; q + 32 * SWEEP_ILP <= len; q += 32 * SWEEP_ILP) {
       int32_t jj[SWEEP_ILP];
 #pragma unroll
-      for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = q + 32 * u < len ? L[q + 32 * u] : -1;
+      for (int u = 0; u < SWEEP_ILP; ++u) jj[u] = L[q + lane + 32 * u];
+      Blk blk = 0;
 #pragma unroll
-      for (int u = 0; u < SWEEP_ILP; ++u)
-        if (jj[u] >= 0) s_ += get(jj[u]);
+      for (int u = 0; u < SWEEP_ILP; ++u) blk += get(jj[u]);
+      s_ += blk;
     }
+#pragma unroll
+    for (int gsz = SWEEP_ILP / 2; gsz >= 1; gsz >>= 1) {
+      if (q + 32 * gsz <= len) {
+        int32_t jj[SWEEP_ILP / 2];
+#pragma unroll
+        for (int u = 0; u < gsz; ++u) jj[u] = L[q + lane + 32 * u];
+        Blk blk = 0;
+#pragma unroll
+        for (int u = 0; u < gsz; ++u) blk += get(jj[u]);
+        s_ += blk;
+        q += 32 * gsz;
+      }
+    }
+    if (q + lane < len) s_ += get(L[q + lane]);
     sum += (u128)s_ * f;
   }
   return sum;
@@ -2600,7 +2621,7 @@ __global__ void __launch_bounds__(THREADS) k_cycles5_hash(DevGraph g, const unsi
         cb_l = g.op[b];
         ce_l = g.R[b + 1];
       }
-      la.v[0] += cycle5_lists(g, cb_l, ce_l, w & ((1u << cb) - 1u), [&](int32_t j) -> uint32_t { return Hw.get(j); });
+      la.v[0] += cycle5_lists<unsigned long long>(g, cb_l, ce_l, w & ((1u << cb) - 1u), [&](int32_t j) -> uint32_t { return Hw.get(j); });
     }
     block_item_flush(la, ids, acc, i, sh);
   }
@@ -2643,7 +2664,7 @@ __global__ void __launch_bounds__(IT_MEDIUM_THREADS) k_cycles5_direct(DevGraph g
         cb_l = g.op[b];
         ce_l = g.R[b + 1];
       }
-      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, [&](int32_t j) -> uint32_t { return tab[j] & 0xffffu; });
+      la.v[0] += cycle5_lists<uint32_t>(g, cb_l, ce_l, f, [&](int32_t j) -> uint32_t { return tab[j] & 0xffffu; });
     }
     block_item_flush(la, ids, acc, i, sh);
   }
@@ -2712,7 +2733,7 @@ __global__ void __launch_bounds__(1024, 1) k_cycles5(DevGraph g, const unsigned 
         cb_l = g.op[b];
         ce_l = g.R[b + 1];
       }
-      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, get);
+      la.v[0] += cycle5_lists<typename CountSum<BIG>::type>(g, cb_l, ce_l, f, get);
     }
     for (unsigned tb = (unsigned)wid * 32; tb < n2; tb += (unsigned)nw * 32) {
       const unsigned t = tb + lane;
@@ -2724,7 +2745,7 @@ __global__ void __launch_bounds__(1024, 1) k_cycles5(DevGraph g, const unsigned 
         ce_l = g.R[b + 1];
         f = p2[b];
       }
-      la.v[0] += cycle5_lists(g, cb_l, ce_l, f, get);
+      la.v[0] += cycle5_lists<typename CountSum<BIG>::type>(g, cb_l, ce_l, f, get);
     }
     __syncthreads();
     for (unsigned t = threadIdx.x; t < n2; t += blockDim.x) p2[tl2[t]] = 0;
