@@ -989,19 +989,52 @@ struct TriLists {
   const int32_t* U;      // sorted common-neighbour ids
   const int64_t* offp;   // per slot: start of the slot's position list
   const int32_t* P;      // per slot (u -> v): positions in row u of the common neighbours, ascending
-  const uint4* rec;      // per slot: off (x, y), the list's length (z), its entries below the core (w; see k_list_records)
+  const uint4* rec;      // per slot: the list the diamond pass reads (see k_list_records)
+  const int32_t* UL;     // id lists of the slots to core vertices, entries below the core only
 };
-// What the diamond pass wants of a slot, in one 16-byte record: it comes to the
-// slots (x -> y) in no order, and the start, the length, the core length and the
-// neighbour in arrays of their own are a sector each.  w: for a slot to a core
-// vertex bit 31 and the number of entries below the core, else the length.
-// R-MAT 19 census 417 -> 412 ms.
-__global__ void k_list_records(DevGraph g, const uint32_t* T, const int64_t* off, const uint32_t* low, int64_t h0,
-                               uint4* rec) {
+// What the diamond pass wants of a slot (x -> y), y above x, in one 16-byte
+// record: it comes to the slots in no order, and the start, the length, the core
+// length and the neighbour in arrays of their own are a sector each.
+//   x, y: start of the list; z: its length; w: 1 for a slot to a core vertex
+// From a list of an edge to a core vertex only the entries below the core are
+// read (core.cu counts the other tips), so these are packed again, end to end: a
+// fraction of the lists, and the pass is bound by their scattered sectors.
+// R-MAT 19 census 417 -> 412 ms with the records, 400 -> 383 with the packed lists
+// (R-MAT 16 24.8 -> 24.0, Chung-Lu 2.1 41.0 -> 39.9).
+__global__ void k_low_counts(DevGraph g, const uint32_t* low, int64_t h0, int64_t* cnt) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t v = warp; v < g.n; v += nwarps) {
+    const int64_t o = g.op[v];
+    for (int64_t p = g.R[v] + lane; p < g.R[v + 1]; p += 32) cnt[p] = p >= o && g.C[p] >= h0 ? (int64_t)low[p] : 0;
+  }
+}
+__global__ void k_low_lists(int64_t nnz, const int64_t* off, const int32_t* U, const int64_t* off_l, int32_t* UL) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t pb = warp * 32; pb < nnz; pb += nwarps * 32) {
+    const int64_t p = pb + lane;
+    const long long to = p < nnz ? off_l[p] : 0, len = p < nnz ? off_l[p + 1] - to : 0;
+    const long long from = len > 0 ? off[p] : 0;
+    unsigned m = __ballot_sync(0xffffffffu, len > 0);
+    while (m) {
+      const int k = __ffs(m) - 1;
+      m &= m - 1;
+      const int32_t* src = U + __shfl_sync(0xffffffffu, from, k);
+      int32_t* dst = UL + __shfl_sync(0xffffffffu, to, k);
+      const long long cnt = __shfl_sync(0xffffffffu, len, k);
+      for (long long q = lane; q < cnt; q += 32) dst[q] = src[q];
+    }
+  }
+}
+__global__ void k_list_records(DevGraph g, const uint32_t* T, const int64_t* off, const uint32_t* low,
+                               const int64_t* off_l, int64_t h0, uint4* rec) {
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < g.nnz; p += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long o = (unsigned long long)off[p];
-    const uint32_t t = T[p];
-    rec[p] = make_uint4((uint32_t)o, (uint32_t)(o >> 32), t, low && g.C[p] >= h0 ? low[p] | 0x80000000u : t);
+    const bool core = off_l && g.C[p] >= h0;
+    const unsigned long long o = (unsigned long long)(core ? off_l[p] : off[p]);
+    rec[p] = make_uint4((uint32_t)o, (uint32_t)(o >> 32), core ? low[p] : T[p], core ? 1u : 0u);
   }
 }
 
@@ -1398,21 +1431,21 @@ __device__ __forceinline__ u128 pair_diamond_chunk(const TriLists& tl3, const Co
   const int lane = threadIdx.x & 31;
   const int32_t i32 = (int32_t)i;
   Sum128 n17;
-  int64_t vb_l = 0;
+  const int32_t* L_l = tl3.U;
   uint32_t len_l = 0;
-  bool cut = false;                             // only the tips below the core: core.cu counts the others
+  bool cut = false;
   if (on) {
     const uint4 e = __ldg(&tl3.rec[xb + tl3.P[r]]);   // slot (x -> y)
-    cut = i >= cv.h0 && (e.w >> 31) != 0;
-    len_l = cut ? e.w & 0x7fffffffu : e.z;
-    vb_l = (int64_t)(((unsigned long long)e.y << 32) | e.x);
+    cut = i >= cv.h0 && e.w != 0;               // every entry is below i
+    len_l = e.z;
+    L_l = (e.w ? tl3.UL : tl3.U) + (int64_t)(((unsigned long long)e.y << 32) | e.x);
   }
   // short lists: each lane walks its own, a few entries in flight, until it
   // passes i (no entry loaded beyond the next few); long ones: the whole warp
   // on one list at a time.  Each term W(i,j) - 2 is below 2^32; a lane adds at
   // most 2^26 of them per list into 64 bits before the carry-counted sum.
   if (on && len_l <= PAIR_SHORT) {
-    const int32_t* L = tl3.U + vb_l;
+    const int32_t* L = L_l;
     const int len = (int)len_l;
     unsigned long long part = 0;
     for (int q = 0; q < len; q += 4) {
@@ -1436,7 +1469,7 @@ __device__ __forceinline__ u128 pair_diamond_chunk(const TriLists& tl3, const Co
   const bool lng = on && len_l > PAIR_SHORT;
   int pre_l = lng && cut ? (int)len_l : 0;
   if (lng && !cut) {
-    const int32_t* L = tl3.U + vb_l;
+    const int32_t* L = L_l;
     int lo = 0, hi = (int)len_l;
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
@@ -1449,7 +1482,8 @@ __device__ __forceinline__ u128 pair_diamond_chunk(const TriLists& tl3, const Co
   while (longm) {
     const int k = __ffs(longm) - 1;
     longm &= longm - 1;
-    const int32_t* L = tl3.U + __shfl_sync(0xffffffffu, vb_l, k) + lane;
+    const int32_t* L = reinterpret_cast<const int32_t*>(
+                           __shfl_sync(0xffffffffu, reinterpret_cast<uintptr_t>(L_l), k)) + lane;
     const int pre = __shfl_sync(0xffffffffu, pre_l, k);
     unsigned long long part = 0;             // x, y are common neighbours of i and every j read here
     int sb = 0;
@@ -4006,7 +4040,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   ESC_TRY(allow_max_smem((const void*)k_tri_lists, smem_optin));
   DevBuf b_rec;
   ESC_TRY(b_rec.alloc(five ? sizeof(uint4) * (size_t)(nnz + 1) : 16));
-  TriLists tl3{off, b_U.as<int32_t>(), offp, b_P.as<int32_t>(), b_rec.as<uint4>()};
+  TriLists tl3{off, b_U.as<int32_t>(), offp, b_P.as<int32_t>(), b_rec.as<uint4>(), nullptr};
 
   // wheel work items: ranks are in degree order, so the large centres are a suffix
   int64_t c0 = n;
@@ -4061,8 +4095,23 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
            g, lo, hR[lo], off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(), d_status), note_launch());
   }
   if (ch > 0) ESC_TRY(core_low(g, T, off, b_U.as<int32_t>(), cv.h0, b_low.as<uint32_t>(), sms, s));
+  DevBuf b_offl, b_UL;
+  if (ch > 0) {                                 // the core's short lists
+    int64_t total = 0;
+    ESC_TRY(b_offl.alloc(sizeof(int64_t) * (nnz + 2)));
+    (k_low_counts<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, b_low.as<uint32_t>(), cv.h0, b_offl.as<int64_t>()),
+     note_launch());
+    ESC_TRY(exclusive_scan_i64(b_offl.as<int64_t>(), b_offl.as<int64_t>(), nnz, true, arena, s));
+    cudaMemcpyAsync(&total, b_offl.as<int64_t>() + nnz, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    ESC_TRY(cudaStreamSynchronize(s));
+    ESC_TRY(b_UL.alloc(sizeof(int32_t) * (size_t)(total + 1)));
+    (k_low_lists<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(nnz, off, b_U.as<int32_t>(), b_offl.as<int64_t>(),
+                                                        b_UL.as<int32_t>()), note_launch());
+    tl3.UL = b_UL.as<int32_t>();
+  }
   if (five && nnz > 0)
-    (k_list_records<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(g, T, off, ch > 0 ? b_low.as<uint32_t>() : nullptr, cv.h0,
+    (k_list_records<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(g, T, off, b_low.as<uint32_t>(),
+                                                          ch > 0 ? b_offl.as<int64_t>() : nullptr, cv.h0,
                                                           b_rec.as<uint4>()), note_launch());
   mark(4, 1, s);
   StreamSet ss_all;
