@@ -3553,9 +3553,10 @@ static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGra
 // Chung-Lu n = 120,000, 5e8 (401), 18.2 / 16.4; Chung-Lu 2.3 n = 250,000, 5e8
 // (134), 52.5 / 52.7; Chung-Lu 2.5 n = 500,000, 9e7 (11), 97.5 / 100.1.
 // The degree limit hardly matters between 16 and 64 (R-MAT 16: 38.5 to 39.0 ms,
-// 96: 45.2), nor the cap from 16,384 up (R-MAT 19: 8,192 760 ms, 16,384 661 ms,
-// 32,768 656 ms); W takes 2 bytes x cap^2.
-static constexpr int CORE_MIN_DEG = 48, CORE_CAP = 16384, CORE_CHUNK_MB = 2048;
+// 96: 45.2), the cap does on large graphs (R-MAT 19: 8,192 482 ms, 16,384 383,
+// 32,768 384, 49,152 385; R-MAT 22: 16,384 15.0 s, 32,768 13.0 s); W takes 2 or 4
+// bytes x cap^2.
+static constexpr int CORE_MIN_DEG = 48, CORE_CAP = 32768, CORE_CHUNK_MB = 2048;
 static constexpr unsigned long long CORE_MIN_D = 1ull << 24, CORE_D_PER_ENTRY = 160;
 static constexpr size_t CORE_W_BYTES = (size_t)24 << 30;
 
