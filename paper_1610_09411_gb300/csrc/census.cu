@@ -10,11 +10,11 @@
 //   Thm 6/7 4-cliques K4(e), K4(t); Thm 10 N10,
 //     N16, N20; Thm 14 5-cliques ............... k_clique_warp / k_clique_large (pass B)
 //   Thm 13's directed tailed triangles ......... k_tri_small / k_tri_large (pass A)
-//   Thm 5 4-cycles C4(e), C4(i) ................ k_cycles4
+//   Thm 5 4-cycles C4(e), C4(i) ................ k_cycles4_*
 //   Thm 12 common-neighbour lists of edges ..... k_tri_lists
-//   Thm 11/12 N13, N17 (pairs and diamonds) .... k_pairs
+//   Thm 11/12 N13, N17 (pairs and diamonds) .... k_pairs_*, core.cu
 //   Thm 11 N18 (wheels) ........................ k_wheels_warp / k_wheels_cta
-//   Thm 13 5-cycles ............................ k_cycles5
+//   Thm 13 5-cycles ............................ k_cycles5*
 //   Thm 3 + App. B assembly .................... k_assemble
 #include "common.cuh"
 #include "core.cuh"
