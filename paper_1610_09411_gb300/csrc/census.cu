@@ -3926,6 +3926,9 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
       cbuf.bits = b_cbits.p;
       cbuf.blocks = b_cblk.p;
       cbuf.tiles = b_ctile.p;
+      // ESC_CORE_WAIT_US, ESC_CORE_GIVE_UP: a shorter limit, a wait that runs out (tests)
+      cbuf.wait_ns = 1000ull * (unsigned long long)env_int("ESC_CORE_WAIT_US", 4000000);
+      cbuf.give_up = (uint32_t)env_int("ESC_CORE_GIVE_UP", 0);
       if (cv.h0 > 0) {
         ESC_TRY(b_cb.alloc((cv.wide ? sizeof(uint32_t) : sizeof(uint16_t)) * (size_t)(cchunks.max_tri + 2)));
         cbuf.b = b_cb.p;

@@ -324,16 +324,17 @@ __device__ __forceinline__ unsigned long long now_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Waits at most CORE_WAIT_NS; false when the wait ran out.
-static constexpr unsigned long long CORE_WAIT_NS = 4000000000ull;
-__device__ __forceinline__ bool mb_wait(uint32_t bar, uint32_t parity) {
+// Waits at most limit_ns (0: not at all); false when the wait ran out.
+static constexpr unsigned long long CORE_DRAIN_NS = 4000000000ull;
+__device__ __forceinline__ bool mb_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
+  if (limit_ns == 0) return false;
   for (int k = 0; k < 16; ++k)
     if (mb_try(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   while (true) {
     for (int k = 0; k < 32; ++k)
       if (mb_try(bar, parity)) return true;
-    if (now_ns() - t0 > CORE_WAIT_NS) return false;
+    if (now_ns() - t0 > limit_ns) return false;
   }
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -382,8 +383,14 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // finished tile from tensor memory while the next one is accumulated in the
 // other half of its 512 columns.  A lane holds one row u and walks the columns,
 // so that the lanes of a warp read W(v, .) and b(v, .) along their rows.
-// Every wait is bounded: a wait that runs out sets the status word and ends the
-// CTA's work.  One centre with d = 16,000 runs at 3.4 PFLOP/s; the many smaller
+// Every wait is bounded (wait_ns): a wait that runs out sets the status word and
+// ends that role's work, after which the other roles' waits run out too.  A
+// reading warp decides with all its lanes at once, as what follows the wait is
+// warp-wide.  However it ends, the copying thread waits until its copies have
+// landed and the issuing thread until its MMAs have finished (CORE_DRAIN_NS at
+// most) before the tensor memory goes back and the CTA ends.  give_up: the
+// reading warps take their wait for this tile (from 1; 0: none) as run out.
+// One centre with d = 16,000 runs at 3.4 PFLOP/s; the many smaller
 // centres of R-MAT 19 (3.3e13 multiply-adds in its triangle's tiles) take 42 ms
 // and are bound by the scattered sectors of W (512 MB, beyond L2) that the
 // entries read, not by the MMAs; the adjacency bits, N20 and the 4-clique sums
@@ -398,7 +405,7 @@ __device__ __forceinline__ bool epi_all(bool ok) {
   return r != 0;
 }
 struct CoreBars {
-  unsigned long long full[CORE_STAGES], empty[CORE_STAGES], accf[2], acce[2];
+  unsigned long long full[CORE_STAGES], empty[CORE_STAGES], accf[2], acce[2], drain;
 };
 static constexpr size_t CORE_SMEM = 1024 + (size_t)CORE_STAGES * CORE_STAGE_BYTES + 2 * CORE_TN * sizeof(void*);
 
@@ -407,7 +414,8 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
                                                               int64_t ntiles, const uint8_t* blocks,
                                                               const uint32_t* bitm, unsigned long long* k4,
                                                               int64_t k4_0, const WT* b_all, const int64_t* tri_off, int64_t s0,
-                                                              AccSet acc, unsigned* status) {
+                                                              AccSet acc, unsigned* status,
+                                                              unsigned long long wait_ns, uint32_t give_up) {
   extern __shared__ uint8_t core_smem_raw[];
   __shared__ CoreBars bars;
   __shared__ uint32_t s_tmem;
@@ -425,6 +433,7 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
       mb_init(smem_u32(&bars.accf[k]), 1);
       mb_init(smem_u32(&bars.acce[k]), CORE_EPI_WARPS);
     }
+    mb_init(smem_u32(&bars.drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (wid == CORE_EPI_WARPS + 1) {
@@ -450,7 +459,7 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
         const bool two = 2 * vt + 1 < nb;
         for (int kb = 0; kb < nb; ++kb, ++fill) {
           const uint32_t sl = fill % CORE_STAGES, ph = (fill / CORE_STAGES) & 1;
-          if (!mb_wait(smem_u32(&bars.empty[sl]), ph ^ 1)) {
+          if (!mb_wait(smem_u32(&bars.empty[sl]), ph ^ 1, wait_ns)) {
             ok = false;
             break;
           }
@@ -463,11 +472,10 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
                      CORE_BLK_BYTES, full);
         }
       }
-      if (!ok) {                                // let the copies in flight land before the CTA ends
-        set_err(status, DEVERR_TIMEOUT);
-        for (uint32_t k = fill > CORE_STAGES ? fill - CORE_STAGES : 0; k < fill; ++k)
-          mb_wait(smem_u32(&bars.full[k % CORE_STAGES]), (k / CORE_STAGES) & 1);
-      }
+      // the copies in flight land before the CTA ends (the issuing thread may have given up on them)
+      for (uint32_t k = fill > CORE_STAGES ? fill - CORE_STAGES : 0; k < fill; ++k)
+        ok = mb_wait(smem_u32(&bars.full[k % CORE_STAGES]), (k / CORE_STAGES) & 1, CORE_DRAIN_NS) && ok;
+      if (!ok) set_err(status, DEVERR_TIMEOUT);
     }
   } else if (wid == CORE_EPI_WARPS + 1) {       // ------------ MMA issue
     if (lane == 0) {
@@ -480,16 +488,15 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
         // D fp32, A and B e4m3, both K-major; N / 8 and M / 16
         const uint32_t idesc = (1u << 4) | ((uint32_t)(ncols >> 3) << 17) | ((CORE_BLK >> 4) << 24);
         const uint32_t buf = it & 1;
-        if (!mb_wait(smem_u32(&bars.acce[buf]), ((it >> 1) & 1) ^ 1)) {
-          set_err(status, DEVERR_TIMEOUT);
+        if (!mb_wait(smem_u32(&bars.acce[buf]), ((it >> 1) & 1) ^ 1, wait_ns)) {
+          ok = false;
           break;
         }
         tc_fence_after();
         const int ksteps = (d + 31) / 32;       // columns beyond d are zero
         for (int kb = 0; kb < nb; ++kb, ++fill) {
           const uint32_t sl = fill % CORE_STAGES;
-          if (!mb_wait(smem_u32(&bars.full[sl]), (fill / CORE_STAGES) & 1)) {
-            set_err(status, DEVERR_TIMEOUT);
+          if (!mb_wait(smem_u32(&bars.full[sl]), (fill / CORE_STAGES) & 1, wait_ns)) {
             ok = false;
             break;
           }
@@ -503,6 +510,10 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
         }
         if (ok) core_commit(smem_u32(&bars.accf[buf]));
       }
+      // every MMA issued, also of a tile given up on, ends before the tensor memory goes back
+      core_commit(smem_u32(&bars.drain));
+      ok = mb_wait(smem_u32(&bars.drain), 0, CORE_DRAIN_NS) && ok;
+      if (!ok) set_err(status, DEVERR_TIMEOUT);
     }
   } else {                                      // ------------ finished tiles
     const int quad = wid & 3, half = wid >> 2, tid = threadIdx.x;
@@ -543,7 +554,8 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core_mma(DevGraph g, CoreVi
       const uint32_t* bw = bitm + (int64_t)td.x * CORE_BIT_WORDS + (td.w & 0xffff) * 4 + quad;
       unsigned long long* k4c = k4 + (g.R[c + 1] - d - k4_0);
       unsigned long long swy = 0, syy = 0, sy = 0, sbb = 0, s20 = 0, sk = 0;
-      const bool ok = mb_wait(smem_u32(&bars.accf[buf]), (it >> 1) & 1);
+      const bool ok = __all_sync(0xffffffffu, mb_wait(smem_u32(&bars.accf[buf]), (it >> 1) & 1,
+                                                      it + 1 == give_up ? 0 : wait_ns));
       tc_fence_after();
       const WT* const* wr = wrow + buf * CORE_TN;
       constexpr int QC = HASB ? 16 : 32;        // columns in flight (registers)
@@ -722,13 +734,13 @@ static cudaError_t core_run_as(const DevGraph& g, const CoreView& cv, const uint
       (k_core_mma<WT, true><<<grid, CORE_THREADS, CORE_SMEM, s>>>(g, cv, (const int4*)cb.tiles, nt,
                                                                   (const uint8_t*)cb.blocks, (const uint32_t*)cb.bits,
                                                                   (unsigned long long*)cb.k4, cb.k4_0, b, d_tri, s0, acc,
-                                                                  status),
+                                                                  status, cb.wait_ns, cb.give_up),
        note_launch());
     else
       (k_core_mma<WT, false><<<grid, CORE_THREADS, CORE_SMEM, s>>>(g, cv, (const int4*)cb.tiles, nt,
                                                                    (const uint8_t*)cb.blocks, (const uint32_t*)cb.bits,
                                                                    (unsigned long long*)cb.k4, cb.k4_0, nullptr, d_tri,
-                                                                   s0, acc, status),
+                                                                   s0, acc, status, cb.wait_ns, cb.give_up),
        note_launch());
     e = cudaGetLastError();
   }

@@ -21,6 +21,8 @@ struct CoreBuffers {
   void* k4 = nullptr;              // zeroed u64 per slot from k4_0, the first one of rank h0
   int64_t k4_0 = 0;
   void* b = nullptr;               // max_tri counts as wide as W's; null when no vertex lies below the core
+  unsigned long long wait_ns = 4000000000ull;   // limit of every wait of the contraction
+  uint32_t give_up = 0;            // tile whose wait runs out at once (tests; 0: none)
 };
 
 // dh, and the prefix sums off (4 x (h + 1)); for a single graph also li and rowb
