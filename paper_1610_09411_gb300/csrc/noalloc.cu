@@ -415,6 +415,11 @@ extern "C" escape_status escape_cycles4_noalloc(int64_t n, const int64_t* row_pt
   if (e == cudaSuccess) e = le;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, ns.status, sizeof(unsigned int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) { cudaGetLastError(); esc::note_cuda_error(e); return ESCAPE_ECUDA; }
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(s);                   // what was queued writes the outputs and the work space
+    cudaGetLastError();
+    esc::note_cuda_error(e);
+    return ESCAPE_ECUDA;
+  }
   return status ? ESCAPE_EINVAL : ESCAPE_OK;
 }
