@@ -34,8 +34,10 @@
 // 57.9 -> 37.4 ms, of Chung-Lu 2.1 n = 262,144 75.9 -> 65.2 ms.
 //
 // Operands are fp8 (e4m3: 0 and 1 are exact) with fp32 accumulation in tensor
-// memory; M < 2^16, so every entry is an exact integer (checked with all-ones
-// operands up to d = 65,536).  k_core_build writes
+// memory: every partial sum is a whole number below d, exact in fp32 below 2^24
+// (a core of CORE_W_BYTES has d below 2^17; the epilogue reads up to 2^23).  The
+// tests put odd sums of up to 65,000, reached in odd steps, through it.
+// k_core_build writes
 // B_c once as blocks of 128 rows x 128 bytes in the 128-byte-swizzled K-major
 // layout the tensor cores read, 16 KB contiguous, so that a plain bulk copy
 // (cp.async.bulk) moves an operand block to shared memory without a tensor map.
