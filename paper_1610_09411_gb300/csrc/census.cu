@@ -3259,6 +3259,11 @@ CacheScope::~CacheScope() {
   t_scope = prev;
 }
 
+void DevBuf::give_back() {
+  if (p) buf_cache().put(dev, p, bytes);
+  p = nullptr;
+  bytes = 0;
+}
 void DevBuf::release() {
   if (!p) return;
   if (t_scope) t_scope->pending.push_back({p, bytes, dev});
@@ -3865,83 +3870,6 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= 65536) hi = mid; else lo = mid + 1; }
     jbig = lo;
   }
-  // core vertices: their core neighbours, places in W and the prefix sums of the work
-  DevBuf b_cdh, b_cli, b_crow, b_coff, b_chl, b_chb, b_cwb, b_low, b_W, b_cblk, b_ctile, b_cb, b_cbits, b_ck4;
-  CoreView cv{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
-  std::vector<int64_t> coff;
-  int64_t wlen = 0;
-  int64_t ch = 0;
-  const int core_min_d = env_int("ESC_CORE_MIN_D", 0);
-  if (five && own.parts <= 1 && env_int("ESC_CORE", 2) != 1 &&
-      pcnt[8] / 2 >= (core_min_d ? (unsigned long long)core_min_d
-                                 : std::max(CORE_MIN_D, CORE_D_PER_ENTRY * (unsigned long long)nnz))) {
-    const int64_t min_deg = env_int("ESC_CORE_MIN_DEG", CORE_MIN_DEG);
-    int64_t lo = 0, hi = n;                     // first rank of degree >= min_deg
-    while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= min_deg) hi = mid; else lo = mid + 1; }
-    ch = n - lo;
-    if (G == 1) ch = std::min<int64_t>(ch, env_int("ESC_CORE_CAP", CORE_CAP));
-  }
-  if (ch > 0) {
-    ESC_TRY(b_cdh.alloc(sizeof(int32_t) * ch));
-    ESC_TRY(b_cli.alloc(sizeof(int32_t) * ch));
-    ESC_TRY(b_crow.alloc(sizeof(int64_t) * ch));
-    ESC_TRY(b_coff.alloc(sizeof(int64_t) * 4 * (ch + 1)));
-    cv.h0 = n - ch;
-    ESC_TRY(core_layout(g, cv.h0, G == 1, b_cdh.as<int32_t>(), b_cli.as<int32_t>(), b_crow.as<int64_t>(),
-                        b_coff.as<int64_t>(), sms, s));
-    if (G > 1) {
-      ESC_TRY(b_chl.alloc(sizeof(int32_t) * ch));
-      ESC_TRY(b_chb.alloc(sizeof(int64_t) * ch));
-      ESC_TRY(b_cwb.alloc(sizeof(int64_t) * (G + 1)));
-      ESC_TRY(core_union(accs.vg, G, cv.h0, ch, b_chl.as<int32_t>(), b_chb.as<int64_t>(), b_cli.as<int32_t>(),
-                         b_crow.as<int64_t>(), b_cwb.as<int64_t>(), arena, sms, s));
-      cudaMemcpyAsync(&wlen, b_cwb.as<int64_t>() + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    } else {
-      wlen = ch * ch;
-    }
-    coff.resize(4 * (size_t)(ch + 1));
-    cudaMemcpyAsync(coff.data(), b_coff.p, sizeof(int64_t) * 4 * (ch + 1), cudaMemcpyDeviceToHost, s);
-    ESC_TRY(cudaStreamSynchronize(s));
-  }
-  // the core's buffers; a core whose W would pass CORE_W_BYTES is left out
-  CoreChunks cchunks;
-  CoreBuffers cbuf;
-  if (ch > 0) {
-    cv.wide = jbig < n ? 1 : 0;
-    const size_t wb = (cv.wide ? sizeof(uint32_t) : sizeof(uint16_t)) * (size_t)(wlen + 1);
-    core_chunks(coff.data(), ch, (int64_t)env_int("ESC_CORE_CHUNK_MB", CORE_CHUNK_MB) << 20, &cchunks);
-    if (wb > CORE_W_BYTES || cchunks.max_tiles == 0) {
-      ch = 0;
-      cv.h0 = n;
-    } else {
-      ESC_TRY(b_low.alloc(sizeof(uint32_t) * (size_t)(nnz + 1)));
-      ESC_TRY(b_W.alloc(wb));
-      ESC_TRY(b_cblk.alloc(core_block_bytes(cchunks)));
-      ESC_TRY(b_ctile.alloc(sizeof(int4) * (size_t)cchunks.max_tiles));
-      ESC_TRY(b_cbits.alloc(core_bit_bytes(cchunks)));
-      cbuf.k4_0 = hR[cv.h0];
-      ESC_TRY(b_ck4.alloc(sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1)));
-      cudaMemsetAsync(b_ck4.p, 0, sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1), s);
-      cbuf.k4 = b_ck4.p;
-      cbuf.bits = b_cbits.p;
-      cbuf.blocks = b_cblk.p;
-      cbuf.tiles = b_ctile.p;
-      // ESC_CORE_WAIT_US, ESC_CORE_GIVE_UP: a shorter limit, a wait that runs out (tests)
-      cbuf.wait_ns = 1000ull * (unsigned long long)env_int("ESC_CORE_WAIT_US", 4000000);
-      cbuf.give_up = (uint32_t)env_int("ESC_CORE_GIVE_UP", 0);
-      if (cv.h0 > 0) {
-        ESC_TRY(b_cb.alloc((cv.wide ? sizeof(uint32_t) : sizeof(uint16_t)) * (size_t)(cchunks.max_tri + 2)));
-        cbuf.b = b_cb.p;
-      }
-      cv.low = b_low.as<uint32_t>();
-      cv.dh = b_cdh.as<int32_t>();
-      cv.li = b_cli.as<int32_t>();
-      cv.rowb = b_crow.as<int64_t>();
-      cv.hl = G > 1 ? b_chl.as<int32_t>() : nullptr;
-      cv.hb = G > 1 ? b_chb.as<int64_t>() : nullptr;
-      cv.W = b_W.p;
-    }
-  }
   // the heavy pair items: clusters sharing one counter array each
   PairPlan pplan;
   int64_t n0 = 0;                               // first rank of degree >= 1 (lower ranks are never counted)
@@ -4081,6 +4009,99 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     ESC_TRY(exclusive_scan_i64(b_wo.as<int64_t>(), b_wo.as<int64_t>(), c0, true, arena, s));
   }
 
+  // ---------------- the dense core
+  // It saves time and nothing else, so it comes after the buffers that the census
+  // cannot do without, and a core whose buffers do not fit the device (or whose W
+  // would pass CORE_W_BYTES) is left out.  ESC_CORE_MAX_MB: a smaller limit (tests).
+  DevBuf b_cdh, b_cli, b_crow, b_coff, b_chl, b_chb, b_cwb, b_low, b_W, b_cblk, b_ctile, b_cb, b_cbits, b_ck4, b_offl,
+      b_UL;
+  CoreView cv{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
+  CoreChunks cchunks;
+  CoreBuffers cbuf;
+  std::vector<int64_t> coff;
+  int64_t ch = 0, wlen = 0;
+  const size_t core_max = (size_t)env_int("ESC_CORE_MAX_MB", 1 << 30) << 20;
+  size_t core_held = 0;
+  struct Want { DevBuf* b; size_t bytes; };
+  // all of them or none (a buffer given back here has not been used yet)
+  auto reserve = [&](std::initializer_list<Want> wants) -> cudaError_t {
+    size_t sum = 0;
+    for (const Want& w : wants) sum += w.bytes;
+    cudaError_t e = core_held + sum > core_max ? cudaErrorMemoryAllocation : cudaSuccess;
+    for (const Want& w : wants)
+      if (e == cudaSuccess && w.bytes) e = w.b->alloc(w.bytes);
+    core_held += sum;
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    for (const Want& w : wants) w.b->give_back();
+    ch = 0;
+    cv = CoreView{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
+    cbuf = CoreBuffers{};
+    return cudaSuccess;
+  };
+  const int core_min_d = env_int("ESC_CORE_MIN_D", 0);
+  if (five && own.parts <= 1 && env_int("ESC_CORE", 2) != 1 &&
+      pcnt[8] / 2 >= (core_min_d ? (unsigned long long)core_min_d
+                                 : std::max(CORE_MIN_D, CORE_D_PER_ENTRY * (unsigned long long)nnz))) {
+    const int64_t min_deg = env_int("ESC_CORE_MIN_DEG", CORE_MIN_DEG);
+    int64_t lo = 0, hi = n;                     // first rank of degree >= min_deg
+    while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (hR[mid + 1] - hR[mid] >= min_deg) hi = mid; else lo = mid + 1; }
+    ch = n - lo;
+    if (G == 1) ch = std::min<int64_t>(ch, env_int("ESC_CORE_CAP", CORE_CAP));
+  }
+  if (ch > 0)
+    ESC_TRY(reserve({{&b_cdh, sizeof(int32_t) * ch}, {&b_cli, sizeof(int32_t) * ch}, {&b_crow, sizeof(int64_t) * ch},
+                     {&b_coff, sizeof(int64_t) * 4 * (ch + 1)}, {&b_chl, G > 1 ? sizeof(int32_t) * ch : 0},
+                     {&b_chb, G > 1 ? sizeof(int64_t) * ch : 0}, {&b_cwb, G > 1 ? sizeof(int64_t) * (G + 1) : 0}}));
+  if (ch > 0) {
+    // core neighbours, places in W and the prefix sums of the work
+    cv.h0 = n - ch;
+    ESC_TRY(core_layout(g, cv.h0, G == 1, b_cdh.as<int32_t>(), b_cli.as<int32_t>(), b_crow.as<int64_t>(),
+                        b_coff.as<int64_t>(), sms, s));
+    if (G > 1) {
+      ESC_TRY(core_union(accs.vg, G, cv.h0, ch, b_chl.as<int32_t>(), b_chb.as<int64_t>(), b_cli.as<int32_t>(),
+                         b_crow.as<int64_t>(), b_cwb.as<int64_t>(), arena, sms, s));
+      cudaMemcpyAsync(&wlen, b_cwb.as<int64_t>() + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    } else {
+      wlen = ch * ch;
+    }
+    coff.resize(4 * (size_t)(ch + 1));
+    cudaMemcpyAsync(coff.data(), b_coff.p, sizeof(int64_t) * 4 * (ch + 1), cudaMemcpyDeviceToHost, s);
+    ESC_TRY(cudaStreamSynchronize(s));
+    cv.wide = jbig < n ? 1 : 0;
+    const size_t word = cv.wide ? sizeof(uint32_t) : sizeof(uint16_t), wb = word * (size_t)(wlen + 1);
+    core_chunks(coff.data(), ch, (int64_t)env_int("ESC_CORE_CHUNK_MB", CORE_CHUNK_MB) << 20, &cchunks);
+    cbuf.k4_0 = hR[cv.h0];
+    const size_t k4b = sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1);
+    if (wb > CORE_W_BYTES || cchunks.max_tiles == 0) {
+      ch = 0;
+      cv.h0 = n;
+    } else {
+      ESC_TRY(reserve({{&b_low, sizeof(uint32_t) * (size_t)(nnz + 1)}, {&b_W, wb}, {&b_cblk, core_block_bytes(cchunks)},
+                       {&b_ctile, sizeof(int4) * (size_t)cchunks.max_tiles}, {&b_cbits, core_bit_bytes(cchunks)},
+                       {&b_ck4, k4b}, {&b_cb, cv.h0 > 0 ? word * (size_t)(cchunks.max_tri + 2) : 0},
+                       {&b_offl, sizeof(int64_t) * (size_t)(nnz + 2)}}));
+    }
+    if (ch > 0) {
+      cudaMemsetAsync(b_ck4.p, 0, k4b, s);
+      cbuf.k4 = b_ck4.p;
+      cbuf.bits = b_cbits.p;
+      cbuf.blocks = b_cblk.p;
+      cbuf.tiles = b_ctile.p;
+      cbuf.b = cv.h0 > 0 ? b_cb.p : nullptr;
+      // ESC_CORE_WAIT_US, ESC_CORE_GIVE_UP: a shorter limit, a wait that runs out (tests)
+      cbuf.wait_ns = 1000ull * (unsigned long long)env_int("ESC_CORE_WAIT_US", 4000000);
+      cbuf.give_up = (uint32_t)env_int("ESC_CORE_GIVE_UP", 0);
+      cv.low = b_low.as<uint32_t>();
+      cv.dh = b_cdh.as<int32_t>();
+      cv.li = b_cli.as<int32_t>();
+      cv.rowb = b_crow.as<int64_t>();
+      cv.hl = G > 1 ? b_chl.as<int32_t>() : nullptr;
+      cv.hb = G > 1 ? b_chb.as<int64_t>() : nullptr;
+      cv.W = b_W.p;
+    }
+  }
+
   // ---------------- concurrent phases on forked streams
   // The common-neighbour lists come first (short when alone); then
   //   s3 (most urgent): wheels      s : pairs
@@ -4099,16 +4120,16 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
            g, lo, hR[lo], off, offp, T, b_U.as<int32_t>(), b_P.as<int32_t>(), d_status), note_launch());
   }
   if (ch > 0) ESC_TRY(core_low(g, T, off, b_U.as<int32_t>(), cv.h0, b_low.as<uint32_t>(), sms, s));
-  DevBuf b_offl, b_UL;
   if (ch > 0) {                                 // the core's short lists
     int64_t total = 0;
-    ESC_TRY(b_offl.alloc(sizeof(int64_t) * (nnz + 2)));
     (k_low_counts<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, b_low.as<uint32_t>(), cv.h0, b_offl.as<int64_t>()),
      note_launch());
     ESC_TRY(exclusive_scan_i64(b_offl.as<int64_t>(), b_offl.as<int64_t>(), nnz, true, arena, s));
     cudaMemcpyAsync(&total, b_offl.as<int64_t>() + nnz, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     ESC_TRY(cudaStreamSynchronize(s));
-    ESC_TRY(b_UL.alloc(sizeof(int32_t) * (size_t)(total + 1)));
+    ESC_TRY(reserve({{&b_UL, sizeof(int32_t) * (size_t)(total + 1)}}));
+  }
+  if (ch > 0) {
     (k_low_lists<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(nnz, off, b_U.as<int32_t>(), b_offl.as<int64_t>(),
                                                         b_UL.as<int32_t>()), note_launch());
     tl3.UL = b_UL.as<int32_t>();

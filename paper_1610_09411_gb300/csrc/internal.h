@@ -53,6 +53,7 @@ struct DevBuf {
   ~DevBuf() { release(); }
   cudaError_t alloc(size_t b);
   void release();
+  void give_back();              // at once, inside a scope too: nothing may have been enqueued on it
   template <class T> T* as() const { return (T*)p; }
 };
 struct CacheScope {
