@@ -3970,9 +3970,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   ESC_TRY(b_gh.alloc(five ? sizeof(int32_t) * 2 * (size_t)ghash_cap * grid_sweep + 16 : 16));
   size_t smem_l = sizeof(int32_t) * 2 * (size_t)hcap_l;
   ESC_TRY(allow_max_smem((const void*)k_tri_lists, smem_optin));
-  DevBuf b_rec;
-  ESC_TRY(b_rec.alloc(five ? sizeof(uint4) * (size_t)(nnz + 1) : 16));
-  TriLists tl3{off, b_U.as<int32_t>(), offp, b_P.as<int32_t>(), b_rec.as<uint4>(), nullptr};
+  TriLists tl3{off, b_U.as<int32_t>(), offp, b_P.as<int32_t>(), nullptr, nullptr};
 
   // wheel work items: ranks are in degree order, so the large centres are a suffix
   int64_t c0 = n;
@@ -4134,10 +4132,17 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
                                                         b_UL.as<int32_t>()), note_launch());
     tl3.UL = b_UL.as<int32_t>();
   }
+  // the slots' records take the place of the arena, which no later phase uses: 16
+  // bytes per entry are its size, and buffers of their own would be a quarter more
+  // than a graph without triangles needs
+  arena.release(0);
+  uint4* rec = (uint4*)arena.alloc(sizeof(uint4) * (size_t)nnz);
+  if (!rec) return cudaErrorMemoryAllocation;
+  tl3.rec = rec;
   if (five && nnz > 0)
     (k_list_records<<<grid_for(nnz, TPB, sms), TPB, 0, s>>>(g, T, off, b_low.as<uint32_t>(),
                                                           ch > 0 ? b_offl.as<int64_t>() : nullptr, cv.h0,
-                                                          b_rec.as<uint4>()), note_launch());
+                                                          rec), note_launch());
   mark(4, 1, s);
   StreamSet ss_all;
   cudaStream_t s1 = s, s2 = s, s3 = s, s4 = s;
