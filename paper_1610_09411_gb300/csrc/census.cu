@@ -18,6 +18,7 @@
 //   Thm 3 + App. B assembly .................... k_assemble
 #include "common.cuh"
 #include "core.cuh"
+#include "estimate.h"
 #include "internal.h"
 
 #include <algorithm>
@@ -3549,8 +3550,8 @@ static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGra
   return e;
 }
 
-// The dense core: vertices of degree CORE_MIN_DEG or more, at most CORE_CAP of
-// a single graph, in graphs (or unions) of at least CORE_MIN_D diamonds and
+// The dense core: vertices of degree CORE_MIN_DEG (estimate.h) or more, at most CORE_CAP
+// of a single graph, in graphs (or unions) of at least CORE_MIN_D diamonds and
 // CORE_D_PER_ENTRY per adjacency entry.  Below that the sweeps' diamonds cost
 // less than the core's launches and passes over the graph (census, ms, without
 // and with a core): ER(800, 0.15), 8e6 diamonds, 1.69 / 1.73; ER(500, 0.3),
@@ -3561,9 +3562,8 @@ static cudaError_t launch_pairs_grp(bool big, const PairPlan& plan, const DevGra
 // 96: 45.2), the cap does on large graphs (R-MAT 19: 8,192 482 ms, 16,384 383,
 // 32,768 384, 49,152 385; R-MAT 22: 16,384 15.0 s, 32,768 13.0 s); W takes 2 or 4
 // bytes x cap^2.
-static constexpr int CORE_MIN_DEG = 48, CORE_CAP = 32768, CORE_CHUNK_MB = 2048;
+static constexpr int CORE_CAP = 32768;
 static constexpr unsigned long long CORE_MIN_D = 1ull << 24, CORE_D_PER_ENTRY = 160;
-static constexpr size_t CORE_W_BYTES = (size_t)24 << 30;
 
 // App. B's matrices are constants of the pattern catalogue (the embedding
 // counts take the host 0.85 ms): built once per process.

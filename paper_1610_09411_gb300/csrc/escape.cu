@@ -2,6 +2,7 @@
 // points, per-element output and the induced/non-induced conversion tables.
 #include "../../include/escape.h"
 #include "common.cuh"
+#include "estimate.h"
 #include "internal.h"
 
 #include <algorithm>
@@ -591,10 +592,8 @@ escape_status escape_census5_batch(int32_t num_graphs, const int64_t* vtx_offset
   int64_t nnz = h[rows];
   if (nnz > 0 && !col) return ESCAPE_EINVAL;
   // Chunks of consecutive graphs, each counted as one block-diagonal union,
-  // sized so that a chunk's work space stays within about half of the free
-  // device memory (at most 64 GiB): per graph the common-neighbour lists
-  // (36 B per triangle, and 3T <= W), per-entry and per-vertex arrays, and per
-  // union vertex the sweeps' per-CTA counters.
+  // sized so that a chunk's estimated work space (estimate.h) stays within about
+  // half of the free device memory (at most 64 GiB).
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
   double budget = std::min((double)free_b * 0.5, (double)((size_t)64 << 30));
@@ -604,17 +603,12 @@ escape_status escape_census5_batch(int32_t num_graphs, const int64_t* vtx_offset
   int32_t k0 = 0;
   while (k0 < num_graphs) {
     int32_t k1 = k0;
-    double used = 0;
+    esc::ChunkEstimate used;
     while (k1 < num_graphs) {
-      double wedges = 0;
-      for (int64_t r = voff[k1]; r < voff[k1 + 1]; ++r) {
-        double d = (double)(h[r + 1] - h[r]);
-        wedges += d * (d - 1) / 2;
-      }
-      const double nk = (double)(voff[k1 + 1] - voff[k1]), ek = (double)(h[voff[k1 + 1]] - h[voff[k1]]);
-      const double need = 12.0 * wedges + 160.0 * ek + 200.0 * nk + 32.0 * 4 * sms * nk;
-      if (k1 > k0 && used + need > budget) break;
-      used += need;
+      esc::ChunkEstimate more = used;
+      more.add(h, voff[k1], voff[k1 + 1], sms);
+      if (k1 > k0 && more.bytes() > budget) break;
+      used = more;
       ++k1;
     }
     // the chunk's offsets and rows, starting at 0

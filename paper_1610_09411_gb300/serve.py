@@ -45,31 +45,65 @@ def triangle_bound(row_ptr: np.ndarray, col: np.ndarray) -> int:
     return int(per_entry.clip(min=0).sum()) // 6
 
 
+CORE_MIN_DEG = 48                 # least degree of a vertex of the census's dense core
+CORE_W_BYTES = 24 << 30           # a core whose wedge counts would take more is left out
+CORE_CHUNK_BYTES = 2 << 30        # operand blocks of the core at a time
+
+
+def core_bytes(vertices: int, max_deg: int) -> int:
+    """Device bytes, from above, of a dense core of that many vertices: its
+    wedge counts (2 B per pair, 4 B where a degree reaches 2^16), and the
+    operand blocks of one chunk of centres with their bits and the below-core
+    counts."""
+    wide = max_deg >= 65536
+    w = (4 if wide else 2) * vertices * vertices
+    if vertices < 2 or w > CORE_W_BYTES:
+        return 0
+    centre = (min(max_deg, vertices) + 127) ** 2
+    blocks = min(vertices * centre, max(CORE_CHUNK_BYTES, centre))
+    return w + blocks * (25 if wide else 17) // 8
+
+
 def footprint_bytes(n: int, m: int, tri_bound: int | None = None, max_deg: int | None = None,
-                    sms: int = 152, cta_per_sm: int = 2) -> int:
+                    sms: int = 152, cta_per_sm: int = 2, core_vertices: int | None = None) -> int:
     """Conservative device bytes for the census of one graph (n vertices, m
-    edges, at most tri_bound triangles, largest degree max_deg): the CSR and
-    its renamed copy and per-edge arrays; the common-neighbour lists, 3T ids
-    and 6T positions (36 B per triangle); and the sweep scratch: per vertex, 8 B
-    for each persistent CTA of the 4-cycle and 5-cycle sweeps (tagged counters)
-    plus 8 B for the 5-cycle P2 counters and their list, 8 B per CTA slot of
-    the pair sweep's counter arrays; per unit of the largest degree, the
-    per-CTA wheel counters and common-neighbour hash tables.  Without a
-    triangle bound, the lists are charged as if every edge were in max_deg
-    triangles.  Used for admission only; the library's cache of released
-    buffers (up to 8 GiB) and its fixed 8 MiB no-allocation array are not
-    part of it."""
+    edges, at most tri_bound triangles, largest degree max_deg, core_vertices
+    of degree CORE_MIN_DEG or more):
+    - per adjacency entry the resident CSR, the batch's and the library's copy
+      of it and its renamed copies, the reverse slots, the per-edge counts, list
+      offsets, sort keys (later the slots' records) and the core's per-slot arrays;
+    - per triangle 3 ids and 6 positions of the common-neighbour lists and 3
+      ids packed again for the core;
+    - per vertex the per-vertex arrays and item lists and, for every persistent
+      CTA of the sweeps' heavy items, 8 B of tagged counters (pairs, 4-cycles,
+      5-cycles) and 8 B of P2 counters and their list;
+    - per unit of the largest degree the list cursors, wheel counters, hash
+      tables and tasks of those CTAs (a task per 512 wedges of an item, which
+      has no more of them than entries or the degree's square);
+    - the clique pass's bit sets and matrices, of an out-degree of at most
+      sqrt(2 m);
+    - the dense core.
+    Without a triangle bound, the lists are charged as if every edge were in
+    max_deg triangles; without core_vertices, as many are assumed as the edges
+    allow.  Used for admission only; the library's cache of released buffers
+    (up to 8 GiB) and its fixed no-allocation array are not part of it."""
     nnz = 2 * m
     if max_deg is None:
         max_deg = n
     if tri_bound is None:
         tri_bound = m * max(max_deg - 1, 0) // 3
+    if core_vertices is None:
+        core_vertices = min(n, nnz // CORE_MIN_DEG) if max_deg >= CORE_MIN_DEG else 0
     grid = sms * cta_per_sm
-    per_edge = nnz * (4 + 4 + 8 + 8 + 8 + 8 + 8 + 8)      # col x2, rev, T, K4, C4, offsets x2
-    lists = 36 * tri_bound
-    per_vertex = n * 8 * 12
-    sweep = n * (grid * (8 + 8 + 8) + 8 * sms * 4) + max_deg * grid * (8 + 16)
-    return int(per_edge + lists + per_vertex + sweep + (64 << 20))
+    per_edge = nnz * (3 * 4 + 4 + 4 + 8 + 4 + 8 + 8 + 16 + 17 + 20)
+    lists = 48 * tri_bound
+    per_vertex = n * 320
+    sweep = n * (8 * sms + 8 * grid + 16 * sms) + max_deg * (sms * (32 + 8 + 32) + grid * 32)
+    sweep += 32 * sms * min(nnz, max_deg * max_deg) // 512
+    dplus = min(max_deg, int(nnz ** 0.5) + 1)
+    words = dplus // 64 + 2
+    cliques = 8 * 4 * sms * dplus * (max_deg // 64 + 1) + min(8 << 30, sms * dplus * (8 * words + 64))
+    return int(per_edge + lists + per_vertex + sweep + cliques + core_bytes(core_vertices, max_deg) + (64 << 20))
 
 
 @dataclass
@@ -126,7 +160,8 @@ class CensusServer:
             return fut
         m = int(row_ptr[-1]) // 2 if n > 0 else 0
         deg = np.diff(row_ptr) if n > 0 else np.zeros(0, np.int64)
-        need = footprint_bytes(n, m, triangle_bound(row_ptr, col), int(deg.max()) if n > 0 else 0)
+        need = footprint_bytes(n, m, triangle_bound(row_ptr, col), int(deg.max()) if n > 0 else 0,
+                               core_vertices=int((deg >= CORE_MIN_DEG).sum()))
         req = Request(n, row_ptr, col, fut, time.perf_counter(), need)
         req.predicted_s = self.predictor.seconds(host_counts(row_ptr, col))
         if req.bytes > self.budget:
