@@ -3209,19 +3209,19 @@ static constexpr size_t kCacheCap = (size_t)8 << 30;
 
 class BufCache {
  public:
-  void* get(int dev, size_t b, size_t* got) {
+  void* get(int dev, size_t b, size_t most, size_t* got) {
     std::lock_guard<std::mutex> lk(mu_);
     auto& m = free_[dev & 63];
     auto it = m.lower_bound(b);
-    if (it == m.end() || it->first > 2 * b) return nullptr;
+    if (it == m.end() || it->first > most) return nullptr;
     void* p = it->second;
     *got = it->first;
     bytes_[dev & 63] -= it->first;
     m.erase(it);
     return p;
   }
-  void put(int dev, void* p, size_t b) {
-    {
+  void put(int dev, void* p, size_t b, bool hold) {
+    if (!hold || b < DevBuf::HOLD_BYTES) {
       std::lock_guard<std::mutex> lk(mu_);
       if (bytes_[dev & 63] + b <= kCacheCap) {
         free_[dev & 63].emplace(b, p);
@@ -3256,19 +3256,19 @@ static thread_local CacheScope* t_scope = nullptr;
 CacheScope::CacheScope(cudaStream_t st) : s(st), prev(t_scope) { t_scope = this; }
 CacheScope::~CacheScope() {
   cudaStreamSynchronize(s);
-  for (auto& b : pending) buf_cache().put(b.dev, b.p, b.bytes);
+  for (auto& b : pending) buf_cache().put(b.dev, b.p, b.bytes, b.hold);
   t_scope = prev;
 }
 
 void DevBuf::give_back() {
-  if (p) buf_cache().put(dev, p, bytes);
+  if (p) buf_cache().put(dev, p, bytes, hold);
   p = nullptr;
   bytes = 0;
 }
 void DevBuf::release() {
   if (!p) return;
-  if (t_scope) t_scope->pending.push_back({p, bytes, dev});
-  else buf_cache().put(dev, p, bytes);
+  if (t_scope) t_scope->pending.push_back({p, bytes, dev, hold});
+  else buf_cache().put(dev, p, bytes, hold);
   p = nullptr;
   bytes = 0;
 }
@@ -3277,7 +3277,7 @@ cudaError_t DevBuf::alloc(size_t b) {
   b = ((b > 0 ? b : 16) + 255) & ~(size_t)255;
   cudaGetDevice(&dev);
   size_t got = 0;
-  if ((p = buf_cache().get(dev, b, &got)) != nullptr) {
+  if ((p = buf_cache().get(dev, b, hold ? b + b / 8 : 2 * b, &got)) != nullptr) {
     bytes = got;
     return cudaSuccess;
   }
@@ -3615,6 +3615,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   arena.cap = arena_bytes;
 
   DevBuf b_perm, b_rank, b_R, b_C, b_op, b_rev;
+  for (DevBuf* b : {&b_perm, &b_rank, &b_R, &b_C, &b_op, &b_rev}) b->hold = or_out != nullptr;
   ESC_TRY(b_perm.alloc(sizeof(int32_t) * (n + 1)));
   ESC_TRY(b_rank.alloc(sizeof(int32_t) * (n + 1)));
   ESC_TRY(b_R.alloc(sizeof(int64_t) * (n + 1)));
@@ -3635,6 +3636,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   const int TPB = 256;
   // ---------------- per-element arrays and accumulators
   DevBuf b_T, b_K4e, b_C4e, b_tv, b_C4v, b_K4v, b_acc, b_ctr;
+  for (DevBuf* b : {&b_T, &b_C4e, &b_K4e, &b_tv, &b_C4v, &b_K4v}) b->hold = pe_out != nullptr;
   ESC_TRY(b_T.alloc(sizeof(uint32_t) * (nnz + 1)));
   ESC_TRY(b_K4e.alloc(sizeof(unsigned long long) * (nnz + 1)));
   ESC_TRY(b_C4e.alloc(sizeof(unsigned long long) * (nnz + 1)));

@@ -373,6 +373,7 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
   }
   esc::CacheScope scope(s);                     // ends after the handle's buffers below have been moved or released
   esc::DevBuf b_rp, b_col, b_status;
+  b_rp.hold = b_col.hold = !(flags & ESCAPE_NORMALIZE);
   cudaError_t e = b_rp.alloc(sizeof(int64_t) * (n + 1));
   if (e == cudaSuccess) e = b_col.alloc(sizeof(int32_t) * (nnz > 0 ? nnz : 1));
   if (e == cudaSuccess) e = b_status.alloc(sizeof(unsigned));
@@ -390,6 +391,7 @@ escape_status escape_load_csr(int64_t n, int64_t nnz, const int64_t* row_ptr, co
     esc::DeviceArena arena;
     size_t ab = (size_t)(2 * nnz + 16) * 8 * 3 + (size_t)((2 * nnz) / 4096 + 2) * 256 * 8 * 2 + (1 << 22);
     esc::DevBuf b_arena, nrp, ncol;
+    nrp.hold = ncol.hold = true;
     e = b_arena.alloc(ab);
     if (e == cudaSuccess) {
       arena.base = b_arena.as<char>();

@@ -31,7 +31,10 @@ struct DeviceArena {
 // cudaFree calls each (cudaFree synchronises the device), so released buffers
 // are kept in a per-device cache, up to 8 GiB, and handed to later ones: a
 // request takes the smallest cached buffer that is large enough and at most
-// twice the size.  If cudaMalloc fails, the cache is emptied and the allocation
+// twice the size.  Buffers that a handle keeps for as long as it lives (hold) fit
+// within an eighth, and those of HOLD_BYTES or more go back to the device, not to
+// the cache: a freed graph leaves its memory to the device's other users.
+// If cudaMalloc fails, the cache is emptied and the allocation
 // tried once more.  A buffer released inside a CacheScope goes back when the
 // scope ends, after the scope's stream has drained, so it never changes hands
 // while kernels may still use it; one released outside any scope goes back at
@@ -40,14 +43,17 @@ struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
   int dev = 0;
+  bool hold = false;             // set before alloc
+  static constexpr size_t HOLD_BYTES = (size_t)64 << 20;
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
-  DevBuf(DevBuf&& o) noexcept : p(o.p), bytes(o.bytes), dev(o.dev) { o.p = nullptr; o.bytes = 0; }
+  DevBuf(DevBuf&& o) noexcept : p(o.p), bytes(o.bytes), dev(o.dev), hold(o.hold) { o.p = nullptr; o.bytes = 0; }
   DevBuf& operator=(DevBuf&& o) noexcept {
     std::swap(p, o.p);
     std::swap(bytes, o.bytes);
     std::swap(dev, o.dev);
+    std::swap(hold, o.hold);
     return *this;
   }
   ~DevBuf() { release(); }
@@ -57,7 +63,7 @@ struct DevBuf {
   template <class T> T* as() const { return (T*)p; }
 };
 struct CacheScope {
-  struct Held { void* p; size_t bytes; int dev; };
+  struct Held { void* p; size_t bytes; int dev; bool hold; };
   cudaStream_t s;
   CacheScope* prev;
   std::vector<Held> pending;
