@@ -145,8 +145,10 @@ escape_status escape_per_element(escape_graph* g, uint64_t* tri_e, uint64_t* c4_
                                  uint64_t* c4_v, uint64_t* k4_v, void* stream);
 
 /* Options: keep_per_element (0/1) makes escape_census5 retain the arrays
- * read by escape_per_element; cta_per_sm sets the persistent-CTA count of the
- * sweep kernels (0 = default, 1..8); serial_phases 1 runs every phase on the
+ * read by escape_per_element; cta_per_sm (1..8) sets the persistent CTAs per SM
+ * of the triangle and common-neighbour list kernels and limits those of the 4-
+ * and 5-cycle sweeps, counted in CTAs of 512 threads (0 = default: 2, and as many
+ * as fit); serial_phases 1 runs every phase on the
  * caller's stream one after another, 0 overlaps the independent sweeps on
  * side streams, and a negative value (the default) chooses by size: one after
  * another for graphs of at least 2^24 adjacency entries (2 x edges), where

@@ -14,8 +14,9 @@ The knobs are environment variables the library reads when it plans a census
                       items, larger ones into CTA items (at most 1024)
   ESC_CLQ_WARP_DIN    clique items with d+ <= 32 and at most this many
                       in-neighbours are counted by one warp (at most 512)
-  ESC_CTA_PER_SM      persistent CTAs per SM of the 4-cycle, 5-cycle and list
-                      sweeps (escape_set_options; 1..4)
+  ESC_CTA_PER_SM      persistent CTAs per SM (escape_set_options; 1..4); applied when
+                      stored, but not searched: without it the cycle sweeps take
+                      as many CTAs as fit, which no value betters
 
 Graphs fall into size classes by their adjacency entries (2m).  tune() runs
 coordinate descent on one representative graph of a class: each knob in turn
@@ -110,7 +111,7 @@ def tune(g, reps: int = 2, knobs=None, log=print) -> dict:
     col = torch.from_numpy(g.col).cuda()
     torch.cuda.synchronize()
     h = esc.escape_load_csr(g.n, rp, col)
-    knobs = knobs or list(KNOBS)
+    knobs = knobs or [k for k in KNOBS if k != "ESC_CTA_PER_SM"]
     try:
         best = {k: KNOBS[k][0] for k in knobs}
         for k in KNOBS:

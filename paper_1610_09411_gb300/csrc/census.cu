@@ -20,6 +20,7 @@
 #include "core.cuh"
 #include "estimate.h"
 #include "internal.h"
+#include "launch.h"
 
 #include <algorithm>
 #include <initializer_list>
@@ -3718,7 +3719,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   mark(1, 0, s);
   int hcap_a = pow2_at_least(2 * dmax);
   size_t smem_a = sizeof(int32_t) * (2 * (size_t)hcap_a) + sizeof(uint32_t) * dmax;
-  int grid_sweep = sms * (cfg.cta_per_sm > 0 ? cfg.cta_per_sm : 1);
+  int grid_sweep = sms * (cfg.cta_per_sm > 0 ? cfg.cta_per_sm : 2);
   if (nsmall > 0)
     (k_tri_small<<<grid_for(nsmall * 32, TPB, sms), TPB, 0, s>>>(g, b_small.as<int32_t>(), nsmall, T, acc_rep),
      note_launch());
@@ -4171,12 +4172,14 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   mark(6, 1, s3);
   // pairs (Thms 11, 12); 16-bit counters when no degree reaches 2^16 (then no W(i,j) can)
   mark(5, 0, s);
-  // CTAs that fit the device at once, at most one per item
-  auto fill = [&](const void* k, int threads, size_t smem, int64_t items, unsigned* grid) -> cudaError_t {
+  // CTAs that fit the device at once, at most one per item (launch.h)
+  const int cta = cfg.cta_per_sm;
+  auto fill = [&](const void* k, int threads, size_t smem, int64_t items, unsigned* grid,
+                  int cta_per_sm = 0) -> cudaError_t {
     ESC_TRY(allow_max_smem(k, smem_optin));
     int per_sm = 1;
     ESC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem));
-    *grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, items);
+    *grid = persistent_grid(per_sm, threads, cta_per_sm, sms, items);
     return cudaSuccess;
   };
   const size_t sm_light = sizeof(uint32_t) << IT_LIGHT_LOG, sm_mid = sizeof(uint32_t) << IT_MID_LOG,
@@ -4267,21 +4270,21 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
          note_launch());
     }
     if (cnt4[1] > 0 && direct) {
-      ESC_TRY(fill((const void*)k_cycles4_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt4[1], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles4_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt4[1], &grid_i, cta));
       (k_cycles4_direct<<<grid_i, IT_MEDIUM_THREADS, sm_direct, s2>>>(gd, l4 + n, (int64_t)cnt4[1], q4 + 1, lc, C4e,
                                                                     accs), note_launch());
     } else if (cnt4[1] > 0) {
-      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt4[1], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt4[1], &grid_i, cta));
       (k_cycles4_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s2>>>(
            g, l4 + n, (int64_t)cnt4[1], q4 + 1, cb, IT_MEDIUM_LOG, C4e, accs, d_status), note_launch());
     }
     if (cnt4[9] > 0) {
-      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt4[9], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt4[9], &grid_i, cta));
       (k_cycles4_hash<IT_MID_THREADS><<<grid_i, IT_MID_THREADS, sm_mid, s2>>>(
            g, l4 + 3 * n, (int64_t)cnt4[9], il4.cnt + 11, cb, IT_MID_LOG, C4e, accs, d_status), note_launch());
     }
     if (cnt4[0] > 0) {
-      ESC_TRY(fill((const void*)k_cycles4_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)cnt4[0], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles4_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, sm_light, (int64_t)cnt4[0], &grid_i, cta));
       (k_cycles4_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, sm_light, s2>>>(
            g, l4, (int64_t)cnt4[0], q4 + 0, cb, IT_LIGHT_LOG, C4e, accs, d_status), note_launch());
     }
@@ -4307,21 +4310,21 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
                                                     win5_words), note_launch());
     }
     if (cnt5[1] > 0 && direct) {
-      ESC_TRY(fill((const void*)k_cycles5_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt5[1], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles5_direct, IT_MEDIUM_THREADS, sm_direct, (int64_t)cnt5[1], &grid_i, cta));
       (k_cycles5_direct<<<grid_i, IT_MEDIUM_THREADS, sm_direct, s4>>>(gd, l5 + n, (int64_t)cnt5[1], q5 + 1, lc, accs),
        note_launch());
     } else if (cnt5[1] > 0) {                   // two tables of half the size
-      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt5[1], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MEDIUM_THREADS>, IT_MEDIUM_THREADS, sm_medium, (int64_t)cnt5[1], &grid_i, cta));
       (k_cycles5_hash<IT_MEDIUM_THREADS><<<grid_i, IT_MEDIUM_THREADS, sm_medium, s4>>>(
            g, l5 + n, (int64_t)cnt5[1], q5 + 1, cb, IT_MEDIUM_LOG - 1, accs, d_status), note_launch());
     }
     if (cnt5[9] > 0) {
-      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt5[9], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_MID_THREADS>, IT_MID_THREADS, sm_mid, (int64_t)cnt5[9], &grid_i, cta));
       (k_cycles5_hash<IT_MID_THREADS><<<grid_i, IT_MID_THREADS, sm_mid, s4>>>(
            g, l5 + 3 * n, (int64_t)cnt5[9], il5.cnt + 11, cb, IT_MID_LOG - 1, accs, d_status), note_launch());
     }
     if (cnt5[0] > 0) {
-      ESC_TRY(fill((const void*)k_cycles5_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, 2 * sm_light, (int64_t)cnt5[0], &grid_i));
+      ESC_TRY(fill((const void*)k_cycles5_hash<IT_LIGHT_THREADS>, IT_LIGHT_THREADS, 2 * sm_light, (int64_t)cnt5[0], &grid_i, cta));
       (k_cycles5_hash<IT_LIGHT_THREADS><<<grid_i, IT_LIGHT_THREADS, 2 * sm_light, s4>>>(
            g, l5, (int64_t)cnt5[0], q5 + 0, cb, IT_LIGHT_LOG, accs, d_status), note_launch());
     }

@@ -17,7 +17,7 @@ struct escape_graph {
   const int64_t* d_rp = nullptr;
   const int32_t* d_col = nullptr;
   int device = 0, sms = 1;
-  int keep_pe = 0, cta_per_sm = 2, serial = -1;   // serial: 1 on, 0 off, -1 by graph size
+  int keep_pe = 0, cta_per_sm = 0, serial = -1;   // serial: 1 on, 0 off, -1 by graph size
   bool has_pe = false;
   esc::PerElement pe;
   esc::Oriented ori;
@@ -438,7 +438,7 @@ escape_status escape_graph_info(const escape_graph* g, int64_t* n, int64_t* m) {
 escape_status escape_set_options(escape_graph* g, int keep_per_element, int cta_per_sm, int serial_phases) {
   if (!g || cta_per_sm < 0 || cta_per_sm > 8) return ESCAPE_EINVAL;
   g->keep_pe = keep_per_element ? 1 : 0;
-  g->cta_per_sm = cta_per_sm ? cta_per_sm : 2;
+  g->cta_per_sm = cta_per_sm;
   g->serial = serial_phases < 0 ? -1 : (serial_phases ? 1 : 0);
   return ESCAPE_OK;
 }
@@ -542,7 +542,6 @@ static escape_status batch_chunk(int32_t num_graphs, const int64_t* voff_h, cons
   if (st == ESCAPE_OK) {
     esc::CensusConfig cfg;
     cfg.sms = sms;
-    cfg.cta_per_sm = 2;
     cfg.d_vtx_offsets = d_voff;
     cfg.num_graphs = num_graphs;
     e = esc::run_census(d_rp, d_col, rows, nnz, cfg, d_out, d_status, nullptr, nullptr, s);

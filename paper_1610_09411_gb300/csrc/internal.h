@@ -127,7 +127,7 @@ struct CensusTimings {
 // cache (allocated inside, sized from the graph).
 struct CensusConfig {
   int sms = 0;                    // SM count of the device
-  int cta_per_sm = 2;             // persistent CTAs per SM for the sweep kernels
+  int cta_per_sm = 0;             // persistent 512-thread CTAs per SM as the caller set them (0: default, see launch.h)
   bool keep_per_element = false;
   bool serial_phases = false;     // run every phase on the caller's stream, one after another
   bool four_only = false;         // 3- and 4-vertex counts only: skip the lists, pairs, wheels and 5-cycles
