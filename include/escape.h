@@ -200,8 +200,8 @@ escape_status escape_last_basis_counts(const escape_graph* g, escape_u128* out);
  *             [0, row_ptr[n]] or decreasing, are skipped and give EINVAL
  *   c4_v      DEVICE uint64[n] output: 4-cycles through each vertex
  *   c4_total  DEVICE uint64[1] output: number of 4-cycles
- * Work space is one fixed device array of ESCAPE_NOALLOC_MAX_N x 64 words
- * (8 MiB) inside the library, shared by every call: calls whose GPU work
+ * Work space is one fixed device array of 2 x ESCAPE_NOALLOC_MAX_N + 64 words
+ * (256 KiB) inside the library, shared by every call: calls whose GPU work
  * overlaps (on different streams or threads) race and must be serialised by
  * the caller.  Each call sets up the work space and clears the outputs before
  * counting.  The array takes its device memory when the library's device

@@ -36,11 +36,11 @@ namespace {
 constexpr int64_t NA_MAX_N = ESCAPE_NOALLOC_MAX_N;  // vertices
 constexpr int NA_LIGHT_DEG = 32, NA_LIGHT_WARPS = 8, NA_LIGHT_LOG = 11, NA_HEAVY_THREADS = 1024;
 constexpr int NA_ILP = 4, NA_PIECE = 256, NA_LONG = 128, NA_HUB_DEG = 256;
-// Work space shared by every call on this device (8 MiB reserved): a header of
-// 64 words (heavy items, queue, status), the order keys and the list of heavy
+// Work space shared by every call on this device (256 KiB): a header of 64
+// words (heavy items, queue, status), the order keys and the list of heavy
 // vertices: those of more than NA_HUB_DEG neighbours from the front, so that
 // they are taken first, the others from the back.
-constexpr int64_t NA_WORDS = (int64_t)64 * NA_MAX_N + 64;
+constexpr int64_t NA_WORDS = 64 + 2 * NA_MAX_N;
 static __device__ __align__(256) unsigned int g_noalloc_scratch[NA_WORDS];
 struct NaSpace {
   unsigned int *hubs, *queue, *status, *others, *key;

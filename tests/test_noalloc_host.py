@@ -100,3 +100,10 @@ def test_an_error_behind_queued_kernels_is_returned_after_they_end(lib, kind, at
     status, trace = _call(lib, kind, at)
     assert status == 3                          # ECUDA
     assert "S" in trace[max(trace.rfind(c) for c in "KX"):]
+
+
+def test_reserved_device_memory(tmp_path):
+    """The header, an order key and a list entry per vertex; nothing unused."""
+    out = _nvcc("-Xptxas", "-v", "-c", SRC, "-o", str(tmp_path / "noalloc.o"))
+    gmem = [int(x) for x in re.findall(r"(\d+) bytes gmem", out)]
+    assert gmem and max(gmem) <= 4 * (64 + 2 * 32768) + 1024
