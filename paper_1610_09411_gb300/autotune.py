@@ -20,8 +20,8 @@ The knobs are environment variables the library reads when it plans a census
 
 Graphs fall into size classes by their adjacency entries (2m).  tune() runs
 coordinate descent on one representative graph of a class: each knob in turn
-over its values, keeping the fastest (CUDA-event time of the census, best of
-`reps`), and stores {class: {knob: value, "ms": best}} in tuning.json beside
+over its values, keeping one that is faster by more than 1% (CUDA-event time of
+the census, best of `reps`), and stores {class: {knob: value, "ms": best}} in tuning.json beside
 this file.  apply(nnz) sets the stored knobs of a graph's class in the process
 environment before a census; the bench calls it.
 
@@ -127,7 +127,7 @@ def tune(g, reps: int = 2, knobs=None, log=print) -> dict:
                 ms = _time_census(h, reps)
                 assert esc.escape_census5(h) == ref, "a launch knob changed the counts"
                 log(f"{g.name} {k}={v}: {ms:.2f} ms (best {best_ms:.2f} ms with {best})")
-                if ms < best_ms:
+                if ms < 0.99 * best_ms:            # runs of one setting differ by up to 1%
                     best_ms, best[k] = ms, v
             os.environ[k] = str(best[k])
     finally:
@@ -162,7 +162,7 @@ def main(argv):
         g = representatives()[name]()
         assert size_class(g.nnz) == name, (name, g.nnz)
         knobs = None
-        if name == "huge":        # a census takes ~30 s here: the knobs that move it
+        if name == "huge":        # a census takes 13 s here: the knobs that move it
             knobs = ["ESC_PAIR_WINDOW", "ESC_PAIR_CLUSTER", "ESC_PAIR_SHAPE", "ESC_WHEEL_WARP_MAX"]
         t0 = time.time()
         table[name] = tune(g, reps[name], knobs)
