@@ -45,7 +45,11 @@ WORKLOADS = {
     "serve": "Poisson stream of Chung-Lu (exponent 2.3, mean degree 16) requests, m log-uniform 1e3-5e6, "
              "120 GB admission budget",
 }
-# per-kernel algorithmic bytes: (phase, kernel, description, function of the oracle sums)
+# the method's work per phase in bytes, 4 B per vertex id of the paper's enumeration:
+# (phase, kernel, description, function of the oracle sums).  The kernels read fewer:
+# the diamonds and wheels among the highest ranks are entries of matrix products
+# (csrc/core.cu), for which no id is read, and most counters stay on chip.  So these
+# are rates of work, not of memory traffic, and no fraction of a bandwidth.
 ALG_BYTES = {
     "wheels": ("k_wheels_cta / k_wheels_warp", "4 B x D (one id read per diamond, Thm 11 wheel sweep)",
                lambda s: 4 * s["D"]),
@@ -170,14 +174,19 @@ DIGEST_SECTIONS = {
 def source_digest(kernel: str = "k_pairs") -> str:
     """Digest of what decides a kernel's DRAM traffic: the section of
     census.cu that holds the kernel and its device helpers, the counter struct
-    it uses and every line naming its constants or launch configuration.
-    Edits elsewhere leave it unchanged; any edit of the kernel changes it (and
-    a failed extraction hashes the whole file, which only makes a stored figure
-    look stale)."""
+    it uses and every line naming its constants or launch configuration; for the
+    pair phase also the whole of core.cu, which runs in it.  Edits elsewhere
+    leave it unchanged; any edit of the kernel changes it (and a failed
+    extraction hashes the whole file, which only makes a stored figure look
+    stale)."""
     path = os.path.join(ROOT, "paper_1610_09411_gb300", "csrc", "census.cu")
     with open(path) as f:
         src = f.read()
     h = hashlib.sha256()
+    core = os.path.join(os.path.dirname(path), "core.cu")
+    if kernel == "k_pairs" and os.path.exists(core):
+        with open(core) as f:
+            h.update(f.read().encode())
     spans, keys = DIGEST_SECTIONS.get(kernel, ([(f" {kernel}(", "\n}\n")], (kernel,)))
     spans = spans + [("struct TaggedCounters {", "\n};\n")]
     cut = []
@@ -332,6 +341,46 @@ def census_alg_bytes(g, sums):
              "cc_wheels": 2 * sums["D"], "paths3": dp}
     total = 4 * sum(terms.values()) + 8 * (n + 3 * g.m)
     return total, {k: int(v) for k, v in terms.items()}
+
+
+def dominant_phase(workload: str, sums, avg_phase: dict, alone_phase: dict):
+    """Rate of work of the dominant kernel: the phase with a byte model that takes
+    longest when every phase runs alone (the ranking of the serialised ncu launch
+    list; overlapped spans inflate the side-stream phases)."""
+    cand = [(alone_phase.get(p, 0.0) or avg_phase.get(p, 0.0), p) for p in ALG_BYTES]
+    cand.sort(reverse=True)
+    peak, peak_src = measured_peak()
+    for _, phase in cand:
+        kernel, desc, fn = ALG_BYTES[phase]
+        ms = avg_phase.get(phase, 0.0)
+        if sums is None or ms <= 0:
+            continue
+        b = fn(sums)
+        if b is None:
+            continue
+        alone = alone_phase.get(phase, 0.0)
+        return {"bound": "latency of dependent list reads", "achieved": b / (ms / 1000.0) / 1e9, "peak": peak,
+                "unit": "GB/s of the byte model", "frac": None,
+                "traffic": stored_traffic(kernel, workload), "kernel": kernel, "phase_ms": ms,
+                "algorithmic_bytes": b, "bytes_model": desc, "peak_source": f"{peak_src} hbm_gbs",
+                "achieved_alone": (b / (alone / 1000.0) / 1e9) if alone > 0 else None,
+                "note": "work per second, not bandwidth: no id is read for the diamonds inside the dense core; "
+                        "phase_ms is timed with the independent sweeps overlapping on side streams; "
+                        "achieved_alone uses the phase's time when every phase runs alone"}
+    return None
+
+
+def census_work(g, sums, ms_per_step: float):
+    """Rate of work of the whole census in the method's bytes (census_alg_bytes)."""
+    if sums is None:
+        return None
+    b_all, terms = census_alg_bytes(g, sums)
+    return {"bound": "latency of dependent list reads", "achieved": b_all / (ms_per_step / 1000.0) / 1e9,
+            "peak": measured_peak()[0], "unit": "GB/s of the byte model", "frac": None,
+            "algorithmic_bytes": b_all, "terms": terms,
+            "bytes_model": "4 B x (2m + sum_{u->v}(d+u + d+v) + 2(W++ + W+-) + W + 2D + DP) + "
+                           "8 B x (n + 3m); 4-clique and bipyramid terms omitted (lower bound)",
+            "note": "work per second, not bandwidth: no id is read for the diamonds and wheels inside the dense core"}
 
 
 def slowest_rank_ms(total_ms: float, world: int, device: str) -> float:
@@ -590,40 +639,10 @@ def main():
             dist.destroy_process_group()
         return
 
-    # roofline of the dominant kernel: the phase with a byte model that takes
-    # longest when every phase runs alone (the ranking of the serialised ncu
-    # launch list; overlapped spans inflate the side-stream phases)
     sums = oracle_sums(args.workload, g)
     avg_phase = {k: v / args.steps for k, v in phase_tot.items()}
-    roof = None
-    cand = [(alone_phase.get(p, 0.0) or avg_phase.get(p, 0.0), p) for p in ALG_BYTES]
-    cand.sort(reverse=True)
-    peak, peak_src = measured_peak()
-    for _, phase in cand:
-        kernel, desc, fn = ALG_BYTES[phase]
-        ms = avg_phase.get(phase, 0.0)
-        if sums is None or ms <= 0:
-            continue
-        b = fn(sums)
-        if b is None:
-            continue
-        achieved = b / (ms / 1000.0) / 1e9
-        alone = alone_phase.get(phase, 0.0)
-        roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": stored_traffic(kernel, args.workload), "kernel": kernel, "phase_ms": ms,
-                "algorithmic_bytes": b, "bytes_model": desc, "peak_source": f"{peak_src} hbm_gbs",
-                "achieved_alone": (b / (alone / 1000.0) / 1e9) if alone > 0 else None,
-                "note": "phase_ms is timed with the independent sweeps overlapping on side streams; "
-                        "achieved_alone uses the phase's time when every phase runs alone"}
-        break
-    census_roof = None
-    if sums is not None:
-        b_all, terms = census_alg_bytes(g, sums)
-        ach = b_all / (ms_per_step / 1000.0) / 1e9
-        census_roof = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-                       "algorithmic_bytes": b_all, "terms": terms,
-                       "bytes_model": "4 B x (2m + sum_{u->v}(d+u + d+v) + 2(W++ + W+-) + W + 2D + DP) + "
-                                      "8 B x (n + 3m); 4-clique and bipyramid terms omitted (lower bound)"}
+    roof = dominant_phase(args.workload, sums, avg_phase, alone_phase)
+    census_roof = census_work(g, sums, ms_per_step)
     cpu = None if args.no_cpu_baseline else cpu_baseline(args.workload)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
