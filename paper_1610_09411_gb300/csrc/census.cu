@@ -376,6 +376,12 @@ __device__ __forceinline__ uint64_t above_mask(int b) { return ~0ull << ((b + 1)
 // R-MAT 19 149 -> 116 ms, on 96 graphs of up to 2,000 vertices 70 -> 41 ms; with
 // the 4-cliques and N20 of the core taken from its contraction 94 and 28.5 ms).
 // dbp += C(candidates, 2) per edge (directed bipyramids).
+// A bit matrix in global memory (SPLIT false) has one b per lane instead, and the
+// lanes go through the words of their candidates together: in the dense graphs
+// that have such out-degrees they then read the same row c at a time, where an
+// even split reads 32 rows (K_1500, clique phase 3,650 -> 2,110 ms; a lane's
+// candidates without the other lanes' words 3,000 ms).
+template <bool SPLIT>
 __device__ __forceinline__ void k5_row(const uint64_t* B, int W, int RS, int a, CliqueWarp* cw, unsigned long long& k5,
                                        u128& dbp) {
   const int lane = threadIdx.x & 31;
@@ -405,6 +411,28 @@ __device__ __forceinline__ void k5_row(const uint64_t* B, int W, int RS, int a, 
         if (n >= 2) dbp += (unsigned long long)n * (n - 1) / 2;
         else n = 0;                             // a lone candidate closes no 5-clique
       }
+      if (!SPLIT) {                             // the lanes go through the words together
+        const uint64_t* rb = B + (int64_t)b * RS;
+        const int wb0 = (b + 1) >> 6;
+        for (int w = __shfl_sync(0xffffffffu, wb0, 0); w < W; ++w) {   // lane 0 holds the lowest b
+          uint64_t cm = n && w >= wb0 ? ra[w] & rb[w] : 0;
+          if (w == wb0) cm &= above_mask(b);
+          while (cm) {
+            const int c = w * 64 + __ffsll((long long)cm) - 1;
+            cm &= cm - 1;
+            const uint64_t* rc = B + (int64_t)c * RS;
+            int u = (c + 1) >> 6;
+            unsigned part = u < W ? __popcll(ra[u] & rb[u] & rc[u] & above_mask(c)) : 0u;
+            for (++u; u + 4 <= W; u += 4)       // independent loads in flight
+              part += __popcll(ra[u] & rb[u] & rc[u]) + __popcll(ra[u + 1] & rb[u + 1] & rc[u + 1]) +
+                      __popcll(ra[u + 2] & rb[u + 2] & rc[u + 2]) + __popcll(ra[u + 3] & rb[u + 3] & rc[u + 3]);
+            for (; u < W; ++u) part += __popcll(ra[u] & rb[u] & rc[u]);
+            k5 += part;
+          }
+          __syncwarp();
+        }
+        continue;
+      }
       unsigned incl = n;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -417,6 +445,7 @@ __device__ __forceinline__ void k5_row(const uint64_t* B, int W, int RS, int a, 
       }
       total += __shfl_sync(0xffffffffu, incl, 31);
     }
+    if (!SPLIT) continue;
     __syncwarp();
     const unsigned share = (total + 31) / 32, p0 = min(total, lane * share), p1 = min(total, p0 + share);
     if (p0 < p1) {
@@ -698,7 +727,7 @@ __global__ void __launch_bounds__(512, 1) k_clique_large(DevGraph g, const int32
         if (!GLOBAL_B && W <= 4) k5_row_reg<4>(B, W, RS, a, k5x2, la.v[5]);
         else if (!GLOBAL_B && W <= 8) k5_row_reg<8>(B, W, RS, a, k5x2, la.v[5]);
         else if (!GLOBAL_B && W <= 12) k5_row_reg<12>(B, W, RS, a, k5x2, la.v[5]);
-        else k5_row(B, W, RS, a, cw, k5, la.v[5]);
+        else k5_row<!GLOBAL_B>(B, W, RS, a, cw, k5, la.v[5]);
       }
       la.v[4] += k5 + k5x2 / 2;                 // a lane's sum of two-fold counts is even
     }
