@@ -4053,6 +4053,11 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
   const size_t core_max = (size_t)env_int("ESC_CORE_MAX_MB", 1 << 30) << 20;
   size_t core_held = 0;
   struct Want { DevBuf* b; size_t bytes; };
+  auto no_core = [&] {
+    ch = 0;
+    cv = CoreView{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
+    cbuf = CoreBuffers{};
+  };
   // all of them or none (a buffer given back here has not been used yet)
   auto reserve = [&](std::initializer_list<Want> wants) -> cudaError_t {
     size_t sum = 0;
@@ -4064,9 +4069,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
     for (const Want& w : wants) w.b->give_back();
-    ch = 0;
-    cv = CoreView{n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
-    cbuf = CoreBuffers{};
+    no_core();
     return cudaSuccess;
   };
   const int core_min_d = env_int("ESC_CORE_MIN_D", 0);
@@ -4089,12 +4092,16 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     ESC_TRY(core_layout(g, cv.h0, G == 1, b_cdh.as<int32_t>(), b_cli.as<int32_t>(), b_crow.as<int64_t>(),
                         b_coff.as<int64_t>(), sms, s));
     if (G > 1) {
-      ESC_TRY(core_union(accs.vg, G, cv.h0, ch, b_chl.as<int32_t>(), b_chb.as<int64_t>(), b_cli.as<int32_t>(),
-                         b_crow.as<int64_t>(), b_cwb.as<int64_t>(), arena, sms, s));
-      cudaMemcpyAsync(&wlen, b_cwb.as<int64_t>() + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+      const cudaError_t e = core_union(accs.vg, G, cv.h0, ch, b_chl.as<int32_t>(), b_chb.as<int64_t>(),
+                                       b_cli.as<int32_t>(), b_crow.as<int64_t>(), b_cwb.as<int64_t>(), arena, sms, s);
+      if (e == cudaErrorMemoryAllocation) no_core();   // more graphs than the arena, sized by the entries, has room for
+      else ESC_TRY(e);
     } else {
       wlen = ch * ch;
     }
+  }
+  if (ch > 0) {
+    if (G > 1) cudaMemcpyAsync(&wlen, b_cwb.as<int64_t>() + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     coff.resize(4 * (size_t)(ch + 1));
     cudaMemcpyAsync(coff.data(), b_coff.p, sizeof(int64_t) * 4 * (ch + 1), cudaMemcpyDeviceToHost, s);
     ESC_TRY(cudaStreamSynchronize(s));
@@ -4104,8 +4111,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     cbuf.k4_0 = hR[cv.h0];
     const size_t k4b = sizeof(unsigned long long) * (size_t)(nnz - cbuf.k4_0 + 1);
     if (wb > CORE_W_BYTES || cchunks.max_tiles == 0) {
-      ch = 0;
-      cv.h0 = n;
+      no_core();
     } else {
       ESC_TRY(reserve({{&b_low, sizeof(uint32_t) * (size_t)(nnz + 1)}, {&b_W, wb}, {&b_cblk, core_block_bytes(cchunks)},
                        {&b_ctile, sizeof(int4) * (size_t)cchunks.max_tiles}, {&b_cbits, core_bit_bytes(cchunks)},
