@@ -234,7 +234,7 @@ __global__ void k_tri_large(DevGraph g, const int32_t* items, int64_t nitems, un
 }
 
 // Copy canonical per-edge values to the reverse slot; per-vertex sums.
-__global__ void k_sym_T(DevGraph g, uint32_t* T, unsigned long long* tv) {
+__global__ void k_sym_T(DevGraph g, uint32_t* T) {
   int lane = threadIdx.x & 31;
   int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -3758,7 +3758,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
         g, b_large.as<int32_t>(), nlarge, ctr + 0, T, acc_rep, hcap_a), note_launch());
   }
   if (n > 0) {
-    (k_sym_T<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T, tv), note_launch());
+    (k_sym_T<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T), note_launch());
     (k_vertex_from_edges_T<<<grid_for(n * 32, TPB, sms), TPB, 0, s>>>(g, T, tv), note_launch());
   }
   mark(1, 1, s);
@@ -4191,7 +4191,7 @@ cudaError_t run_census(const int64_t* rp, const int32_t* col, int64_t n, int64_t
     ESC_TRY(ss_all.fork_from(s));
   }
 
-  // wheels (Thm 11): the longest phase, started first
+  // wheels (Thm 11), on the most urgent stream: few CTAs of long items
   mark(6, 0, s3);
   if (five && c0 < n)
     (k_wheels_cta<<<(unsigned)std::min<int64_t>(sms, std::max<int64_t>(nitems_w, 1)), WHEEL_THREADS, smem_w, s3>>>(

@@ -30,17 +30,17 @@
 // times fewer entries than there are diamonds, so the contraction B_c B_c goes
 // to tcgen05 and only its d^2 / 2 entries per centre are touched by scalar code.
 //
-// Measured (GB300): the census of R-MAT scale 19 971 -> 656 ms, of scale 16
-// 57.9 -> 37.4 ms, of Chung-Lu 2.1 n = 262,144 75.9 -> 65.2 ms.
+// Measured (GB300), the census without and with the core: R-MAT scale 19 726 and
+// 380 ms, scale 16 50.6 and 24.2 ms, Chung-Lu 2.1 n = 262,144 53.2 and 39.8 ms.
 //
 // Operands are fp8 (e4m3: 0 and 1 are exact) with fp32 accumulation in tensor
 // memory: every partial sum is a whole number below d, exact in fp32 below 2^24
 // (a core of CORE_W_BYTES has d below 2^17; the epilogue reads up to 2^23).  The
 // tests put odd sums of up to 65,000, reached in odd steps, through it.
-// k_core_build writes
-// B_c once as blocks of 128 rows x 128 bytes in the 128-byte-swizzled K-major
-// layout the tensor cores read, 16 KB contiguous, so that a plain bulk copy
-// (cp.async.bulk) moves an operand block to shared memory without a tensor map.
+// k_core_build writes B_c once as blocks of 128 rows x 128 bytes in the
+// 128-byte-swizzled K-major layout the tensor cores read, 16 KB contiguous, so
+// that a plain bulk copy (cp.async.bulk) moves an operand block to shared memory
+// without a tensor map.
 #include "core.cuh"
 
 #include <algorithm>
@@ -396,7 +396,9 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // centres of R-MAT 19 (3.3e13 multiply-adds in its triangle's tiles) take 42 ms
 // and are bound by the scattered sectors of W (512 MB, beyond L2) that the
 // entries read, not by the MMAs; the adjacency bits, N20 and the 4-clique sums
-// cost 4 ms of it and save the clique pass 22 ms.
+// cost 4 ms of it and save the clique pass 22 ms.  On R-MAT 22, with 32-bit
+// counts, the contraction reads 3.54 TB in 0.62 s (5.7 TB/s, 0.84 of the measured
+// copy rate).
 template <typename WT> struct CoreSum { typedef uint32_t type; };   // 32 terms below 2^18
 template <> struct CoreSum<uint32_t> { typedef unsigned long long type; };
 // barrier of the eight reading warps; true when ok holds on every thread
@@ -709,8 +711,7 @@ static cudaError_t core_run_as(const DevGraph& g, const CoreView& cv, const uint
                                const CoreBuffers& cb, const AccSet& acc, unsigned* status, int sms, int smem_optin,
                                cudaStream_t s) {
   const int64_t h = g.n - cv.h0;
-  const int64_t *rb = off, *blk = off + (h + 1), *til = off + 2 * (h + 1), *tri = off + 3 * (h + 1);
-  (void)blk;
+  const int64_t *rb = off, *til = off + 2 * (h + 1), *tri = off + 3 * (h + 1);
   const int bit_words = (int)ck.max_row_blocks * 4;
   const size_t smem_b = sizeof(uint32_t) * 8 * (size_t)bit_words;
   cudaError_t e = cudaFuncSetAttribute((const void*)k_core_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
