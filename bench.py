@@ -359,12 +359,16 @@ def dominant_phase(workload: str, sums, avg_phase: dict, alone_phase: dict):
         if b is None:
             continue
         alone = alone_phase.get(phase, 0.0)
+        traffic = stored_traffic(kernel, workload)
+        dram = traffic / ((alone or ms) / 1000.0) / 1e9 if traffic else None
         return {"bound": "latency of dependent list reads", "achieved": b / (ms / 1000.0) / 1e9, "peak": peak,
                 "unit": "GB/s of the byte model", "frac": None,
-                "traffic": stored_traffic(kernel, workload), "kernel": kernel, "phase_ms": ms,
+                "traffic": traffic, "traffic_gbs": dram, "traffic_frac": dram / peak if dram else None,
+                "kernel": kernel, "phase_ms": ms,
                 "algorithmic_bytes": b, "bytes_model": desc, "peak_source": f"{peak_src} hbm_gbs",
                 "achieved_alone": (b / (alone / 1000.0) / 1e9) if alone > 0 else None,
-                "note": "work per second, not bandwidth: no id is read for the diamonds inside the dense core; "
+                "note": "achieved is work per second, not bandwidth: no id is read for the diamonds inside the dense "
+                        "core; traffic_gbs is the DRAM traffic of the stored ncu capture over the phase's time; "
                         "phase_ms is timed with the independent sweeps overlapping on side streams; "
                         "achieved_alone uses the phase's time when every phase runs alone"}
     return None
