@@ -260,7 +260,7 @@ escape_status escape_census5_finish(escape_graph* g, const escape_part* total, e
 /* Number of meaningful entries of escape_part.sums. */
 int escape_part_sum_count(void);
 
-/* Frees a handle (NULL: no-op).  Its device buffers of 64 MiB or more are freed,
+/* Frees a handle (NULL: no-op).  Its device buffers of 128 MiB or more are freed,
  * the smaller ones join the kept ones described at escape_census5. */
 void escape_free(escape_graph* g);
 

@@ -22,22 +22,23 @@ class ChunkEstimate {
  public:
   // graph of the rows [r0, r1) of rp
   void add(const int64_t* rp, int64_t r0, int64_t r1, int sms) {
-    double wedges = 0, sq = 0, biggest = 0, top = 0, cores = 0;
+    // whole numbers without a branch, for the compiler's vectors: a batch has many rows
+    uint64_t wedges2 = 0, sq = 0, cores = 0;
+    uint32_t top = 0;
     for (int64_t r = r0; r < r1; ++r) {
-      const double d = (double)(rp[r + 1] - rp[r]);
-      wedges += d * (d - 1) / 2;
+      const uint32_t d = (uint32_t)(rp[r + 1] - rp[r]);
+      const uint64_t in = d >= (uint32_t)CORE_MIN_DEG ? ~0ull : 0ull;
+      wedges2 += (uint64_t)d * (d - 1u);        // d = 0: 0 x (2^32 - 1)
+      sq += ((uint64_t)(d + 127u) * (d + 127u)) & in;
+      cores -= in;
       top = std::max(top, d);
-      if (d >= CORE_MIN_DEG) {
-        cores += 1;
-        sq += (d + 127) * (d + 127);
-        biggest = std::max(biggest, (d + 127) * (d + 127));
-      }
     }
-    sweeps_ += 16.0 * wedges + 160.0 * (double)(rp[r1] - rp[r0]) + (260.0 + 32.0 * 4 * sms) * (double)(r1 - r0);
-    w_ += 4.0 * cores * cores;
+    const double big = (double)top + 127;
+    sweeps_ += 8.0 * (double)wedges2 + 160.0 * (double)(rp[r1] - rp[r0]) + (260.0 + 32.0 * 4 * sms) * (double)(r1 - r0);
+    w_ += 4.0 * (double)cores * (double)cores;
     wide_ = wide_ || top >= 65536;
-    blocks_ += sq;
-    block_ = std::max(block_, biggest);
+    blocks_ += (double)sq;
+    if (cores) block_ = std::max(block_, big * big);
   }
   double bytes() const {
     const double w = wide_ ? w_ : w_ / 2;

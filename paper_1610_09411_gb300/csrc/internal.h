@@ -44,7 +44,7 @@ struct DevBuf {
   size_t bytes = 0;
   int dev = 0;
   bool hold = false;             // set before alloc
-  static constexpr size_t HOLD_BYTES = (size_t)64 << 20;
+  static constexpr size_t HOLD_BYTES = (size_t)128 << 20;
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;

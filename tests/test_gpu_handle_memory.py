@@ -31,33 +31,33 @@ def free():
 MB = 1 << 20
 """
 SCRIPTS = {
-    # rows of 40 MB, entries of 80 MB
+    # rows of 80 MB, entries of 160 MB
     "loaded": """
-g = ring(5000000, 4)
+g = ring(10000000, 4)
 before = free()
 h = esc.escape_load_csr(g.n, g.row_ptr, g.col)
-assert before - free() >= 110 * MB
+assert before - free() >= 220 * MB
 esc.escape_free(h)
-assert before - free() <= 45 * MB, (before - free()) / MB
+assert before - free() <= 90 * MB, (before - free()) / MB
 """,
-    # T 80, C4 160, K4 160, renamed entries 80, reverse slots 160 and the loaded entries 80 MB
+    # T 160, C4 320, K4 320, renamed entries 160, reverse slots 320 and the loaded entries 160 MB
     "elements": """
-g = ring(5000000, 4)
+g = ring(10000000, 4)
 h = esc.escape_load_csr(g.n, g.row_ptr, g.col)
 esc.escape_set_options(h, keep_per_element=True)
 esc.escape_census5(h)
 held = free()
 esc.escape_free(h)
-assert free() - held >= 680 * MB, (free() - held) / MB
+assert free() - held >= 1360 * MB, (free() - held) / MB
 """,
     # raw entries of twice the size are not part of the handle
     "normalised": """
-g = ring(5000000, 4)
+g = ring(10000000, 4)
 before = free()
 h = esc.escape_load_csr(g.n, g.row_ptr, g.col, flags=esc.ESCAPE_NORMALIZE)
 held = free()
 esc.escape_free(h)
-assert free() - held >= 76 * MB, (free() - held) / MB
+assert free() - held >= 152 * MB, (free() - held) / MB
 """,
     # a kept buffer of 60 MB is not taken for 32 MB of entries
     "tight": """
